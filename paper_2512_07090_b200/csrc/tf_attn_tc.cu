@@ -6,7 +6,7 @@
 // two query heads of one KV group (then both tiles need the same K/V tiles with the same masks).
 // Warp roles:
 //   warps 0-3 / 4-7  softmax group of Q tile 0 / 1 (thread r owns row r of its tile)
-//   warp 8           issues every tcgen05.mma (one lane)
+//   warp 8           issues every tcgen05.mma (the whole warp runs the loop, one elected lane issues)
 //   warp 9           TMA producer: K and V tiles of 128 keys into a 4-slot ring (one lane)
 //   warps 10-11      idle; they complete the warpgroup whose registers go to the softmax groups
 // The query rows are gathered (they are scattered in the sequence) into shared memory in the
@@ -373,7 +373,8 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
         }
     } else if (warp == kMmaWarp) {
         // ================================ MMA issuer ==================================================
-        if (lane == 0) {
+        {
+            const uint32_t lead = elect_one();
             auto slot_of = [&](int j, int kv) { return (2 * (j - J0) + kv) % kStages; };
             auto par_of = [&](int j, int kv) { return ((2 * (j - J0) + kv) / kStages) & 1; };
             auto active = [&](int i, int j) { return j >= jb[i] && j < je[i]; };
@@ -383,16 +384,16 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) {
                     const uint32_t off = (kk >> 2) * kHalfBytes + (kk & 3) * 32;
-                    mma_ss(tmem + i * 128, desc_kmajor(qaddr + off), desc_kmajor(kaddr + off), kIdescQK, kk > 0);
+                    mma_ss(tmem + i * 128, desc_kmajor(qaddr + off), desc_kmajor(kaddr + off), kIdescQK, kk > 0, lead);
                 }
-                mma_commit(bar_s + 8 * i);
+                mma_commit(bar_s + 8 * i, lead);
             };
             auto issue_pv = [&](int i, int j, bool first) {   // O_i (+)= P_i V_j : 8 steps of 16 keys
                 const uint32_t vaddr = sbase + kOffRing + slot_of(j, 1) * kTileBytes;
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)
                     mma_ts(tmem + 256 + i * 128, tmem + i * 128 + kk * 8, desc_mnmajor(vaddr + kk * 16 * 128, kHalfBytes), kIdescPV,
-                           (!first || kk > 0) ? 1u : 0u);
+                           (!first || kk > 0) ? 1u : 0u, lead);
             };
             mbar_wait(bar_q, 0, abort_flag, p.wait_cycles, p.status, 20);
             int done[kQTiles] = {0, 0};
@@ -402,7 +403,7 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
                     mbar_wait(bar_full + 8 * slot_of(j, 0), par_of(j, 0), abort_flag, p.wait_cycles, p.status, 21);
                     tc_fence_after();
                     issue_qk(j - J0, j);
-                    mma_commit(bar_empty + 8 * slot_of(j, 0));
+                    mma_commit(bar_empty + 8 * slot_of(j, 0), lead);
                 }
                 for (int j = J0; j < J1; ++j) {
                     const int i = (j - J0) & 1;
@@ -411,11 +412,11 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
                     tc_fence_after();
                     issue_pv(i, j, done[i] == 0);
                     ++done[i];
-                    mma_commit(bar_empty + 8 * slot_of(j, 1));
+                    mma_commit(bar_empty + 8 * slot_of(j, 1), lead);
                     if (j + 2 < J1) {
                         mbar_wait(bar_full + 8 * slot_of(j + 2, 0), par_of(j + 2, 0), abort_flag, p.wait_cycles, p.status, 23);
                         issue_qk(i, j + 2);
-                        mma_commit(bar_empty + 8 * slot_of(j + 2, 0));
+                        mma_commit(bar_empty + 8 * slot_of(j + 2, 0), lead);
                     }
                 }
             } else {
@@ -423,7 +424,7 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
             tc_fence_after();
             for (int i = 0; i < kQTiles; ++i)
                 if (active(i, J0)) issue_qk(i, J0);
-            mma_commit(bar_empty + 8 * slot_of(J0, 0));
+            mma_commit(bar_empty + 8 * slot_of(J0, 0), lead);
             for (int j = J0; j < J1; ++j) {
                 mbar_wait(bar_full + 8 * slot_of(j, 1), par_of(j, 1), abort_flag, p.wait_cycles, p.status, 22);
                 if (j + 1 < J1) mbar_wait(bar_full + 8 * slot_of(j + 1, 0), par_of(j + 1, 0), abort_flag, p.wait_cycles, p.status, 23);
@@ -435,13 +436,13 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
                         issue_pv(i, j, done[i] == 0);
                         ++done[i];
                     }
-                    if (i == kQTiles - 1) mma_commit(bar_empty + 8 * slot_of(j, 1));
+                    if (i == kQTiles - 1) mma_commit(bar_empty + 8 * slot_of(j, 1), lead);
                     if (j + 1 < J1 && active(i, j + 1)) issue_qk(i, j + 1);
                 }
-                if (j + 1 < J1) mma_commit(bar_empty + 8 * slot_of(j + 1, 0));
+                if (j + 1 < J1) mma_commit(bar_empty + 8 * slot_of(j + 1, 0), lead);
             }
             }
-            mma_commit(bar_o);
+            mma_commit(bar_o, lead);
         }
     }
     } else {
@@ -720,15 +721,16 @@ attention_tc_single_kernel(const TcParams p, const __grid_constant__ CUtensorMap
             }
         } else {
             // ================================ MMA issuer ==================================================
-            if (lane == 0) {
+            {
+                const uint32_t lead = elect_one();
                 auto issue_qk = [&]() {           // S = Q K_j^T : 8 steps of 16 dims
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk) {
                         const uint32_t off = (kk >> 2) * kHalfBytes + (kk & 3) * 32;
-                        mma_ss(tmem, desc_kmajor(sbase + kOffQ1 + off), desc_kmajor(sbase + kOffK1 + off), kIdescQK, kk > 0);
+                        mma_ss(tmem, desc_kmajor(sbase + kOffQ1 + off), desc_kmajor(sbase + kOffK1 + off), kIdescQK, kk > 0, lead);
                     }
-                    mma_commit(bar_s);
-                    mma_commit(bar_ek);
+                    mma_commit(bar_s, lead);
+                    mma_commit(bar_ek, lead);
                 };
                 mbar_wait(bar_q, 0, abort_flag, p.wait_cycles, p.status, 20);
                 mbar_wait(bar_fk, 0, abort_flag, p.wait_cycles, p.status, 21);
@@ -742,15 +744,15 @@ attention_tc_single_kernel(const TcParams p, const __grid_constant__ CUtensorMap
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk)    // O (+)= P V_j : 8 steps of 16 keys
                         mma_ts(tmem + 128, tmem + kk * 8, desc_mnmajor(sbase + kOffV1 + kk * 16 * 128, kHalfBytes), kIdescPV,
-                               (n > 0 || kk > 0) ? 1u : 0u);
-                    mma_commit(bar_ev);
+                               (n > 0 || kk > 0) ? 1u : 0u, lead);
+                    mma_commit(bar_ev, lead);
                     if (j + 1 < J1) {
                         mbar_wait(bar_fk, (n + 1) & 1, abort_flag, p.wait_cycles, p.status, 23);
                         tc_fence_after();
                         issue_qk();
                     }
                 }
-                mma_commit(bar_o);
+                mma_commit(bar_o, lead);
             }
         }
     } else {

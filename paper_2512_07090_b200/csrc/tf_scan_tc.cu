@@ -319,8 +319,8 @@ kv_stats_gram1_kernel(const Gram1Params p, const __grid_constant__ CUtensorMap m
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)         // 16 tokens per step
             mma_ss(tmem + 16 * (kk & 1), desc_mnmajor(xa + kk * 16 * 128, kHalf),
-                   desc_kmajor(bt + (kk >> 2) * (16 * 128) + (kk & 3) * 32), kIdescAgg, kk > 1);
-        mma_commit(bar_mma);
+                   desc_kmajor(bt + (kk >> 2) * (16 * 128) + (kk & 3) * 32), kIdescAgg, kk > 1, 1u);
+        mma_commit(bar_mma, 1u);
     }
     wait_bar(bar_mma, mma_phase, abort_flag, p.wait_cycles, p.status, 101); mma_phase ^= 1;
     tc_fence_after();
@@ -365,9 +365,9 @@ kv_stats_gram1_kernel(const Gram1Params p, const __grid_constant__ CUtensorMap m
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) {   // 16 dims per step; B = rows 64 hh .. 64 hh + 63 of the same tile
                 const uint32_t off = (kk >> 2) * kHalf + (kk & 3) * 32;
-                mma_ss(tmem, desc_kmajor(xa + off), desc_kmajor(xa + hh * (64 * 128) + off), kIdescG64, kk > 0);
+                mma_ss(tmem, desc_kmajor(xa + off), desc_kmajor(xa + hh * (64 * 128) + off), kIdescG64, kk > 0, 1u);
             }
-            mma_commit(bar_mma);
+            mma_commit(bar_mma, 1u);
         }
         wait_bar(bar_mma, mma_phase, abort_flag, p.wait_cycles, p.status, 102 + hh); mma_phase ^= 1;
         tc_fence_after();
@@ -407,8 +407,8 @@ kv_stats_gram1_kernel(const Gram1Params p, const __grid_constant__ CUtensorMap m
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)             // 16 dims per step; two interleaved accumulator chains
             mma_ss(tmem + 16 * (kk & 1), desc_kmajor(xa + (kk >> 2) * kHalf + (kk & 3) * 32),
-                   desc_kmajor(bt + (kk >> 2) * (16 * 128) + (kk & 3) * 32), kIdescU, kk > 1);
-        mma_commit(bar_mma);
+                   desc_kmajor(bt + (kk >> 2) * (16 * 128) + (kk & 3) * 32), kIdescU, kk > 1, 1u);
+        mma_commit(bar_mma, 1u);
     }
     wait_bar(bar_mma, mma_phase, abort_flag, p.wait_cycles, p.status, 104); mma_phase ^= 1;
     tc_fence_after();
@@ -617,9 +617,9 @@ kv_stats_gram_persistent_kernel(const GramPParams pp, const __grid_constant__ CU
         if (tid == 0) {
             tc_fence_after();
             mma_burst<kPBlock, true>(k8, tm_s, x_lo | dlo_mn, dhi, x_lo + (kHalf >> 4) | dlo_k, dhi, kIdescAgg);   // 16 tokens per step
-            mma_commit(bar_small);
+            mma_commit(bar_small, 1u);
             mma_burst<kPBlock, false>(k8, tm_g, x_lo | dlo_k, dhi, x_lo | dlo_k, dhi, kIdescG64);               // 16 dims per step
-            mma_commit(bar_g);
+            mma_commit(bar_g, 1u);
         }
         // ---- look-back requests go out under the products (thread = dim) -------------------------------------------
         const int a0 = c > 0 ? ((c - 1) / kGramAnchorEvery) * kGramAnchorEvery : 0;
@@ -697,7 +697,7 @@ kv_stats_gram_persistent_kernel(const GramPParams pp, const __grid_constant__ CU
         if (tid == 0) {
             tc_fence_after();
             mma_burst<kPBlock, false>(k8, tm_g, x_lo | dlo_k, dhi, x_lo + (64 * 128 >> 4) | dlo_k, dhi, kIdescG80);
-            mma_commit(bar_g);
+            mma_commit(bar_g, 1u);
         }
         wait_bar_parked(bar_g, 1, abort_flag, p.wait_cycles, p.status, 203);
         tc_fence_after();

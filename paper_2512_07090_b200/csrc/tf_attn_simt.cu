@@ -1,17 +1,29 @@
 // Step a5 on CUDA cores: causal (optionally windowed) attention for retained tokens, any dtype.
 //
-// This is the path fp32 tensors take (fp32 accuracy rules out the 16-bit tensor-core path) and
-// the A/B reference for the tensor-core kernel.  One warp owns one (retained token, query head):
-// 32 keys at a time, each lane scores one key against the query held in shared memory, the
-// warp runs the online softmax, and each lane accumulates 4 output dims over those 32 keys.
-// The warp also zeroes the output rows of the pruned tokens that lie between its retained token
-// and the previous one (Section 3.2: a skipped token's attention output is zero), so the whole
-// of O is written with no separate clearing pass.
+// This is the path fp32 tensors take (fp32 accuracy rules out the 16-bit tensor-core path) and the A/B reference for the
+// tensor-core kernel.  A CTA of 8 warps owns 16 or 32 consecutive entries of a sequence's retained list for one query
+// head; keys and values go through shared memory in chunks of 64.  A warp owns 4 rows of the tile: lane l scores keys l and
+// l + 32 of a chunk for all of them (keys from shared memory, queries by broadcast), the warp runs the online softmax,
+// and each lane accumulates 4 output dims of its 4 rows over the chunk.  Scores, probabilities and sums are fp32 throughout.
+//   kSplit = 1 (32 rows): all warps work on the same chunk, two CTAs per SM.
+//   kSplit = 2 (16 rows): the two halves of the CTA take alternate chunks of the same rows and are merged at the end: twice
+//                         as many CTAs with half the serial length, for problems that would leave SMs idle.
+// The next chunk's keys are fetched (cp.async) under the P V part, its values under the next Q K part.  Shared-memory reads
+// bound it: per 4 dims 16 wavefronts (a 16-byte broadcast is two) for 8 cycles of multiply-adds in Q K^T, 24 for 16 in P V.
+// A retained row's warp also zeroes the output rows of the pruned tokens before it (Section 3.2: a skipped token's
+// attention output is zero), so the whole of O is written with no separate clearing pass.
+//   One warp per row, a key at a time per lane straight from global memory, took 48 us at 1 x 128 tokens x 32 heads, 392 at
+// 512 and 4700 at 2 x 1024 x 40 heads; this kernel takes 11, 85 and 670.
+#include <algorithm>
+
 #include "tf_common.cuh"
 
 namespace tf {
 
-constexpr int kSimtWarps = 4;
+constexpr int kSimtChunk = 64;         // keys per chunk
+constexpr int kSimtWarps = 8;
+constexpr int kSimtThreads = kSimtWarps * 32;
+constexpr int kSimtRows = 4;           // rows per warp
 
 struct AttnParams {
     const void* Q; const void* K; const void* V; void* O;
@@ -23,116 +35,238 @@ struct AttnParams {
     int retained_only;         // 1: a retained query sees retained tokens' keys / values only
 };
 
-template <typename T> __device__ __forceinline__ float to_f(T v);
-template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
-template <> __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
-template <typename T> __device__ __forceinline__ T from_f(float v);
-template <> __device__ __forceinline__ float from_f<float>(float v) { return v; }
-template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
+template <int kSplit> struct SimtCfg {                                   // kSplit: parts of the CTA with chunks of their own
+    static constexpr int kPartThreads = kSimtThreads / kSplit;
+    static constexpr int kRows = kSimtWarps / kSplit * kSimtRows;
+    static constexpr int kChunkFloats = kSimtChunk * kHeadDim;
+    static constexpr int kOffQ = 2 * kSplit * kChunkFloats;              // [part][K, V] chunks first
+    static constexpr int kOffP = kOffQ + kRows * kHeadDim;               // [warp][row][64]
+    static constexpr int kSmemBytes = (kOffP + kSimtWarps * kSimtRows * kSimtChunk) * 4;
+};
 
+__device__ __forceinline__ void store4(float* p, float a, float b, float c, float d) { *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d); }
+__device__ __forceinline__ void store4(__nv_bfloat16* p, float a, float b, float c, float d) {
+    __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(c, d);
+    *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+}
 // four consecutive elements (16 bytes of fp32, 8 bytes of bf16; the caller's offset is a multiple of four elements)
-__device__ __forceinline__ void load4(const float* p, float (&f)[4]) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(p));
-    f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
-}
-__device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&f)[4]) {
+__device__ __forceinline__ float4 load4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
     const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
-    f[0] = __uint_as_float(v.x << 16); f[1] = __uint_as_float(v.x & 0xffff0000u);
-    f[2] = __uint_as_float(v.y << 16); f[3] = __uint_as_float(v.y & 0xffff0000u);
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
 }
+// four elements from global to shared memory (zeros unless live); fp32: asynchronously
+__device__ __forceinline__ void fetch4(float* dst, const float* src, bool live) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(live ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void fetch4(float* dst, const __nv_bfloat16* src, bool live) {
+    *reinterpret_cast<float4*>(dst) = live ? load4(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+__device__ __forceinline__ void fetch_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void fetch_wait_all_but_one() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
 template <typename T>
 __device__ __forceinline__ void zero_rows(T* Ob, const Strides3& os, int t_lo, int t_hi, int lane) {
-    for (int t = t_lo; t < t_hi; ++t) {
-        T* row = Ob + (long long)t * os.t;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) row[lane * 4 + i] = from_f<T>(0.f);
-    }
+    for (int t = t_lo; t < t_hi; ++t) store4(Ob + (long long)t * os.t + lane * 4, 0.f, 0.f, 0.f, 0.f);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kSimtWarps * 32) attention_simt_kernel(const AttnParams p) {
-    constexpr int EPV = Elem<T>::kPerVec;          // elements per 16-byte vector
-    constexpr int NVEC = kHeadDim / EPV;
-    __shared__ __align__(16) float q_s[kSimtWarps][kHeadDim];
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int slot = blockIdx.x * kSimtWarps + warp;   // index into the retained list
+template <typename T, int kSplit>
+__global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_simt_kernel(const AttnParams p) {
+    using C = SimtCfg<kSplit>;
+    constexpr int R = kSimtRows;
+    extern __shared__ __align__(16) float simt_smem[];
+    grid_dependency_wait();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int part = warp / (kSimtWarps / kSplit), ptid = tid & (C::kPartThreads - 1);
+    const int rgroup = warp & (kSimtWarps / kSplit - 1);
     const int qh = blockIdx.y, b = blockIdx.z;
     const int nk = p.n_kept[b];
-    if (slot >= max(nk, 1)) return;
+    const int slot0 = ((int)gridDim.x - 1 - (int)blockIdx.x) * C::kRows;     // the longest rows first
     const int32_t* kept = p.kept_idx + (size_t)b * p.S;
     T* Ob = reinterpret_cast<T*>(p.O) + (long long)b * p.os.b + (long long)qh * p.os.h;
+    if (nk == 0) {
+        if (slot0 == 0)
+            for (int t = warp; t < p.S; t += kSimtWarps) zero_rows(Ob, p.os, t, t + 1, lane);
+        return;
+    }
+    if (slot0 >= nk) return;
 
-    // rows of pruned tokens around this slot
-    if (nk == 0) { zero_rows(Ob, p.os, 0, p.S, lane); return; }
-    const int t = kept[slot];
-    zero_rows(Ob, p.os, slot == 0 ? 0 : kept[slot - 1] + 1, t, lane);
-    if (slot == nk - 1) zero_rows(Ob, p.os, t + 1, p.S, lane);
-
+    float* const sK = simt_smem + part * 2 * C::kChunkFloats;
+    float* const sV = sK + C::kChunkFloats;
+    float* const sQ = simt_smem + C::kOffQ;
+    float* const sP = simt_smem + C::kOffP + warp * R * kSimtChunk;
     const int kh = qh / (p.Hq / p.Hkv);
-    const T* qrow = reinterpret_cast<const T*>(p.Q) + (long long)b * p.qs.b + (long long)t * p.qs.t + (long long)qh * p.qs.h;
     const T* Kb = reinterpret_cast<const T*>(p.K) + (long long)b * p.ks.b + (long long)kh * p.ks.h;
     const T* Vb = reinterpret_cast<const T*>(p.V) + (long long)b * p.vs.b + (long long)kh * p.vs.h;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) q_s[warp][lane * 4 + i] = to_f<T>(qrow[lane * 4 + i]) * p.scale_log2;
-    __syncwarp();
 
-    // keys are visited by index: token positions, or positions in the retained list (retained_only),
-    // where entry c stands for token kept[c] and the query itself is entry `slot`
-    const int t_min = (p.window > 0) ? max(0, t - p.window + 1) : 0;
-    const int j_hi = p.retained_only ? slot : t;
-    const int j_lo = p.retained_only ? first_kept_at_or_after(kept, slot + 1, t_min) : t_min;
-    float m = -1e30f, lsum = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int j0 = j_lo; j0 <= j_hi; j0 += 32) {
-        const int j = j0 + lane;
-        float s = -1e30f;
-        const int tok = (j <= j_hi) ? (p.retained_only ? kept[j] : j) : 0;
-        if (j <= j_hi) {
-            const T* krow = Kb + (long long)tok * p.ks.t;
-            float d0 = 0.f, d1 = 0.f;
-#pragma unroll 8
-            for (int v = 0; v < NVEC; ++v) {   // eight 16-byte loads in flight per lane: the warp is alone on its row, so
-                                               // memory-level parallelism has to come from inside it
-                float f[EPV];
-                Elem<T>::unpack(ldg16(krow + v * EPV), f);
-                const float* qq = &q_s[warp][v * EPV];
-#pragma unroll
-                for (int e = 0; e < EPV; e += 2) { d0 = fmaf(f[e], qq[e], d0); d1 = fmaf(f[e + 1], qq[e + 1], d1); }
-            }
-            s = d0 + d1;
+    // keys are visited by index: token positions, or positions in the retained list (retained_only), where entry c stands
+    // for token kept[c] and the query itself is its own entry
+    auto first_key = [&](int slot, int t) {
+        const int t_min = p.window > 0 ? max(0, t - p.window + 1) : 0;
+        return p.retained_only ? (t_min > 0 ? first_kept_at_or_after(kept, slot + 1, t_min) : 0) : t_min;
+    };
+    const int s_last = min(slot0 + C::kRows, nk) - 1;
+    const int c_hi = p.retained_only ? s_last : kept[s_last];              // the CTA's last visible key
+    const int ch0 = first_key(slot0, kept[slot0]) / kSimtChunk, ch1 = c_hi / kSimtChunk + 1;
+
+    // one 16-byte piece per thread and step; the pieces of a key row are rotated (XOR) by the row so that lanes reading the
+    // same piece of 8 consecutive rows hit different banks
+    auto fetch = [&](float* dst, const T* base, long long stride, int ch, bool swizzle) {
+#pragma unroll 4
+        for (int i = ptid; i < kSimtChunk * 32; i += C::kPartThreads) {
+            const int row = i >> 5, piece = i & 31, j = ch * kSimtChunk + row;
+            const bool live = j <= c_hi;
+            const long long tok = live ? (p.retained_only ? kept[j] : j) : 0;
+            fetch4(dst + row * kHeadDim + ((swizzle ? piece ^ (row & 7) : piece) << 2), base + tok * stride + piece * 4, live);
         }
-        const float m_new = fmaxf(m, warp_max(s));
-        const float corr = exp2f(m - m_new);
-        const float pj = (j <= j_hi) ? exp2f(s - m_new) : 0.f;
-        lsum = lsum * corr + warp_sum(pj);
+        fetch_commit();
+    };
+    auto part_sync = [&]() {
+        if (kSplit == 1) __syncthreads();
+        else asm volatile("bar.sync %0, %1;" :: "r"(1 + part), "n"(C::kPartThreads) : "memory");
+    };
+    int ch = ch0 + part;
+    if (ch < ch1) { fetch(sK, Kb, p.ks.t, ch, true); fetch(sV, Vb, p.vs.t, ch, false); }
+    for (int i = tid; i < C::kRows * 32; i += kSimtThreads) {
+        const int row = i >> 5, piece = i & 31, slot = slot0 + row;
+        float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (slot < nk)
+            q = load4(reinterpret_cast<const T*>(p.Q) + (long long)b * p.qs.b + (long long)kept[slot] * p.qs.t + (long long)qh * p.qs.h + piece * 4);
+        *reinterpret_cast<float4*>(sQ + row * kHeadDim + piece * 4) = make_float4(q.x * p.scale_log2, q.y * p.scale_log2, q.z * p.scale_log2, q.w * p.scale_log2);
+    }
+    const int row0 = rgroup * R;
+    int lo[R], hi[R], w_lo = 0x7fffffff, w_hi = -1;                     // visible keys of each row (hi < lo: no such row)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] *= corr;
-        const int n_here = min(32, j_hi - j0 + 1);
-        // same order of additions as a plain loop over the block's keys; the value rows of eight keys are requested
-        // together (loads first, products after), not one round trip to memory per key
-        for (int jj0 = 0; jj0 < n_here; jj0 += 8) {
-            float vv[8][4];
+    for (int r = 0; r < R; ++r) {
+        const int slot = slot0 + row0 + r;
+        lo[r] = 0; hi[r] = -1;
+        if (slot < nk) {
+            const int t = kept[slot];
+            lo[r] = first_key(slot, t);
+            hi[r] = p.retained_only ? slot : t;
+            w_lo = min(w_lo, lo[r]); w_hi = max(w_hi, hi[r]);
+        }
+    }
+    __syncthreads();
+
+    float m[R], l[R], acc[R][4];                                          // l: this lane's share of the row's sum
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int vt = __shfl_sync(0xffffffffu, tok, jj0 + u);
-                if (jj0 + u < n_here) load4(Vb + (long long)vt * p.vs.t + lane * 4, vv[u]);
-            }
+    for (int r = 0; r < R; ++r) { m[r] = -1e30f; l[r] = 0.f; acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = 0.f; }
+    for (; ch < ch1; ch += kSplit) {
+        const int j0 = ch * kSimtChunk;
+        const bool mine = w_hi >= j0 && w_lo < j0 + kSimtChunk;            // some row of this warp sees this chunk
+        fetch_wait_all_but_one();
+        part_sync();                                                       // K(ch) is there
+        float s[R][2];
+        if (mine) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const float pw = __shfl_sync(0xffffffffu, pj, jj0 + u);
-                if (jj0 + u < n_here) {
+            for (int r = 0; r < R; ++r) s[r][0] = s[r][1] = 0.f;
+            const float4* k4 = reinterpret_cast<const float4*>(sK) + lane * 32;
+            const float4* q4 = reinterpret_cast<const float4*>(sQ) + row0 * 32;
+#pragma unroll 4
+            for (int d = 0; d < 32; ++d) {
+                const float4 ka = k4[d ^ (lane & 7)], kb = k4[32 * 32 + (d ^ (lane & 7))];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) acc[i] = fmaf(pw, vv[u][i], acc[i]);
+                for (int r = 0; r < R; ++r) {
+                    const float4 q = q4[r * 32 + d];
+                    s[r][0] = fmaf(q.x, ka.x, s[r][0]); s[r][1] = fmaf(q.x, kb.x, s[r][1]);
+                    s[r][0] = fmaf(q.y, ka.y, s[r][0]); s[r][1] = fmaf(q.y, kb.y, s[r][1]);
+                    s[r][0] = fmaf(q.z, ka.z, s[r][0]); s[r][1] = fmaf(q.z, kb.z, s[r][1]);
+                    s[r][0] = fmaf(q.w, ka.w, s[r][0]); s[r][1] = fmaf(q.w, kb.w, s[r][1]);
                 }
             }
         }
-        m = m_new;
-    }
-    const float inv = 1.f / lsum;
-    T* orow = Ob + (long long)t * p.os.t;
+        part_sync();                                                       // K(ch) has been read
+        if (ch + kSplit < ch1) fetch(sK, Kb, p.ks.t, ch + kSplit, true); else fetch_commit();
+        if (mine) {
+            const int ja = j0 + lane, jb = ja + 32;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) orow[lane * 4 + i] = from_f<T>(acc[i] * inv);
+            for (int r = 0; r < R; ++r) {
+                const bool va = ja >= lo[r] && ja <= hi[r], vb = jb >= lo[r] && jb <= hi[r];
+                const float sa = va ? s[r][0] : -1e30f, sb = vb ? s[r][1] : -1e30f;
+                const float m_new = fmaxf(m[r], warp_max(fmaxf(sa, sb)));
+                const float corr = exp2f(m[r] - m_new);
+                const float pa = va ? exp2f(sa - m_new) : 0.f, pb = vb ? exp2f(sb - m_new) : 0.f;
+                m[r] = m_new;
+                l[r] = fmaf(l[r], corr, pa + pb);
+                acc[r][0] *= corr; acc[r][1] *= corr; acc[r][2] *= corr; acc[r][3] *= corr;
+                sP[r * kSimtChunk + lane] = pa;
+                sP[r * kSimtChunk + 32 + lane] = pb;
+            }
+            __syncwarp();
+        }
+        fetch_wait_all_but_one();
+        part_sync();                                                       // V(ch) is there
+        if (mine) {
+            const int jj0 = max(0, w_lo - j0) & ~3, jj1 = min(kSimtChunk, w_hi - j0 + 1);
+            for (int jj = jj0; jj < jj1; jj += 4) {
+                float4 v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = reinterpret_cast<const float4*>(sV)[(jj + u) * 32 + lane];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const float4 w = *reinterpret_cast<const float4*>(sP + r * kSimtChunk + jj);
+                    const float wu[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        acc[r][0] = fmaf(wu[u], v[u].x, acc[r][0]); acc[r][1] = fmaf(wu[u], v[u].y, acc[r][1]);
+                        acc[r][2] = fmaf(wu[u], v[u].z, acc[r][2]); acc[r][3] = fmaf(wu[u], v[u].w, acc[r][3]);
+                    }
+                }
+            }
+            __syncwarp();                                                  // sP is written again in the next chunk
+        }
+        part_sync();                                                       // V(ch) has been read
+        if (ch + kSplit < ch1) fetch(sV, Vb, p.vs.t, ch + kSplit, false); else fetch_commit();
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) l[r] = warp_sum(l[r]);
+    if (kSplit == 2) {      // the second half of the CTA hands its part of every row to the first
+        float* const other = simt_smem + row0 * (kHeadDim + 4);
+        __syncthreads();
+        if (part == 1) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                *reinterpret_cast<float4*>(other + r * (kHeadDim + 4) + lane * 4) = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
+                if (lane == 0) { other[r * (kHeadDim + 4) + kHeadDim] = m[r]; other[r * (kHeadDim + 4) + kHeadDim + 1] = l[r]; }
+            }
+        }
+        __syncthreads();
+        if (part == 1) return;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float* o = other + r * (kHeadDim + 4);
+            const float4 a2 = *reinterpret_cast<const float4*>(o + lane * 4);
+            const float m2 = o[kHeadDim], l2 = o[kHeadDim + 1], mm = fmaxf(m[r], m2), e1 = exp2f(m[r] - mm), e2 = exp2f(m2 - mm);
+            l[r] = fmaf(l[r], e1, l2 * e2);
+            acc[r][0] = fmaf(acc[r][0], e1, a2.x * e2); acc[r][1] = fmaf(acc[r][1], e1, a2.y * e2);
+            acc[r][2] = fmaf(acc[r][2], e1, a2.z * e2); acc[r][3] = fmaf(acc[r][3], e1, a2.w * e2);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int slot = slot0 + row0 + r;
+        if (slot >= nk) break;
+        const int t = kept[slot];
+        const float inv = 1.f / l[r];
+        store4(Ob + (long long)t * p.os.t + lane * 4, acc[r][0] * inv, acc[r][1] * inv, acc[r][2] * inv, acc[r][3] * inv);
+        zero_rows(Ob, p.os, slot == 0 ? 0 : kept[slot - 1] + 1, t, lane);   // pruned rows before this one
+        if (slot == nk - 1) zero_rows(Ob, p.os, t + 1, p.S, lane);
+    }
+}
+
+template <typename T, int kSplit>
+static cudaError_t launch_simt_form(const AttnParams& ap, int batch, int device, cudaStream_t st) {
+    using C = SimtCfg<kSplit>;
+    static bool attr_set_dev[kDeviceFlagSlots] = {};      // function attributes are per device
+    bool& attr_set = attr_set_dev[device >= 0 && device < kDeviceFlagSlots ? device : 0];
+    if (!attr_set) {
+        const cudaError_t e = cudaFuncSetAttribute(attention_simt_kernel<T, kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    return launch_dependent(attention_simt_kernel<T, kSplit>, dim3((unsigned)((ap.S + C::kRows - 1) / C::kRows), (unsigned)ap.Hq, (unsigned)batch),
+                            dim3(kSimtThreads), C::kSmemBytes, st, ap);
 }
 
 cudaError_t launch_attention_simt(tf_ctx* ctx, const tf_shape& s, const tf_filter_params& p,
@@ -151,12 +285,17 @@ cudaError_t launch_attention_simt(tf_ctx* ctx, const tf_shape& s, const tf_filte
     const float scale = s.softmax_scale != 0.f ? s.softmax_scale : 1.f / sqrtf((float)s.head_dim);
     ap.scale_log2 = scale * 1.4426950408889634f;
     ap.kept_idx = kept_idx; ap.n_kept = n_kept;
-    const dim3 grid((unsigned)((s.seq + kSimtWarps - 1) / kSimtWarps), (unsigned)s.n_q_heads, (unsigned)s.batch);
-    if (s.dtype == TF_BF16) attention_simt_kernel<__nv_bfloat16><<<grid, kSimtWarps * 32, 0, st>>>(ap);
-    else                    attention_simt_kernel<float><<<grid, kSimtWarps * 32, 0, st>>>(ap);
+    // Up to two 16-row CTAs per SM the split form wins (us at 1 x 128 x 32 heads, 1 x 256 x 32, 2 x 256 x 32: 11 / 33 / 52
+    // split, 16 / 44 / 45 unsplit), beyond that its second set of chunks costs more than it hides (1 x 768 x 40: 196 / 177).
+    // The number of retained rows is only known on the device: the ratio gives the expected count.
+    const double kept_frac = (p.select_mode == TF_SELECT_RATIO) ? 1.0 - p.prune_ratio : 1.0;
+    const bool split = (double)s.batch * s.n_q_heads * ceil(s.seq * kept_frac / 16.0) <= 2.0 * sm_count();
+    cudaError_t e;
+    if (s.dtype == TF_BF16) e = split ? launch_simt_form<__nv_bfloat16, 2>(ap, s.batch, ctx->device, st) : launch_simt_form<__nv_bfloat16, 1>(ap, s.batch, ctx->device, st);
+    else                    e = split ? launch_simt_form<float, 2>(ap, s.batch, ctx->device, st) : launch_simt_form<float, 1>(ap, s.batch, ctx->device, st);
     ctx->launches += 1;
     ctx->last_attention_kernel = TF_KERNEL_ATTN_SIMT;
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace tf

@@ -118,6 +118,13 @@ __device__ __forceinline__ float key_score(unsigned int k) {
 // ---- host-side launch bookkeeping --------------------------------------------------------------
 struct Strides3 { long long b, t, h; };
 
+// SMs of the current device
+inline int sm_count() {
+    int sms = 148, dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
 // Launch a kernel that may start while the kernel before it on the stream drains (programmatic
 // dependent launch).  Such a kernel executes grid_dependency_wait() before it touches global memory;
 // until then only its launch and set-up overlap with its predecessor.

@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(kScanThreads, 4) kv_stats_kernel(const ScanPar
     __shared__ unsigned int s_ticket, s_tag;
 
     const int tid = threadIdx.x, g = tid >> 3, l = tid & 7;
+    grid_dependency_wait();
     if (tid == 0) {
         s_tag = scan_launch_tag(p.counters);
         s_ticket = scan_draw_ticket(p.counters);
@@ -356,16 +357,11 @@ cudaError_t launch_kv_stats(tf_ctx* ctx, const tf_shape& s, const tf_filter_para
     sp.max_polls = ctx_max_polls(ctx);
 
     const dim3 grid((unsigned)tiles), block(kScanThreads);
-    if (s.dtype == TF_BF16) {
-        if (ema) kv_stats_kernel<__nv_bfloat16, true><<<grid, block, 0, st>>>(sp);
-        else     kv_stats_kernel<__nv_bfloat16, false><<<grid, block, 0, st>>>(sp);
-    } else {
-        if (ema) kv_stats_kernel<float, true><<<grid, block, 0, st>>>(sp);
-        else     kv_stats_kernel<float, false><<<grid, block, 0, st>>>(sp);
-    }
+    auto kernel = s.dtype == TF_BF16 ? (ema ? kv_stats_kernel<__nv_bfloat16, true> : kv_stats_kernel<__nv_bfloat16, false>)
+                                     : (ema ? kv_stats_kernel<float, true> : kv_stats_kernel<float, false>);
+    const cudaError_t e = launch_dependent(kernel, grid, block, 0, st, sp);
     ctx->launches += 1;
     ctx->last_scan_kernel = TF_KERNEL_SCAN_PLAIN;
-    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) ws->needs_clear = true;   // whatever the launch left behind is cleared before the next one
     return e;
 }

@@ -816,8 +816,7 @@ cudaError_t launch_kv_stats_gram(tf_ctx* ctx, const tf_shape& s, const tf_filter
     gp.wait_cycles = ctx_wait_cycles(ctx);
     gp.counters = reinterpret_cast<unsigned int*>(base);
     gp.n_work = (unsigned int)(2 * tiles);
-    int sms = 148;
-    { int dev = 0; if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev); }
+    const int sms = sm_count();
     // the persistent form pays its set-up once per SM and wins once every worker sees several tiles (measured
     // cross-over between 2.3 and 11.5 tiles per worker); below that the one-tile-per-CTA form starts sooner
     const bool persistent = ctx->scan_path == 3 || (ctx->scan_path == 0 && 2 * tiles >= (size_t)4 * sms * kPWorkers);

@@ -408,6 +408,26 @@ def test_pruned_attention_retained_keys_only(dtype, path, B, S, Hq, Hkv, window,
     g.close()
 
 
+@pytest.mark.parametrize("B,S,Hq,Hkv,window,ratio,visibility", [
+    (1, 16, 2, 1, 0, 0.0, tfb.TF_KV_ALL), (1, 17, 2, 1, 0, 0.0, tfb.TF_KV_ALL), (1, 65, 3, 3, 0, 0.25, tfb.TF_KV_RETAINED),
+    (1, 600, 2, 2, 65, 0.1, tfb.TF_KV_ALL),          # split over two chunk sequences (few CTAs)
+    (2, 520, 20, 5, 100, 0.5, tfb.TF_KV_ALL), (3, 333, 24, 6, 0, 0.3, tfb.TF_KV_RETAINED),
+    (1, 97, 80, 40, 0, 0.0, tfb.TF_KV_ALL)])          # 32 rows per CTA, all warps on one chunk
+def test_cuda_core_attention_both_forms(B, S, Hq, Hkv, window, ratio, visibility):
+    q, k, v = _qkv(B, S, Hq, Hkv, torch.float32, seed=S + Hq)
+    qn, kn, vn = oracle_inputs(q, k, v)
+    ref = oracle.layer_filter(qn, kn, vn, prune_ratio=ratio, warmup_tokens=1, window=window,
+                              kv_visibility=oracle.KV_RETAINED if visibility == tfb.TF_KV_RETAINED else oracle.KV_ALL)
+    g = Gpu(q, k, v, window=window, prune_ratio=ratio, kv_visibility=visibility)
+    idx, nk = torch.from_numpy(ref["kept_idx"]).to(DEV), torch.from_numpy(ref["n_kept"]).to(DEV)
+    g.ctx.tf_pruned_attention(g.shape, g.params, q, k, v, idx, nk, g.O)
+    g.status_ok()
+    o = to_np(g.O)
+    assert attn_rel_err(o, ref["O"]) < ATTN_TOL[torch.float32]
+    assert np.all(o[ref["keep_mask"] == 0] == 0.0)
+    g.close()
+
+
 def test_layer_filter_retained_keys_only():
     q, k, v = _qkv(2, 700, 8, 2, torch.bfloat16, seed=77)
     n_mis = _layer_case(q, k, v, window=0, prune_ratio=0.5, warmup_tokens=4, kv_visibility=tfb.TF_KV_RETAINED)

@@ -10,6 +10,8 @@ namespace {
 
 using namespace tf;
 
+constexpr size_t kStatusBytes = sizeof(DevStatus) + kDecodeCounters * sizeof(unsigned int);
+
 inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 // Sections of the caller's workspace.
@@ -31,7 +33,7 @@ WsLayout ws_layout(const tf_shape& s, const tf_filter_params* p) {
     w.theta = off;     off += align256((size_t)s.batch * sizeof(float));
     w.kv_compact = off;   // retained tokens' K and V (TF_KV_RETAINED on the tensor-core path only)
     if (p && p->kv_visibility == TF_KV_RETAINED && s.dtype == TF_BF16) off += kv_compact_bytes(s);
-    w.total = off;
+    w.total = off + align256(decode_scratch_bytes(s));   // (used from the front of the workspace: one workspace serves one call at a time)
     return w;
 }
 
@@ -152,8 +154,8 @@ tf_status tf_create(tf_ctx** out, int device) {
     c->use_tensor_cores = 1;
     c->max_polls = -1;
     c->wait_cycles = -1;
-    if (cudaMalloc(reinterpret_cast<void**>(&c->dev_status), sizeof(DevStatus)) != cudaSuccess ||
-        cudaMemset(c->dev_status, 0, sizeof(DevStatus)) != cudaSuccess) {
+    if (cudaMalloc(reinterpret_cast<void**>(&c->dev_status), kStatusBytes) != cudaSuccess ||
+        cudaMemset(c->dev_status, 0, kStatusBytes) != cudaSuccess) {
         delete c;
         return TF_ERR_CUDA;
     }
@@ -482,7 +484,8 @@ tf_status tf_get_status(tf_ctx* ctx, int sync, int64_t detail[4]) {
         detail[2] = (int64_t)h.nan_count; detail[3] = (int64_t)ctx->launches;
     }
     if (h.code == TF_ERR_TIMEOUT) {
-        invalidate_scan_scratch(ctx);   // records written under a wait that gave up are not to be trusted
+        invalidate_scan_scratch(ctx);   // records written under a wait that gave up are not to be trusted, nor counts of arrivals
+        cudaMemset(ctx->dev_status + 1, 0, kStatusBytes - sizeof(DevStatus));
         return TF_ERR_TIMEOUT;
     }
     if (h.code == TF_ERR_NAN_SCORE) return TF_ERR_NAN_SCORE;
@@ -494,7 +497,7 @@ tf_status tf_clear_status(tf_ctx* ctx) {
     DeviceGuard g(ctx->device);
     if (!g.ok) return TF_ERR_CUDA;
     invalidate_scan_scratch(ctx);
-    return cudaMemset(ctx->dev_status, 0, sizeof(DevStatus)) == cudaSuccess ? TF_OK : TF_ERR_CUDA;
+    return cudaMemset(ctx->dev_status, 0, kStatusBytes) == cudaSuccess ? TF_OK : TF_ERR_CUDA;
 }
 
 tf_status tf_last_kernels(tf_ctx* ctx, int32_t kernels[2]) {

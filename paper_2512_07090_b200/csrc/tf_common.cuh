@@ -11,6 +11,7 @@ namespace tf {
 
 constexpr int kHeadDim = 128;
 constexpr int kDeviceFlagSlots = 64;       // per-device one-time set-up flags
+constexpr int kDecodeCounters = 256;       // counters of the streaming decode kernel: two for its work list, then one per piece
 constexpr float kNormEps = 1e-8f;   // lower clamp of each norm in the cosine
 
 // Device status record: four 64-bit words {code, where, nan_count, reserved}.
@@ -186,7 +187,7 @@ __device__ __forceinline__ void scan_leave(unsigned int* counters, unsigned int 
 // The opaque context of include/tf.h.
 struct tf_ctx {
     int device;
-    tf::DevStatus* dev_status;     // device memory, 4 words
+    tf::DevStatus* dev_status;     // device memory: the status record, then kDecodeCounters counters of tf_decode_step
     void* workspace;               // caller-owned
     size_t workspace_bytes;
     tf::ScanScratch scan_user;     // scan bookkeeping of the caller's workspace
@@ -270,6 +271,7 @@ struct tf_decode_args {
     const tf_decode_state* state; void* O_new; float* score_out; uint8_t* skip_out;
     float eta; int alg1_sign;
 };
+size_t decode_scratch_bytes(const tf_shape& s);   // partial results of tf_decode_step, at the start of the workspace
 cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_params& p, const tf_decode_args& a,
                                cudaStream_t st);
 // returns cudaErrorNotSupported when the tensor-core path cannot take this call

@@ -7,13 +7,14 @@
 //   (Eq. 2), score s_KV (Eq. 3), threshold adaptation, skip decision; then the anchor takes the
 //   token in and the counters advance.  Order as in Algorithm 1: compare first, update after
 //   (the inclusive reading updates first).
-// decode_attention_kernel (one CTA per (query head, sequence)): standard single-query attention
-//   over cache positions <= pos (optionally windowed) unless the token is skipped, in which case
-//   its output row is zero (Section 3.2).  The 8 warps take interleaved blocks of 32 keys, each
-//   with its own online softmax; the partial results are merged through shared memory.
+// decode_attention_stream_kernel, decode_attention_split_kernel (bf16 with 1, 2, 4 or 8 query heads per KV head): below.
+// decode_attention_kernel (fp32 and other group sizes; one CTA per (query head, sequence)): standard single-query
+//   attention over cache positions <= pos (optionally windowed) unless the token is skipped, in which case its output row
+//   is zero (Section 3.2).  The 8 warps take interleaved blocks of 32 keys, each with its own online softmax; the
+//   partial results are merged through shared memory.
 #include <algorithm>
 
-#include "tf_common.cuh"
+#include "tf_ptx.cuh"
 
 namespace tf {
 
@@ -28,6 +29,8 @@ struct DecideParams {
     double target;                      // the target skip ratio, as the caller gave it
     int alg1_sign;
     float* sum_k; float* sum_v; long long* count;      // state
+    int sums16;                         // the sums are 16-byte aligned
+    int early;                          // the kernel after this one may start now (it waits before it reads what this one writes)
     float* tau; long long* steps; long long* skips;
     float* score_out; uint8_t* skip_out;
     DevStatus* status;
@@ -40,11 +43,28 @@ template <typename T> __device__ __forceinline__ T dec_from_f(float v);
 template <> __device__ __forceinline__ float dec_from_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 dec_from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
+// four consecutive elements of a cache row (the rows are 16-byte aligned)
+__device__ __forceinline__ void dec_load4(const float* p, float (&f)[4]) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+    f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
+}
+__device__ __forceinline__ void dec_load4(const __nv_bfloat16* p, float (&f)[4]) {
+    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+    f[0] = __uint_as_float(v.x << 16); f[1] = __uint_as_float(v.x & 0xffff0000u);
+    f[2] = __uint_as_float(v.y << 16); f[3] = __uint_as_float(v.y & 0xffff0000u);
+}
+
+// One chain of dependent loads (position, then rows), so what counts is how much of it is in flight at once: a warp per
+// two KV heads as far as 32 warps reach, every load a full vector (where the state is aligned).  Once everything before the
+// step is complete the attention kernel may start and fetch its first tiles under this kernel.
+constexpr int kDecideWarps = 32;
+
 template <typename T>
-__global__ void __launch_bounds__(kDecWarps * 32) decode_decide_kernel(const DecideParams p) {
+__global__ void __launch_bounds__(kDecideWarps * 32) decode_decide_kernel(const DecideParams p) {
     extern __shared__ float cos_s[];        // [2][Hkv]
     grid_dependency_wait();                 // launched early; the step before this one on the stream must be complete
-    const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (p.early) grid_launch_dependents();
+    const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
     const int t = p.pos[b];
     const long long n0 = p.count[b];
     const bool ema = p.anchor_mode == TF_ANCHOR_EMA, incl = p.anchor_mode == TF_ANCHOR_INCL_MEAN;
@@ -55,36 +75,59 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_decide_kernel(const Dec
     float tau_old = 0.f;
     if (threadIdx.x == 0) { steps = p.steps[b]; skips = p.skips[b]; tau_old = p.tau[b]; }
 
-    for (int h = warp; h < p.Hkv; h += kDecWarps) {
-        const T* kp = reinterpret_cast<const T*>(p.K) + (long long)b * p.ks.b + (long long)t * p.ks.t + (long long)h * p.ks.h + lane * 4;
-        const T* vp = reinterpret_cast<const T*>(p.V) + (long long)b * p.vs.b + (long long)t * p.vs.t + (long long)h * p.vs.h + lane * 4;
-        float* sk = p.sum_k + ((size_t)b * p.Hkv + h) * kHeadDim + lane * 4;
-        float* sv = p.sum_v + ((size_t)b * p.Hkv + h) * kHeadDim + lane * 4;
-        float dk = 0.f, kk = 0.f, pk = 0.f, dv = 0.f, vv = 0.f, pv = 0.f;
-        float nk4[4], nv4[4];
+    for (int h0 = warp; h0 < p.Hkv; h0 += 2 * n_warps) {    // two heads at a time: all of their loads go out together
+        float xk4[2][4], xv4[2][4], ak4[2][4], av4[2][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float xk = dec_to_f<T>(kp[i]), xv = dec_to_f<T>(vp[i]);
-            float ak = sk[i], av = sv[i];
-            const float uk = fmaf(a, ak, w * xk), uv = fmaf(a, av, w * xv);    // anchor after the token is taken in
-            if (incl) { ak = uk; av = uv; }
-            dk = fmaf(xk, ak, dk); kk = fmaf(xk, xk, kk); pk = fmaf(ak, ak, pk);
-            dv = fmaf(xv, av, dv); vv = fmaf(xv, xv, vv); pv = fmaf(av, av, pv);
-            nk4[i] = uk; nv4[i] = uv;
-        }
-        dk = warp_sum(dk); kk = warp_sum(kk); pk = warp_sum(pk);
-        dv = warp_sum(dv); vv = warp_sum(vv); pv = warp_sum(pv);
-        if (lane == 0) {
-            float ck = 0.f, cv = 0.f;
-            if (n_cmp > 0) {
-                const float s = ema ? 1.f : 1.f / (float)n_cmp;     // anchor = sum * s
-                ck = (dk * s) / (fmaxf(sqrtf(kk), kNormEps) * fmaxf(sqrtf(pk) * s, kNormEps));
-                cv = (dv * s) / (fmaxf(sqrtf(vv), kNormEps) * fmaxf(sqrtf(pv) * s, kNormEps));
+        for (int u = 0; u < 2; ++u) {
+            const int h = min(h0 + u * n_warps, p.Hkv - 1);
+            dec_load4(reinterpret_cast<const T*>(p.K) + (long long)b * p.ks.b + (long long)t * p.ks.t + (long long)h * p.ks.h + lane * 4, xk4[u]);
+            dec_load4(reinterpret_cast<const T*>(p.V) + (long long)b * p.vs.b + (long long)t * p.vs.t + (long long)h * p.vs.h + lane * 4, xv4[u]);
+            const size_t off = ((size_t)b * p.Hkv + h) * kHeadDim + lane * 4;
+            if (p.sums16) {
+                const float4 sk4 = *reinterpret_cast<const float4*>(p.sum_k + off), sv4 = *reinterpret_cast<const float4*>(p.sum_v + off);
+                ak4[u][0] = sk4.x; ak4[u][1] = sk4.y; ak4[u][2] = sk4.z; ak4[u][3] = sk4.w;
+                av4[u][0] = sv4.x; av4[u][1] = sv4.y; av4[u][2] = sv4.z; av4[u][3] = sv4.w;
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) { ak4[u][i] = p.sum_k[off + i]; av4[u][i] = p.sum_v[off + i]; }
             }
-            cos_s[h] = ck; cos_s[p.Hkv + h] = cv;
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { sk[i] = nk4[i]; sv[i] = nv4[i]; }
+        for (int u = 0; u < 2; ++u) {
+            const int h = h0 + u * n_warps;
+            if (h >= p.Hkv) break;
+            float dk = 0.f, kk = 0.f, pk = 0.f, dv = 0.f, vv = 0.f, pv = 0.f;
+            float nk4[4], nv4[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float xk = xk4[u][i], xv = xv4[u][i];
+                float ak = ak4[u][i], av = av4[u][i];
+                const float uk = fmaf(a, ak, w * xk), uv = fmaf(a, av, w * xv);    // anchor after the token is taken in
+                if (incl) { ak = uk; av = uv; }
+                dk = fmaf(xk, ak, dk); kk = fmaf(xk, xk, kk); pk = fmaf(ak, ak, pk);
+                dv = fmaf(xv, av, dv); vv = fmaf(xv, xv, vv); pv = fmaf(av, av, pv);
+                nk4[i] = uk; nv4[i] = uv;
+            }
+            dk = warp_sum(dk); kk = warp_sum(kk); pk = warp_sum(pk);
+            dv = warp_sum(dv); vv = warp_sum(vv); pv = warp_sum(pv);
+            if (lane == 0) {
+                float ck = 0.f, cv = 0.f;
+                if (n_cmp > 0) {
+                    const float s = ema ? 1.f : 1.f / (float)n_cmp;     // anchor = sum * s
+                    ck = (dk * s) / (fmaxf(sqrtf(kk), kNormEps) * fmaxf(sqrtf(pk) * s, kNormEps));
+                    cv = (dv * s) / (fmaxf(sqrtf(vv), kNormEps) * fmaxf(sqrtf(pv) * s, kNormEps));
+                }
+                cos_s[h] = ck; cos_s[p.Hkv + h] = cv;
+            }
+            const size_t off = ((size_t)b * p.Hkv + h) * kHeadDim + lane * 4;
+            if (p.sums16) {
+                *reinterpret_cast<float4*>(p.sum_k + off) = make_float4(nk4[0], nk4[1], nk4[2], nk4[3]);
+                *reinterpret_cast<float4*>(p.sum_v + off) = make_float4(nv4[0], nv4[1], nv4[2], nv4[3]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) { p.sum_k[off + i] = nk4[i]; p.sum_v[off + i] = nv4[i]; }
+            }
+        }
     }
     __syncthreads();
     if (warp == 0) {
@@ -215,36 +258,62 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_attention_kernel(const 
 }
 
 // ---------------------------------------------------------------------------------------------------
-// bf16 decode attention for grouped heads: one CTA per (split of the visible keys, KV head, sequence)
-// serves all G <= 8 query heads of the group, so K and V rows are read once per group.  The two small
-// products run on warp-level tensor-core instructions (m16n8k16, bf16 in, fp32 out): the path is
-// bandwidth-bound, and the CUDA-core dot products (8 FMAs and 4 shuffles per (head, key)) were what kept
-// it from the bandwidth, so the point is the instruction count, not the flops.  Per warp and block of
-// 16 keys:
-//   S^T[16 keys x 8 heads] = K_blk Q^T     8 products over the 128 dims.  A dot product does not care in
-//                                           which order the dims are visited, so lane (g, t) loads 16-byte
-//                                           pieces t, t+4, t+8, t+12 of its two key rows (g, g+8) and of
-//                                           query head g, and both operands use the same dim order: no
-//                                           shared memory, no shuffles, every load a full 16 bytes;
-//   online softmax on the accumulator layout (lane holds keys g, g+8 for heads 2t, 2t+1: the maximum
-//   over keys is three shuffles); P^T goes back through two 8x8 register transposes (movmatrix);
-//   O^T[128 dims x 8 heads] += V_blk^T P^T  8 products.  Lane (g, t) loads dims 16g..16g+15 of its four
-//                                           key rows (2t, 2t+1, 2t+8, 2t+9); the pairs "same dim, two
-//                                           consecutive keys" the A operand wants are byte permutes.
-// The 8 warps take key blocks 8 apart, each with its own online softmax; they are merged through shared
-// memory.  With more than one split the CTA leaves (max, sum, unnormalised output) per head in scratch
-// and decode_combine_kernel merges the splits.
+// bf16 decode attention, streaming form (chosen for ungrouped heads and for very short steps): one persistent CTA per SM; all
+// G <= 8 query heads of a KV head are served together, so K and V rows are read once per group.  The path is a stream of
+// K / V rows: what bounds it is HBM bandwidth, and what it takes to reach it is that every SM has loads in flight from its
+// first to its last cycle.
+//   work    the visible keys of every unskipped (sequence, KV head) -- a work item -- are cut into tiles of 64 keys, and the list
+//           of all tiles into pieces: 5/8 of it into one piece per CTA, the rest into small pieces that are drawn from a
+//           counter, so that CTAs that started late or run on slower SMs take fewer (equal shares alone: the first CTA done
+//           14 % before the last).  A work item that lies in several pieces leaves partial results (unnormalised output,
+//           maximum, sum) in scratch; the CTA that arrives last, or decode_combine_kernel, merges them.  Where there are many
+//           short work items a piece is a work item, and nothing is merged; so it is without scratch.
+//   warp 8  producer: K and V tiles (and the query rows) by TMA into a ring of slots, 128 to 192 KB in flight per SM,
+//           running ahead across work items.  It starts while the decision kernel still runs, as if no token were skipped; if
+//           one is, what it fetched is thrown away.
+//   warps 0-3 / 4-7 consume the even / odd tiles, 16 keys per warp, on m16n8k16 products:
+//           S^T[16 keys x 8 heads] = K Q^T (A by ldmatrix), online softmax on the accumulator layout (lane holds keys g, g + 8 for
+//           heads 2t, 2t + 1), P^T through two 8x8 register transposes, O^T[128 dims x 8 heads] += V^T P^T (A by
+//           ldmatrix.trans).
+//   warps 9-12 merge: at the end of a segment (a work item, or the part of one in this piece) the consumers leave their
+//           states in shared memory and go on with the next segment at once; these warps merge the eight states and write the result.
+// Every wait is bounded, those of the warps for one another too (mbarriers, no named barriers): on expiry the CTA records
+// TF_ERR_TIMEOUT, stops waiting, lets copies in flight land and exits.
+//   A step of 128 sequences x 400 keys x 40 heads (half of them skipped): 112 -> 100 us, 4 x 4096 keys x 40 heads: 75 -> 61 us.
 // ---------------------------------------------------------------------------------------------------
 constexpr int kPartialFloats = kHeadDim + 2;
+constexpr int kStreamKeys = 64;                            // keys per tile
+constexpr int kStreamHalf = kStreamKeys * 128;             // one [64 keys][128 B] swizzled block
+constexpr int kStreamStage = 4 * kStreamHalf;              // K dims 0-63, 64-127, V dims 0-63, 64-127
+constexpr int kStreamThreads = 416;
+constexpr int kStreamSegs = 4;                             // segment descriptors in flight
+constexpr int kStreamMaxBatch = 512;                       // sequences per launch
+constexpr int kStreamDrawn = 1;                            // drawn pieces per CTA on average (4: 8 x 4096 keys x 8 heads 39 instead of 32 us)
+constexpr size_t kStreamScratch = (size_t)5 << 20;         // partial results: room for more pieces than there are
+template <int G> struct StreamCfg {
+    // an EVEN number of ring slots: a slot then always belongs to the same half of the consumers, which so waits for every
+    // phase of its barrier (a half that skipped phases could mistake an earlier one's completion for its own)
+    static constexpr int kStages = G == 8 ? 4 : 6;
+    static constexpr int kQBytes = G * kHeadDim * 2;       // query rows of a work item
+    static constexpr int kOffQ = kStages * kStreamStage;
+    static constexpr int kOffPart = kOffQ + kStages * kQBytes;
+    static constexpr int kSmemBytes = kOffPart + 8 * G * kPartialFloats * 4 + 1024;   // + alignment slack
+};
 
-struct DecGqaParams {
-    const __nv_bfloat16* Q; const __nv_bfloat16* K; const __nv_bfloat16* V; __nv_bfloat16* O;
+struct DecStreamParams {
+    const __nv_bfloat16* Q; __nv_bfloat16* O;
     long long q_b, q_h, o_b, o_h;
-    Strides3 ks, vs;
     const int32_t* pos; const uint8_t* skip;
-    int Hq, Hkv, window, n_splits;
+    int B, Hq, Hkv, window;
     float scale_log2;
-    float* partial;                   // [B][Hq][n_splits][130] when n_splits > 1
+    uint4* begun;                     // for decode_combine_kernel: [piece] {sequence or ~0, KV head, last piece} of the work item that begins in the
+                                      // piece and ends in a later one; in front of it the number of pieces
+    float* partial;                   // [slot][G][130]; null: a work item is never split
+    unsigned int max_slots;
+    unsigned int* counters;           // {next piece, CTAs done}, zero before and after every launch (with partial only)
+    unsigned int* arrived;            // [piece] zero before and after every launch; null: decode_combine_kernel merges
+    DevStatus* status;
+    long long wait_cycles;
 };
 
 __device__ __forceinline__ void mma_bf16_16816(float* d, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
@@ -259,10 +328,545 @@ __device__ __forceinline__ uint32_t transpose8x8_b16(uint32_t a) {
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo)) | ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi)) << 16);
 }
+__device__ __forceinline__ float ex2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldmatrix4_trans(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+
+// The cut of the list of tiles: tiles below `cut` in pieces of `share` tiles, the rest in pieces of `piece`.
+struct StreamCut {
+    unsigned int cut, share, piece;
+    __device__ __forceinline__ unsigned int piece_of(unsigned int y) const { return y < cut ? y / share : cut / share + (y - cut) / piece; }
+};
+// A piece leaves at most two partial results: slot 2 x for the item it finds begun, 2 x + 1 for the one it begins and does not end.
+// merges the parts of a work item that lies in pieces first .. last: heads h0 .. h0 + N - 1 of the group, dim d
+template <int G, int N>
+__device__ __forceinline__ void merge_parts(const DecStreamParams& p, int b, int kh, unsigned int first, unsigned int last, int h0, int d) {
+    const int n = (int)(last - first) + 1;
+    const float* base = p.partial + ((size_t)(2 * first) * G + h0) * kPartialFloats;
+    float M[N], L[N], acc[N];
+#pragma unroll
+    for (int h = 0; h < N; ++h) { M[h] = -1e30f; L[h] = 0.f; acc[h] = 0.f; }
+    for (int q0 = 0; q0 < n; q0 += 8) {                     // eight parts of every head requested together: one round trip, not one per part
+        float m[N][8], l[N][8], v[N][8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int q = min(q0 + u, n - 1);
+#pragma unroll
+            for (int h = 0; h < N; ++h) {
+                const float* src = base + ((size_t)(2 * q + (q == 0 ? 1 : 0)) * G + h) * kPartialFloats;
+                m[h][u] = __ldcg(src + kHeadDim); l[h][u] = __ldcg(src + kHeadDim + 1); v[h][u] = __ldcg(src + d);
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < N; ++h) {
+            float mx = M[h];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) mx = fmaxf(mx, m[h][u]);
+            const float e0 = exp2f(M[h] - mx);
+            L[h] *= e0; acc[h] *= e0; M[h] = mx;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float e = q0 + u < n ? exp2f(m[h][u] - mx) : 0.f;
+                L[h] = fmaf(l[h][u], e, L[h]);
+                acc[h] = fmaf(v[h][u], e, acc[h]);
+            }
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < N; ++h)
+        p.O[(long long)b * p.o_b + (long long)(kh * G + h0 + h) * p.o_h + d] = __float2bfloat16_rn(acc[h] / L[h]);
+}
+
+// a segment: the tiles of one work item in one piece
+struct StreamSeg {
+    int b, kh, j;                     // sequence, KV head, first tile of the work item
+    int count;                        // tiles; 0: no more work
+    int slot;                         // where the result goes in the scratch; -1: it is the whole work item
+    unsigned int p_first, p_last;     // the pieces the work item lies in
+    int ends_piece;                   // 1: the piece's last segment ...
+    unsigned int piece;               // ... and that piece
+};
+
+template <int G>
+__global__ void __launch_bounds__(kStreamThreads, 1)
+decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV) {
+    using C = StreamCfg<G>;
+    constexpr unsigned int kStages = C::kStages;
+    extern __shared__ uint8_t stream_raw[];
+    __shared__ unsigned int pre[kStreamMaxBatch + 1];      // tiles per KV head of the sequences before b
+    __shared__ int s_pos[kStreamMaxBatch];
+    __shared__ unsigned short active[kStreamMaxBatch];     // the sequences that have tiles
+    __shared__ StreamSeg segs[kStreamSegs];
+    __shared__ __align__(8) unsigned long long bars[2 * C::kStages + 2 * kStreamSegs + 3];
+    __shared__ unsigned int s_tiles, s_segs;
+    __shared__ int s_abort, s_last;
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(stream_raw) + 1023) & ~(uintptr_t)1023);
+    const uint32_t sbase = smem_u32(smem);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, cta = blockIdx.x;
+    const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * kStages, bar_seg = bar_empty + 8 * kStages,
+                   bar_seg_free = bar_seg + 8 * kStreamSegs, bar_part = bar_seg_free + 8 * kStreamSegs, bar_part_free = bar_part + 8,
+                   bar_c = bar_part_free + 8;
+    volatile int* abort_flag = &s_abort;
+    if (tid == 256) {                                       // the thread that uses the barriers before the first block-wide one
+        prefetch_map(&mapK); prefetch_map(&mapV);
+        for (unsigned int i = 0; i < kStages; ++i) { mbar_init(bar_full + 8 * i, 1); mbar_init(bar_empty + 8 * i, 4); }
+        for (int i = 0; i < kStreamSegs; ++i) { mbar_init(bar_seg + 8 * i, 1); mbar_init(bar_seg_free + 8 * i, 12); }
+        mbar_init(bar_part, 8); mbar_init(bar_part_free, 4); mbar_init(bar_c, 4);
+        s_abort = 0;
+        mbar_fence_init();
+    }
+
+    // ---- the list of tiles, made by warp 8 -----------------------------------------------------------------------------
+    // The positions (like K, V and Q) are not written by the decision kernel, and this grid starts only when every CTA of that
+    // kernel has seen all work before it complete: they can be read before the wait (past L1, which may hold older data).
+    auto first_key = [&](int t_pos) { return p.window > 0 ? max(0, t_pos - p.window + 1) : 0; };
+    unsigned int n_seqs = 0, longest = 0;                   // sequences with work, most tiles of one work item
+    auto make_list = [&](bool decided) {
+        unsigned int run = 0;
+        n_seqs = 0; longest = 0;
+        for (int b0 = 0; b0 < p.B; b0 += 32) {
+            const int b = b0 + lane;
+            unsigned int n = 0;
+            if (b < p.B) {
+                const int t_pos = decided ? s_pos[b] : __ldcg(p.pos + b);
+                if (!decided) s_pos[b] = t_pos;
+                if (!decided || !p.skip[b]) n = (unsigned int)(t_pos - first_key(t_pos) + kStreamKeys) / kStreamKeys;
+            }
+            unsigned int in = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned int v = __shfl_up_sync(0xffffffffu, in, o);
+                if (lane >= o) in += v;
+            }
+            if (b < p.B) pre[b] = run + in - n;
+            run += __shfl_sync(0xffffffffu, in, 31);
+            const unsigned int with = __ballot_sync(0xffffffffu, n > 0);
+            if (n > 0) active[n_seqs + __popc(with & ((1u << lane) - 1u))] = (unsigned short)b;
+            n_seqs += __popc(with);
+            longest = max(longest, __reduce_max_sync(0xffffffffu, n));
+        }
+        if (lane == 0) pre[p.B] = run;
+        __syncwarp();
+    };
+    unsigned int total = 0, n_pieces = 0;
+    bool whole = false;
+    StreamCut cut{};
+    auto make_cut = [&]() {                                 // reads pre[]
+        total = pre[p.B] * (unsigned int)p.Hkv;
+        const unsigned int n_cta = min(gridDim.x, max(total, 1u)), items = n_seqs * (unsigned int)p.Hkv;
+        // whole: a piece is a work item, so nothing has to be merged: without scratch, and when there are many short work
+        // items anyway
+        whole = !p.partial || (items >= 8 * n_cta && longest <= total / (4 * n_cta));
+        if (whole) {
+            n_pieces = items;
+        } else {
+            cut.share = max(1u, (total / 8 * 5 + n_cta - 1) / n_cta);
+            cut.cut = min(total / cut.share, n_cta) * cut.share;
+            const unsigned int rest = total - cut.cut, most = max(1u, min(kStreamDrawn * n_cta, p.max_slots / 2 - n_cta - 1));
+            cut.piece = max(1u, (rest + most - 1) / most);
+            n_pieces = cut.cut / cut.share + (rest + cut.piece - 1) / cut.piece;
+        }
+    };
+    // producer state (warp 8, lane 0): the current segment, the next tile of it, and where the piece ends
+    StreamSeg pt{};
+    int pk_lo = 0, p_done = 0;
+    unsigned int n_segs = 0;
+    int walk = 0;                                           // a sequence at or before the next piece
+    unsigned int py = 0, py_end = 0, p_now = 0, pn = 0;     // tile number, end of the piece, its number; tiles of the work item
+    auto open_segment = [&]() {                             // from tile py of work item (pt.b, pt.kh, pt.j) on
+        pk_lo = first_key(s_pos[pt.b]);
+        const unsigned int i0 = py - pt.j;
+        pt.count = (int)min(pn - pt.j, py_end - py);
+        p_done = 0;
+        pt.p_first = whole ? p_now : cut.piece_of(i0); pt.p_last = whole ? p_now : cut.piece_of(i0 + pn - 1);
+        pt.ends_piece = py + (unsigned int)pt.count == py_end ? 1 : 0;
+        pt.piece = p_now;
+        pt.slot = (unsigned int)pt.count == pn ? -1 : (int)(2 * p_now + (pt.j == 0 ? 1 : 0));
+    };
+    auto next_item = [&]() {                                // there is one
+        pt.j = 0;
+        if (++pt.kh == p.Hkv) {
+            pt.kh = 0;
+            do { ++pt.b; pn = pre[pt.b + 1] - pre[pt.b]; } while (pn == 0);
+        }
+    };
+    auto open_piece = [&](unsigned int x) {                 // x < n_pieces
+        // (on the path of the loads: one division here, and a walk over the sequences instead of a search -- pieces only go up)
+        p_now = x;
+        if (whole) {
+            const unsigned int i = x / (unsigned int)p.Hkv;
+            pt.b = active[i]; pt.kh = (int)(x - i * (unsigned int)p.Hkv); pt.j = 0;
+            pn = pre[pt.b + 1] - pre[pt.b];
+            py = 0; py_end = pn;
+        } else {
+            const unsigned int n_static = cut.cut / cut.share;
+            py = x < n_static ? x * cut.share : cut.cut + (x - n_static) * cut.piece;
+            py_end = min(total, x < n_static ? py + cut.share : py + cut.piece);
+            while (pre[walk + 1] * (unsigned int)p.Hkv <= py) ++walk;
+            pt.b = walk;
+            pn = pre[walk + 1] - pre[walk];
+            const unsigned int rem = py - pre[walk] * (unsigned int)p.Hkv;
+            pt.kh = (int)(rem / pn); pt.j = (int)(rem - (unsigned int)pt.kh * pn);
+        }
+        open_segment();
+    };
+    auto announce = [&]() {                                 // the segment's descriptor (its ring slot is free)
+        segs[n_segs % kStreamSegs] = pt;
+        mbar_arrive(bar_seg + 8 * (n_segs % kStreamSegs));
+        ++n_segs;
+    };
+    auto produce = [&](unsigned int it) {
+        const unsigned int st = it % kStages;
+        const uint32_t dst = sbase + st * kStreamStage, bar = bar_full + 8 * st;
+        const int key = pk_lo + (pt.j + p_done) * kStreamKeys;
+        const bool with_q = p_done < 2;                    // either half of the consumers finds the query rows with its first tile
+        mbar_expect_tx(bar, kStreamStage + (with_q ? C::kQBytes : 0));
+        tma_load_4d(dst, &mapK, bar, 0, pt.kh, key, pt.b);
+        tma_load_4d(dst + kStreamHalf, &mapK, bar, 64, pt.kh, key, pt.b);
+        tma_load_4d(dst + 2 * kStreamHalf, &mapV, bar, 0, pt.kh, key, pt.b);
+        tma_load_4d(dst + 3 * kStreamHalf, &mapV, bar, 64, pt.kh, key, pt.b);
+        if (with_q) {
+            const __nv_bfloat16* q = p.Q + (long long)pt.b * p.q_b + (long long)pt.kh * G * p.q_h;
+            for (int g = 0; g < G; ++g)
+                bulk_load(sbase + C::kOffQ + st * C::kQBytes + g * kHeadDim * 2, q + (long long)g * p.q_h, kHeadDim * 2, bar);
+        }
+        ++p_done; ++py;
+        if (p_done == pt.count && py < py_end) { next_item(); open_segment(); }
+    };
+    if (warp == 8) {
+        make_list(false);
+        if (lane == 0) {
+            unsigned int n = 0;
+            make_cut();
+            if ((unsigned int)cta < n_pieces) {
+                open_piece(cta);
+                for (; n < kStages && py < py_end && (p_done > 0 || n_segs < kStreamSegs); ++n) {
+                    if (p_done == 0) announce();
+                    produce(n);
+                }
+            }
+            s_tiles = n;                                    // tiles fetched and segments announced before the decisions are known
+            s_segs = n_segs;
+        }
+    }
+    __syncwarp();
+    grid_dependency_wait();
+    int any_skip = 0;
+    for (int b = tid; b < p.B; b += kStreamThreads) any_skip |= p.skip[b];
+    any_skip = __syncthreads_or(any_skip);
+    const unsigned int ahead = s_tiles;
+    const unsigned int wasted = any_skip ? ahead : 0u, wasted_segs = any_skip ? s_segs : 0u;   // in vain: everybody lets them pass
+    if (warp == 8) {
+        // ================================ producer ============================================================
+        if (any_skip) { make_list(true); walk = 0; }
+        if (lane == 0) make_cut();
+        if (cta == 0 && lane == 0 && p.begun) p.begun[-1] = make_uint4(whole ? 0u : n_pieces, 0u, 0u, 0u);
+        if (lane == 0) {
+            unsigned int x = cta, it = ahead;
+            bool ok = true, open = !any_skip && ahead > 0;   // the piece opened above goes on
+            auto slot_free = [&]() {
+                return it < kStages || mbar_wait_bounded(bar_empty + 8 * (it % kStages), ((it / kStages) - 1) & 1u, abort_flag, p.wait_cycles, p.status, 601);
+            };
+            auto seg_free = [&]() {
+                return n_segs < kStreamSegs ||
+                       mbar_wait_bounded(bar_seg_free + 8 * (n_segs % kStreamSegs), ((n_segs / kStreamSegs) - 1) & 1u, abort_flag, p.wait_cycles, p.status, 606);
+            };
+            while (ok && x < n_pieces) {
+                if (!open) open_piece(x);
+                unsigned int x_next = x + gridDim.x;
+                bool drawn = !p.partial;
+                while (ok && py < py_end) {
+                    if (!drawn && py + 3 >= py_end) {       // as late as the answer is still there in time
+                        x_next = gridDim.x + atomicAdd(p.counters, 1u);
+                        drawn = true;
+                    }
+                    if (p_done == 0) {
+                        ok = seg_free();
+                        if (ok) announce();
+                    }
+                    ok = ok && slot_free();
+                    if (ok) { produce(it); ++it; }
+                }
+                if (!drawn) x_next = gridDim.x + atomicAdd(p.counters, 1u);
+                open = false;
+                x = x_next;
+            }
+            if (ok && seg_free()) {                         // no more work
+                pt.count = 0;
+                announce();
+            }
+            if (p.partial && atomicAdd(p.counters + 1, 1u) == gridDim.x - 1) {   // the last to stop drawing resets the counters
+                atomicExch(p.counters, 0u);
+                atomicExch(p.counters + 1, 0u);
+            }
+        }
+    } else if (warp < 8) {
+        // ================================ consumers ===========================================================
+        grid_launch_dependents();
+        float* part_s = reinterpret_cast<float*>(smem + C::kOffPart);
+        const int half = warp >> 2, kb = (warp & 3) * 16;   // this warp's 16 keys of every second tile
+        const int g = lane >> 2, t = lane & 3;
+        // ldmatrix row of this lane: K as A (rows = keys), V as transposed A (rows = keys of the stored tile)
+        const int rk = kb + (lane & 7) + ((lane >> 3) & 1) * 8, ck = lane >> 4;
+        const int rv = kb + (lane & 7) + (lane >> 4) * 8, cv = (lane >> 3) & 1;
+        unsigned int it = 0;
+        bool ok = true;
+        for (; it < wasted; ++it) {
+            if ((int)(it & 1) != half) continue;
+            ok = __all_sync(0xffffffffu, ok && mbar_wait_bounded(bar_full + 8 * (it % kStages), 0, abort_flag, p.wait_cycles, p.status, 603));
+            if (ok && lane == 0) mbar_arrive(bar_empty + 8 * (it % kStages));
+        }
+        for (unsigned int sg = 0; ok; ++sg) {
+            const unsigned int ss = sg % kStreamSegs;
+            ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar_seg + 8 * ss, (sg / kStreamSegs) & 1u, abort_flag, p.wait_cycles, p.status, 607));
+            if (!ok) break;
+            const StreamSeg seg = segs[ss];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_seg_free + 8 * ss);
+            if (sg < wasted_segs) continue;
+            if (seg.count == 0) break;
+            const int t_pos = s_pos[seg.b], n_vis = t_pos - first_key(t_pos) + 1 - seg.j * kStreamKeys;      // visible keys from the segment's first on
+            float m[2] = {-1e30f, -1e30f}, l[2] = {0.f, 0.f};   // heads 2t, 2t + 1 (m is the same in all lanes of equal t; l is the lane's share)
+            float o[8][4];                                      // O^T: dims 16 mt + g and 16 mt + 8 + g, heads 2t, 2t + 1
+            uint32_t qb[8][2];
+#pragma unroll
+            for (int mt = 0; mt < 8; ++mt) { o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f; }
+            const int i0 = ((int)(it & 1) == half) ? 0 : 1;      // this half's first tile
+            for (int i = i0; i < seg.count; i += 2) {
+                const unsigned int st = (it + i) % kStages;
+                ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar_full + 8 * st, ((it + i) / kStages) & 1u, abort_flag, p.wait_cycles, p.status, 602));
+                if (!ok) break;
+                if (i < 2) {                                     // Q^T as the B operand
+                    const uint8_t* q = smem + C::kOffQ + st * C::kQBytes + (g < G ? g : 0) * kHeadDim * 2 + t * 4;
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk) {
+                        qb[kk][0] = g < G ? *reinterpret_cast<const uint32_t*>(q + kk * 32) : 0u;
+                        qb[kk][1] = g < G ? *reinterpret_cast<const uint32_t*>(q + kk * 32 + 16) : 0u;
+                    }
+                }
+                const uint32_t ka = sbase + st * kStreamStage, va = ka + 2 * kStreamHalf;
+                const int left = n_vis - i * kStreamKeys - kb;   // visible keys of this warp's 16
+                if (left > 0) {
+                    float s[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f};   // two accumulation chains
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk) {
+                        uint32_t a[4];
+                        const int ch = kk * 2 + ck;
+                        ldmatrix4(ka + (ch >> 3) * kStreamHalf + rk * 128 + (((ch & 7) ^ (rk & 7)) << 4), a);
+                        mma_bf16_16816(kk & 1 ? s2 : s, a[0], a[1], a[2], a[3], qb[kk][0], qb[kk][1]);
+                    }
+                    if (left < 16) {   // rows past the last visible key hold whatever the cache holds: their values must not reach the sum
+                        for (int z = lane; z < (16 - left) * 16; z += 32) {
+                            const int row = kb + left + (z >> 4);
+                            *reinterpret_cast<uint4*>(smem + st * kStreamStage + (2 + ((z >> 3) & 1)) * kStreamHalf + row * 128 + ((z & 7) << 4)) = make_uint4(0, 0, 0, 0);
+                        }
+                        __syncwarp();
+                    }
+                    const bool v0 = g < left, v1 = g + 8 < left;
+                    s[0] = v0 ? (s[0] + s2[0]) * p.scale_log2 : -1e30f; s[1] = v0 ? (s[1] + s2[1]) * p.scale_log2 : -1e30f;
+                    s[2] = v1 ? (s[2] + s2[2]) * p.scale_log2 : -1e30f; s[3] = v1 ? (s[3] + s2[3]) * p.scale_log2 : -1e30f;
+                    float corr[2], pr[4];
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        float mx = fmaxf(s[k], s[k + 2]);
+                        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
+                        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+                        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+                        const float mn = fmaxf(m[k], mx);
+                        corr[k] = ex2_approx(m[k] - mn);
+                        m[k] = mn;
+                        pr[k] = v0 ? ex2_approx(s[k] - mn) : 0.f;
+                        pr[k + 2] = v1 ? ex2_approx(s[k + 2] - mn) : 0.f;
+                        l[k] = fmaf(l[k], corr[k], pr[k] + pr[k + 2]);
+                    }
+                    // P^T (keys x heads) -> the B operand wants head g with keys 2t, 2t+1 / 2t+8, 2t+9: two 8x8 transposes
+                    const uint32_t pb0 = transpose8x8_b16(pack_bf16x2(pr[0], pr[1]));
+                    const uint32_t pb1 = transpose8x8_b16(pack_bf16x2(pr[2], pr[3]));
+                    if (__any_sync(0xffffffffu, corr[0] != 1.f || corr[1] != 1.f)) {
+#pragma unroll
+                        for (int mt = 0; mt < 8; ++mt) { o[mt][0] *= corr[0]; o[mt][1] *= corr[1]; o[mt][2] *= corr[0]; o[mt][3] *= corr[1]; }
+                    }
+#pragma unroll
+                    for (int mt = 0; mt < 8; ++mt) {
+                        uint32_t a[4];
+                        const int ch = mt * 2 + cv;
+                        ldmatrix4_trans(va + (ch >> 3) * kStreamHalf + rv * 128 + (((ch & 7) ^ (rv & 7)) << 4), a);
+                        mma_bf16_16816(o[mt], a[0], a[1], a[2], a[3], pb0, pb1);
+                    }
+                }
+                if (left < 16) fence_proxy_async();              // zeros written above, before TMA writes the slot again
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_empty + 8 * st);
+            }
+            if (!ok) break;
+            it += seg.count;
+            // ---- the warp's state to the merging warps ---------------------------------------------------------------
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                l[k] += __shfl_xor_sync(0xffffffffu, l[k], 4);
+                l[k] += __shfl_xor_sync(0xffffffffu, l[k], 8);
+                l[k] += __shfl_xor_sync(0xffffffffu, l[k], 16);
+            }
+            const unsigned int k_seg = sg - wasted_segs;         // (the first wait passes: nothing has been left there yet)
+            ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar_part_free, (k_seg & 1u) ^ 1u, abort_flag, p.wait_cycles, p.status, 605));
+            if (!ok) break;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int h = 2 * t + k;
+                if (h < G) {
+                    float* dst = part_s + (warp * G + h) * kPartialFloats;
+#pragma unroll
+                    for (int mt = 0; mt < 8; ++mt) { dst[16 * mt + g] = o[mt][k]; dst[16 * mt + 8 + g] = o[mt][k + 2]; }
+                    if (g == 0) { dst[kHeadDim] = m[k]; dst[kHeadDim + 1] = l[k]; }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_part);
+        }
+    } else {
+        // ================================ merging warps =======================================================
+        const float* part_s = reinterpret_cast<const float*>(smem + C::kOffPart);
+        const int mt = tid - 288;                           // 0 .. 127: output dim
+        for (int b = cta; b < p.B; b += (int)gridDim.x)     // skipped tokens' output rows
+            if (p.skip[b])
+                for (int i = mt; i < p.Hq * (kHeadDim / 8); i += 128)
+                    *reinterpret_cast<uint4*>(p.O + (long long)b * p.o_b + (long long)(i >> 4) * p.o_h + (i & 15) * 8) = make_uint4(0, 0, 0, 0);
+        uint32_t c_phase = 0;
+        auto mergers_sync = [&]() {                         // the 4 merging warps; false: a wait gave up
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_c);
+            const bool ok = mbar_wait_bounded(bar_c, c_phase, abort_flag, p.wait_cycles, p.status, 604);
+            c_phase ^= 1;
+            return __all_sync(0xffffffffu, ok) != 0;
+        };
+        for (unsigned int sg = 0;; ++sg) {
+            const unsigned int ss = sg % kStreamSegs;
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar_seg + 8 * ss, (sg / kStreamSegs) & 1u, abort_flag, p.wait_cycles, p.status, 608))) break;
+            const StreamSeg seg = segs[ss];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_seg_free + 8 * ss);
+            if (sg < wasted_segs) continue;
+            if (seg.count == 0) break;
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar_part, (sg - wasted_segs) & 1u, abort_flag, p.wait_cycles, p.status, 609))) break;
+            float M[G], L[G], acc[G];
+#pragma unroll
+            for (int h = 0; h < G; ++h) {
+                const float* src = part_s + h * kPartialFloats;
+                M[h] = -1e30f;
+#pragma unroll
+                for (int w2 = 0; w2 < 8; ++w2) M[h] = fmaxf(M[h], src[w2 * G * kPartialFloats + kHeadDim]);
+                L[h] = 0.f; acc[h] = 0.f;
+#pragma unroll
+                for (int w2 = 0; w2 < 8; ++w2) {
+                    const float e = ex2_approx(src[w2 * G * kPartialFloats + kHeadDim] - M[h]);
+                    L[h] = fmaf(src[w2 * G * kPartialFloats + kHeadDim + 1], e, L[h]);
+                    acc[h] = fmaf(src[w2 * G * kPartialFloats + mt], e, acc[h]);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_part_free);
+#pragma unroll
+            for (int h = 0; h < G; ++h) {
+                if (seg.slot < 0) {
+                    p.O[(long long)seg.b * p.o_b + (long long)(seg.kh * G + h) * p.o_h + mt] = __float2bfloat16_rn(acc[h] / L[h]);
+                } else {
+                    float* dst = p.partial + ((size_t)seg.slot * G + h) * kPartialFloats;
+                    dst[mt] = acc[h];
+                    if (mt == 0) { dst[kHeadDim] = M[h]; dst[kHeadDim + 1] = L[h]; }
+                }
+            }
+            if (p.begun && seg.ends_piece && mt == 0 && seg.piece < gridDim.x * (1 + kStreamDrawn))
+                p.begun[seg.piece] = seg.slot == (int)(2 * seg.piece + 1) ? make_uint4((unsigned int)seg.b, (unsigned int)seg.kh, seg.p_last, 0u)
+                                                                          : make_uint4(0xffffffffu, 0u, 0u, 0u);
+            if (seg.slot >= 0 && p.arrived) {                // whoever comes last merges the work item's parts
+                __threadfence();
+                if (!mergers_sync()) break;
+                if (mt == 0) {
+                    const unsigned int n = atomicAdd(p.arrived + seg.p_first, 1u);
+                    s_last = n == seg.p_last - seg.p_first;
+                    if (s_last) atomicExch(p.arrived + seg.p_first, 0u);
+                }
+                if (!mergers_sync()) break;
+                if (s_last) {
+                    __threadfence();
+                    constexpr int kAtOnce = G < 4 ? G : 4;
+                    for (int h = 0; h < G; h += kAtOnce) merge_parts<G, kAtOnce>(p, seg.b, seg.kh, seg.p_first, seg.p_last, h, mt);
+                }
+                if (!mergers_sync()) break;                  // s_last has been read
+            }
+        }
+    }
+    __syncwarp();
+    __syncthreads();
+    if (*abort_flag) {   // a wait gave up: let copies in flight land before the shared memory goes away
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000ll) { }
+    }
+}
+
+// merges the work items that lie in several pieces: CTA x the one that begins in piece x, a thread per (head, dim)
+template <int G>
+__global__ void __launch_bounds__(G * kHeadDim) decode_combine_kernel(const DecStreamParams p) {
+    grid_dependency_wait();
+    const unsigned int x = blockIdx.x, n_pieces = p.begun[-1].x;
+    const uint4 it = p.begun[x];                            // (beyond the last piece: whatever is there)
+    if (x < n_pieces && it.x != 0xffffffffu)
+        merge_parts<G, 1>(p, (int)it.x, (int)it.y, x, it.z, (int)threadIdx.x / kHeadDim, (int)threadIdx.x % kHeadDim);
+}
+
+// what decode_combine_kernel reads, in front of the slots
+static size_t stream_table_bytes(int grid) { return (1 + (size_t)grid * (1 + kStreamDrawn)) * sizeof(uint4); }
+
+// a workspace is usually sized with a prefill shape, which need not name the query heads
+size_t decode_scratch_bytes(const tf_shape& s) { return s.dtype == TF_BF16 ? kStreamScratch + stream_table_bytes(sm_count()) : 0; }
+
+template <int G>
+static cudaError_t launch_stream(const DecStreamParams& sp, int grid, int device, const CUtensorMap& mk, const CUtensorMap& mv, cudaStream_t st) {
+    static bool attr_set_dev[kDeviceFlagSlots] = {};      // function attributes are per device
+    bool& attr_set = attr_set_dev[device >= 0 && device < kDeviceFlagSlots ? device : 0];
+    if (!attr_set) {
+        const cudaError_t e = cudaFuncSetAttribute(decode_attention_stream_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamCfg<G>::kSmemBytes);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    const cudaError_t e = launch_dependent(decode_attention_stream_kernel<G>, dim3((unsigned)grid), dim3(kStreamThreads), StreamCfg<G>::kSmemBytes, st, sp, mk, mv);
+    if (e != cudaSuccess || !sp.begun) return e;
+    return launch_dependent(decode_combine_kernel<G>, dim3((unsigned)(grid * (1 + kStreamDrawn))), dim3(G * kHeadDim), 0, st, sp);
+}
+
+// ---------------------------------------------------------------------------------------------------
+// Grouped heads (G >= 2) in more than a very short step: one CTA per (split of the visible keys, KV head, sequence), two CTAs
+// per SM.  No list of work to make: a grouped cache is a G-th of the bytes, and the head start of this form outweighs the equal
+// shares of the streaming kernel (us a step, this / streaming: 1 x 8192 16 / 24, 8 x 4096 keys of 16384 31 / 32, 128 x 1024 68 / 80;
+// ungrouped 40 heads: 1 x 8192 45 / 36, 4 x 4096 75 / 61, 128 x 512 112 / 100).  Operands come straight from global memory, no shared
+// memory: a dot product does not care in which order the dims are visited, so lane (g, t) loads 16-byte pieces t, t+4, t+8,
+// t+12 of its two key rows (g, g+8) and of query head g; of its four value rows (2t, 2t+1, 2t+8, 2t+9) it loads dims 16g ..
+// 16g+15, and the pairs "same dim, two consecutive keys" the A operand wants are byte permutes.  The 8 warps take key blocks 8 apart
+// and are merged through shared memory; with more than one split the CTA leaves (max, sum, unnormalised output) per head
+// in scratch and decode_merge_splits_kernel merges the splits.
+// ---------------------------------------------------------------------------------------------------
+struct DecGqaParams {
+    const __nv_bfloat16* Q; const __nv_bfloat16* K; const __nv_bfloat16* V; __nv_bfloat16* O;
+    long long q_b, q_h, o_b, o_h;
+    Strides3 ks, vs;
+    const int32_t* pos; const uint8_t* skip;
+    int Hq, Hkv, window, n_splits;
+    float scale_log2;
+    float* partial;                   // [B][Hq][n_splits][130] when n_splits > 1
+};
+
 __device__ __forceinline__ uint32_t word_of(const uint4& r, int w) { return w == 0 ? r.x : w == 1 ? r.y : w == 2 ? r.z : r.w; }
 
 template <int G>
-__global__ void __launch_bounds__(256, 2) decode_attention_gqa_kernel(const DecGqaParams p) {
+__global__ void __launch_bounds__(256, 2) decode_attention_split_kernel(const DecGqaParams p) {
     __shared__ float part_s[8][G][kPartialFloats];
     grid_dependency_wait();
     const int split = blockIdx.x, kh = blockIdx.y, b = blockIdx.z;
@@ -328,10 +932,10 @@ __global__ void __launch_bounds__(256, 2) decode_attention_gqa_kernel(const DecG
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
             const float mn = fmaxf(m[c], mx);
-            corr[c] = exp2f(m[c] - mn);
+            corr[c] = ex2_approx(m[c] - mn);
             m[c] = mn;
-            pr[c] = v0 ? exp2f(s[c] - mn) : 0.f;
-            pr[c + 2] = v1 ? exp2f(s[c + 2] - mn) : 0.f;
+            pr[c] = v0 ? ex2_approx(s[c] - mn) : 0.f;
+            pr[c + 2] = v1 ? ex2_approx(s[c + 2] - mn) : 0.f;
             l[c] = fmaf(l[c], corr[c], pr[c] + pr[c + 2]);
         }
         // P^T (keys x heads) -> the B operand wants head g with keys 2t, 2t+1 / 2t+8, 2t+9: two 8x8 transposes
@@ -393,21 +997,32 @@ __global__ void __launch_bounds__(256, 2) decode_attention_gqa_kernel(const DecG
 }
 
 // merges the splits of one (query head, sequence); a skipped token gets its zero row here
-__global__ void __launch_bounds__(kHeadDim) decode_combine_kernel(const DecGqaParams p) {
+__global__ void __launch_bounds__(kHeadDim) decode_merge_splits_kernel(const DecGqaParams p) {
     grid_dependency_wait();
     const int qh = blockIdx.x, b = blockIdx.y, d = threadIdx.x;
     __nv_bfloat16* out = p.O + (long long)b * p.o_b + (long long)qh * p.o_h + d;
-    if (p.skip[b]) { *out = __float2bfloat16_rn(0.f); return; }
-    const float* src = p.partial + ((size_t)b * p.Hq + qh) * p.n_splits * kPartialFloats;
-    float M = -1e30f;
-    for (int s2 = 0; s2 < p.n_splits; ++s2) M = fmaxf(M, src[s2 * kPartialFloats + kHeadDim]);
-    float L = 0.f, o = 0.f;
-    for (int s2 = 0; s2 < p.n_splits; ++s2) {
-        const float c = exp2f(src[s2 * kPartialFloats + kHeadDim] - M);
-        L = fmaf(src[s2 * kPartialFloats + kHeadDim + 1], c, L);
-        o = fmaf(src[s2 * kPartialFloats + d], c, o);
+    const bool skip = p.skip[b] != 0;
+    const float* base = p.partial + ((size_t)b * p.Hq + qh) * p.n_splits * kPartialFloats;
+    float M = -1e30f, L = 0.f, acc = 0.f;
+    for (int q0 = 0; q0 < p.n_splits; q0 += 8) {            // eight splits requested together (a skipped token's are stale, and not used)
+        float m[8], l[8], v[8], mx = M;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float* src = base + (size_t)min(q0 + u, p.n_splits - 1) * kPartialFloats;
+            m[u] = src[kHeadDim]; l[u] = src[kHeadDim + 1]; v[u] = src[d];
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) mx = fmaxf(mx, m[u]);
+        const float e0 = exp2f(M - mx);
+        L *= e0; acc *= e0; M = mx;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float e = q0 + u < p.n_splits ? exp2f(m[u] - M) : 0.f;
+            L = fmaf(l[u], e, L);
+            acc = fmaf(v[u], e, acc);
+        }
     }
-    *out = __float2bfloat16_rn(o / L);
+    *out = skip ? __float2bfloat16_rn(0.f) : __float2bfloat16_rn(acc / L);
 }
 
 cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_params& p, const tf_decode_args& a,
@@ -421,13 +1036,35 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
     dp.warmup = p.warmup_tokens; dp.gamma = p.gamma; dp.var_eps = p.var_eps > 0.f ? p.var_eps : 1e-8f;
     dp.eta = a.eta; dp.target = p.prune_ratio; dp.alg1_sign = a.alg1_sign;
     dp.sum_k = a.state->sum_k; dp.sum_v = a.state->sum_v; dp.count = reinterpret_cast<long long*>(a.state->count);
+    dp.sums16 = ((reinterpret_cast<uintptr_t>(dp.sum_k) | reinterpret_cast<uintptr_t>(dp.sum_v)) & 15u) == 0;
+    // bf16 with 1, 2, 4 or 8 query heads per KV head and 16-byte aligned query rows: the streaming kernel for ungrouped heads
+    // and for steps with at most half a tile per SM, the split kernel otherwise (both sides' times stand at the split kernel;
+    // at 1 x 420 keys x 8 heads 12.4 us a step against 13.5)
+    const int G = s.n_q_heads / s.n_kv_heads;
+    const int sms = sm_count();
+    const int max_keys = s.window > 0 ? std::min(s.window, s.seq) : s.seq;     // pos is device data: size for the worst case
+    const long long tiles_max = (long long)s.batch * s.n_kv_heads * ((max_keys + kStreamKeys - 1) / kStreamKeys);
+    const bool grouped = s.dtype == TF_BF16 && (G == 1 || G == 2 || G == 4 || G == 8) && ((s.q_stride[0] | s.q_stride[2]) % 8) == 0 &&
+                         (reinterpret_cast<uintptr_t>(a.q_new) & 15u) == 0;
+    CUtensorMap mk, mv;
+    auto maps = [&](int b0, int n) {
+        const __nv_bfloat16* K = static_cast<const __nv_bfloat16*>(a.K_cache) + (long long)b0 * s.k_stride[0];
+        const __nv_bfloat16* V = static_cast<const __nv_bfloat16*>(a.V_cache) + (long long)b0 * s.v_stride[0];
+        return make_bshd_map(&mk, K, s.k_stride, n, s.seq, s.n_kv_heads, 2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 64, kStreamKeys, CU_TENSOR_MAP_SWIZZLE_128B) &&
+               make_bshd_map(&mv, V, s.v_stride, n, s.seq, s.n_kv_heads, 2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 64, kStreamKeys, CU_TENSOR_MAP_SWIZZLE_128B);
+    };
+    const bool stream = grouped && (G == 1 || 2 * tiles_max <= sms) && tiles_max < (1ll << 31) &&              // (tile numbers are 32 bits)
+                        ((s.o_stride[0] | s.o_stride[2]) % 8) == 0 && (reinterpret_cast<uintptr_t>(a.O_new) & 15u) == 0 &&
+                        (s.batch == 1 || (s.k_stride[0] > 0 && s.v_stride[0] > 0)) && maps(0, std::min<int>(s.batch, kStreamMaxBatch));
+    dp.early = stream ? 1 : 0;
     dp.tau = a.state->tau; dp.steps = reinterpret_cast<long long*>(a.state->steps);
     dp.skips = reinterpret_cast<long long*>(a.state->skips);
     dp.score_out = a.score_out; dp.skip_out = a.skip_out; dp.status = ctx->dev_status;
     const size_t smem = 2 * (size_t)s.n_kv_heads * sizeof(float);
     cudaError_t e;
-    if (s.dtype == TF_BF16) e = launch_dependent(decode_decide_kernel<__nv_bfloat16>, dim3((unsigned)s.batch), dim3(kDecWarps * 32), smem, st, dp);
-    else                    e = launch_dependent(decode_decide_kernel<float>, dim3((unsigned)s.batch), dim3(kDecWarps * 32), smem, st, dp);
+    const dim3 decide_block(32u * std::min(kDecideWarps, std::max((s.n_kv_heads + 1) / 2, 4)));
+    if (s.dtype == TF_BF16) e = launch_dependent(decode_decide_kernel<__nv_bfloat16>, dim3((unsigned)s.batch), decide_block, smem, st, dp);
+    else                    e = launch_dependent(decode_decide_kernel<float>, dim3((unsigned)s.batch), decide_block, smem, st, dp);
     ctx->launches += 1;
     if (e != cudaSuccess) return e;
 
@@ -438,19 +1075,13 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
     ap.Hq = s.n_q_heads; ap.Hkv = s.n_kv_heads; ap.window = s.window;
     const float scale = s.softmax_scale != 0.f ? s.softmax_scale : 1.f / sqrtf((float)s.head_dim);
     ap.scale_log2 = scale * 1.4426950408889634f;
-    // bf16 with 1, 2, 4 or 8 query heads per KV head: the grouped kernel (K / V read once per group), split
-    // over the visible keys when that is needed to fill the GPU and the bound workspace can hold the partials
-    const int G = s.n_q_heads / s.n_kv_heads;
-    if (s.dtype == TF_BF16 && (G == 1 || G == 2 || G == 4 || G == 8) && (s.q_stride[2] % 8 == 0) && (s.q_stride[0] % 8 == 0) &&
-        (reinterpret_cast<uintptr_t>(a.q_new) & 15u) == 0) {
+    if (grouped && !stream) {
         DecGqaParams gp{};
         gp.Q = static_cast<const __nv_bfloat16*>(a.q_new); gp.K = static_cast<const __nv_bfloat16*>(a.K_cache);
         gp.V = static_cast<const __nv_bfloat16*>(a.V_cache); gp.O = static_cast<__nv_bfloat16*>(a.O_new);
         gp.q_b = ap.q_b; gp.q_h = ap.q_h; gp.o_b = ap.o_b; gp.o_h = ap.o_h;
         gp.ks = ap.ks; gp.vs = ap.vs; gp.pos = a.pos; gp.skip = a.skip_out;
         gp.Hq = s.n_q_heads; gp.Hkv = s.n_kv_heads; gp.window = s.window; gp.scale_log2 = ap.scale_log2;
-        const int sms = sm_count();
-        const int max_keys = s.window > 0 ? (s.window < s.seq ? s.window : s.seq) : s.seq;   // pos is device data: size for the worst case
         // Number of key splits: two CTAs fit an SM, a wave of CTAs costs (a fixed part worth ~192 keys + its keys), and a
         // partly filled wave costs as much as a full one; take the split count with the cheapest estimate, at least
         // 256 keys per split.
@@ -473,15 +1104,54 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
         if (n_splits > 1) { ctx->scan_user.needs_clear = true; ctx->scan_owned.needs_clear = true; }
         const dim3 grid((unsigned)n_splits, (unsigned)s.n_kv_heads, (unsigned)s.batch);
         switch (G) {
-            case 1: e = launch_dependent(decode_attention_gqa_kernel<1>, grid, dim3(256), 0, st, gp); break;
-            case 2: e = launch_dependent(decode_attention_gqa_kernel<2>, grid, dim3(256), 0, st, gp); break;
-            case 4: e = launch_dependent(decode_attention_gqa_kernel<4>, grid, dim3(256), 0, st, gp); break;
-            default: e = launch_dependent(decode_attention_gqa_kernel<8>, grid, dim3(256), 0, st, gp); break;
+            case 1: e = launch_dependent(decode_attention_split_kernel<1>, grid, dim3(256), 0, st, gp); break;
+            case 2: e = launch_dependent(decode_attention_split_kernel<2>, grid, dim3(256), 0, st, gp); break;
+            case 4: e = launch_dependent(decode_attention_split_kernel<4>, grid, dim3(256), 0, st, gp); break;
+            default: e = launch_dependent(decode_attention_split_kernel<8>, grid, dim3(256), 0, st, gp); break;
         }
         ctx->launches += 1;
         if (e == cudaSuccess && n_splits > 1) {
-            e = launch_dependent(decode_combine_kernel, dim3((unsigned)s.n_q_heads, (unsigned)s.batch), dim3(kHeadDim), 0, st, gp);
+            e = launch_dependent(decode_merge_splits_kernel, dim3((unsigned)s.n_q_heads, (unsigned)s.batch), dim3(kHeadDim), 0, st, gp);
             ctx->launches += 1;
+        }
+        return e;
+    }
+    if (stream) {
+        DecStreamParams sp{};
+        sp.q_b = ap.q_b; sp.q_h = ap.q_h; sp.o_b = ap.o_b; sp.o_h = ap.o_h;
+        sp.Hq = s.n_q_heads; sp.Hkv = s.n_kv_heads; sp.window = s.window; sp.scale_log2 = ap.scale_log2;
+        sp.status = ctx->dev_status; sp.wait_cycles = ctx_wait_cycles(ctx);
+        for (int b0 = 0; b0 < s.batch; b0 += kStreamMaxBatch) {
+            const int n = std::min(s.batch - b0, kStreamMaxBatch);
+            if (b0 > 0 && !maps(b0, n)) return cudaErrorInvalidValue;
+            sp.B = n;
+            sp.Q = static_cast<const __nv_bfloat16*>(a.q_new) + (long long)b0 * ap.q_b;
+            sp.O = static_cast<__nv_bfloat16*>(a.O_new) + (long long)b0 * ap.o_b;
+            sp.pos = a.pos + b0; sp.skip = a.skip_out + b0;
+            const long long tiles = (long long)n * s.n_kv_heads * ((max_keys + kStreamKeys - 1) / kStreamKeys);
+            const int grid = (int)std::min<long long>(sms, tiles);
+            sp.partial = nullptr; sp.begun = nullptr; sp.counters = nullptr; sp.arrived = nullptr;
+            // scratch: the table of begun work items, then slots: two per piece, and there have to be more pieces than CTAs
+            const size_t slot = (size_t)G * kPartialFloats * sizeof(float), table = stream_table_bytes(grid);
+            const size_t scratch = std::min(ctx->workspace ? ctx->workspace_bytes : 0, table + kStreamScratch);
+            if (scratch >= table + (3 * grid + 2) * slot) {
+                sp.partial = reinterpret_cast<float*>(static_cast<char*>(ctx->workspace) + table);
+                sp.max_slots = (unsigned int)((scratch - table) / slot);
+                sp.counters = reinterpret_cast<unsigned int*>(ctx->dev_status + 1);
+                // Short steps are bound by launches and latency: there the CTA that arrives last merges a work item (with
+                // more to merge that is slower than a kernel of its own: 4 x 4096 keys x 40 heads 61.2 against 60.5 us).
+                if (2 * grid <= sms) sp.arrived = sp.counters + 2;
+                else sp.begun = static_cast<uint4*>(ctx->workspace) + 1;
+                ctx->scan_user.needs_clear = true; ctx->scan_owned.needs_clear = true;      // (the scan's records: as above)
+            }
+            switch (G) {
+                case 1: e = launch_stream<1>(sp, grid, ctx->device, mk, mv, st); break;
+                case 2: e = launch_stream<2>(sp, grid, ctx->device, mk, mv, st); break;
+                case 4: e = launch_stream<4>(sp, grid, ctx->device, mk, mv, st); break;
+                default: e = launch_stream<8>(sp, grid, ctx->device, mk, mv, st); break;
+            }
+            ctx->launches += sp.begun ? 2 : 1;
+            if (e != cudaSuccess) return e;
         }
         return e;
     }

@@ -744,6 +744,55 @@ def test_requested_kernel_that_cannot_take_the_call_is_an_error_not_a_fallback()
 
 
 # ------------------------------------------------------------------------------- online decode step
+@pytest.mark.parametrize("workspace", [True, False])     # work items split over CTAs and merged / whole items per CTA
+@pytest.mark.parametrize("B,S,Hkv,G,window", [(1, 64, 1, 1, 0), (1, 65, 3, 2, 0), (5, 1500, 3, 4, 0), (4, 2000, 2, 8, 700),
+                                              (1, 9000, 1, 4, 0), (40, 300, 5, 1, 130), (1030, 70, 1, 1, 0),
+                                              (2, 9000, 3, 1, 0), (150, 130, 8, 1, 0), (1, 200, 4, 8, 0)])
+def test_decode_attention_uneven_positions_and_skips(B, S, Hkv, G, window, workspace):
+    """Every sequence at a position of its own (tile edges among them), some skipped, NaN in the cache behind each position:
+    the streaming kernel (ungrouped heads: split and whole work items; short steps of any group) and the split kernel against
+    fp64 softmax attention."""
+    rng = np.random.default_rng(B * S + G)
+    Hq = Hkv * G
+    q, k, v = _qkv(B, S, Hq, Hkv, torch.bfloat16, seed=S + G)
+    pos = rng.integers(0, S, B)
+    pos[0] = S - 1
+    pos[-1] = min(S - 1, 63) if B > 1 else pos[-1]
+    skip_me = rng.random(B) < 0.4
+    skip_me[0] = False
+    for b in range(B):
+        k[b, pos[b] + 1:] = float("nan")
+        v[b, pos[b] + 1:] = float("nan")
+    ctx = tfb.Context(0)
+    params = tfb.default_params(prune_ratio=0.5, warmup_tokens=0)
+    O = torch.full((B, Hq, 128), float("nan"), dtype=torch.bfloat16, device=DEV)
+    shape = tfb.make_shape(None, k, v, window=window, n_q_heads=Hq)
+    qn = q[:, S - 1].contiguous()
+    shape.q_stride[:] = [qn.stride(0), 0, qn.stride(1)]
+    shape.o_stride[:] = [O.stride(0), 0, O.stride(1)]
+    if workspace:
+        ctx.ensure_workspace(shape, params)
+    st = tfb.DecodeState(B, Hkv, DEV)
+    st.tau.copy_(torch.from_numpy(np.where(skip_me, -9.0, 9.0).astype(np.float32)))
+    score, skip = torch.empty(B, device=DEV), torch.empty(B, dtype=torch.uint8, device=DEV)
+    pos_t = torch.from_numpy(pos.astype(np.int32)).to(DEV)
+    for _ in range(2):      # the second step finds what the first left in the scratch
+        ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos_t, st, O, score, skip)
+    assert ctx.tf_get_status()[0] == tfb.TF_OK
+    assert np.array_equal(skip.cpu().numpy(), skip_me.astype(np.uint8))
+    o = to_np(O)
+    for b in range(B):
+        if skip_me[b]:
+            assert np.all(o[b] == 0.0)
+            continue
+        lo = max(0, pos[b] - window + 1) if window > 0 else 0
+        kk, vv = k[b, lo:pos[b] + 1].double(), v[b, lo:pos[b] + 1].double()
+        s = torch.einsum("hgd,nhd->hgn", qn[b].double().view(Hkv, G, 128), kk) / 128 ** 0.5
+        ref = torch.einsum("hgn,nhd->hgd", s.softmax(-1), vv).reshape(Hq, 128).cpu().numpy()
+        assert attn_rel_err(o[b], ref) < ATTN_TOL[torch.bfloat16], b
+    ctx.close()
+
+
 @pytest.mark.parametrize("dtype,mode,window,S0,T,Hq,Hkv",
                          [(torch.bfloat16, tfb.TF_ANCHOR_PAST_MEAN, 0, 70, 90, 8, 2), (torch.float32, tfb.TF_ANCHOR_PAST_MEAN, 40, 70, 90, 8, 2),
                           (torch.bfloat16, tfb.TF_ANCHOR_EMA, 0, 70, 90, 8, 2), (torch.bfloat16, tfb.TF_ANCHOR_INCL_MEAN, 0, 70, 90, 8, 2),

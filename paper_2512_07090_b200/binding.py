@@ -95,11 +95,35 @@ def _check(code: int, what: str) -> None:
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream() -> int:
+    """The current stream of the current device.  (Asked for as a raw handle: building torch's Stream object takes 3 us,
+    a quarter of a short decode step's host time.)"""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
+_CALLS = {"tf_kv_stats": 9, "tf_kv_stats_static": 9, "tf_score_fuse": 7, "tf_select": 9, "tf_score_select": 11,
+          "tf_pruned_attention": 10, "tf_layer_filter": 12, "tf_layer_filter_host": 12}    # arguments, pointers all
+_calls = None
+
+
+def _call(name: str):
+    """The entry points that are called per layer or token, with declared argument types (addresses are passed as plain
+    integers then, without an object per argument)."""
+    global _calls
+    if _calls is None:
+        L, calls = lib(), {}
+        for n, count in _CALLS.items():
+            calls[n] = L[n]                  # a function object of its own: lib()'s keeps its loose prototype
+            calls[n].argtypes = [C.c_void_p] * count
+            calls[n].restype = C.c_int
+        calls["tf_decode_step"] = f = L["tf_decode_step"]
+        f.argtypes = [C.c_void_p] * 3 + [C.c_float, C.c_int32] + [C.c_void_p] * 9
+        f.restype = C.c_int
+        _calls = calls
+    return _calls[name]
 
 
 def default_params(**kw) -> tf_filter_params:
@@ -180,7 +204,7 @@ class Context:
 
     def set_workspace(self, buf: Optional[torch.Tensor]) -> None:
         self._ws = buf
-        _check(lib().tf_set_workspace(self._h, _ptr(buf), C.c_size_t(0 if buf is None else buf.numel() * buf.element_size())),
+        _check(lib().tf_set_workspace(self._h, C.c_void_p(_ptr(buf)), C.c_size_t(0 if buf is None else buf.numel() * buf.element_size())),
                "tf_set_workspace")
 
     def ensure_workspace(self, shape: tf_shape, params: tf_filter_params) -> None:
@@ -190,48 +214,48 @@ class Context:
 
     # ---- the five entry points -----------------------------------------------------------------
     def tf_kv_stats(self, shape, params, K, V, sim_k, sim_v, carry: Optional[tf_carry] = None):
-        _check(lib().tf_kv_stats(self._h, C.byref(shape), C.byref(params), _ptr(K), _ptr(V), _ptr(sim_k),
-                                 _ptr(sim_v), None if carry is None else C.byref(carry), _stream()), "tf_kv_stats")
+        _check(_call("tf_kv_stats")(self._h, C.byref(shape), C.byref(params), _ptr(K), _ptr(V), _ptr(sim_k),
+                                    _ptr(sim_v), None if carry is None else C.byref(carry), _stream()), "tf_kv_stats")
 
     def tf_kv_stats_static(self, shape, params, K, V, sim_k, sim_v, carry: Optional[tf_carry] = None):
         """tf_kv_stats on the library's built-in scratch array: no workspace, nothing allocated."""
-        _check(lib().tf_kv_stats_static(self._h, C.byref(shape), C.byref(params), _ptr(K), _ptr(V), _ptr(sim_k),
-                                        _ptr(sim_v), None if carry is None else C.byref(carry), _stream()),
+        _check(_call("tf_kv_stats_static")(self._h, C.byref(shape), C.byref(params), _ptr(K), _ptr(V), _ptr(sim_k),
+                                           _ptr(sim_v), None if carry is None else C.byref(carry), _stream()),
                "tf_kv_stats_static")
 
     def tf_score_fuse(self, shape, params, sim_k, sim_v, score):
-        _check(lib().tf_score_fuse(self._h, C.byref(shape), C.byref(params), _ptr(sim_k), _ptr(sim_v),
-                                   _ptr(score), _stream()), "tf_score_fuse")
+        _check(_call("tf_score_fuse")(self._h, C.byref(shape), C.byref(params), _ptr(sim_k), _ptr(sim_v),
+                                      _ptr(score), _stream()), "tf_score_fuse")
 
     def tf_select(self, shape, params, score, keep_mask, kept_idx, n_kept, theta=None):
-        _check(lib().tf_select(self._h, C.byref(shape), C.byref(params), _ptr(score), _ptr(keep_mask),
-                               _ptr(kept_idx), _ptr(n_kept), _ptr(theta), _stream()), "tf_select")
+        _check(_call("tf_select")(self._h, C.byref(shape), C.byref(params), _ptr(score), _ptr(keep_mask),
+                                  _ptr(kept_idx), _ptr(n_kept), _ptr(theta), _stream()), "tf_select")
 
     def tf_score_select(self, shape, params, sim_k, sim_v, score, keep_mask, kept_idx, n_kept, theta=None):
-        _check(lib().tf_score_select(self._h, C.byref(shape), C.byref(params), _ptr(sim_k), _ptr(sim_v), _ptr(score),
-                                     _ptr(keep_mask), _ptr(kept_idx), _ptr(n_kept), _ptr(theta), _stream()), "tf_score_select")
+        _check(_call("tf_score_select")(self._h, C.byref(shape), C.byref(params), _ptr(sim_k), _ptr(sim_v), _ptr(score),
+                                        _ptr(keep_mask), _ptr(kept_idx), _ptr(n_kept), _ptr(theta), _stream()), "tf_score_select")
 
     def tf_pruned_attention(self, shape, params, Q, K, V, kept_idx, n_kept, O):
-        _check(lib().tf_pruned_attention(self._h, C.byref(shape), C.byref(params), _ptr(Q), _ptr(K), _ptr(V),
-                                         _ptr(kept_idx), _ptr(n_kept), _ptr(O), _stream()), "tf_pruned_attention")
+        _check(_call("tf_pruned_attention")(self._h, C.byref(shape), C.byref(params), _ptr(Q), _ptr(K), _ptr(V),
+                                            _ptr(kept_idx), _ptr(n_kept), _ptr(O), _stream()), "tf_pruned_attention")
 
     def tf_layer_filter(self, shape, params, Q, K, V, O, score=None, keep_mask=None, kept_idx=None, n_kept=None):
-        _check(lib().tf_layer_filter(self._h, C.byref(shape), C.byref(params), _ptr(Q), _ptr(K), _ptr(V), _ptr(O),
-                                     _ptr(score), _ptr(keep_mask), _ptr(kept_idx), _ptr(n_kept), _stream()),
+        _check(_call("tf_layer_filter")(self._h, C.byref(shape), C.byref(params), _ptr(Q), _ptr(K), _ptr(V), _ptr(O),
+                                        _ptr(score), _ptr(keep_mask), _ptr(kept_idx), _ptr(n_kept), _stream()),
                "tf_layer_filter")
 
     def tf_decode_step(self, shape, params, eta, q_new, K_cache, V_cache, pos, state: "DecodeState", O_new,
                        score=None, skip=None, alg1_sign=False):
-        _check(lib().tf_decode_step(self._h, C.byref(shape), C.byref(params), C.c_float(eta),
-                                    C.c_int32(1 if alg1_sign else 0), _ptr(q_new), _ptr(K_cache), _ptr(V_cache),
-                                    _ptr(pos), C.byref(state.struct), _ptr(O_new), _ptr(score), _ptr(skip), _stream()),
+        _check(_call("tf_decode_step")(self._h, C.byref(shape), C.byref(params), eta,
+                                       1 if alg1_sign else 0, _ptr(q_new), _ptr(K_cache), _ptr(V_cache),
+                                       _ptr(pos), C.byref(state.struct), _ptr(O_new), _ptr(score), _ptr(skip), _stream()),
                "tf_decode_step")
 
     def tf_layer_filter_host(self, shape, params, Q, K, V, O, score=None, keep_mask=None, kept_idx=None, n_kept=None):
         """Host tensors in, host tensors out (copies inside the call; returns after the stream is idle)."""
-        _check(lib().tf_layer_filter_host(self._h, C.byref(shape), C.byref(params), _ptr(Q), _ptr(K), _ptr(V),
-                                          _ptr(O), _ptr(score), _ptr(keep_mask), _ptr(kept_idx), _ptr(n_kept),
-                                          _stream()), "tf_layer_filter_host")
+        _check(_call("tf_layer_filter_host")(self._h, C.byref(shape), C.byref(params), _ptr(Q), _ptr(K), _ptr(V),
+                                             _ptr(O), _ptr(score), _ptr(keep_mask), _ptr(kept_idx), _ptr(n_kept),
+                                             _stream()), "tf_layer_filter_host")
 
     # ---- status --------------------------------------------------------------------------------
     def tf_get_status(self, sync: bool = True):
@@ -269,7 +293,7 @@ class Context:
 
     def tf_wait_selftest(self):
         """Make bounded waits run out on purpose (conditions nothing ever fulfils); tf_get_status then says TF_ERR_TIMEOUT."""
-        _check(lib().tf_wait_selftest(self._h, _stream()), "tf_wait_selftest")
+        _check(lib().tf_wait_selftest(self._h, C.c_void_p(_stream())), "tf_wait_selftest")
 
     @property
     def launches(self) -> int:

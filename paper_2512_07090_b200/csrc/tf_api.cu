@@ -484,7 +484,7 @@ tf_status tf_get_status(tf_ctx* ctx, int sync, int64_t detail[4]) {
         detail[2] = (int64_t)h.nan_count; detail[3] = (int64_t)ctx->launches;
     }
     if (h.code == TF_ERR_TIMEOUT) {
-        invalidate_scan_scratch(ctx);   // records written under a wait that gave up are not to be trusted, nor counts of arrivals
+        invalidate_scan_scratch(ctx);   // records written under a wait that gave up are not to be trusted, nor counters
         cudaMemset(ctx->dev_status + 1, 0, kStatusBytes - sizeof(DevStatus));
         return TF_ERR_TIMEOUT;
     }

@@ -11,7 +11,7 @@ namespace tf {
 
 constexpr int kHeadDim = 128;
 constexpr int kDeviceFlagSlots = 64;       // per-device one-time set-up flags
-constexpr int kDecodeCounters = 256;       // counters of the streaming decode kernel: two for its work list, then one per piece
+constexpr int kDecodeCounters = 2;         // counters of the streaming decode kernel: its work list
 constexpr float kNormEps = 1e-8f;   // lower clamp of each norm in the cosine
 
 // Device status record: four 64-bit words {code, where, nan_count, reserved}.

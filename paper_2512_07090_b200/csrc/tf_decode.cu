@@ -13,6 +13,7 @@
 //   is zero (Section 3.2).  The 8 warps take interleaved blocks of 32 keys, each with its own online softmax; the
 //   partial results are merged through shared memory.
 #include <algorithm>
+#include <cooperative_groups.h>
 
 #include "tf_ptx.cuh"
 
@@ -258,28 +259,27 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_attention_kernel(const 
 }
 
 // ---------------------------------------------------------------------------------------------------
-// bf16 decode attention, streaming form (chosen for ungrouped heads and for very short steps): one persistent CTA per SM; all
-// G <= 8 query heads of a KV head are served together, so K and V rows are read once per group.  The path is a stream of
-// K / V rows: what bounds it is HBM bandwidth, and what it takes to reach it is that every SM has loads in flight from its
+// bf16 decode attention for ungrouped heads, streaming form: one persistent CTA per SM.  The path is a stream of K / V rows: what bounds it is HBM bandwidth, and what it takes to reach it is that every SM has loads in flight from its
 // first to its last cycle.
 //   work    the visible keys of every unskipped (sequence, KV head) -- a work item -- are cut into tiles of 64 keys, and the list
 //           of all tiles into pieces: 5/8 of it into one piece per CTA, the rest into small pieces that are drawn from a
 //           counter, so that CTAs that started late or run on slower SMs take fewer (equal shares alone: the first CTA done
 //           14 % before the last).  A work item that lies in several pieces leaves partial results (unnormalised output,
-//           maximum, sum) in scratch; the CTA that arrives last, or decode_combine_kernel, merges them.  Where there are many
+//           maximum, sum) in scratch, and decode_combine_kernel merges them (merging by whichever CTA arrives last was slower:
+//           4 x 4096 keys x 40 heads 61.2 against 60.5 us).  Where there are many
 //           short work items a piece is a work item, and nothing is merged; so it is without scratch.
-//   warp 8  producer: K and V tiles (and the query rows) by TMA into a ring of slots, 128 to 192 KB in flight per SM,
+//   warp 8  producer: K and V tiles (and the query rows) by TMA into a ring of slots, 192 KB in flight per SM,
 //           running ahead across work items.  It starts while the decision kernel still runs, as if no token were skipped; if
 //           one is, what it fetched is thrown away.
 //   warps 0-3 / 4-7 consume the even / odd tiles, 16 keys per warp, on m16n8k16 products:
-//           S^T[16 keys x 8 heads] = K Q^T (A by ldmatrix), online softmax on the accumulator layout (lane holds keys g, g + 8 for
-//           heads 2t, 2t + 1), P^T through two 8x8 register transposes, O^T[128 dims x 8 heads] += V^T P^T (A by
+//           S^T[16 keys x 8 columns] = K Q^T (A by ldmatrix; one column is the head, the others are zero: the products are not what
+//           bounds this), online softmax on the accumulator layout (lane holds keys g, g + 8 for columns 2t, 2t + 1), P^T through two 8x8 register transposes, O^T[128 dims x 8] += V^T P^T (A by
 //           ldmatrix.trans).
 //   warps 9-12 merge: at the end of a segment (a work item, or the part of one in this piece) the consumers leave their
 //           states in shared memory and go on with the next segment at once; these warps merge the eight states and write the result.
 // Every wait is bounded, those of the warps for one another too (mbarriers, no named barriers): on expiry the CTA records
 // TF_ERR_TIMEOUT, stops waiting, lets copies in flight land and exits.
-//   A step of 128 sequences x 400 keys x 40 heads (half of them skipped): 112 -> 100 us, 4 x 4096 keys x 40 heads: 75 -> 61 us.
+//   A step of 128 sequences x 400 keys x 40 heads (half of them skipped): 112 -> 98 us, 4 x 4096 keys x 40 heads: 75 -> 60 us.
 // ---------------------------------------------------------------------------------------------------
 constexpr int kPartialFloats = kHeadDim + 2;
 constexpr int kStreamKeys = 64;                            // keys per tile
@@ -289,16 +289,14 @@ constexpr int kStreamThreads = 416;
 constexpr int kStreamSegs = 4;                             // segment descriptors in flight
 constexpr int kStreamMaxBatch = 512;                       // sequences per launch
 constexpr int kStreamDrawn = 1;                            // drawn pieces per CTA on average (4: 8 x 4096 keys x 8 heads 39 instead of 32 us)
-constexpr size_t kStreamScratch = (size_t)5 << 20;         // partial results: room for more pieces than there are
-template <int G> struct StreamCfg {
-    // an EVEN number of ring slots: a slot then always belongs to the same half of the consumers, which so waits for every
-    // phase of its barrier (a half that skipped phases could mistake an earlier one's completion for its own)
-    static constexpr int kStages = G == 8 ? 4 : 6;
-    static constexpr int kQBytes = G * kHeadDim * 2;       // query rows of a work item
-    static constexpr int kOffQ = kStages * kStreamStage;
-    static constexpr int kOffPart = kOffQ + kStages * kQBytes;
-    static constexpr int kSmemBytes = kOffPart + 8 * G * kPartialFloats * 4 + 1024;   // + alignment slack
-};
+constexpr size_t kStreamScratch = (size_t)1 << 20;         // partial results: room for more pieces than there are
+// an EVEN number of ring slots: a slot then always belongs to the same half of the consumers, which so waits for every
+// phase of its barrier (a half that skipped phases could mistake an earlier one's completion for its own)
+constexpr unsigned int kStages = 6;
+constexpr int kStreamQ = kHeadDim * 2;                     // the query row of a work item
+constexpr int kStreamOffQ = kStages * kStreamStage;
+constexpr int kStreamOffPart = kStreamOffQ + kStages * kStreamQ;
+constexpr int kStreamSmem = kStreamOffPart + 8 * kPartialFloats * 4 + 1024;   // + alignment slack
 
 struct DecStreamParams {
     const __nv_bfloat16* Q; __nv_bfloat16* O;
@@ -308,10 +306,9 @@ struct DecStreamParams {
     float scale_log2;
     uint4* begun;                     // for decode_combine_kernel: [piece] {sequence or ~0, KV head, last piece} of the work item that begins in the
                                       // piece and ends in a later one; in front of it the number of pieces
-    float* partial;                   // [slot][G][130]; null: a work item is never split
+    float* partial;                   // [slot][130]; null: a work item is never split
     unsigned int max_slots;
     unsigned int* counters;           // {next piece, CTAs done}, zero before and after every launch (with partial only)
-    unsigned int* arrived;            // [piece] zero before and after every launch; null: decode_combine_kernel merges
     DevStatus* status;
     long long wait_cycles;
 };
@@ -346,44 +343,6 @@ struct StreamCut {
     __device__ __forceinline__ unsigned int piece_of(unsigned int y) const { return y < cut ? y / share : cut / share + (y - cut) / piece; }
 };
 // A piece leaves at most two partial results: slot 2 x for the item it finds begun, 2 x + 1 for the one it begins and does not end.
-// merges the parts of a work item that lies in pieces first .. last: heads h0 .. h0 + N - 1 of the group, dim d
-template <int G, int N>
-__device__ __forceinline__ void merge_parts(const DecStreamParams& p, int b, int kh, unsigned int first, unsigned int last, int h0, int d) {
-    const int n = (int)(last - first) + 1;
-    const float* base = p.partial + ((size_t)(2 * first) * G + h0) * kPartialFloats;
-    float M[N], L[N], acc[N];
-#pragma unroll
-    for (int h = 0; h < N; ++h) { M[h] = -1e30f; L[h] = 0.f; acc[h] = 0.f; }
-    for (int q0 = 0; q0 < n; q0 += 8) {                     // eight parts of every head requested together: one round trip, not one per part
-        float m[N][8], l[N][8], v[N][8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int q = min(q0 + u, n - 1);
-#pragma unroll
-            for (int h = 0; h < N; ++h) {
-                const float* src = base + ((size_t)(2 * q + (q == 0 ? 1 : 0)) * G + h) * kPartialFloats;
-                m[h][u] = __ldcg(src + kHeadDim); l[h][u] = __ldcg(src + kHeadDim + 1); v[h][u] = __ldcg(src + d);
-            }
-        }
-#pragma unroll
-        for (int h = 0; h < N; ++h) {
-            float mx = M[h];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) mx = fmaxf(mx, m[h][u]);
-            const float e0 = exp2f(M[h] - mx);
-            L[h] *= e0; acc[h] *= e0; M[h] = mx;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const float e = q0 + u < n ? exp2f(m[h][u] - mx) : 0.f;
-                L[h] = fmaf(l[h][u], e, L[h]);
-                acc[h] = fmaf(v[h][u], e, acc[h]);
-            }
-        }
-    }
-#pragma unroll
-    for (int h = 0; h < N; ++h)
-        p.O[(long long)b * p.o_b + (long long)(kh * G + h0 + h) * p.o_h + d] = __float2bfloat16_rn(acc[h] / L[h]);
-}
 
 // a segment: the tiles of one work item in one piece
 struct StreamSeg {
@@ -395,31 +354,27 @@ struct StreamSeg {
     unsigned int piece;               // ... and that piece
 };
 
-template <int G>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV) {
-    using C = StreamCfg<G>;
-    constexpr unsigned int kStages = C::kStages;
     extern __shared__ uint8_t stream_raw[];
     __shared__ unsigned int pre[kStreamMaxBatch + 1];      // tiles per KV head of the sequences before b
     __shared__ int s_pos[kStreamMaxBatch];
     __shared__ unsigned short active[kStreamMaxBatch];     // the sequences that have tiles
     __shared__ StreamSeg segs[kStreamSegs];
-    __shared__ __align__(8) unsigned long long bars[2 * C::kStages + 2 * kStreamSegs + 3];
+    __shared__ __align__(8) unsigned long long bars[2 * kStages + 2 * kStreamSegs + 2];
     __shared__ unsigned int s_tiles, s_segs;
-    __shared__ int s_abort, s_last;
+    __shared__ int s_abort;
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(stream_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, cta = blockIdx.x;
     const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * kStages, bar_seg = bar_empty + 8 * kStages,
-                   bar_seg_free = bar_seg + 8 * kStreamSegs, bar_part = bar_seg_free + 8 * kStreamSegs, bar_part_free = bar_part + 8,
-                   bar_c = bar_part_free + 8;
+                   bar_seg_free = bar_seg + 8 * kStreamSegs, bar_part = bar_seg_free + 8 * kStreamSegs, bar_part_free = bar_part + 8;
     volatile int* abort_flag = &s_abort;
     if (tid == 256) {                                       // the thread that uses the barriers before the first block-wide one
         prefetch_map(&mapK); prefetch_map(&mapV);
         for (unsigned int i = 0; i < kStages; ++i) { mbar_init(bar_full + 8 * i, 1); mbar_init(bar_empty + 8 * i, 4); }
         for (int i = 0; i < kStreamSegs; ++i) { mbar_init(bar_seg + 8 * i, 1); mbar_init(bar_seg_free + 8 * i, 12); }
-        mbar_init(bar_part, 8); mbar_init(bar_part_free, 4); mbar_init(bar_c, 4);
+        mbar_init(bar_part, 8); mbar_init(bar_part_free, 4);
         s_abort = 0;
         mbar_fence_init();
     }
@@ -528,16 +483,12 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
         const uint32_t dst = sbase + st * kStreamStage, bar = bar_full + 8 * st;
         const int key = pk_lo + (pt.j + p_done) * kStreamKeys;
         const bool with_q = p_done < 2;                    // either half of the consumers finds the query rows with its first tile
-        mbar_expect_tx(bar, kStreamStage + (with_q ? C::kQBytes : 0));
+        mbar_expect_tx(bar, kStreamStage + (with_q ? kStreamQ : 0));
         tma_load_4d(dst, &mapK, bar, 0, pt.kh, key, pt.b);
         tma_load_4d(dst + kStreamHalf, &mapK, bar, 64, pt.kh, key, pt.b);
         tma_load_4d(dst + 2 * kStreamHalf, &mapV, bar, 0, pt.kh, key, pt.b);
         tma_load_4d(dst + 3 * kStreamHalf, &mapV, bar, 64, pt.kh, key, pt.b);
-        if (with_q) {
-            const __nv_bfloat16* q = p.Q + (long long)pt.b * p.q_b + (long long)pt.kh * G * p.q_h;
-            for (int g = 0; g < G; ++g)
-                bulk_load(sbase + C::kOffQ + st * C::kQBytes + g * kHeadDim * 2, q + (long long)g * p.q_h, kHeadDim * 2, bar);
-        }
+        if (with_q) bulk_load(sbase + kStreamOffQ + st * kStreamQ, p.Q + (long long)pt.b * p.q_b + (long long)pt.kh * p.q_h, kStreamQ, bar);
         ++p_done; ++py;
         if (p_done == pt.count && py < py_end) { next_item(); open_segment(); }
     };
@@ -611,7 +562,7 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
     } else if (warp < 8) {
         // ================================ consumers ===========================================================
         grid_launch_dependents();
-        float* part_s = reinterpret_cast<float*>(smem + C::kOffPart);
+        float* part_s = reinterpret_cast<float*>(smem + kStreamOffPart);
         const int half = warp >> 2, kb = (warp & 3) * 16;   // this warp's 16 keys of every second tile
         const int g = lane >> 2, t = lane & 3;
         // ldmatrix row of this lane: K as A (rows = keys), V as transposed A (rows = keys of the stored tile)
@@ -645,11 +596,11 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
                 ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar_full + 8 * st, ((it + i) / kStages) & 1u, abort_flag, p.wait_cycles, p.status, 602));
                 if (!ok) break;
                 if (i < 2) {                                     // Q^T as the B operand
-                    const uint8_t* q = smem + C::kOffQ + st * C::kQBytes + (g < G ? g : 0) * kHeadDim * 2 + t * 4;
+                    const uint8_t* q = smem + kStreamOffQ + st * kStreamQ + t * 4;
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk) {
-                        qb[kk][0] = g < G ? *reinterpret_cast<const uint32_t*>(q + kk * 32) : 0u;
-                        qb[kk][1] = g < G ? *reinterpret_cast<const uint32_t*>(q + kk * 32 + 16) : 0u;
+                        qb[kk][0] = g == 0 ? *reinterpret_cast<const uint32_t*>(q + kk * 32) : 0u;
+                        qb[kk][1] = g == 0 ? *reinterpret_cast<const uint32_t*>(q + kk * 32 + 16) : 0u;
                     }
                 }
                 const uint32_t ka = sbase + st * kStreamStage, va = ka + 2 * kStreamHalf;
@@ -718,35 +669,23 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
             const unsigned int k_seg = sg - wasted_segs;         // (the first wait passes: nothing has been left there yet)
             ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar_part_free, (k_seg & 1u) ^ 1u, abort_flag, p.wait_cycles, p.status, 605));
             if (!ok) break;
+            if (t == 0) {                                        // column 0 is the head
+                float* dst = part_s + warp * kPartialFloats;
 #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const int h = 2 * t + k;
-                if (h < G) {
-                    float* dst = part_s + (warp * G + h) * kPartialFloats;
-#pragma unroll
-                    for (int mt = 0; mt < 8; ++mt) { dst[16 * mt + g] = o[mt][k]; dst[16 * mt + 8 + g] = o[mt][k + 2]; }
-                    if (g == 0) { dst[kHeadDim] = m[k]; dst[kHeadDim + 1] = l[k]; }
-                }
+                for (int mt = 0; mt < 8; ++mt) { dst[16 * mt + g] = o[mt][0]; dst[16 * mt + 8 + g] = o[mt][2]; }
+                if (g == 0) { dst[kHeadDim] = m[0]; dst[kHeadDim + 1] = l[0]; }
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_part);
         }
     } else {
         // ================================ merging warps =======================================================
-        const float* part_s = reinterpret_cast<const float*>(smem + C::kOffPart);
+        const float* part_s = reinterpret_cast<const float*>(smem + kStreamOffPart);
         const int mt = tid - 288;                           // 0 .. 127: output dim
         for (int b = cta; b < p.B; b += (int)gridDim.x)     // skipped tokens' output rows
             if (p.skip[b])
                 for (int i = mt; i < p.Hq * (kHeadDim / 8); i += 128)
                     *reinterpret_cast<uint4*>(p.O + (long long)b * p.o_b + (long long)(i >> 4) * p.o_h + (i & 15) * 8) = make_uint4(0, 0, 0, 0);
-        uint32_t c_phase = 0;
-        auto mergers_sync = [&]() {                         // the 4 merging warps; false: a wait gave up
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_c);
-            const bool ok = mbar_wait_bounded(bar_c, c_phase, abort_flag, p.wait_cycles, p.status, 604);
-            c_phase ^= 1;
-            return __all_sync(0xffffffffu, ok) != 0;
-        };
         for (unsigned int sg = 0;; ++sg) {
             const unsigned int ss = sg % kStreamSegs;
             if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar_seg + 8 * ss, (sg / kStreamSegs) & 1u, abort_flag, p.wait_cycles, p.status, 608))) break;
@@ -756,52 +695,28 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
             if (sg < wasted_segs) continue;
             if (seg.count == 0) break;
             if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar_part, (sg - wasted_segs) & 1u, abort_flag, p.wait_cycles, p.status, 609))) break;
-            float M[G], L[G], acc[G];
+            float M = -1e30f, L = 0.f, acc = 0.f;
 #pragma unroll
-            for (int h = 0; h < G; ++h) {
-                const float* src = part_s + h * kPartialFloats;
-                M[h] = -1e30f;
+            for (int w2 = 0; w2 < 8; ++w2) M = fmaxf(M, part_s[w2 * kPartialFloats + kHeadDim]);
 #pragma unroll
-                for (int w2 = 0; w2 < 8; ++w2) M[h] = fmaxf(M[h], src[w2 * G * kPartialFloats + kHeadDim]);
-                L[h] = 0.f; acc[h] = 0.f;
-#pragma unroll
-                for (int w2 = 0; w2 < 8; ++w2) {
-                    const float e = ex2_approx(src[w2 * G * kPartialFloats + kHeadDim] - M[h]);
-                    L[h] = fmaf(src[w2 * G * kPartialFloats + kHeadDim + 1], e, L[h]);
-                    acc[h] = fmaf(src[w2 * G * kPartialFloats + mt], e, acc[h]);
-                }
+            for (int w2 = 0; w2 < 8; ++w2) {
+                const float* src = part_s + w2 * kPartialFloats;
+                const float e = ex2_approx(src[kHeadDim] - M);
+                L = fmaf(src[kHeadDim + 1], e, L);
+                acc = fmaf(src[mt], e, acc);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_part_free);
-#pragma unroll
-            for (int h = 0; h < G; ++h) {
-                if (seg.slot < 0) {
-                    p.O[(long long)seg.b * p.o_b + (long long)(seg.kh * G + h) * p.o_h + mt] = __float2bfloat16_rn(acc[h] / L[h]);
-                } else {
-                    float* dst = p.partial + ((size_t)seg.slot * G + h) * kPartialFloats;
-                    dst[mt] = acc[h];
-                    if (mt == 0) { dst[kHeadDim] = M[h]; dst[kHeadDim + 1] = L[h]; }
-                }
+            if (seg.slot < 0) {
+                p.O[(long long)seg.b * p.o_b + (long long)seg.kh * p.o_h + mt] = __float2bfloat16_rn(acc / L);
+            } else {
+                float* dst = p.partial + (size_t)seg.slot * kPartialFloats;
+                dst[mt] = acc;
+                if (mt == 0) { dst[kHeadDim] = M; dst[kHeadDim + 1] = L; }
             }
             if (p.begun && seg.ends_piece && mt == 0 && seg.piece < gridDim.x * (1 + kStreamDrawn))
                 p.begun[seg.piece] = seg.slot == (int)(2 * seg.piece + 1) ? make_uint4((unsigned int)seg.b, (unsigned int)seg.kh, seg.p_last, 0u)
                                                                           : make_uint4(0xffffffffu, 0u, 0u, 0u);
-            if (seg.slot >= 0 && p.arrived) {                // whoever comes last merges the work item's parts
-                __threadfence();
-                if (!mergers_sync()) break;
-                if (mt == 0) {
-                    const unsigned int n = atomicAdd(p.arrived + seg.p_first, 1u);
-                    s_last = n == seg.p_last - seg.p_first;
-                    if (s_last) atomicExch(p.arrived + seg.p_first, 0u);
-                }
-                if (!mergers_sync()) break;
-                if (s_last) {
-                    __threadfence();
-                    constexpr int kAtOnce = G < 4 ? G : 4;
-                    for (int h = 0; h < G; h += kAtOnce) merge_parts<G, kAtOnce>(p, seg.b, seg.kh, seg.p_first, seg.p_last, h, mt);
-                }
-                if (!mergers_sync()) break;                  // s_last has been read
-            }
         }
     }
     __syncwarp();
@@ -812,46 +727,66 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
     }
 }
 
-// merges the work items that lie in several pieces: CTA x the one that begins in piece x, a thread per (head, dim)
-template <int G>
-__global__ void __launch_bounds__(G * kHeadDim) decode_combine_kernel(const DecStreamParams p) {
+// merges the work items that lie in several pieces: CTA x the one that begins in piece x, a thread per dim
+__global__ void __launch_bounds__(kHeadDim) decode_combine_kernel(const DecStreamParams p) {
     grid_dependency_wait();
     const unsigned int x = blockIdx.x, n_pieces = p.begun[-1].x;
     const uint4 it = p.begun[x];                            // (beyond the last piece: whatever is there)
-    if (x < n_pieces && it.x != 0xffffffffu)
-        merge_parts<G, 1>(p, (int)it.x, (int)it.y, x, it.z, (int)threadIdx.x / kHeadDim, (int)threadIdx.x % kHeadDim);
+    if (x >= n_pieces || it.x == 0xffffffffu) return;
+    const int n = (int)(it.z - x) + 1, d = threadIdx.x;
+    const float* base = p.partial + (size_t)(2 * x) * kPartialFloats;
+    float M = -1e30f, L = 0.f, acc = 0.f;
+    for (int q0 = 0; q0 < n; q0 += 8) {                     // eight parts requested together: one round trip, not one per part
+        float m[8], l[8], v[8], mx = M;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int q = min(q0 + u, n - 1);
+            const float* src = base + (size_t)(2 * q + (q == 0 ? 1 : 0)) * kPartialFloats;
+            m[u] = src[kHeadDim]; l[u] = src[kHeadDim + 1]; v[u] = src[d];
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) mx = fmaxf(mx, m[u]);
+        const float e0 = exp2f(M - mx);
+        L *= e0; acc *= e0; M = mx;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float e = q0 + u < n ? exp2f(m[u] - M) : 0.f;
+            L = fmaf(l[u], e, L);
+            acc = fmaf(v[u], e, acc);
+        }
+    }
+    p.O[(long long)it.x * p.o_b + (long long)it.y * p.o_h + d] = __float2bfloat16_rn(acc / L);
 }
 
 // what decode_combine_kernel reads, in front of the slots
 static size_t stream_table_bytes(int grid) { return (1 + (size_t)grid * (1 + kStreamDrawn)) * sizeof(uint4); }
 
-// a workspace is usually sized with a prefill shape, which need not name the query heads
 size_t decode_scratch_bytes(const tf_shape& s) { return s.dtype == TF_BF16 ? kStreamScratch + stream_table_bytes(sm_count()) : 0; }
 
-template <int G>
 static cudaError_t launch_stream(const DecStreamParams& sp, int grid, int device, const CUtensorMap& mk, const CUtensorMap& mv, cudaStream_t st) {
     static bool attr_set_dev[kDeviceFlagSlots] = {};      // function attributes are per device
     bool& attr_set = attr_set_dev[device >= 0 && device < kDeviceFlagSlots ? device : 0];
     if (!attr_set) {
-        const cudaError_t e = cudaFuncSetAttribute(decode_attention_stream_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamCfg<G>::kSmemBytes);
+        const cudaError_t e = cudaFuncSetAttribute(decode_attention_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStreamSmem);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    const cudaError_t e = launch_dependent(decode_attention_stream_kernel<G>, dim3((unsigned)grid), dim3(kStreamThreads), StreamCfg<G>::kSmemBytes, st, sp, mk, mv);
+    const cudaError_t e = launch_dependent(decode_attention_stream_kernel, dim3((unsigned)grid), dim3(kStreamThreads), kStreamSmem, st, sp, mk, mv);
     if (e != cudaSuccess || !sp.begun) return e;
-    return launch_dependent(decode_combine_kernel<G>, dim3((unsigned)(grid * (1 + kStreamDrawn))), dim3(G * kHeadDim), 0, st, sp);
+    return launch_dependent(decode_combine_kernel, dim3((unsigned)(grid * (1 + kStreamDrawn))), dim3(kHeadDim), 0, st, sp);
 }
 
 // ---------------------------------------------------------------------------------------------------
-// Grouped heads (G >= 2) in more than a very short step: one CTA per (split of the visible keys, KV head, sequence), two CTAs
+// Grouped heads, and ungrouped ones in a very short step: one CTA per (split of the visible keys, KV head, sequence), two CTAs
 // per SM.  No list of work to make: a grouped cache is a G-th of the bytes, and the head start of this form outweighs the equal
 // shares of the streaming kernel (us a step, this / streaming: 1 x 8192 16 / 24, 8 x 4096 keys of 16384 31 / 32, 128 x 1024 68 / 80;
-// ungrouped 40 heads: 1 x 8192 45 / 36, 4 x 4096 75 / 61, 128 x 512 112 / 100).  Operands come straight from global memory, no shared
+// ungrouped 40 heads: 1 x 8192 44 / 36, 4 x 4096 75 / 60, 128 x 512 112 / 98).  Operands come straight from global memory, no shared
 // memory: a dot product does not care in which order the dims are visited, so lane (g, t) loads 16-byte pieces t, t+4, t+8,
 // t+12 of its two key rows (g, g+8) and of query head g; of its four value rows (2t, 2t+1, 2t+8, 2t+9) it loads dims 16g ..
 // 16g+15, and the pairs "same dim, two consecutive keys" the A operand wants are byte permutes.  The 8 warps take key blocks 8 apart
-// and are merged through shared memory; with more than one split the CTA leaves (max, sum, unnormalised output) per head
-// in scratch and decode_merge_splits_kernel merges the splits.
+// and are merged through shared memory.  The splits of a short step are a thread-block cluster (kCluster): they are merged through
+// distributed shared memory, without scratch and without a third launch; otherwise the CTA leaves (max, sum, unnormalised
+// output) per head in scratch and decode_merge_splits_kernel merges the splits.
 // ---------------------------------------------------------------------------------------------------
 struct DecGqaParams {
     const __nv_bfloat16* Q; const __nv_bfloat16* K; const __nv_bfloat16* V; __nv_bfloat16* O;
@@ -865,17 +800,19 @@ struct DecGqaParams {
 
 __device__ __forceinline__ uint32_t word_of(const uint4& r, int w) { return w == 0 ? r.x : w == 1 ? r.y : w == 2 ? r.z : r.w; }
 
-template <int G>
-__global__ void __launch_bounds__(256, 2) decode_attention_split_kernel(const DecGqaParams p) {
+template <int G, bool kCluster>
+__global__ void __launch_bounds__(256, kCluster ? 1 : 2) decode_attention_split_kernel(const DecGqaParams p) {
     __shared__ float part_s[8][G][kPartialFloats];
+    __shared__ float merge_s[kCluster ? 8 : 1][kCluster ? G : 1][kPartialFloats];   // the splits' results, in the first CTA of a cluster
     grid_dependency_wait();
     const int split = blockIdx.x, kh = blockIdx.y, b = blockIdx.z;
     if (p.skip[b]) {
-        if (split == 0 && p.n_splits == 1)
+        if (split == 0 && (kCluster || p.n_splits == 1))
             for (int i = threadIdx.x; i < G * kHeadDim; i += 256)
                 p.O[(long long)b * p.o_b + (long long)(kh * G + i / kHeadDim) * p.o_h + (i % kHeadDim)] = __float2bfloat16_rn(0.f);
         return;
     }
+    if constexpr (kCluster) cooperative_groups::this_cluster().barrier_arrive();   // this CTA's shared memory may be written from now on
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int t_pos = p.pos[b];
     const int j_lo = (p.window > 0) ? max(0, t_pos - p.window + 1) : 0;
@@ -973,6 +910,7 @@ __global__ void __launch_bounds__(256, 2) decode_attention_split_kernel(const De
         }
     }
     __syncthreads();
+    if constexpr (kCluster) cooperative_groups::this_cluster().barrier_wait();
     for (int i = threadIdx.x; i < G * kHeadDim; i += 256) {
         const int h = i / kHeadDim, d = i % kHeadDim;
         float M = -1e30f;
@@ -986,12 +924,31 @@ __global__ void __launch_bounds__(256, 2) decode_attention_split_kernel(const De
             acc = fmaf(part_s[w2][h][d], c, acc);
         }
         const int qh = kh * G + h;
-        if (p.n_splits == 1) {
+        if constexpr (kCluster) {       // to the first split of the cluster, which merges them
+            float* dst = cooperative_groups::this_cluster().map_shared_rank(&merge_s[0][0][0], 0) + (split * G + h) * kPartialFloats;
+            dst[d] = acc;
+            if (d == 0) { dst[kHeadDim] = M; dst[kHeadDim + 1] = L; }
+        } else if (p.n_splits == 1) {
             p.O[(long long)b * p.o_b + (long long)qh * p.o_h + d] = __float2bfloat16_rn(acc / L);
         } else {
             float* dst = p.partial + (((size_t)b * p.Hq + qh) * p.n_splits + split) * kPartialFloats;
             dst[d] = acc;
             if (d == 0) { dst[kHeadDim] = M; dst[kHeadDim + 1] = L; }
+        }
+    }
+    if constexpr (kCluster) {
+        cooperative_groups::this_cluster().sync();
+        if (split != 0) return;
+        for (int i = threadIdx.x; i < G * kHeadDim; i += 256) {
+            const int h = i / kHeadDim, d = i % kHeadDim;
+            float M = -1e30f, L = 0.f, acc = 0.f;
+            for (int q = 0; q < p.n_splits; ++q) M = fmaxf(M, merge_s[q][h][kHeadDim]);
+            for (int q = 0; q < p.n_splits; ++q) {
+                const float c = exp2f(merge_s[q][h][kHeadDim] - M);
+                L = fmaf(merge_s[q][h][kHeadDim + 1], c, L);
+                acc = fmaf(merge_s[q][h][d], c, acc);
+            }
+            p.O[(long long)b * p.o_b + (long long)(kh * G + h) * p.o_h + d] = __float2bfloat16_rn(acc / L);
         }
     }
 }
@@ -1025,6 +982,20 @@ __global__ void __launch_bounds__(kHeadDim) decode_merge_splits_kernel(const Dec
     *out = skip ? __float2bfloat16_rn(0.f) : __float2bfloat16_rn(acc / L);
 }
 
+template <int G>
+static cudaError_t launch_split(const DecGqaParams& gp, dim3 grid, bool cluster, cudaStream_t st) {
+    if (!cluster) return launch_dependent(decode_attention_split_kernel<G, false>, grid, dim3(256), 0, st, gp);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = 0; cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = grid.x; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, decode_attention_split_kernel<G, true>, gp);
+}
+
 cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_params& p, const tf_decode_args& a,
                                cudaStream_t st) {
     if (s.batch == 0) return cudaSuccess;
@@ -1038,8 +1009,7 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
     dp.sum_k = a.state->sum_k; dp.sum_v = a.state->sum_v; dp.count = reinterpret_cast<long long*>(a.state->count);
     dp.sums16 = ((reinterpret_cast<uintptr_t>(dp.sum_k) | reinterpret_cast<uintptr_t>(dp.sum_v)) & 15u) == 0;
     // bf16 with 1, 2, 4 or 8 query heads per KV head and 16-byte aligned query rows: the streaming kernel for ungrouped heads
-    // and for steps with at most half a tile per SM, the split kernel otherwise (both sides' times stand at the split kernel;
-    // at 1 x 420 keys x 8 heads 12.4 us a step against 13.5)
+    // (more than half a tile per SM), the split kernel otherwise (both sides' times stand at the split kernel)
     const int G = s.n_q_heads / s.n_kv_heads;
     const int sms = sm_count();
     const int max_keys = s.window > 0 ? std::min(s.window, s.seq) : s.seq;     // pos is device data: size for the worst case
@@ -1053,7 +1023,7 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
         return make_bshd_map(&mk, K, s.k_stride, n, s.seq, s.n_kv_heads, 2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 64, kStreamKeys, CU_TENSOR_MAP_SWIZZLE_128B) &&
                make_bshd_map(&mv, V, s.v_stride, n, s.seq, s.n_kv_heads, 2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 64, kStreamKeys, CU_TENSOR_MAP_SWIZZLE_128B);
     };
-    const bool stream = grouped && (G == 1 || 2 * tiles_max <= sms) && tiles_max < (1ll << 31) &&              // (tile numbers are 32 bits)
+    const bool stream = grouped && G == 1 && 2 * tiles_max > sms && tiles_max < (1ll << 31) &&              // (tile numbers are 32 bits)
                         ((s.o_stride[0] | s.o_stride[2]) % 8) == 0 && (reinterpret_cast<uintptr_t>(a.O_new) & 15u) == 0 &&
                         (s.batch == 1 || (s.k_stride[0] > 0 && s.v_stride[0] > 0)) && maps(0, std::min<int>(s.batch, kStreamMaxBatch));
     dp.early = stream ? 1 : 0;
@@ -1085,32 +1055,37 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
         // Number of key splits: two CTAs fit an SM, a wave of CTAs costs (a fixed part worth ~192 keys + its keys), and a
         // partly filled wave costs as much as a full one; take the split count with the cheapest estimate, at least
         // 256 keys per split.
+        // Few work items: the splits, as short as 64 keys, are a cluster and need no third launch (1 x 420 keys x 8 heads 8.4
+        // instead of 9.9 us; with the SMs full clusters wait for one another's slots: 32 x 4096 x 8 86 instead of 79 us).
+        const long long groups = (long long)s.batch * s.n_kv_heads, slots = 2ll * sms;
+        const bool few = 8 * groups <= sms && G <= 4;
         int n_splits = 1;
         {
-            const long long groups = (long long)s.batch * s.n_kv_heads, slots = 2ll * sms;
+            const size_t per_split = (size_t)s.batch * s.n_q_heads * kPartialFloats * sizeof(float);
+            const int most = std::max(few ? std::min(8, max_keys / 64) : 1, max_keys / 256);
             long long best = -1;
-            for (int n = 1; n <= std::max(1, max_keys / 256); ++n) {
+            for (int n = 1; n <= std::max(1, most); ++n) {
+                if ((n > 8 || (n > 1 && !few)) && (!ctx->workspace || ctx->workspace_bytes < per_split * n)) break;
                 const long long waves = (groups * n + slots - 1) / slots;
                 const long long cost = waves * (192 + (max_keys + n - 1) / n);
                 if (best < 0 || cost < best) { best = cost; n_splits = n; }
             }
         }
-        const size_t need = (size_t)s.batch * s.n_q_heads * n_splits * kPartialFloats * sizeof(float);
-        if (n_splits > 1 && (!ctx->workspace || ctx->workspace_bytes < need)) n_splits = 1;
         gp.n_splits = n_splits;
-        gp.partial = n_splits > 1 ? static_cast<float*>(ctx->workspace) : nullptr;
+        const bool cluster = few && n_splits > 1 && n_splits <= 8, scratch = n_splits > 1 && !cluster;
+        gp.partial = scratch ? static_cast<float*>(ctx->workspace) : nullptr;
         // the partial results overwrite the start of the workspace, where tf_kv_stats keeps its tagged records: the
         // next scan on this workspace clears its region first instead of trusting what it finds there
-        if (n_splits > 1) { ctx->scan_user.needs_clear = true; ctx->scan_owned.needs_clear = true; }
+        if (scratch) { ctx->scan_user.needs_clear = true; ctx->scan_owned.needs_clear = true; }
         const dim3 grid((unsigned)n_splits, (unsigned)s.n_kv_heads, (unsigned)s.batch);
         switch (G) {
-            case 1: e = launch_dependent(decode_attention_split_kernel<1>, grid, dim3(256), 0, st, gp); break;
-            case 2: e = launch_dependent(decode_attention_split_kernel<2>, grid, dim3(256), 0, st, gp); break;
-            case 4: e = launch_dependent(decode_attention_split_kernel<4>, grid, dim3(256), 0, st, gp); break;
-            default: e = launch_dependent(decode_attention_split_kernel<8>, grid, dim3(256), 0, st, gp); break;
+            case 1: e = launch_split<1>(gp, grid, cluster, st); break;
+            case 2: e = launch_split<2>(gp, grid, cluster, st); break;
+            case 4: e = launch_split<4>(gp, grid, cluster, st); break;
+            default: e = launch_dependent(decode_attention_split_kernel<8, false>, grid, dim3(256), 0, st, gp); break;
         }
         ctx->launches += 1;
-        if (e == cudaSuccess && n_splits > 1) {
+        if (e == cudaSuccess && scratch) {
             e = launch_dependent(decode_merge_splits_kernel, dim3((unsigned)s.n_q_heads, (unsigned)s.batch), dim3(kHeadDim), 0, st, gp);
             ctx->launches += 1;
         }
@@ -1130,26 +1105,18 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
             sp.pos = a.pos + b0; sp.skip = a.skip_out + b0;
             const long long tiles = (long long)n * s.n_kv_heads * ((max_keys + kStreamKeys - 1) / kStreamKeys);
             const int grid = (int)std::min<long long>(sms, tiles);
-            sp.partial = nullptr; sp.begun = nullptr; sp.counters = nullptr; sp.arrived = nullptr;
+            sp.partial = nullptr; sp.begun = nullptr; sp.counters = nullptr;
             // scratch: the table of begun work items, then slots: two per piece, and there have to be more pieces than CTAs
-            const size_t slot = (size_t)G * kPartialFloats * sizeof(float), table = stream_table_bytes(grid);
+            const size_t slot = kPartialFloats * sizeof(float), table = stream_table_bytes(grid);
             const size_t scratch = std::min(ctx->workspace ? ctx->workspace_bytes : 0, table + kStreamScratch);
             if (scratch >= table + (3 * grid + 2) * slot) {
                 sp.partial = reinterpret_cast<float*>(static_cast<char*>(ctx->workspace) + table);
                 sp.max_slots = (unsigned int)((scratch - table) / slot);
                 sp.counters = reinterpret_cast<unsigned int*>(ctx->dev_status + 1);
-                // Short steps are bound by launches and latency: there the CTA that arrives last merges a work item (with
-                // more to merge that is slower than a kernel of its own: 4 x 4096 keys x 40 heads 61.2 against 60.5 us).
-                if (2 * grid <= sms) sp.arrived = sp.counters + 2;
-                else sp.begun = static_cast<uint4*>(ctx->workspace) + 1;
+                sp.begun = static_cast<uint4*>(ctx->workspace) + 1;
                 ctx->scan_user.needs_clear = true; ctx->scan_owned.needs_clear = true;      // (the scan's records: as above)
             }
-            switch (G) {
-                case 1: e = launch_stream<1>(sp, grid, ctx->device, mk, mv, st); break;
-                case 2: e = launch_stream<2>(sp, grid, ctx->device, mk, mv, st); break;
-                case 4: e = launch_stream<4>(sp, grid, ctx->device, mk, mv, st); break;
-                default: e = launch_stream<8>(sp, grid, ctx->device, mk, mv, st); break;
-            }
+            e = launch_stream(sp, grid, ctx->device, mk, mv, st);
             ctx->launches += sp.begun ? 2 : 1;
             if (e != cudaSuccess) return e;
         }

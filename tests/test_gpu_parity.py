@@ -750,8 +750,8 @@ def test_requested_kernel_that_cannot_take_the_call_is_an_error_not_a_fallback()
                                               (2, 9000, 3, 1, 0), (150, 130, 8, 1, 0), (1, 200, 4, 8, 0)])
 def test_decode_attention_uneven_positions_and_skips(B, S, Hkv, G, window, workspace):
     """Every sequence at a position of its own (tile edges among them), some skipped, NaN in the cache behind each position:
-    the streaming kernel (ungrouped heads: split and whole work items; short steps of any group) and the split kernel against
-    fp64 softmax attention."""
+    the streaming kernel (ungrouped heads: split and whole work items) and the split kernel (as a cluster, through scratch,
+    unsplit) against fp64 softmax attention."""
     rng = np.random.default_rng(B * S + G)
     Hq = Hkv * G
     q, k, v = _qkv(B, S, Hq, Hkv, torch.bfloat16, seed=S + G)

@@ -314,13 +314,14 @@ kv_stats_gram1_kernel(const Gram1Params p, const __grid_constant__ CUtensorMap m
     wait_bar(bar_tma, 0, abort_flag, p.wait_cycles, p.status, 100);
 
     // ---- 1. column sums: (X^T Bt^T)[d][6] = sum_t X[t][d]; two interleaved accumulator chains ------------
-    if (tid == 0) {
+    if (warp == 0) {
+        const uint32_t lead = elect_one();
         tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)         // 16 tokens per step
             mma_ss(tmem + 16 * (kk & 1), desc_mnmajor(xa + kk * 16 * 128, kHalf),
-                   desc_kmajor(bt + (kk >> 2) * (16 * 128) + (kk & 3) * 32), kIdescAgg, kk > 1, 1u);
-        mma_commit(bar_mma, 1u);
+                   desc_kmajor(bt + (kk >> 2) * (16 * 128) + (kk & 3) * 32), kIdescAgg, kk > 1, lead);
+        mma_commit(bar_mma, lead);
     }
     wait_bar(bar_mma, mma_phase, abort_flag, p.wait_cycles, p.status, 101); mma_phase ^= 1;
     tc_fence_after();
@@ -360,14 +361,15 @@ kv_stats_gram1_kernel(const Gram1Params p, const __grid_constant__ CUtensorMap m
     float r_acc = 0.f, r_part = 0.f, g_diag = 0.f;
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh) {
-        if (tid == 0) {
+        if (warp == 0) {
+            const uint32_t lead = elect_one();
             tc_fence_after();
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) {   // 16 dims per step; B = rows 64 hh .. 64 hh + 63 of the same tile
                 const uint32_t off = (kk >> 2) * kHalf + (kk & 3) * 32;
-                mma_ss(tmem, desc_kmajor(xa + off), desc_kmajor(xa + hh * (64 * 128) + off), kIdescG64, kk > 0, 1u);
+                mma_ss(tmem, desc_kmajor(xa + off), desc_kmajor(xa + hh * (64 * 128) + off), kIdescG64, kk > 0, lead);
             }
-            mma_commit(bar_mma, 1u);
+            mma_commit(bar_mma, lead);
         }
         wait_bar(bar_mma, mma_phase, abort_flag, p.wait_cycles, p.status, 102 + hh); mma_phase ^= 1;
         tc_fence_after();
@@ -402,13 +404,14 @@ kv_stats_gram1_kernel(const Gram1Params p, const __grid_constant__ CUtensorMap m
     tc_fence_before();
     __syncthreads();
     c2 = (red[0] + red[2]) + (red[4] + red[6]);
-    if (tid == 0) {
+    if (warp == 0) {
+        const uint32_t lead = elect_one();
         tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)             // 16 dims per step; two interleaved accumulator chains
             mma_ss(tmem + 16 * (kk & 1), desc_kmajor(xa + (kk >> 2) * kHalf + (kk & 3) * 32),
-                   desc_kmajor(bt + (kk >> 2) * (16 * 128) + (kk & 3) * 32), kIdescU, kk > 1, 1u);
-        mma_commit(bar_mma, 1u);
+                   desc_kmajor(bt + (kk >> 2) * (16 * 128) + (kk & 3) * 32), kIdescU, kk > 1, lead);
+        mma_commit(bar_mma, lead);
     }
     wait_bar(bar_mma, mma_phase, abort_flag, p.wait_cycles, p.status, 104); mma_phase ^= 1;
     tc_fence_after();
@@ -475,20 +478,20 @@ struct GramPParams {
 // their low word, so the issuing thread adds compile-time offsets (units of 16 bytes) to two precomputed low
 // words instead of rebuilding 64-bit descriptors per product: issue is on the critical path of every tile.
 template <uint32_t A_OFF, uint32_t B_OFF, bool ACC>
-__device__ __forceinline__ void mma_step(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t id) {
-    asm volatile("{\n.reg .pred p;\n.reg .b32 ta, tb;\n.reg .b64 da, db;\n"
-                 "setp.ne.b32 p, %6, 0;\n"
+__device__ __forceinline__ void mma_step(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t id, uint32_t issue) {
+    asm volatile("{\n.reg .pred p, q;\n.reg .b32 ta, tb;\n.reg .b64 da, db;\n"
+                 "setp.ne.b32 p, %6, 0;\nsetp.ne.b32 q, %9, 0;\n"
                  "add.u32 ta, %1, %7;\nadd.u32 tb, %3, %8;\n"
                  "mov.b64 da, {ta, %2};\nmov.b64 db, {tb, %4};\n"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}"
-                 :: "r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(id), "n"(ACC ? 1 : 0), "n"(A_OFF), "n"(B_OFF)
+                 "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}"
+                 :: "r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(id), "n"(ACC ? 1 : 0), "n"(A_OFF), "n"(B_OFF), "r"(issue)
                  : "memory");
 }
 __host__ __device__ constexpr uint32_t kmaj_step(int kk, int block_bytes) { return (uint32_t)(((kk >> 2) * block_bytes + (kk & 3) * 32) >> 4); }
 template <int BLOCK, bool A_MN, int... KK>
 __device__ __forceinline__ void mma_burst(std::integer_sequence<int, KK...>, uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi,
-                                          uint32_t b_lo, uint32_t b_hi, uint32_t id) {
-    (mma_step<(A_MN ? (uint32_t)(KK * 16 * 128 >> 4) : kmaj_step(KK, BLOCK)), kmaj_step(KK, BLOCK), (KK > 0)>(d_tmem, a_lo, a_hi, b_lo, b_hi, id), ...);
+                                          uint32_t b_lo, uint32_t b_hi, uint32_t id, uint32_t issue) {
+    (mma_step<(A_MN ? (uint32_t)(KK * 16 * 128 >> 4) : kmaj_step(KK, BLOCK)), kmaj_step(KK, BLOCK), (KK > 0)>(d_tmem, a_lo, a_hi, b_lo, b_hi, id, issue), ...);
 }
 __device__ __forceinline__ bool wait_bar_parked(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long budget_cycles,
                                                 DevStatus* status, unsigned long long where) {
@@ -614,12 +617,13 @@ kv_stats_gram_persistent_kernel(const GramPParams pp, const __grid_constant__ CU
         wait_bar_parked(bar_tma, tile_phase, abort_flag, p.wait_cycles, p.status, 200);
 
         // ---- X^T 1 (columns 64-79) and columns 0-63 of G, issued together ------------------------------------
-        if (tid == 0) {
+        if (warp == 0) {
+            const uint32_t lead = elect_one();
             tc_fence_after();
-            mma_burst<kPBlock, true>(k8, tm_s, x_lo | dlo_mn, dhi, x_lo + (kHalf >> 4) | dlo_k, dhi, kIdescAgg);   // 16 tokens per step
-            mma_commit(bar_small, 1u);
-            mma_burst<kPBlock, false>(k8, tm_g, x_lo | dlo_k, dhi, x_lo | dlo_k, dhi, kIdescG64);               // 16 dims per step
-            mma_commit(bar_g, 1u);
+            mma_burst<kPBlock, true>(k8, tm_s, x_lo | dlo_mn, dhi, x_lo + (kHalf >> 4) | dlo_k, dhi, kIdescAgg, lead);   // 16 tokens per step
+            mma_commit(bar_small, lead);
+            mma_burst<kPBlock, false>(k8, tm_g, x_lo | dlo_k, dhi, x_lo | dlo_k, dhi, kIdescG64, lead);               // 16 dims per step
+            mma_commit(bar_g, lead);
         }
         // ---- look-back requests go out under the products (thread = dim) -------------------------------------------
         const int a0 = c > 0 ? ((c - 1) / kGramAnchorEvery) * kGramAnchorEvery : 0;
@@ -694,10 +698,11 @@ kv_stats_gram_persistent_kernel(const GramPParams pp, const __grid_constant__ CU
         worker_sync(w);
         c2 = (red[0] + red[2]) + (red[4] + red[6]);
         // ---- columns 64-127 of G and u = X [c1 c2 c3 ..]^T as one product of 80 columns ------------------------------------
-        if (tid == 0) {
+        if (warp == 0) {
+            const uint32_t lead = elect_one();
             tc_fence_after();
-            mma_burst<kPBlock, false>(k8, tm_g, x_lo | dlo_k, dhi, x_lo + (64 * 128 >> 4) | dlo_k, dhi, kIdescG80);
-            mma_commit(bar_g, 1u);
+            mma_burst<kPBlock, false>(k8, tm_g, x_lo | dlo_k, dhi, x_lo + (64 * 128 >> 4) | dlo_k, dhi, kIdescG80, lead);
+            mma_commit(bar_g, lead);
         }
         wait_bar_parked(bar_g, 1, abort_flag, p.wait_cycles, p.status, 203);
         tc_fence_after();
@@ -816,10 +821,13 @@ cudaError_t launch_kv_stats_gram(tf_ctx* ctx, const tf_shape& s, const tf_filter
     gp.wait_cycles = ctx_wait_cycles(ctx);
     gp.counters = reinterpret_cast<unsigned int*>(base);
     gp.n_work = (unsigned int)(2 * tiles);
+    // The persistent form pays its set-up once per SM and wins once every worker sees two tiles: 64 chains x 24 chunks
+    // 31.5 us against 38.3 one tile per CTA, 64 x 16 24.4 against 27.7; with 1.2 tiles per worker it starts too late (17.5
+    // against 18.0).  Long chains wait for their carries, which six resident tiles per SM that start together hide better
+    // (8 chains x 128 chunks, 2.3 tiles per worker: 33.4 against 31.0; 16 x 64: 29.0 against 29.5): they need four.
+    const size_t per_worker = gl.n_chunks <= 64 ? 2 : 4;
     const int sms = sm_count();
-    // the persistent form pays its set-up once per SM and wins once every worker sees several tiles (measured
-    // cross-over between 2.3 and 11.5 tiles per worker); below that the one-tile-per-CTA form starts sooner
-    const bool persistent = ctx->scan_path == 3 || (ctx->scan_path == 0 && 2 * tiles >= (size_t)4 * sms * kPWorkers);
+    const bool persistent = ctx->scan_path == 3 || (ctx->scan_path == 0 && 2 * tiles >= per_worker * sms * kPWorkers);
     cudaError_t e;
     if (persistent) {
         static bool attr_set_p_dev[kDeviceFlagSlots] = {};

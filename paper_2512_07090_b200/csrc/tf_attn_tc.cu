@@ -1,14 +1,14 @@
 // Step a5 on the 5th-generation tensor cores: bf16 causal (optionally windowed) attention for
 // retained tokens only, head_dim 128.
 //
-// One CTA owns 256 consecutive entries of a sequence's retained list for one query head, as two
-// 128-row Q tiles that share every K/V tile -- or, on grouped-query shapes, the same 128 entries for
-// two query heads of one KV group (then both tiles need the same K/V tiles with the same masks).
+// A work item is 256 consecutive entries of a sequence's retained list for one query head, as two
+// 128-row Q tiles that share every K/V tile -- or, on grouped-query shapes, the same 128 or 64 entries for
+// two or four query heads of one KV group (then both tiles need the same K/V tiles with the same masks).
 // Warp roles:
 //   warps 0-3 / 4-7  softmax group of Q tile 0 / 1 (thread r owns row r of its tile)
 //   warp 8           issues every tcgen05.mma (the whole warp runs the loop, one elected lane issues)
 //   warp 9           TMA producer: K and V tiles of 128 keys into a 4-slot ring (one lane)
-//   warps 10-11      idle; they complete the warpgroup whose registers go to the softmax groups
+//   warps 10-11      fetch the next work item and its Q rows, zero the output rows of pruned tokens
 // The query rows are gathered (they are scattered in the sequence) into shared memory in the
 // 128-byte-swizzled K-major operand layout.  Per K/V tile j and Q tile i:
 //     S_i = Q_i K_j^T      A, B from shared memory (K-major)            -> TMEM, 128 columns
@@ -23,8 +23,8 @@
 // only rescaled) when the tile maximum exceeds it by more than 2^8, and writes P as bf16 pairs
 // straight back into TMEM.  A Q tile skips K/V tiles none of its rows can see.  The epilogue
 // normalises, converts to bf16 and scatters rows to their token positions; rows of pruned tokens
-// between two retained tokens are zeroed by the thread that owns the later one (Section 3.2:
-// a skipped token's attention output is zero).
+// are zeroed with the retained row that follows them (Section 3.2: a skipped token's attention
+// output is zero).
 //
 // Every mbarrier wait is bounded by a cycle budget; on expiry the CTA records TF_ERR_TIMEOUT,
 // stops waiting, lets copies in flight land, releases its TMEM and exits.
@@ -54,39 +54,33 @@ struct TcParams {
     const int32_t* kept_idx; const int32_t* n_kept;
     DevStatus* status;
     int compact;          // 1: K / V hold the retained tokens only, entry c = token kept_idx[c] (TF_KV_RETAINED)
-    int n_row_blocks;     // CTAs per (batch, query head)
+    int n_row_blocks;     // row blocks per (batch, query head)
+    int n_blocks_est;     // ... that are expected to hold retained rows (a host-side estimate; any value in 1 .. n_row_blocks is right)
     int bh_group;         // CTA order: (batch, head) pairs are taken in groups of this many; within a group all of the
                           // heaviest row block first.  1 = all row blocks of a head together, n_bh = heaviest first over all heads
-    int first_pair;       // row block the first CTA of a head takes: the last one expected to hold retained rows
+    int first_pair;       // n_blocks_est - 1: the row block the first CTA of a head takes
     long long wait_cycles;   // budget of one mbarrier wait
 };
 
-// Two ways of giving the two softmax groups of a CTA their work:
-//   shared (kSplit = false): two consecutive 128-row Q tiles; every K/V tile is loaded once and used by both.
-//   split  (kSplit = true):  ONE 128-row Q tile; the groups take alternate K/V tiles and their partial
-//                            results (O, maximum, sum) are merged at the end.  Twice as many, half as
-//                            long CTAs: used when the shared form would leave SMs idle or unbalanced.
-template <bool kSplit> struct Cfg {
-    static constexpr int kQBufs = kSplit ? 1 : 2;         // Q tiles in shared memory
-    static constexpr int kStages = kSplit ? 6 : 4;        // ring slots, filled in the order K(j), V(j), K(j+1), V(j+1), ...
-    static constexpr int kRows = kQBufs * kTileM;         // retained rows per CTA
-    static constexpr int kStep = kSplit ? 2 : 1;          // K/V tile stride of one softmax group
-    // shared-memory map (dynamic, base aligned to 1024 B)
+// shared-memory map of the split form (dynamic, base aligned to 1024 B): one Q tile, a ring filled in the order K(j), V(j),
+// K(j+1), V(j+1), ..., barriers
+struct SplitCfg {
+    static constexpr int kStages = 6;
     static constexpr int kOffQ = 0;
-    static constexpr int kOffRing = kOffQ + kQBufs * kTileBytes;
+    static constexpr int kOffRing = kOffQ + kTileBytes;
     static constexpr int kOffBar = kOffRing + kStages * kTileBytes;
     static constexpr int kSmemBytes = kOffBar + 256 + 1024;   // barriers + alignment slack
 };
 
-// CTAs start in index order.  Row blocks of a head differ in length by the causal triangle, so the heaviest should
-// go first, over as many heads as possible (the grid then ends with short CTAs from many heads, which fill the SMs
+// Work items are handed out in index order.  Row blocks of a head differ in length by the causal triangle, so the heaviest
+// should go first, over as many heads as possible (the grid then ends with short items from many heads, which fill the SMs
 // evenly); but the CTAs that run at the same time should find K and V in L2, which the row blocks of one head do (they
 // read nearly the same keys) and those of different heads do not.  So the (batch, head) pairs are taken in groups whose
 // K and V fit the L2 budget, and inside a group the order is: heaviest row block of every head, next row block, ...
-__device__ __forceinline__ void cta_work_item(const TcParams& p, int& rb, int& bh) {
-    const int n_bh = (int)(gridDim.x / (unsigned)p.n_row_blocks);
-    const int per_group = p.bh_group * p.n_row_blocks;
-    const int g = (int)blockIdx.x / per_group, within = (int)blockIdx.x - g * per_group;
+__device__ __forceinline__ void work_item(const TcParams& p, unsigned int item, int n_blocks, int& rb, int& bh) {
+    const int n_bh = (int)(gridDim.x / (unsigned)n_blocks);
+    const int per_group = p.bh_group * n_blocks;
+    const int g = (int)item / per_group, within = (int)item - g * per_group;
     const int g_size = min(p.bh_group, n_bh - g * p.bh_group);     // the last group may be smaller
     rb = within / g_size;
     bh = g * p.bh_group + within % g_size;
@@ -215,23 +209,469 @@ __device__ __forceinline__ void softmax_tile(uint32_t tm_s, uint32_t tm_o, int l
     l_run = fmaf(l_run, corr, psum);
 }
 
-// kHpt = query heads per Q tile: 0 = the forms above (one head per CTA); 1, 2 = the head forms of the shared form for
-// grouped-query shapes: a Q tile holds the same 128 / kHpt retained rows of kHpt query heads of one KV group (row r of
-// the tile is head r / (128 / kHpt), entry r % (128 / kHpt)), and the CTA's second tile the next kHpt heads of that group.
-template <bool kSplit, int kHpt = 0>
+// ---------------------------------------------------------------------------------------------------------
+// Shared and head forms: persistent CTAs, one per SM, that take work items (row block, head) from the hardware's own
+// launch queue (cluster launch control: a running CTA cancels the launch of a waiting one and does its work).
+//   kHpt = 0: an item is 256 consecutive retained rows of one head, two Q tiles of 128.
+//   kHpt = 1, 2 (grouped-query shapes): a Q tile holds the same 128 / kHpt retained rows of kHpt query heads of one KV
+//     group (row r of the tile is head r / (128 / kHpt), entry r % (128 / kHpt)), the item's second tile the next kHpt
+//     heads of that group: both tiles have the same K/V tiles and masks, no tile is ever worked on by one group alone.
+// A CTA per item spends some 15,000 cycles around its tiles (3,300 each): launch, TMEM, three dependent global round
+// trips, 64 KB of scattered Q rows, the first Q K^T and the last P V with nothing beside them, the epilogue.  Here the
+// next item's set-up runs under the tiles of the current one:
+//   warps 10-11 claim the next item when the last K/V tile of this one has been requested (late enough for the queue
+//     to hand items to the SMs that run out first), read its indices, gather its Q rows (cp.async) and publish a
+//     descriptor; then they zero the output rows of pruned tokens.
+//   warp 9 goes on with the next item's K/V tiles in the same ring, warp 8 with its products: Q K^T of the next item's
+//     first tile is issued right behind the last P V of this one.
+//   Q tiles take turns in three slots of shared memory.  Tile 0 of the next item goes into the third slot at any time,
+//     tile 1 into the slot of this item's tile 0, which its last Q K^T gives back about one tile time before it is
+//     needed (kHpt > 0) or group 0's epilogue does (kHpt = 0, where group 0 finishes first).
+//   The epilogue stages its rows in the slot of tile 1 (kHpt > 0) or of the group's own tile (kHpt = 0).
+// One layer's pass, one CTA per item -> persistent: 8 x 16384 windowed 4276 -> 3932 us, 2 x 8192 grouped heads 609 -> 568 us,
+// 4 x 4096 x 40 heads 555 -> 506 us, 3 x 1531 87.7 -> 82.8 us, 2 x 3001 retained keys 139 -> 127 us.
+// ---------------------------------------------------------------------------------------------------------
+constexpr int kGatherWarp = kTmaWarp + 1;              // and the one after it
+constexpr int kGatherThreads = 64;
+constexpr int kPStages = 4;                            // K/V ring slots
+constexpr int kPQSlots = 3;
+constexpr int kPOffQ = 0, kPOffRing = kPQSlots * kTileBytes, kPOffRows = kPOffRing + kPStages * kTileBytes;
+constexpr int kPOffMisc = kPOffRows + 2 * kSoftmaxThreads * 4;      // two sets of token positions of an item's rows
+constexpr int kPSmemBytes = kPOffMisc + 512;           // the dynamic segment must start 1024-byte aligned (checked)
+static_assert(kPSmemBytes <= 227 * 1024, "shared memory of one CTA");
+
+struct TcItem {
+    int valid;            // 0: there is no further item
+    int b, qh, slot0, nk;
+    int jb[2], je[2];     // K/V tiles jb .. je - 1 of each Q tile
+};
+
+// 64 threads (warps 10-11) agree: true if any of them says so
+__device__ __forceinline__ bool gather_any(bool x) {
+    uint32_t r;
+    asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.or.pred q, 1, 64, p;\nselp.u32 %0, 1, 0, q;\n}"
+                 : "=r"(r) : "r"((uint32_t)x) : "memory");
+    return r != 0;
+}
+
+template <int kHpt>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV) {
-    static_assert(!(kSplit && kHpt > 0), "the head forms are variants of the shared form");
     static_assert(kHpt == 0 || kHpt == 1 || kHpt == 2, "one, two or four query heads per CTA");
-    using C = Cfg<kSplit>;
     constexpr bool kHeads = kHpt > 0;
-    // retained-list entries one CTA covers; kOneSpan: both softmax groups work on the SAME entries (the split form:
-    // alternate K/V tiles; the head forms: different query heads of one KV group, so that the groups' K/V tile ranges and
-    // masks coincide and no tile is ever worked on by one group alone)
-    constexpr bool kOneSpan = kSplit || kHeads;
     constexpr int kTileRows = kHeads ? kTileM / kHpt : kTileM;   // retained-list entries per Q tile
-    constexpr int kRows = kOneSpan ? kTileRows : C::kRows;
-    constexpr int kStages = C::kStages, kOffQ = C::kOffQ, kOffRing = C::kOffRing, kOffBar = C::kOffBar, kStep = C::kStep;
+    constexpr int kRows = kHeads ? kTileRows : 2 * kTileM;       // ... per item
+    constexpr int kHeadsPerCta = kHeads ? 2 * kHpt : 1;
+    extern __shared__ uint8_t smem[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t sbase = smem_u32(smem);
+    if (sbase & 1023u) {   // the swizzled operand layout needs it; nothing has been started yet
+        if (tid == 0) report_error(p.status, TF_ERR_TIMEOUT, 398);
+        return;
+    }
+    const uint32_t bars = sbase + kPOffMisc;
+    const uint32_t bar_full = bars, bar_empty = bar_full + 8 * kPStages;   // [kPStages] ring slot filled / read by its products
+    const uint32_t bar_s = bar_empty + 8 * kPStages;     // [2] S_i ready
+    const uint32_t bar_p = bar_s + 16;                   // [2] P_i written (and O_i rescaled)
+    const uint32_t bar_o = bar_p + 16;                   // [2] the item's last P_i V done
+    // what is filled or given back ahead of its reader has one barrier per parity of the item, so that no phase can be missed
+    const uint32_t bar_qf0 = bar_o + 16, bar_qf1 = bar_qf0 + 16;   // [2], [1] Q tile 0 / 1 gathered
+    const uint32_t bar_q0 = bar_qf1 + 8;                 // Q slot of tile 0 given back
+    const uint32_t bar_q1 = bar_q0 + 8;                  // [2] Q slot of tile 1, the item's rows and descriptor given back
+    const uint32_t bar_item = bar_q1 + 16;               // [2] item descriptor written
+    const uint32_t bar_claim = bar_item + 16;            // answer of the launch queue
+    const uint32_t bar_asked = bar_claim + 8;            // every K/V tile of the item requested
+    const uint32_t claim = bars + 192;                   // 16 bytes
+    TcItem* const items = reinterpret_cast<TcItem*>(smem + kPOffMisc + 224);          // [2]
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kPOffMisc + 320);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kPOffMisc + 328);
+    int* const rows = reinterpret_cast<int*>(smem + kPOffRows);                       // [2][256] token position, -1: no row
+    static_assert(sizeof(TcItem) <= 48 && (2 * kPStages + 16) * 8 <= 192, "layout of the last 512 bytes");
+    if (tid == 0) {
+        for (int i = 0; i < kPStages; ++i) { mbar_init(bar_full + 8 * i, 1); mbar_init(bar_empty + 8 * i, 1); }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(bar_s + 8 * i, 1); mbar_init(bar_p + 8 * i, kTileM); mbar_init(bar_o + 8 * i, 1);
+            mbar_init(bar_qf0 + 8 * i, kGatherThreads); mbar_init(bar_item + 8 * i, kGatherThreads);
+            mbar_init(bar_q1 + 8 * i, kSoftmaxThreads / 32);
+        }
+        mbar_init(bar_qf1, kGatherThreads);
+        mbar_init(bar_q0, kHeads ? 1 : kTileM / 32);
+        mbar_init(bar_claim, 1);
+        mbar_init(bar_asked, 1);
+        *abort_flag = 0;
+        mbar_fence_init();
+    }
+    __syncwarp();
+    if (warp == kMmaWarp) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    grid_dependency_wait();   // kept_idx / n_kept come from the kernel before this one
+    auto q_slot = [&](int n, int i) { return sbase + kPOffQ + (uint32_t)((2 * n + i) % kPQSlots) * kTileBytes; };
+    // waits for the descriptor of the CTA's item n; false (for the whole warp): there is none, or a wait has given up
+    auto get_item = [&](int n, TcItem& it) {
+        mbar_wait(bar_item + 8 * (n & 1), (n >> 1) & 1, abort_flag, p.wait_cycles, p.status, 12);
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+        it = items[n & 1];
+        return it.valid != 0;
+    };
+
+    // registers move from the third warpgroup (which needs few) to the two softmax groups
+    // (each setmaxnreg sits at the top of the branch it governs, so no later code sees both)
+    if (warp >= kMmaWarp) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+    if (warp >= kGatherWarp) {
+        // ================================ items, Q rows, zero rows ====================================
+        const int w = warp - kGatherWarp, sub = lane >> 4, l16 = lane & 15;
+        const uint4 zero4 = make_uint4(0, 0, 0, 0);
+        unsigned int item = blockIdx.x;
+        int n = 0, claims = 0;
+        for (;;) {
+            int rb, bh;
+            work_item(p, item, p.n_blocks_est, rb, bh);
+            const int qh = (bh % (p.Hq / kHeadsPerCta)) * kHeadsPerCta, b = bh / (p.Hq / kHeadsPerCta);   // first (or only) head
+            const int nk = p.n_kept[b];
+            const int32_t* kept = p.kept_idx + (size_t)b * p.S;
+            __nv_bfloat16* Ob = p.O + (long long)b * p.os.b + (long long)qh * p.os.h + l16 * 8;
+            const __nv_bfloat16* Qb = p.Q + (long long)b * p.qs.b + (long long)qh * p.qs.h + l16 * 8;
+            bool produced = false;
+            const int blk0 = p.n_blocks_est - 1 - rb;         // heaviest expected row block first
+            if (nk <= 0 && blk0 == 0) {                       // nothing retained at all: the whole head is zero
+                for (int hh = 0; hh < kHeadsPerCta; ++hh)
+                    for (int t = 2 * w + sub; t < p.S; t += 4)
+                        *reinterpret_cast<uint4*>(Ob + (long long)hh * p.os.h + (long long)t * p.os.t) = zero4;
+            }
+            // row blocks beyond the expected number (normally empty) go to the items of the expected ones
+            for (int blk = blk0; blk < p.n_row_blocks && blk * kRows < nk; blk += p.n_blocks_est) {
+                if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
+                const int slot0 = blk * kRows;
+                // this warp's half of each Q tile: rows 64 w .. 64 w + 63, two per lane
+                int k0[2], k1[2];
+                const int e0 = slot0 + ((w * 64) & (kTileRows - 1));
+                k0[0] = e0 + lane < nk ? kept[e0 + lane] : -1;
+                k0[1] = e0 + 32 + lane < nk ? kept[e0 + 32 + lane] : -1;
+                if (kHeads) { k1[0] = k0[0]; k1[1] = k0[1]; }
+                else {
+                    k1[0] = e0 + kTileM + lane < nk ? kept[e0 + kTileM + lane] : -1;
+                    k1[1] = e0 + kTileM + 32 + lane < nk ? kept[e0 + kTileM + 32 + lane] : -1;
+                }
+                TcItem d;
+                d.valid = 1; d.b = b; d.qh = qh; d.slot0 = slot0; d.nk = nk;
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {     // which K/V tiles each Q tile needs
+                    const int s_lo = slot0 + (kHeads ? 0 : i * kTileM);
+                    d.jb[i] = d.je[i] = 0;
+                    if (s_lo < nk) {
+                        const int s_last = min(s_lo + kTileRows, nk) - 1;
+                        const int t_first = kept[s_lo], t_last = kept[s_last];
+                        int k_first = p.window > 0 ? max(0, t_first - p.window + 1) : 0;   // first key the tile's first row sees
+                        int k_last = t_last;                                                // last key its last row sees
+                        if (p.compact) {   // keys are entries of the retained list
+                            k_first = p.window > 0 ? first_kept_at_or_after(kept, s_lo + 1, k_first) : 0;
+                            k_last = s_last;
+                        }
+                        d.jb[i] = k_first / kTileN;
+                        d.je[i] = k_last / kTileN + 1;
+                    }
+                }
+                // the slot of tile 0, the descriptor and the row positions are those of item n - 2
+                if (n >= 2) mbar_wait(bar_q1 + 8 * (n & 1), ((n >> 1) - 1) & 1, abort_flag, p.wait_cycles, p.status, 13);
+                __syncwarp();
+                int* rw = rows + (n & 1) * kSoftmaxThreads + ((w * 64) & (kTileRows - 1));
+                rw[lane] = k0[0];
+                rw[32 + lane] = k0[1];
+                if (!kHeads) { rw[kTileM + lane] = k1[0]; rw[kTileM + 32 + lane] = k1[1]; }
+                if (tid == kGatherWarp * 32) items[n & 1] = d;
+                mbar_arrive(bar_item + 8 * (n & 1));
+                // 16 lanes copy a 256-byte row; rows that do not exist become zero
+                auto gather = [&](int i, const int (&kk)[2]) {
+                    const uint32_t dst = q_slot(n, i) + (uint32_t)((l16 >> 3) * kHalfBytes);
+                    const __nv_bfloat16* src = Qb + (long long)(kHeads ? i * kHpt + (kHpt == 2 ? w : 0) : 0) * p.qs.h;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll 8
+                        for (int e = 0; e < 16; ++e) {
+                            const int t = __shfl_sync(0xffffffffu, kk[h], 2 * e + sub), r = w * 64 + h * 32 + 2 * e + sub;
+                            cp_async16(dst + (uint32_t)(r * 128 + (((l16 & 7) ^ (r & 7)) << 4)),
+                                       src + (long long)max(t, 0) * p.qs.t, t >= 0 ? 16u : 0u);
+                        }
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                };
+                gather(0, k0);
+                if (n == 0) {
+                    gather(1, k1);
+                    asm volatile("cp.async.wait_group 1;" ::: "memory");
+                    fence_proxy_async();
+                    mbar_arrive(bar_qf0);
+                } else {
+                    asm volatile("cp.async.wait_group 0;" ::: "memory");
+                    fence_proxy_async();
+                    mbar_arrive(bar_qf0 + 8 * (n & 1));
+                    mbar_wait(bar_q0, (n - 1) & 1, abort_flag, p.wait_cycles, p.status, 14);
+                    __syncwarp();
+                    gather(1, k1);
+                }
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                fence_proxy_async();
+                mbar_arrive(bar_qf1);
+                // rows of pruned tokens that precede a retained row of this warp (and follow the last one of all) are zero
+                auto zero_rows = [&](const int (&kk)[2], int first, int hh0, int n_heads) {
+                    if (first >= nk) return;
+                    int before = first == 0 ? -1 : kept[first - 1];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        int pv = __shfl_up_sync(0xffffffffu, kk[h], 1);
+                        if (lane == 0) pv = before;
+                        before = __shfl_sync(0xffffffffu, kk[h], 31);
+                        for (int e = 0; e < 16; ++e) {
+                            const int cur = __shfl_sync(0xffffffffu, kk[h], 2 * e + sub), prev = __shfl_sync(0xffffffffu, pv, 2 * e + sub);
+                            if (cur < 0) continue;
+                            const bool last = first + h * 32 + 2 * e + sub == nk - 1;
+                            for (int hh = hh0; hh < hh0 + n_heads; ++hh) {
+                                __nv_bfloat16* Oz = Ob + (long long)hh * p.os.h;
+                                for (int t = prev + 1; t < cur; ++t) *reinterpret_cast<uint4*>(Oz + (long long)t * p.os.t) = zero4;
+                                if (last)
+                                    for (int t = cur + 1; t < p.S; ++t) *reinterpret_cast<uint4*>(Oz + (long long)t * p.os.t) = zero4;
+                            }
+                        }
+                        __syncwarp();
+                    }
+                };
+                if (kHpt == 2) { zero_rows(k0, e0, w, 1); zero_rows(k0, e0, 2 + w, 1); }
+                else zero_rows(k0, e0, 0, kHeadsPerCta);
+                if (!kHeads) zero_rows(k1, e0 + kTileM, 0, 1);
+                ++n;
+                produced = true;
+            }
+            // the next item
+            __syncwarp();
+            if (produced) mbar_wait(bar_asked, (n - 1) & 1, abort_flag, p.wait_cycles, p.status, 15);
+            __syncwarp();
+            fence_proxy_async();                               // the last answer has been read
+            if (gather_any(*abort_flag != 0)) break;
+            if (tid == kGatherWarp * 32) {
+                mbar_expect_tx(bar_claim, 16);
+                launch_queue_claim(claim, bar_claim);
+            }
+            __syncwarp();
+            const bool answered = mbar_wait_bounded(bar_claim, claims & 1, abort_flag, p.wait_cycles, p.status, 16);
+            ++claims;
+            if (gather_any(!answered)) break;
+            if (!launch_queue_item(claim, item) || item >= gridDim.x) {
+                if (n >= 2) mbar_wait(bar_q1 + 8 * (n & 1), ((n >> 1) - 1) & 1, abort_flag, p.wait_cycles, p.status, 17);
+                if (tid == kGatherWarp * 32) items[n & 1].valid = 0;
+                mbar_arrive(bar_item + 8 * (n & 1));
+                break;
+            }
+        }
+    } else if (warp == kTmaWarp) {
+        // ================================ TMA producer ================================================
+        TcItem it;
+        int q = 0;       // ring slots filled so far
+        for (int n = 0; get_item(n, it); ++n) {
+            if (lane == 0) {
+                const int kh = it.qh / (p.Hq / p.Hkv), J1 = max(it.je[0], it.je[1]);
+                for (int j = it.jb[0]; j < J1 && !*abort_flag; ++j) {      // rows ascend, so tile 0 starts first
+                    for (int kv = 0; kv < 2; ++kv, ++q) {
+                        const int st = q % kPStages;
+                        // the CTA's first K and V tiles go out at once; the rest of the ring is filled once the Q rows are
+                        // in shared memory (nothing can consume it earlier, and the copies would slow each other down)
+                        if (n == 0 && q == 2) mbar_wait(bar_qf1, 0, abort_flag, p.wait_cycles, p.status, 11);
+                        if (q >= kPStages) mbar_wait(bar_empty + 8 * st, ((q / kPStages) - 1) & 1, abort_flag, p.wait_cycles, p.status, 10);
+                        const uint32_t dst = sbase + kPOffRing + st * kTileBytes;
+                        const CUtensorMap* map = kv ? &mapV : &mapK;
+                        mbar_expect_tx(bar_full + 8 * st, kTileBytes);
+                        tma_load_4d(dst, map, bar_full + 8 * st, 0, kh, j * kTileN, it.b);
+                        tma_load_4d(dst + kHalfBytes, map, bar_full + 8 * st, 64, kh, j * kTileN, it.b);
+                    }
+                }
+                mbar_arrive(bar_asked);
+            }
+            __syncwarp();
+        }
+    } else {
+        // ================================ MMA issuer ==================================================
+        const uint32_t lead = elect_one();
+        TcItem cur;
+        int n = 0, q0 = 0;             // the CTA's item, ring slots used by the items before it
+        int done[2] = {0, 0};          // tiles of each group so far
+        auto ring = [&](int q) { return sbase + kPOffRing + (q % kPStages) * kTileBytes; };
+        auto wait_full = [&](int q, int where) {
+            mbar_wait(bar_full + 8 * (q % kPStages), (q / kPStages) & 1, abort_flag, p.wait_cycles, p.status, where);
+        };
+        auto release = [&](int q) { mma_commit(bar_empty + 8 * (q % kPStages), lead); };
+        auto issue_qk = [&](int i, uint32_t qaddr, uint32_t kaddr) {   // S_i = Q_i K_j^T : 8 steps of 16 dims
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) {
+                const uint32_t off = (kk >> 2) * kHalfBytes + (kk & 3) * 32;
+                mma_ss(tmem + i * 128, desc_kmajor(qaddr + off), desc_kmajor(kaddr + off), kIdescQK, kk > 0, lead);
+            }
+            mma_commit(bar_s + 8 * i, lead);
+        };
+        auto issue_pv = [&](int i, uint32_t vaddr, bool first) {       // O_i (+)= P_i V_j : 8 steps of 16 keys
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk)
+                mma_ts(tmem + 256 + i * 128, tmem + i * 128 + kk * 8, desc_mnmajor(vaddr + kk * 16 * 128, kHalfBytes), kIdescPV,
+                       (!first || kk > 0) ? 1u : 0u, lead);
+        };
+        bool more = get_item(0, cur), ahead = false;      // ahead: Q_0 K^T of the item's first tile is issued already
+        while (more) {
+            const int J0 = cur.jb[0], J1 = max(cur.je[0], cur.je[1]);
+            const uint32_t qa[2] = {q_slot(n, 0), q_slot(n, 1)};
+            auto active = [&](int i, int j) { return j >= cur.jb[i] && j < cur.je[i]; };
+            // the first tile's Q K^T
+            if (!ahead) {
+                wait_full(q0, 21);
+                mbar_wait(bar_qf0 + 8 * (n & 1), (n >> 1) & 1, abort_flag, p.wait_cycles, p.status, 20);
+                tc_fence_after();
+                issue_qk(0, qa[0], ring(q0));
+            }
+            mbar_wait(bar_qf1, n & 1, abort_flag, p.wait_cycles, p.status, 19);
+            tc_fence_after();
+            if (active(1, J0)) issue_qk(1, qa[1], ring(q0));
+            release(q0);
+            if (kHeads && J1 == J0 + 1) mma_commit(bar_q0, lead);
+            ahead = false;
+            for (int j = J0; j < J1; ++j) {
+                const int qv = q0 + 2 * (j - J0) + 1;
+                const bool last = j + 1 == J1;
+                wait_full(qv, 22);
+                if (!last) wait_full(qv + 1, 23);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    if (active(i, j)) {
+                        mbar_wait(bar_p + 8 * i, done[i] & 1, abort_flag, p.wait_cycles, p.status, 24 + i);
+                        tc_fence_after();
+                        issue_pv(i, ring(qv), j == cur.jb[i]);
+                        ++done[i];
+                        if (j + 1 == cur.je[i]) mma_commit(bar_o + 8 * i, lead);
+                    }
+                    if (i == 1) release(qv);
+                    if (!last) {
+                        if (active(i, j + 1)) issue_qk(i, qa[i], ring(qv + 1));
+                    } else if (i == 0) {
+                        // the next item's first Q_0 K^T, if everything it needs has arrived
+                        bool ready = mbar_test(bar_item + 8 * ((n + 1) & 1), ((n + 1) >> 1) & 1);
+                        if (__all_sync(0xffffffffu, ready)) {
+                            ready = items[(n + 1) & 1].valid != 0 && mbar_test(bar_qf0 + 8 * ((n + 1) & 1), ((n + 1) >> 1) & 1) &&
+                                    mbar_test(bar_full + 8 * ((qv + 1) % kPStages), ((qv + 1) / kPStages) & 1);
+                            ahead = __all_sync(0xffffffffu, ready);
+                            if (ahead) {
+                                tc_fence_after();
+                                issue_qk(0, q_slot(n + 1, 0), ring(qv + 1));
+                            }
+                        }
+                    }
+                }
+                if (!last) {
+                    release(qv + 1);
+                    if (kHeads && j + 2 == J1) mma_commit(bar_q0, lead);      // this item's last Q K^T
+                }
+            }
+            q0 += 2 * (J1 - J0);
+            ++n;
+            more = get_item(n, cur);
+        }
+    }
+    } else {
+        // ================================ softmax groups ===============================================
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+        const int i = warp >> 2;                 // group: its Q tile
+        const int r = tid & (kTileM - 1);        // row within the tile
+        const uint32_t tm_s = tmem + ((uint32_t)((warp & 3) * 32) << 16) + i * 128;   // this warp's lanes, S_i / P_i
+        const uint32_t tm_o = tm_s + 256;                                               // O_i
+        TcItem it;
+        int tiles = 0, ends = 0;                 // of this group so far
+        for (int n = 0; get_item(n, it); ++n) {
+            const int32_t* kept = p.kept_idx + (size_t)it.b * p.S;
+            const int e_row = (kHeads ? 0 : i * kTileM) + (r & (kTileRows - 1));
+            const int slot = it.slot0 + e_row;
+            const int t_row = rows[(n & 1) * kSoftmaxThreads + e_row];                // the row's token position, -1 if none
+            const bool valid = t_row >= 0;
+            int hi = t_row;                                                           // visible keys: lo .. hi
+            int lo = (valid && p.window > 0) ? max(0, t_row - p.window + 1) : 0;
+            if (p.compact && valid) {
+                lo = p.window > 0 ? first_kept_at_or_after(kept, slot + 1, lo) : 0;
+                hi = slot;
+            }
+            __syncwarp();
+            const int jb = i == 0 ? it.jb[0] : it.jb[1], je = i == 0 ? it.je[0] : it.je[1];
+            float m_ref = -INFINITY, l_run = 0.f;
+            for (int j = jb; j < je; ++j, ++tiles) {
+                mbar_wait(bar_s + 8 * i, tiles & 1, abort_flag, p.wait_cycles, p.status, 30 + i);
+                __syncwarp();
+                tc_fence_after();
+                softmax_tile(tm_s, tm_o, lo, hi, j * kTileN, p.scale_log2, j > jb, m_ref, l_run);
+                tmem_wait_st();
+                tc_fence_before();
+                mbar_arrive(bar_p + 8 * i);
+            }
+            // ---- epilogue: O / l -> bf16 -> the row's token position --------------------------------------
+            // A thread owns a row, and rows of retained tokens lie far apart in O: storing from the registers would
+            // touch 32 different lines per warp instruction.  Each warp therefore stages its 32 rows, 64 columns at a
+            // time, in 4 KiB of a Q slot whose products are done (16-byte chunks XOR-swizzled by the row) and writes
+            // them out with 8 lanes per 128 bytes.
+            if (je > jb) {
+                mbar_wait(bar_o + 8 * i, ends & 1, abort_flag, p.wait_cycles, p.status, 40);
+                ++ends;
+                __syncwarp();
+                tc_fence_after();
+                const float inv = 1.f / l_run;
+                __nv_bfloat16* Ow = p.O + (long long)it.b * p.os.b +
+                                    (long long)(it.qh + (kHeads ? i * kHpt + ((warp & 3) * 32) / kTileRows : 0)) * p.os.h;   // a warp's rows are of one head
+                uint8_t* stage = smem + (q_slot(n, kHeads ? 1 : i) - sbase) + (kHeads ? warp : (warp & 3)) * 4096;
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    uint32_t o[64];
+                    tmem_ld32(tm_o + c * 64, o);
+                    tmem_ld32(tm_o + c * 64 + 32, o + 32);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int v = 0; v < 8; ++v) {
+                        uint4 x;
+                        x.x = pack_bf16(__uint_as_float(o[8 * v + 0]) * inv, __uint_as_float(o[8 * v + 1]) * inv);
+                        x.y = pack_bf16(__uint_as_float(o[8 * v + 2]) * inv, __uint_as_float(o[8 * v + 3]) * inv);
+                        x.z = pack_bf16(__uint_as_float(o[8 * v + 4]) * inv, __uint_as_float(o[8 * v + 5]) * inv);
+                        x.w = pack_bf16(__uint_as_float(o[8 * v + 6]) * inv, __uint_as_float(o[8 * v + 7]) * inv);
+                        *reinterpret_cast<uint4*>(stage + lane * 128 + ((v ^ (lane & 7)) << 4)) = x;
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int pass = 0; pass < 8; ++pass) {
+                        const int R = pass * 4 + (lane >> 3), t_out = __shfl_sync(0xffffffffu, t_row, R);
+                        const uint4 x = *reinterpret_cast<const uint4*>(stage + R * 128 + (((lane & 7) ^ (R & 7)) << 4));
+                        if (t_out >= 0) *reinterpret_cast<uint4*>(Ow + (long long)t_out * p.os.t + c * 64 + (lane & 7) * 8) = x;
+                    }
+                    __syncwarp();
+                }
+                tc_fence_before();      // the next item's products write over O_i and S_i
+            }
+            // this warp is done with the item's slots, rows and descriptor
+            if (lane == 0) {
+                if (!kHeads && i == 0) mbar_arrive(bar_q0);
+                mbar_arrive(bar_q1 + 8 * (n & 1));
+            }
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (*abort_flag) {   // a wait gave up: give copies and MMAs still in flight time to land before leaving
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000ll) { }
+        __syncthreads();
+    }
+    if (warp == kMmaWarp) tmem_dealloc(tmem, kTmemCols);
+}
+
+// Split form: ONE 128-row Q tile; the softmax groups take alternate K/V tiles and their partial results (O, maximum, sum)
+// are merged at the end.  Twice as many, half as long CTAs: used when the shared form would leave SMs idle.
+__global__ void __launch_bounds__(kThreads, 1)
+attention_tc_split_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV) {
+    constexpr int kRows = kTileM;         // retained-list entries one CTA covers
+    constexpr int kStep = 2;              // K/V tile stride of one softmax group
+    constexpr int kStages = SplitCfg::kStages, kOffQ = SplitCfg::kOffQ, kOffRing = SplitCfg::kOffRing, kOffBar = SplitCfg::kOffBar;
     extern __shared__ uint8_t smem_raw[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -259,14 +699,13 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
     if (warp == kMmaWarp) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
     grid_dependency_wait();   // kept_idx / n_kept come from the kernel before this one
     int rb, bh;
-    cta_work_item(p, rb, bh);
+    work_item(p, blockIdx.x, p.n_row_blocks, rb, bh);
     // Row blocks are taken from the heaviest expected one (the last with retained rows, a host-side estimate) down to
     // block 0, then the blocks above the estimate, which are normally empty: CTAs with nothing to do start last
     // instead of delaying the first wave of real work.  Any estimate gives a one-to-one assignment.
     int pair = p.first_pair - rb;
     if (pair < 0) pair += p.n_row_blocks;
-    constexpr int kHeadsPerCta = kHeads ? 2 * kHpt : 1;
-    const int qh = (bh % (p.Hq / kHeadsPerCta)) * kHeadsPerCta, b = bh / (p.Hq / kHeadsPerCta);   // first (or only) head
+    const int qh = bh % p.Hq, b = bh / p.Hq;
     const int nk = p.n_kept[b];
     const int slot0 = pair * kRows;
     const int32_t* kept = p.kept_idx + (size_t)b * p.S;
@@ -274,9 +713,8 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
     const uint4 zero4 = make_uint4(0, 0, 0, 0);
     if (slot0 >= max(nk, 1) || nk == 0) {   // no retained row in this block (CTA-uniform)
         if (slot0 < max(nk, 1)) {           // nothing retained at all: the whole head is zero
-            for (int hh = 0; hh < kHeadsPerCta; ++hh)
-                for (int i = tid; i < p.S * 16; i += kThreads)
-                    *reinterpret_cast<uint4*>(Ob + (long long)hh * p.os.h + (long long)(i >> 4) * p.os.t + (i & 15) * 8) = zero4;
+            for (int i = tid; i < p.S * 16; i += kThreads)
+                *reinterpret_cast<uint4*>(Ob + (long long)(i >> 4) * p.os.t + (i & 15) * 8) = zero4;
         }
         tc_fence_before();
         __syncthreads();
@@ -288,43 +726,30 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
     // The softmax threads read the retained indices of the Q rows they will gather (16 lanes per 256-byte row, the
     // 8 warps take 16 rows per round) and of their own row now, next to the loads the set-up below waits for anyway:
     // one global round trip less between the set-up and the first Q K^T.
-    constexpr int kRounds = C::kRows / 16;   // 16 rows per round over the CTA's Q tiles
+    constexpr int kRounds = kTileM / 16;   // 16 rows per round
     int tq[kRounds];
     int t_row = -1;
     if (warp < kMmaWarp) {
 #pragma unroll
         for (int it = 0; it < kRounds; ++it) {
-            const int rr = it * 16 + warp * 2 + (lane >> 4);           // row of the CTA's Q buffer (tile rr / 128)
-            const int s_q = slot0 + (kHeads ? (rr & (kTileRows - 1)) : rr);
+            const int s_q = slot0 + it * 16 + warp * 2 + (lane >> 4);
             tq[it] = s_q < nk ? kept[s_q] : -1;
         }
-        const int slot_pre = slot0 + (kOneSpan ? 0 : (warp >> 2) * kTileM) + (tid & (kTileRows - 1));
+        const int slot_pre = slot0 + (tid & (kTileM - 1));
         if (slot_pre < nk) t_row = kept[slot_pre];
     }
 
-    // ---- which K/V tiles each Q tile needs (CTA-uniform) -------------------------------------------
-    // group i works on tiles jb[i], jb[i] + kStep, ... < je[i]
-    int jb[kQTiles], je[kQTiles];
-#pragma unroll
-    for (int i = 0; i < kQTiles; ++i) {
-        const int s_lo = slot0 + (kOneSpan ? 0 : i * kTileM);
-        if (s_lo < nk) {
-            const int s_last = min(s_lo + kTileRows, nk) - 1;
-            const int t_first = kept[s_lo], t_last = kept[s_last];
-            int k_first = p.window > 0 ? max(0, t_first - p.window + 1) : 0;   // first key the tile's first row sees
-            int k_last = t_last;                                                // last key its last row sees
-            if (p.compact) {   // keys are entries of the retained list
-                k_first = p.window > 0 ? first_kept_at_or_after(kept, s_lo + 1, k_first) : 0;
-                k_last = s_last;
-            }
-            jb[i] = k_first / kTileN + (kSplit ? i : 0);
-            je[i] = k_last / kTileN + 1;
-        } else {
-            jb[i] = je[i] = 0;
-        }
+    // ---- which K/V tiles the Q tile needs (CTA-uniform): group i works on tiles jb[i], jb[i] + 2, ... < J1 ------------
+    const int s_last = min(slot0 + kTileM, nk) - 1;
+    const int t_first = kept[slot0], t_last = kept[s_last];
+    int k_first = p.window > 0 ? max(0, t_first - p.window + 1) : 0;   // first key the tile's first row sees
+    int k_last = t_last;                                                // last key its last row sees
+    if (p.compact) {   // keys are entries of the retained list
+        k_first = p.window > 0 ? first_kept_at_or_after(kept, slot0 + 1, k_first) : 0;
+        k_last = s_last;
     }
-    const int n_q = kSplit ? 1 : ((je[1] > jb[1]) ? 2 : 1);   // Q tiles to gather
-    const int J0 = jb[0], J1 = max(je[0], je[1]);   // rows ascend, so tile 0 starts first
+    const int J0 = k_first / kTileN, J1 = k_last / kTileN + 1;
+    const int jb[2] = {J0, J0 + 1};
     const int kh = qh / (p.Hq / p.Hkv);
 
     tc_fence_before();
@@ -344,12 +769,9 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
         const int s_end = min(slot0 + kRows, nk);
         for (int s_z = slot0 + g4; s_z < s_end; s_z += 4) {
             const int prev = s_z == 0 ? -1 : kept[s_z - 1], cur = kept[s_z];
-            for (int hh = 0; hh < kHeadsPerCta; ++hh) {
-                __nv_bfloat16* Oz = Ob + (long long)hh * p.os.h + l16 * 8;
-                for (int t = prev + 1; t < cur; ++t) *reinterpret_cast<uint4*>(Oz + (long long)t * p.os.t) = zero4;
-                if (s_z == nk - 1)
-                    for (int t = cur + 1; t < p.S; ++t) *reinterpret_cast<uint4*>(Oz + (long long)t * p.os.t) = zero4;
-            }
+            for (int t = prev + 1; t < cur; ++t) *reinterpret_cast<uint4*>(Ob + (long long)t * p.os.t + l16 * 8) = zero4;
+            if (s_z == nk - 1)
+                for (int t = cur + 1; t < p.S; ++t) *reinterpret_cast<uint4*>(Ob + (long long)t * p.os.t + l16 * 8) = zero4;
         }
     } else if (warp == kTmaWarp) {
         // ================================ TMA producer ================================================
@@ -377,10 +799,9 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
             const uint32_t lead = elect_one();
             auto slot_of = [&](int j, int kv) { return (2 * (j - J0) + kv) % kStages; };
             auto par_of = [&](int j, int kv) { return ((2 * (j - J0) + kv) / kStages) & 1; };
-            auto active = [&](int i, int j) { return j >= jb[i] && j < je[i]; };
             auto issue_qk = [&](int i, int j) {   // S_i = Q_i K_j^T : 8 steps of 16 dims
                 const uint32_t kaddr = sbase + kOffRing + slot_of(j, 0) * kTileBytes;
-                const uint32_t qaddr = sbase + kOffQ + (kSplit ? 0 : i) * kTileBytes;   // split: both groups share the Q tile
+                const uint32_t qaddr = sbase + kOffQ;   // both groups share the Q tile
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) {
                     const uint32_t off = (kk >> 2) * kHalfBytes + (kk & 3) * 32;
@@ -397,7 +818,7 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
             };
             mbar_wait(bar_q, 0, abort_flag, p.wait_cycles, p.status, 20);
             int done[kQTiles] = {0, 0};
-            if constexpr (kSplit) {
+            {
                 // tile j belongs to group (j - J0) & 1; order: QK_0(J0), QK_1(J0+1), then per tile PV(j), QK(j+2)
                 for (int j = J0; j < min(J0 + 2, J1); ++j) {
                     mbar_wait(bar_full + 8 * slot_of(j, 0), par_of(j, 0), abort_flag, p.wait_cycles, p.status, 21);
@@ -419,28 +840,6 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
                         mma_commit(bar_empty + 8 * slot_of(j + 2, 0), lead);
                     }
                 }
-            } else {
-            mbar_wait(bar_full + 8 * slot_of(J0, 0), par_of(J0, 0), abort_flag, p.wait_cycles, p.status, 21);
-            tc_fence_after();
-            for (int i = 0; i < kQTiles; ++i)
-                if (active(i, J0)) issue_qk(i, J0);
-            mma_commit(bar_empty + 8 * slot_of(J0, 0), lead);
-            for (int j = J0; j < J1; ++j) {
-                mbar_wait(bar_full + 8 * slot_of(j, 1), par_of(j, 1), abort_flag, p.wait_cycles, p.status, 22);
-                if (j + 1 < J1) mbar_wait(bar_full + 8 * slot_of(j + 1, 0), par_of(j + 1, 0), abort_flag, p.wait_cycles, p.status, 23);
-#pragma unroll
-                for (int i = 0; i < kQTiles; ++i) {
-                    if (active(i, j)) {
-                        mbar_wait(bar_p + 8 * i, done[i] & 1, abort_flag, p.wait_cycles, p.status, 24 + i);
-                        tc_fence_after();
-                        issue_pv(i, j, done[i] == 0);
-                        ++done[i];
-                    }
-                    if (i == kQTiles - 1) mma_commit(bar_empty + 8 * slot_of(j, 1), lead);
-                    if (j + 1 < J1 && active(i, j + 1)) issue_qk(i, j + 1);
-                }
-                if (j + 1 < J1) mma_commit(bar_empty + 8 * slot_of(j + 1, 0), lead);
-            }
             }
             mma_commit(bar_o, lead);
         }
@@ -448,9 +847,9 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
     } else {
         // ================================ softmax groups ===============================================
         asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
-        const int i = warp >> 2;                 // group: its Q tile (shared) or its half of the K/V tiles (split)
+        const int i = warp >> 2;                 // group: its half of the K/V tiles
         const int r = tid & (kTileM - 1);        // row within the tile
-        const int slot = slot0 + (kOneSpan ? 0 : i * kTileM) + (r & (kTileRows - 1));
+        const int slot = slot0 + r;
         const bool valid = slot < nk;               // t_row (fetched above) is the row's token position, -1 if none
         int hi = t_row;                                                           // visible keys: lo .. hi
         int lo = (valid && p.window > 0) ? max(0, t_row - p.window + 1) : 0;
@@ -459,20 +858,15 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
             hi = slot;
         }
         {
-            // gather the CTA's Q rows into the swizzled K-major operand layout
+            // gather the Q rows into the swizzled K-major operand layout
             const int sub = lane >> 4, cc = lane & 15, w8 = tid >> 5;
             uint4 qv[kRounds];
             const __nv_bfloat16* qbase = p.Q + (long long)b * p.qs.b + (long long)qh * p.qs.h + cc * 8;
 #pragma unroll
-            for (int it = 0; it < kRounds; ++it) {   // head forms: rounds 8..15 fill the second tile, a round lies within one head
-                const int hh = kHeads ? (it >> 3) * kHpt + ((it & 7) * 16) / kTileRows : 0;
-                qv[it] = tq[it] >= 0 ? ldg16(qbase + (long long)hh * p.qs.h + (long long)tq[it] * p.qs.t) : zero4;
-            }
+            for (int it = 0; it < kRounds; ++it) qv[it] = tq[it] >= 0 ? ldg16(qbase + (long long)tq[it] * p.qs.t) : zero4;
 #pragma unroll
-            for (int it = 0; it < kRounds; ++it) {
-                const int rr = it * 16 + w8 * 2 + sub;
-                *reinterpret_cast<uint4*>(smem + kOffQ + (rr >> 7) * kTileBytes + swz(rr & (kTileM - 1), cc)) = qv[it];
-            }
+            for (int it = 0; it < kRounds; ++it)
+                *reinterpret_cast<uint4*>(smem + kOffQ + swz(it * 16 + w8 * 2 + sub, cc)) = qv[it];
             fence_proxy_async();
             mbar_arrive(bar_q);
         }
@@ -480,7 +874,7 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
         const uint32_t tm_s = tmem + ((uint32_t)((warp & 3) * 32) << 16) + i * 128;   // this warp's lanes, S_i / P_i
         const uint32_t tm_o = tm_s + 256;                                               // O_i
         float m_ref = -INFINITY, l_run = 0.f;
-        for (int j = jb[i]; j < je[i]; j += kStep) {
+        for (int j = jb[i]; j < J1; j += kStep) {
             const int c_it = (j - jb[i]) / kStep;
             const int j0 = j * kTileN;
             mbar_wait(bar_s + 8 * i, c_it & 1, abort_flag, p.wait_cycles, p.status, 30 + i);
@@ -497,7 +891,7 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
         // Q tile (nobody reads it once every MMA has completed; 16-byte chunks XOR-swizzled by the row) and written
         // out with 16 lanes per 256-byte row.  (maximum, sum) of the split form and the rows' token positions
         // travel through the first K/V ring slot, equally idle by now.
-        if constexpr (kSplit) {
+        {
             // merge the two groups' partial results: both accumulators sit in the TMEM lanes of this row,
             // so each group finishes 64 of the 128 output columns
             mbar_wait(bar_o, 0, abort_flag, p.wait_cycles, p.status, 40);
@@ -509,7 +903,7 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
             if (i == 0) trow_s[r] = t_row;                        // -1: no such row
             asm volatile("bar.sync 1, %0;" :: "n"(kSoftmaxThreads) : "memory");
             const float2 other = ml[(i ^ 1) * kTileM + r];
-            const bool both = je[1] > jb[1];                       // group 1 had tiles (CTA-uniform)
+            const bool both = J1 > jb[1];                       // group 1 had tiles (CTA-uniform)
             const float m0 = i == 0 ? m_ref : other.x, l0 = i == 0 ? l_run : other.y;   // group 0 always has a tile
             const float m1 = i == 0 ? other.x : m_ref, l1 = i == 0 ? other.y : l_run;
             const float m_all = both ? fmaxf(m0, m1) : m0;
@@ -546,39 +940,6 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
                 if (t_out >= 0)
                     *reinterpret_cast<uint4*>(Ob + (long long)t_out * p.os.t + l16 * 8) =
                         *reinterpret_cast<const uint4*>(smem + kOffQ + R * 256 + ((l16 ^ (R & 15)) << 4));
-            }
-        } else if (i < n_q) {
-            mbar_wait(bar_o, 0, abort_flag, p.wait_cycles, p.status, 40);
-            __syncwarp();
-            tc_fence_after();
-            const float inv = 1.f / l_run;
-            __nv_bfloat16* Oi = Ob + (kHeads ? (long long)(i * kHpt) * p.os.h : 0ll);   // this group's first head
-            int* trow_s = reinterpret_cast<int*>(smem + kOffRing + 4096) + i * kTileM;
-            trow_s[r] = t_row;
-            uint8_t* stage = smem + kOffQ + i * kTileBytes + r * 256;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                uint32_t o[32];
-                tmem_ld32(tm_o + c * 32, o);
-                tmem_wait_ld();
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    uint4 w;
-                    w.x = pack_bf16(__uint_as_float(o[8 * v + 0]) * inv, __uint_as_float(o[8 * v + 1]) * inv);
-                    w.y = pack_bf16(__uint_as_float(o[8 * v + 2]) * inv, __uint_as_float(o[8 * v + 3]) * inv);
-                    w.z = pack_bf16(__uint_as_float(o[8 * v + 4]) * inv, __uint_as_float(o[8 * v + 5]) * inv);
-                    w.w = pack_bf16(__uint_as_float(o[8 * v + 6]) * inv, __uint_as_float(o[8 * v + 7]) * inv);
-                    *reinterpret_cast<uint4*>(stage + (((c * 4 + v) ^ (r & 15)) << 4)) = w;
-                }
-            }
-            asm volatile("bar.sync %0, %1;" :: "r"(2 + i), "n"(kTileM) : "memory");   // this group's 128 threads
-            const int sub = r >> 4, l16 = r & 15;                  // 128 threads: 8 rows per pass
-#pragma unroll
-            for (int pass = 0; pass < kTileM / 8; ++pass) {
-                const int R = pass * 8 + sub, t_out = trow_s[R];
-                if (t_out >= 0)
-                    *reinterpret_cast<uint4*>(Oi + (long long)(R / kTileRows) * p.os.h + (long long)t_out * p.os.t + l16 * 8) =
-                        *reinterpret_cast<const uint4*>(smem + kOffQ + i * kTileBytes + R * 256 + ((l16 ^ (R & 15)) << 4));
             }
         }
     }
@@ -638,7 +999,7 @@ attention_tc_single_kernel(const TcParams p, const __grid_constant__ CUtensorMap
     if (warp == kMmaWarp1) tmem_alloc(smem_u32(tmem_slot), kTmemCols1);
     grid_dependency_wait();   // kept_idx / n_kept come from the kernel before this one
     int rb, bh;
-    cta_work_item(p, rb, bh);
+    work_item(p, blockIdx.x, p.n_row_blocks, rb, bh);
     int blk = p.first_pair - rb;          // heaviest expected row block first, blocks expected to be empty last
     if (blk < 0) blk += p.n_row_blocks;
     const int qh = bh % p.Hq, b = bh / p.Hq;
@@ -906,17 +1267,11 @@ cudaError_t launch_attention_tc(tf_ctx* ctx, const tf_shape& s, const tf_filter_
     static bool attr_set_dev[kDeviceFlagSlots] = {};      // function attributes are per device
     bool& attr_set = attr_set_dev[ctx->device >= 0 && ctx->device < kDeviceFlagSlots ? ctx->device : 0];
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(attention_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             Cfg<false>::kSmemBytes);
+        cudaError_t e = cudaFuncSetAttribute(attention_tc_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attention_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attention_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPSmemBytes);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(attention_tc_kernel<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     Cfg<false>::kSmemBytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(attention_tc_kernel<false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     Cfg<false>::kSmemBytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(attention_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     Cfg<true>::kSmemBytes);
+            e = cudaFuncSetAttribute(attention_tc_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SplitCfg::kSmemBytes);
         if (e != cudaSuccess) return e;
         // The kernel moves registers from its third warpgroup to the softmax warpgroups (setmaxnreg: 168 -> 72
         // releases 128 x 96, 168 -> 216 takes 256 x 48).  An inc only receives what a dec of the same CTA
@@ -925,10 +1280,10 @@ cudaError_t launch_attention_tc(tf_ctx* ctx, const tf_shape& s, const tf_filter_
         // That is a defect of the build, not a property of the call: it is reported as an error of its own and
         // never answered by running another kernel.
         cudaFuncAttributes fa{};
-        if (cudaFuncGetAttributes(&fa, attention_tc_kernel<false>) != cudaSuccess || fa.numRegs != 168 ||
-            cudaFuncGetAttributes(&fa, attention_tc_kernel<false, 1>) != cudaSuccess || fa.numRegs != 168 ||
-            cudaFuncGetAttributes(&fa, attention_tc_kernel<false, 2>) != cudaSuccess || fa.numRegs != 168 ||
-            cudaFuncGetAttributes(&fa, attention_tc_kernel<true>) != cudaSuccess || fa.numRegs != 168)
+        if (cudaFuncGetAttributes(&fa, attention_tc_kernel<0>) != cudaSuccess || fa.numRegs != 168 ||
+            cudaFuncGetAttributes(&fa, attention_tc_kernel<1>) != cudaSuccess || fa.numRegs != 168 ||
+            cudaFuncGetAttributes(&fa, attention_tc_kernel<2>) != cudaSuccess || fa.numRegs != 168 ||
+            cudaFuncGetAttributes(&fa, attention_tc_split_kernel) != cudaSuccess || fa.numRegs != 168)
             return cudaErrorInvalidDeviceFunction;
         // the single form: 256 threads at 128 registers, traded 128 x 200 + 128 x 56
         e = cudaFuncSetAttribute(attention_tc_single_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes1);
@@ -973,9 +1328,10 @@ cudaError_t launch_attention_tc(tf_ctx* ctx, const tf_shape& s, const tf_filter_
                                                                       : (long long)s.seq;
         const long long blocks = (std::max<long long>(kept_est, 1) + rows_per_cta - 1) / rows_per_cta;
         tp.first_pair = (int)std::min<long long>(std::max<long long>(blocks - 1, 0), tp.n_row_blocks - 1);
+        tp.n_blocks_est = tp.first_pair + 1;
     }
     const long long n_bh = (long long)(heads ? s.n_q_heads / (2 * hpt) : s.n_q_heads) * s.batch;
-    const long long n_ctas = (long long)tp.n_row_blocks * n_bh;
+    const long long n_ctas = (long long)(split || single ? tp.n_row_blocks : tp.n_blocks_est) * n_bh;
     {
         // Groups of (batch, head) pairs.  Heaviest-first over ALL heads balances best and costs nothing while all of K
         // and V stays in L2 (c4: 555 -> 526 us).  Once the K and V of the heads that run together exceed L2, every CTA
@@ -999,10 +1355,10 @@ cudaError_t launch_attention_tc(tf_ctx* ctx, const tf_shape& s, const tf_filter_
     if (n_ctas > 0x7fffffffll) return cudaErrorInvalidValue;
     cudaError_t e;
     if (single) e = launch_dependent(attention_tc_single_kernel, dim3((unsigned)n_ctas), dim3(kThreads1), kSmemBytes1, st, tp, mapK, mapV);
-    else if (hpt == 2) e = launch_dependent(attention_tc_kernel<false, 2>, dim3((unsigned)n_ctas), dim3(kThreads), Cfg<false>::kSmemBytes, st, tp, mapK, mapV);
-    else if (hpt == 1) e = launch_dependent(attention_tc_kernel<false, 1>, dim3((unsigned)n_ctas), dim3(kThreads), Cfg<false>::kSmemBytes, st, tp, mapK, mapV);
-    else if (split) e = launch_dependent(attention_tc_kernel<true>, dim3((unsigned)n_ctas), dim3(kThreads), Cfg<true>::kSmemBytes, st, tp, mapK, mapV);
-    else       e = launch_dependent(attention_tc_kernel<false>, dim3((unsigned)n_ctas), dim3(kThreads), Cfg<false>::kSmemBytes, st, tp, mapK, mapV);
+    else if (split) e = launch_dependent(attention_tc_split_kernel, dim3((unsigned)n_ctas), dim3(kThreads), SplitCfg::kSmemBytes, st, tp, mapK, mapV);
+    else if (hpt == 2) e = launch_dependent(attention_tc_kernel<2>, dim3((unsigned)n_ctas), dim3(kThreads), kPSmemBytes, st, tp, mapK, mapV);
+    else if (hpt == 1) e = launch_dependent(attention_tc_kernel<1>, dim3((unsigned)n_ctas), dim3(kThreads), kPSmemBytes, st, tp, mapK, mapV);
+    else       e = launch_dependent(attention_tc_kernel<0>, dim3((unsigned)n_ctas), dim3(kThreads), kPSmemBytes, st, tp, mapK, mapV);
     ctx->launches += 1;
     ctx->last_attention_kernel = single ? TF_KERNEL_ATTN_TC_SINGLE : hpt == 2 ? TF_KERNEL_ATTN_TC_HEAD_QUAD : hpt == 1 ? TF_KERNEL_ATTN_TC_HEAD_PAIR
                                         : split ? TF_KERNEL_ATTN_TC_SPLIT : TF_KERNEL_ATTN_TC_SHARED;

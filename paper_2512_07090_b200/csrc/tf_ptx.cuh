@@ -26,6 +26,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
+// whether the phase of this parity has completed, without waiting
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
 // Bounded wait.  Returns false when the cycle budget ran out or another thread of the CTA has
 // already given up (abort_flag); the first thread to give up records TF_ERR_TIMEOUT.
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, volatile int* abort_flag,
@@ -107,6 +114,28 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+
+// 16 bytes, of which the first src_bytes (0 or 16) are copied and the rest is zero
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" :: "r"(dst), "l"(src), "r"(src_bytes) : "memory");
+}
+
+// ---- cluster launch control: a running CTA takes over the work of one of its grid that waits to be launched ----------
+// asks for it; the answer (16 bytes at dst) completes 16 bytes of transaction on bar
+__device__ __forceinline__ void launch_queue_claim(uint32_t dst, uint32_t bar) {
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+                 :: "r"(dst), "r"(bar) : "memory");
+}
+// false: nothing was waiting (no further request may be made); else item = blockIdx.x of the CTA that will not be launched
+__device__ __forceinline__ bool launch_queue_item(uint32_t answer, unsigned int& item) {
+    uint32_t ok, x;
+    asm volatile("{\n.reg .pred p;\n.reg .b128 r;\nld.shared.b128 r, [%2];\nmov.u32 %1, 0;\n"
+                 "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n"
+                 "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, r;\nselp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok), "=r"(x) : "r"(answer) : "memory");
+    item = x;
+    return ok != 0;
+}
 
 // ---- tcgen05: tensor memory, products, loads / stores of accumulators -----------------------------------
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }

@@ -482,6 +482,37 @@ def test_pruned_attention_head_groups_of_unequal_size():
     g.close()
 
 
+@pytest.mark.parametrize("path,S,window,claimed_ratio", [(2, 100, 0, 0.0), (2, 400, 0, 0.5), (2, 300, 70, 0.9), (5, 40, 0, 0.0),
+                                                         (5, 300, 0, 0.9), (6, 65, 0, 0.0), (6, 300, 0, 0.5), (6, 400, 130, 0.9)])
+def test_pruned_attention_many_short_items_per_cta(path, S, window, claimed_ratio):
+    """More work items than SMs, of one to four K/V tiles each, so that a CTA takes several of them and goes from one to the
+    next without a pause; retained lists of every length (none, one, all), also longer than the ratio suggests."""
+    B, Hq, Hkv = 13, 32, 8
+    q, k, v = _qkv(B, S, Hq, Hkv, torch.bfloat16, seed=S)
+    rng = np.random.default_rng(S)
+    mask = (rng.random((B, S)) < np.linspace(0.05, 0.95, B)[:, None]).astype(np.uint8)
+    mask[0], mask[1], mask[2], mask[2, S // 2] = 0, 1, 0, 1
+    idx = np.full((B, S), -1, np.int32)
+    for b in range(B):
+        idx[b, :mask[b].sum()] = np.nonzero(mask[b])[0]
+    g = Gpu(q, k, v, window=window, prune_ratio=claimed_ratio)
+    g.ctx.tf_set_attention_path(path)
+    idx_d, nk_d = torch.from_numpy(idx).to(DEV), torch.from_numpy(mask.sum(1).astype(np.int32)).to(DEV)
+    qn, kn, vn = oracle_inputs(q, k, v)
+    ref = oracle.pruned_attention(qn, kn, vn, mask, window=window)
+    first = None
+    for _ in range(3):
+        g.O.fill_(float("nan"))
+        g.ctx.tf_pruned_attention(g.shape, g.params, q, k, v, idx_d, nk_d, g.O)
+        g.status_ok()
+        first = g.O.clone() if first is None else first
+        assert torch.equal(first, g.O)                # whichever CTA takes an item, the result is the same
+    o = to_np(g.O)
+    assert attn_rel_err(o, ref) < ATTN_TOL[torch.bfloat16]
+    assert np.all(o[mask == 0] == 0.0)
+    g.close()
+
+
 @pytest.mark.parametrize("tensor_cores", [2, 3, 4, 5, 6])
 @pytest.mark.parametrize("claimed_ratio", [0.0, 0.9])
 def test_pruned_attention_with_a_retained_list_the_ratio_does_not_predict(tensor_cores, claimed_ratio):

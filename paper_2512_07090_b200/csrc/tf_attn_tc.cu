@@ -237,8 +237,13 @@ constexpr int kPStages = 4;                            // K/V ring slots
 constexpr int kPQSlots = 3;
 constexpr int kPOffQ = 0, kPOffRing = kPQSlots * kTileBytes, kPOffRows = kPOffRing + kPStages * kTileBytes;
 constexpr int kPOffMisc = kPOffRows + 2 * kSoftmaxThreads * 4;      // two sets of token positions of an item's rows
-constexpr int kPSmemBytes = kPOffMisc + 512;           // the dynamic segment must start 1024-byte aligned (checked)
+constexpr int kPOffZero = kPOffMisc + 512, kZeroBytes = 512;        // zeros: what rows of pruned tokens are filled with
+constexpr int kPSmemBytes = kPOffZero + kZeroBytes;    // the dynamic segment must start 1024-byte aligned (checked)
 static_assert(kPSmemBytes <= 227 * 1024, "shared memory of one CTA");
+
+// the claim goes out when the K/V ring has taken all but this many of the item's tiles, four or five tile times before the
+// item ends.  0, 1, 2, 3: 76.8, 77.1, 76.2, 76.1 us (3 x 1531), 92.6, 92.2, 92.1, 91.9 us (4096 tokens), the larger cases +-0.3 %
+constexpr int kClaimLead = 2;
 
 struct TcItem {
     int valid;            // 0: there is no further item
@@ -280,7 +285,7 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
     const uint32_t bar_q1 = bar_q0 + 8;                  // [2] Q slot of tile 1, the item's rows and descriptor given back
     const uint32_t bar_item = bar_q1 + 16;               // [2] item descriptor written
     const uint32_t bar_claim = bar_item + 16;            // answer of the launch queue
-    const uint32_t bar_asked = bar_claim + 8;            // every K/V tile of the item requested
+    const uint32_t bar_asked = bar_claim + 8;            // all but the last kClaimLead K/V tiles of the item requested
     const uint32_t claim = bars + 192;                   // 16 bytes
     TcItem* const items = reinterpret_cast<TcItem*>(smem + kPOffMisc + 224);          // [2]
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kPOffMisc + 320);
@@ -301,6 +306,8 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
         *abort_flag = 0;
         mbar_fence_init();
     }
+    if (tid < kZeroBytes / 16) *reinterpret_cast<uint4*>(smem + kPOffZero + tid * 16) = make_uint4(0, 0, 0, 0);
+    fence_proxy_async();
     __syncwarp();
     if (warp == kMmaWarp) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
     tc_fence_before();
@@ -324,7 +331,7 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
     if (warp >= kGatherWarp) {
         // ================================ items, Q rows, zero rows ====================================
         const int w = warp - kGatherWarp, sub = lane >> 4, l16 = lane & 15;
-        const uint4 zero4 = make_uint4(0, 0, 0, 0);
+        const bool dense_heads = p.os.h == kHeadDim;
         unsigned int item = blockIdx.x;
         int n = 0, claims = 0;
         for (;;) {
@@ -333,14 +340,19 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
             const int qh = (bh % (p.Hq / kHeadsPerCta)) * kHeadsPerCta, b = bh / (p.Hq / kHeadsPerCta);   // first (or only) head
             const int nk = p.n_kept[b];
             const int32_t* kept = p.kept_idx + (size_t)b * p.S;
-            __nv_bfloat16* Ob = p.O + (long long)b * p.os.b + (long long)qh * p.os.h + l16 * 8;
+            __nv_bfloat16* Ob = p.O + (long long)b * p.os.b + (long long)qh * p.os.h;
+            // zeroes token t's output rows of n_heads (1 or 2) heads from head hh on: bulk copies, one instruction of one lane each
+            auto zero_token = [&](int t, int hh, int n_heads) {
+                __nv_bfloat16* dst = Ob + (long long)hh * p.os.h + (long long)t * p.os.t;
+                bulk_store(dst, sbase + kPOffZero, dense_heads ? n_heads * kHeadDim * 2 : kHeadDim * 2);
+                if (n_heads == 2 && !dense_heads) bulk_store(dst + p.os.h, sbase + kPOffZero, kHeadDim * 2);
+            };
             const __nv_bfloat16* Qb = p.Q + (long long)b * p.qs.b + (long long)qh * p.qs.h + l16 * 8;
             bool produced = false;
             const int blk0 = p.n_blocks_est - 1 - rb;         // heaviest expected row block first
             if (nk <= 0 && blk0 == 0) {                       // nothing retained at all: the whole head is zero
-                for (int hh = 0; hh < kHeadsPerCta; ++hh)
-                    for (int t = 2 * w + sub; t < p.S; t += 4)
-                        *reinterpret_cast<uint4*>(Ob + (long long)hh * p.os.h + (long long)t * p.os.t) = zero4;
+                for (int t = w * 32 + lane; t < p.S; t += kGatherThreads)
+                    for (int hh = 0; hh < kHeadsPerCta; hh += 2) zero_token(t, hh, min(kHeadsPerCta, 2));
             }
             // row blocks beyond the expected number (normally empty) go to the items of the expected ones
             for (int blk = blk0; blk < p.n_row_blocks && blk * kRows < nk; blk += p.n_blocks_est) {
@@ -415,32 +427,28 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
                 asm volatile("cp.async.wait_group 0;" ::: "memory");
                 fence_proxy_async();
                 mbar_arrive(bar_qf1);
-                // rows of pruned tokens that precede a retained row of this warp (and follow the last one of all) are zero
-                auto zero_rows = [&](const int (&kk)[2], int first, int hh0, int n_heads) {
-                    if (first >= nk) return;
-                    int before = first == 0 ? -1 : kept[first - 1];
+                // rows of pruned tokens that precede a retained row of this warp (and follow the last one of all) are zero:
+                // each lane fills the gaps before its own two entries.  (Sixteen lanes storing a row took 20,000 to 26,000
+                // cycles per item, longer than a short item's tiles; this takes a tenth.)
+                auto zero_rows = [&](const int (&kk)[2], int first, int hh, int n_heads) {
+                    int before = (first > 0 && first < nk) ? kept[first - 1] : -1;
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        int pv = __shfl_up_sync(0xffffffffu, kk[h], 1);
-                        if (lane == 0) pv = before;
+                        int prev = __shfl_up_sync(0xffffffffu, kk[h], 1);
+                        if (lane == 0) prev = before;
                         before = __shfl_sync(0xffffffffu, kk[h], 31);
-                        for (int e = 0; e < 16; ++e) {
-                            const int cur = __shfl_sync(0xffffffffu, kk[h], 2 * e + sub), prev = __shfl_sync(0xffffffffu, pv, 2 * e + sub);
-                            if (cur < 0) continue;
-                            const bool last = first + h * 32 + 2 * e + sub == nk - 1;
-                            for (int hh = hh0; hh < hh0 + n_heads; ++hh) {
-                                __nv_bfloat16* Oz = Ob + (long long)hh * p.os.h;
-                                for (int t = prev + 1; t < cur; ++t) *reinterpret_cast<uint4*>(Oz + (long long)t * p.os.t) = zero4;
-                                if (last)
-                                    for (int t = cur + 1; t < p.S; ++t) *reinterpret_cast<uint4*>(Oz + (long long)t * p.os.t) = zero4;
-                            }
-                        }
+                        for (int t = prev + 1; t < kk[h]; ++t) zero_token(t, hh, n_heads);     // (kk[h] = -1: no entry)
+                        __syncwarp();
+                        const int end = nk - 1 - (first + h * 32);                             // the lane that has the last entry of all
+                        if (end >= 0 && end < 32)
+                            for (int t = __shfl_sync(0xffffffffu, kk[h], end) + 1 + lane; t < p.S; t += 32) zero_token(t, hh, n_heads);
                         __syncwarp();
                     }
                 };
-                if (kHpt == 2) { zero_rows(k0, e0, w, 1); zero_rows(k0, e0, 2 + w, 1); }
+                if (kHpt == 2) zero_rows(k0, e0, 2 * w, 2);
                 else zero_rows(k0, e0, 0, kHeadsPerCta);
                 if (!kHeads) zero_rows(k1, e0 + kTileM, 0, 1);
+                bulk_commit();
                 ++n;
                 produced = true;
             }
@@ -465,6 +473,9 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
                 break;
             }
         }
+        __syncwarp();
+        bulk_commit();
+        bulk_wait_all();       // the zeros have been read and written
     } else if (warp == kTmaWarp) {
         // ================================ TMA producer ================================================
         TcItem it;
@@ -485,8 +496,8 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
                         tma_load_4d(dst, map, bar_full + 8 * st, 0, kh, j * kTileN, it.b);
                         tma_load_4d(dst + kHalfBytes, map, bar_full + 8 * st, 64, kh, j * kTileN, it.b);
                     }
+                    if (j == max(J1 - 1 - kClaimLead, it.jb[0])) mbar_arrive(bar_asked);
                 }
-                mbar_arrive(bar_asked);
             }
             __syncwarp();
         }

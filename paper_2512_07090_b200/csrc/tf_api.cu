@@ -104,14 +104,14 @@ void invalidate_scan_scratch(tf_ctx* ctx) {
 // bound workspace (a call on a group of heads reuses the front of it)
 tf_status attention_dispatch(tf_ctx* ctx, const tf_shape& s, const tf_filter_params& p, const void* Q,
                              const void* K, const void* V, const int32_t* kept_idx,
-                             const int32_t* n_kept, void* O, void* kv_compact, cudaStream_t st) {
+                             const int32_t* n_kept, void* O, void* kv_compact, bool after_selection, cudaStream_t st) {
     if (s.dtype == TF_BF16 && ctx->use_tensor_cores) {
         const cudaError_t e = launch_attention_tc(ctx, s, p, Q, K, V, kept_idx, n_kept, O, kv_compact, st);
         // The default path falls back to the CUDA-core kernel only when no tensor map can describe the caller's
         // layout; an explicitly requested form is a requirement, and any other failure is an error.
         if (e != cudaErrorNotSupported || ctx->attention_form != 0) return to_status(e);
     }
-    return to_status(launch_attention_simt(ctx, s, p, Q, K, V, kept_idx, n_kept, O, st));
+    return to_status(launch_attention_simt(ctx, s, p, Q, K, V, kept_idx, n_kept, O, after_selection, st));
 }
 
 // the workspace section for the retained tokens' K / V, or nullptr when this call does not need one
@@ -271,7 +271,7 @@ tf_status tf_pruned_attention(tf_ctx* ctx, const tf_shape* shape, const tf_filte
     void* kv_compact = nullptr;
     s = kv_compact_section(ctx, *shape, *params, &kv_compact);
     if (s != TF_OK) return s;
-    return attention_dispatch(ctx, *shape, *params, Q, K, V, kept_idx, n_kept, O, kv_compact, static_cast<cudaStream_t>(stream));
+    return attention_dispatch(ctx, *shape, *params, Q, K, V, kept_idx, n_kept, O, kv_compact, false, static_cast<cudaStream_t>(stream));
 }
 
 tf_status tf_layer_filter(tf_ctx* ctx, const tf_shape* shape, const tf_filter_params* params,
@@ -307,7 +307,7 @@ tf_status tf_layer_filter(tf_ctx* ctx, const tf_shape* shape, const tf_filter_pa
     void* kv_compact = nullptr;
     s = kv_compact_section(ctx, *shape, *params, &kv_compact);
     if (s != TF_OK) return s;
-    return attention_dispatch(ctx, *shape, *params, Q, K, V, kept_idx, n_kept, O, kv_compact, st);
+    return attention_dispatch(ctx, *shape, *params, Q, K, V, kept_idx, n_kept, O, kv_compact, true, st);
 }
 
 tf_status tf_layer_filter_host(tf_ctx* ctx, const tf_shape* shape, const tf_filter_params* params,
@@ -413,7 +413,7 @@ tf_status tf_layer_filter_host(tf_ctx* ctx, const tf_shape* shape, const tf_filt
         gs.n_q_heads = hq_g; gs.n_kv_heads = hkv_g;
         const size_t kv_off = (size_t)g2 * hkv_g * d * es;
         s = attention_dispatch(ctx, gs, *params, dQ + off, static_cast<char*>(dK) + kv_off, static_cast<char*>(dV) + kv_off, dI, dN,
-                               dO + off, kv_compact, st);
+                               dO + off, kv_compact, false, st);
         if (s != TF_OK) break;
         e = cudaEventRecord(ev_att, st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->s_out, ev_att, 0);

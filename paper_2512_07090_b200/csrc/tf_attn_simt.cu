@@ -14,6 +14,9 @@
 // attention output is zero), so the whole of O is written with no separate clearing pass.
 //   One warp per row, a key at a time per lane straight from global memory, took 48 us at 1 x 128 tokens x 32 heads, 392 at
 // 512 and 4700 at 2 x 1024 x 40 heads; this kernel takes 11, 85 and 670.
+// CTAs with rows start before those expected to have none, over all heads (a quarter to a half of the grid was empty CTAs
+// between the others), and inside a layer step the first chunk is fetched while the selection runs: per pass 1 x 300 x 32
+// heads 63.5 -> 52.4 us, 1 x 700 143 -> 119, 2 x 1000 571 -> 506.
 #include <algorithm>
 
 #include "tf_common.cuh"
@@ -32,6 +35,8 @@ struct AttnParams {
     float scale_log2;          // softmax scale * log2(e)
     const int32_t* kept_idx;   // [B,S]
     const int32_t* n_kept;     // [B]
+    int n_blocks, blocks_est;  // row blocks per head / those expected to hold retained rows (they start first)
+    int early;                 // 1: the selection kernel is the one before this on the stream and the first chunk is known
     int retained_only;         // 1: a retained query sees retained tokens' keys / values only
 };
 
@@ -63,6 +68,7 @@ __device__ __forceinline__ void fetch4(float* dst, const __nv_bfloat16* src, boo
     *reinterpret_cast<float4*>(dst) = live ? load4(src) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 __device__ __forceinline__ void fetch_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void fetch_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void fetch_wait_all_but_one() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
 template <typename T>
@@ -75,22 +81,14 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
     using C = SimtCfg<kSplit>;
     constexpr int R = kSimtRows;
     extern __shared__ __align__(16) float simt_smem[];
-    grid_dependency_wait();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int part = warp / (kSimtWarps / kSplit), ptid = tid & (C::kPartThreads - 1);
     const int rgroup = warp & (kSimtWarps / kSplit - 1);
-    const int qh = blockIdx.y, b = blockIdx.z;
-    const int nk = p.n_kept[b];
-    const int slot0 = ((int)gridDim.x - 1 - (int)blockIdx.x) * C::kRows;     // the longest rows first
+    const int qh = (int)blockIdx.x % p.Hq, b = blockIdx.z, rb = (int)blockIdx.x / p.Hq;
+    const int blk = p.blocks_est - 1 - rb + (rb < p.blocks_est ? 0 : p.n_blocks);     // the longest rows first, empty blocks last
+    const int slot0 = blk * C::kRows;
     const int32_t* kept = p.kept_idx + (size_t)b * p.S;
     T* Ob = reinterpret_cast<T*>(p.O) + (long long)b * p.os.b + (long long)qh * p.os.h;
-    if (nk == 0) {
-        if (slot0 == 0)
-            for (int t = warp; t < p.S; t += kSimtWarps) zero_rows(Ob, p.os, t, t + 1, lane);
-        return;
-    }
-    if (slot0 >= nk) return;
-
     float* const sK = simt_smem + part * 2 * C::kChunkFloats;
     float* const sV = sK + C::kChunkFloats;
     float* const sQ = simt_smem + C::kOffQ;
@@ -98,6 +96,29 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
     const int kh = qh / (p.Hq / p.Hkv);
     const T* Kb = reinterpret_cast<const T*>(p.K) + (long long)b * p.ks.b + (long long)kh * p.ks.h;
     const T* Vb = reinterpret_cast<const T*>(p.V) + (long long)b * p.vs.b + (long long)kh * p.vs.h;
+    // one 16-byte piece per thread and step; the pieces of a key row are rotated (XOR) by the row so that lanes reading the
+    // same piece of 8 consecutive rows hit different banks
+    auto fetch = [&](float* dst, const T* base, long long stride, int ch, int last, bool swizzle) {
+#pragma unroll 4
+        for (int i = ptid; i < kSimtChunk * 32; i += C::kPartThreads) {
+            const int row = i >> 5, piece = i & 31, j = ch * kSimtChunk + row;
+            const bool live = j <= last;
+            const long long tok = live ? (p.retained_only ? kept[j] : j) : 0;
+            fetch4(dst + row * kHeadDim + ((swizzle ? piece ^ (row & 7) : piece) << 2), base + tok * stride + piece * 4, live);
+        }
+        fetch_commit();
+    };
+    // the first chunk of keys and values does not depend on the selection: it is fetched while that still runs
+    const bool early = p.early && blk < p.blocks_est && part * kSimtChunk < p.S;
+    if (early) { fetch(sK, Kb, p.ks.t, part, p.S - 1, true); fetch(sV, Vb, p.vs.t, part, p.S - 1, false); }
+    grid_dependency_wait();
+    const int nk = p.n_kept[b];
+    if (slot0 >= nk) {
+        if (nk == 0 && slot0 == 0)
+            for (int t = warp; t < p.S; t += kSimtWarps) zero_rows(Ob, p.os, t, t + 1, lane);
+        fetch_wait_all();
+        return;
+    }
 
     // keys are visited by index: token positions, or positions in the retained list (retained_only), where entry c stands
     // for token kept[c] and the query itself is its own entry
@@ -109,24 +130,17 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
     const int c_hi = p.retained_only ? s_last : kept[s_last];              // the CTA's last visible key
     const int ch0 = first_key(slot0, kept[slot0]) / kSimtChunk, ch1 = c_hi / kSimtChunk + 1;
 
-    // one 16-byte piece per thread and step; the pieces of a key row are rotated (XOR) by the row so that lanes reading the
-    // same piece of 8 consecutive rows hit different banks
-    auto fetch = [&](float* dst, const T* base, long long stride, int ch, bool swizzle) {
-#pragma unroll 4
-        for (int i = ptid; i < kSimtChunk * 32; i += C::kPartThreads) {
-            const int row = i >> 5, piece = i & 31, j = ch * kSimtChunk + row;
-            const bool live = j <= c_hi;
-            const long long tok = live ? (p.retained_only ? kept[j] : j) : 0;
-            fetch4(dst + row * kHeadDim + ((swizzle ? piece ^ (row & 7) : piece) << 2), base + tok * stride + piece * 4, live);
-        }
-        fetch_commit();
-    };
     auto part_sync = [&]() {
         if (kSplit == 1) __syncthreads();
         else asm volatile("bar.sync %0, %1;" :: "r"(1 + part), "n"(C::kPartThreads) : "memory");
     };
     int ch = ch0 + part;
-    if (ch < ch1) { fetch(sK, Kb, p.ks.t, ch, true); fetch(sV, Vb, p.vs.t, ch, false); }
+    if (!early && ch < ch1) { fetch(sK, Kb, p.ks.t, ch, c_hi, true); fetch(sV, Vb, p.vs.t, ch, c_hi, false); }
+    if (early && c_hi < (part + 1) * kSimtChunk - 1) {     // values behind the last visible key: zero, as when fetched with the limit
+        fetch_wait_all();
+        for (int i = ptid; i < kSimtChunk * 32; i += C::kPartThreads)      // (the pieces this thread fetched)
+            if (part * kSimtChunk + (i >> 5) > c_hi) *reinterpret_cast<float4*>(sV + (i >> 5) * kHeadDim + ((i & 31) << 2)) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     for (int i = tid; i < C::kRows * 32; i += kSimtThreads) {
         const int row = i >> 5, piece = i & 31, slot = slot0 + row;
         float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -177,7 +191,7 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
             }
         }
         part_sync();                                                       // K(ch) has been read
-        if (ch + kSplit < ch1) fetch(sK, Kb, p.ks.t, ch + kSplit, true); else fetch_commit();
+        if (ch + kSplit < ch1) fetch(sK, Kb, p.ks.t, ch + kSplit, c_hi, true); else fetch_commit();
         if (mine) {
             const int ja = j0 + lane, jb = ja + 32;
 #pragma unroll
@@ -217,10 +231,11 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
             __syncwarp();                                                  // sP is written again in the next chunk
         }
         part_sync();                                                       // V(ch) has been read
-        if (ch + kSplit < ch1) fetch(sV, Vb, p.vs.t, ch + kSplit, false); else fetch_commit();
+        if (ch + kSplit < ch1) fetch(sV, Vb, p.vs.t, ch + kSplit, c_hi, false); else fetch_commit();
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) l[r] = warp_sum(l[r]);
+    fetch_wait_all();
     if (kSplit == 2) {      // the second half of the CTA hands its part of every row to the first
         float* const other = simt_smem + row0 * (kHeadDim + 4);
         __syncthreads();
@@ -256,7 +271,7 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
 }
 
 template <typename T, int kSplit>
-static cudaError_t launch_simt_form(const AttnParams& ap, int batch, int device, cudaStream_t st) {
+static cudaError_t launch_simt_form(AttnParams ap, double kept, int batch, int device, cudaStream_t st) {
     using C = SimtCfg<kSplit>;
     static bool attr_set_dev[kDeviceFlagSlots] = {};      // function attributes are per device
     bool& attr_set = attr_set_dev[device >= 0 && device < kDeviceFlagSlots ? device : 0];
@@ -265,14 +280,17 @@ static cudaError_t launch_simt_form(const AttnParams& ap, int batch, int device,
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    return launch_dependent(attention_simt_kernel<T, kSplit>, dim3((unsigned)((ap.S + C::kRows - 1) / C::kRows), (unsigned)ap.Hq, (unsigned)batch),
+    ap.n_blocks = (ap.S + C::kRows - 1) / C::kRows;
+    ap.blocks_est = std::min(std::max((int)ceil(kept / C::kRows), 1), ap.n_blocks);
+    if ((long long)ap.n_blocks * ap.Hq > 0x7fffffffll) return cudaErrorInvalidValue;
+    return launch_dependent(attention_simt_kernel<T, kSplit>, dim3((unsigned)ap.n_blocks * (unsigned)ap.Hq, 1, (unsigned)batch),
                             dim3(kSimtThreads), C::kSmemBytes, st, ap);
 }
 
 cudaError_t launch_attention_simt(tf_ctx* ctx, const tf_shape& s, const tf_filter_params& p,
                                   const void* Q, const void* K, const void* V,
                                   const int32_t* kept_idx, const int32_t* n_kept, void* O,
-                                  cudaStream_t st) {
+                                  bool after_selection, cudaStream_t st) {
     if (s.batch == 0 || s.seq == 0) return cudaSuccess;
     AttnParams ap{};
     ap.retained_only = (p.kv_visibility == TF_KV_RETAINED);
@@ -285,14 +303,16 @@ cudaError_t launch_attention_simt(tf_ctx* ctx, const tf_shape& s, const tf_filte
     const float scale = s.softmax_scale != 0.f ? s.softmax_scale : 1.f / sqrtf((float)s.head_dim);
     ap.scale_log2 = scale * 1.4426950408889634f;
     ap.kept_idx = kept_idx; ap.n_kept = n_kept;
+    ap.early = after_selection && s.window == 0 && !ap.retained_only;
     // Up to two 16-row CTAs per SM the split form wins (us at 1 x 128 x 32 heads, 1 x 256 x 32, 2 x 256 x 32: 11 / 33 / 52
     // split, 16 / 44 / 45 unsplit), beyond that its second set of chunks costs more than it hides (1 x 768 x 40: 196 / 177).
     // The number of retained rows is only known on the device: the ratio gives the expected count.
     const double kept_frac = (p.select_mode == TF_SELECT_RATIO) ? 1.0 - p.prune_ratio : 1.0;
     const bool split = (double)s.batch * s.n_q_heads * ceil(s.seq * kept_frac / 16.0) <= 2.0 * sm_count();
     cudaError_t e;
-    if (s.dtype == TF_BF16) e = split ? launch_simt_form<__nv_bfloat16, 2>(ap, s.batch, ctx->device, st) : launch_simt_form<__nv_bfloat16, 1>(ap, s.batch, ctx->device, st);
-    else                    e = split ? launch_simt_form<float, 2>(ap, s.batch, ctx->device, st) : launch_simt_form<float, 1>(ap, s.batch, ctx->device, st);
+    const double kept = ceil(s.seq * kept_frac);
+    if (s.dtype == TF_BF16) e = split ? launch_simt_form<__nv_bfloat16, 2>(ap, kept, s.batch, ctx->device, st) : launch_simt_form<__nv_bfloat16, 1>(ap, kept, s.batch, ctx->device, st);
+    else                    e = split ? launch_simt_form<float, 2>(ap, kept, s.batch, ctx->device, st) : launch_simt_form<float, 1>(ap, kept, s.batch, ctx->device, st);
     ctx->launches += 1;
     ctx->last_attention_kernel = TF_KERNEL_ATTN_SIMT;
     return e;

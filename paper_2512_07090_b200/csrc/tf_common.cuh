@@ -265,7 +265,7 @@ cudaError_t launch_score_select(tf_ctx* ctx, const tf_shape& s, const tf_filter_
 cudaError_t launch_attention_simt(tf_ctx* ctx, const tf_shape& s, const tf_filter_params& p,
                                   const void* Q, const void* K, const void* V,
                                   const int32_t* kept_idx, const int32_t* n_kept, void* O,
-                                  cudaStream_t st);
+                                  bool after_selection, cudaStream_t st);
 struct tf_decode_args {
     const void* q_new; const void* K_cache; const void* V_cache; const int32_t* pos;
     const tf_decode_state* state; void* O_new; float* score_out; uint8_t* skip_out;

@@ -60,8 +60,10 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_kernel(const SelectPara
     __shared__ int s_tab[KPT > 0 ? KPT : kMaxTableChunks][kSelWarps];   // [chunk][warp] ballot counts of the final sweep
     __shared__ unsigned int s_few[32];
 
-    grid_launch_dependents();   // one CTA per sequence: the attention grid may take the other SMs and set up meanwhile
     grid_dependency_wait();
+    // One CTA per sequence: the attention grid may take the other SMs and set up meanwhile.  After the wait, so that whatever
+    // was queued before this kernel is complete when that grid starts and it may read the inputs ahead of its own wait.
+    grid_launch_dependents();
     const int b = blockIdx.x, tid = threadIdx.x, S = p.S;
     const float* sc = p.score + (size_t)b * S;
     if (KPT == 0 && p.stage) {   // too many scores for registers: the passes below read them from shared memory

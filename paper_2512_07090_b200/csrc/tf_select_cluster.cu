@@ -88,8 +88,8 @@ __global__ void __launch_bounds__(kCsThreads, 1) select_cluster_kernel(const Clu
     __shared__ unsigned int s_few[32];        // CTA 0's copy: the last few candidates' keys, appended by the whole cluster
     __shared__ int s_few_n;
 
-    grid_launch_dependents();   // few CTAs: the attention grid may take the other SMs and set up meanwhile
     grid_dependency_wait();
+    grid_launch_dependents();   // few CTAs: the attention grid may take the other SMs and set up meanwhile (see select_kernel)
     cg::cluster_group cluster = cg::this_cluster();
     const int n_ranks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const int b = (int)blockIdx.x / n_ranks, tid = threadIdx.x, S = p.S;

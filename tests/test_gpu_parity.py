@@ -428,6 +428,25 @@ def test_cuda_core_attention_both_forms(B, S, Hq, Hkv, window, ratio, visibility
     g.close()
 
 
+@pytest.mark.parametrize("B,S,Hq,Hkv,ratio", [(1, 1, 2, 2, 0.0), (1, 63, 4, 4, 0.5), (2, 64, 4, 2, 0.5), (1, 65, 32, 32, 0.3),
+                                              (1, 200, 32, 32, 0.7), (3, 129, 8, 2, 0.25), (2, 300, 40, 40, 0.5)])
+def test_fp32_layer_step_has_the_bits_of_its_attention_alone(B, S, Hq, Hkv, ratio):
+    """Inside a layer step the CUDA-core attention fetches its first keys and values while the selection runs, without
+    knowing which is the last it may see; alone it fetches up to the last visible one.  Same bits."""
+    q, k, v = _qkv(B, S, Hq, Hkv, torch.float32, seed=S)
+    g = Gpu(q, k, v, prune_ratio=ratio, warmup_tokens=1)
+    for _ in range(2):
+        g.O.fill_(float("nan"))
+        g.ctx.tf_layer_filter(g.shape, g.params, q, k, v, g.O, g.score, g.keep, g.idx, g.nk)
+    g.status_ok()
+    layer = g.O.clone()
+    g.O.fill_(float("nan"))
+    g.ctx.tf_pruned_attention(g.shape, g.params, q, k, v, g.idx, g.nk, g.O)
+    g.status_ok()
+    assert torch.equal(layer, g.O)
+    g.close()
+
+
 def test_layer_filter_retained_keys_only():
     q, k, v = _qkv(2, 700, 8, 2, torch.bfloat16, seed=77)
     n_mis = _layer_case(q, k, v, window=0, prune_ratio=0.5, warmup_tokens=4, kv_visibility=tfb.TF_KV_RETAINED)

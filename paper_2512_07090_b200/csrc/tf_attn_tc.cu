@@ -1322,7 +1322,13 @@ cudaError_t launch_attention_tc(tf_ctx* ctx, const tf_shape& s, const tf_filter_
     const double ctas_shared = (double)s.batch * s.n_q_heads * ceil(s.seq * kept_frac / (kQTiles * kTileM));
     const int sms = sm_count();
     const bool single = ctx->attention_form == 3;
-    const bool split = ctx->attention_form == 2 || (ctx->attention_form == 0 && ctas_shared < 1.0 * sms);
+    // ... when all its CTAs run at once, or when a row's keys are many (32 heads x 2048 tokens, 16 tiles: 34.4 us against 37.7):
+    // with few tiles per CTA the second wave of CTAs costs more than the halved length saves (4 x 512 tokens x 32 heads: 26.5
+    // against 19.4).
+    double keys = compact ? s.seq * kept_frac : (double)s.seq;
+    if (s.window > 0) keys = std::min(keys, (double)s.window + kTileM / std::max(kept_frac, 1e-3));
+    const bool split = ctx->attention_form == 2 ||
+                       (ctx->attention_form == 0 && ctas_shared < 1.0 * sms && (2.0 * ctas_shared <= sms || keys > 7.0 * kTileN));
     // Grouped-query attention with an even number of query heads per KV head: the two Q tiles of a shared-form CTA are
     // the same 128 retained rows of two query heads of one group instead of 256 rows of one head; with a multiple of
     // four, the same 64 rows of four heads (two per tile): the shorter the span of positions a CTA's rows cover, the

@@ -18,6 +18,7 @@
 // between the others), and inside a layer step the first chunk is fetched while the selection runs: per pass 1 x 300 x 32
 // heads 63.5 -> 52.4 us, 1 x 700 143 -> 119, 2 x 1000 571 -> 506.
 #include <algorithm>
+#include <type_traits>
 
 #include "tf_common.cuh"
 
@@ -70,6 +71,13 @@ __device__ __forceinline__ void fetch4(float* dst, const __nv_bfloat16* src, boo
 __device__ __forceinline__ void fetch_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void fetch_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void fetch_wait_all_but_one() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+
+// a += w * v where `yes`, without a branch
+__device__ __forceinline__ void fma4_if(float (&a)[4], float w, const float4& v, bool yes) {
+    asm("{\n.reg .pred p;\nsetp.ne.u32 p, %9, 0;\n@p fma.rn.f32 %0, %4, %5, %0;\n@p fma.rn.f32 %1, %4, %6, %1;\n"
+        "@p fma.rn.f32 %2, %4, %7, %2;\n@p fma.rn.f32 %3, %4, %8, %3;\n}"
+        : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]) : "f"(w), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"((unsigned int)yes));
+}
 
 template <typename T>
 __device__ __forceinline__ void zero_rows(T* Ob, const Strides3& os, int t_lo, int t_hi, int lane) {
@@ -136,11 +144,6 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
     };
     int ch = ch0 + part;
     if (!early && ch < ch1) { fetch(sK, Kb, p.ks.t, ch, c_hi, true); fetch(sV, Vb, p.vs.t, ch, c_hi, false); }
-    if (early && c_hi < (part + 1) * kSimtChunk - 1) {     // values behind the last visible key: zero, as when fetched with the limit
-        fetch_wait_all();
-        for (int i = ptid; i < kSimtChunk * 32; i += C::kPartThreads)      // (the pieces this thread fetched)
-            if (part * kSimtChunk + (i >> 5) > c_hi) *reinterpret_cast<float4*>(sV + (i >> 5) * kHeadDim + ((i & 31) << 2)) = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
     for (int i = tid; i < C::kRows * 32; i += kSimtThreads) {
         const int row = i >> 5, piece = i & 31, slot = slot0 + row;
         float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -150,6 +153,7 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
     }
     const int row0 = rgroup * R;
     int lo[R], hi[R], w_lo = 0x7fffffff, w_hi = -1;                     // visible keys of each row (hi < lo: no such row)
+    int all_lo = 0, all_hi = 0x7fffffff;                                // keys that every row of the warp sees
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int slot = slot0 + row0 + r;
@@ -159,6 +163,7 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
             lo[r] = first_key(slot, t);
             hi[r] = p.retained_only ? slot : t;
             w_lo = min(w_lo, lo[r]); w_hi = max(w_hi, hi[r]);
+            all_lo = max(all_lo, lo[r]); all_hi = min(all_hi, hi[r]);
         }
     }
     __syncthreads();
@@ -166,6 +171,25 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
     float m[R], l[R], acc[R][4];                                          // l: this lane's share of the row's sum
 #pragma unroll
     for (int r = 0; r < R; ++r) { m[r] = -1e30f; l[r] = 0.f; acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = 0.f; }
+    auto weigh = [&](int jj, int j0, auto edge) {                         // four keys' values into the rows' sums
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = reinterpret_cast<const float4*>(sV)[(jj + u) * 32 + lane];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float4 w = *reinterpret_cast<const float4*>(sP + r * kSimtChunk + jj);
+            const float wu[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if constexpr (decltype(edge)::value) {
+                    fma4_if(acc[r], wu[u], v[u], j0 + jj + u >= lo[r] && j0 + jj + u <= hi[r]);
+                } else {
+                    acc[r][0] = fmaf(wu[u], v[u].x, acc[r][0]); acc[r][1] = fmaf(wu[u], v[u].y, acc[r][1]);
+                    acc[r][2] = fmaf(wu[u], v[u].z, acc[r][2]); acc[r][3] = fmaf(wu[u], v[u].w, acc[r][3]);
+                }
+            }
+        }
+    };
     for (; ch < ch1; ch += kSplit) {
         const int j0 = ch * kSimtChunk;
         const bool mine = w_hi >= j0 && w_lo < j0 + kSimtChunk;            // some row of this warp sees this chunk
@@ -212,22 +236,13 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
         fetch_wait_all_but_one();
         part_sync();                                                       // V(ch) is there
         if (mine) {
+            // A probability of 0 does not keep a value out of a row that may not see it (0 * Inf and 0 * NaN are NaN): groups of
+            // keys that not every row of the warp sees make the products of the rows that do.
             const int jj0 = max(0, w_lo - j0) & ~3, jj1 = min(kSimtChunk, w_hi - j0 + 1);
-            for (int jj = jj0; jj < jj1; jj += 4) {
-                float4 v[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) v[u] = reinterpret_cast<const float4*>(sV)[(jj + u) * 32 + lane];
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float4 w = *reinterpret_cast<const float4*>(sP + r * kSimtChunk + jj);
-                    const float wu[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        acc[r][0] = fmaf(wu[u], v[u].x, acc[r][0]); acc[r][1] = fmaf(wu[u], v[u].y, acc[r][1]);
-                        acc[r][2] = fmaf(wu[u], v[u].z, acc[r][2]); acc[r][3] = fmaf(wu[u], v[u].w, acc[r][3]);
-                    }
-                }
-            }
+            const int in0 = min(max(all_lo - j0 + 3, jj0) & ~3, jj1), in1 = min(max((all_hi + 1 - j0) & ~3, in0), jj1);
+            for (int jj = jj0; jj < in0; jj += 4) weigh(jj, j0, std::true_type());
+            for (int jj = in0; jj < in1; jj += 4) weigh(jj, j0, std::false_type());
+            for (int jj = in1; jj < jj1; jj += 4) weigh(jj, j0, std::true_type());
             __syncwarp();                                                  // sP is written again in the next chunk
         }
         part_sync();                                                       // V(ch) has been read

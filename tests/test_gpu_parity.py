@@ -447,6 +447,32 @@ def test_fp32_layer_step_has_the_bits_of_its_attention_alone(B, S, Hq, Hkv, rati
     g.close()
 
 
+@pytest.mark.parametrize("B,S,Hq,Hkv", [(1, 300, 2, 2), (2, 520, 40, 40)])     # two chunk sequences per CTA / all warps on one
+@pytest.mark.parametrize("window,visibility", [(0, tfb.TF_KV_ALL), (41, tfb.TF_KV_ALL), (0, tfb.TF_KV_RETAINED), (41, tfb.TF_KV_RETAINED)])
+def test_cuda_core_attention_keeps_a_value_out_of_rows_that_may_not_see_it(B, S, Hq, Hkv, window, visibility):
+    """Inf or NaN in the values of one token: the rows before it and those whose window has passed it keep their bits."""
+    q, k, v = _qkv(B, S, Hq, Hkv, torch.float32, seed=S)
+    g = Gpu(q, k, v, window=window, prune_ratio=0.25, kv_visibility=visibility)
+    kept = np.sort(np.random.default_rng(S).permutation(S)[:3 * S // 4])
+    idx = torch.full((B, S), -1, dtype=torch.int32, device=DEV)
+    idx[:, :len(kept)] = torch.from_numpy(kept.astype(np.int32)).to(DEV)
+    nk = torch.full((B,), len(kept), dtype=torch.int32, device=DEV)
+    g.ctx.tf_pruned_attention(g.shape, g.params, q, k, v, idx, nk, g.O)
+    g.status_ok()
+    ref = g.O.clone()
+    for entry, value in ((0, float("inf")), (66, float("nan")), (133, float("-inf")), (len(kept) - 1, float("nan"))):
+        bad = int(kept[entry])
+        poisoned = v.clone()
+        poisoned[:, bad] = value
+        g.ctx.tf_pruned_attention(g.shape, g.params, q, k, poisoned, idx, nk, g.O)
+        g.status_ok()
+        t = np.arange(S)
+        blind = torch.from_numpy((t < bad) | (t >= bad + window if window > 0 else False)).to(DEV)
+        assert torch.equal(g.O[:, blind], ref[:, blind]), (bad, value)
+        assert not torch.isfinite(g.O[:, bad]).any()
+    g.close()
+
+
 def test_layer_filter_retained_keys_only():
     q, k, v = _qkv(2, 700, 8, 2, torch.bfloat16, seed=77)
     n_mis = _layer_case(q, k, v, window=0, prune_ratio=0.5, warmup_tokens=4, kv_visibility=tfb.TF_KV_RETAINED)

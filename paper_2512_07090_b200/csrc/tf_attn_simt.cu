@@ -197,22 +197,31 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
         part_sync();                                                       // K(ch) is there
         float s[R][2];
         if (mine) {
+            // the even and the odd dims of a score are summed apart, two products per instruction.  One chain of 128 left an
+            // error of 5.9e-7 (2-norm over 2-norm, 1 x 700 tokens, against 64 bits), two chains of 64 leave 3.8e-7.
+            uint64_t s2[R][2];
 #pragma unroll
-            for (int r = 0; r < R; ++r) s[r][0] = s[r][1] = 0.f;
-            const float4* k4 = reinterpret_cast<const float4*>(sK) + lane * 32;
-            const float4* q4 = reinterpret_cast<const float4*>(sQ) + row0 * 32;
+            for (int r = 0; r < R; ++r) s2[r][0] = s2[r][1] = 0ull;
+            const ulonglong2* k4 = reinterpret_cast<const ulonglong2*>(sK) + lane * 32;
+            const ulonglong2* q4 = reinterpret_cast<const ulonglong2*>(sQ) + row0 * 32;
 #pragma unroll 4
             for (int d = 0; d < 32; ++d) {
-                const float4 ka = k4[d ^ (lane & 7)], kb = k4[32 * 32 + (d ^ (lane & 7))];
+                const ulonglong2 ka = k4[d ^ (lane & 7)], kb = k4[32 * 32 + (d ^ (lane & 7))];
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
-                    const float4 q = q4[r * 32 + d];
-                    s[r][0] = fmaf(q.x, ka.x, s[r][0]); s[r][1] = fmaf(q.x, kb.x, s[r][1]);
-                    s[r][0] = fmaf(q.y, ka.y, s[r][0]); s[r][1] = fmaf(q.y, kb.y, s[r][1]);
-                    s[r][0] = fmaf(q.z, ka.z, s[r][0]); s[r][1] = fmaf(q.z, kb.z, s[r][1]);
-                    s[r][0] = fmaf(q.w, ka.w, s[r][0]); s[r][1] = fmaf(q.w, kb.w, s[r][1]);
+                    const ulonglong2 q = q4[r * 32 + d];
+                    s2[r][0] = fma2(q.x, ka.x, s2[r][0]); s2[r][1] = fma2(q.x, kb.x, s2[r][1]);
+                    s2[r][0] = fma2(q.y, ka.y, s2[r][0]); s2[r][1] = fma2(q.y, kb.y, s2[r][1]);
                 }
             }
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    float even, odd;
+                    unpack2(s2[r][c], even, odd);
+                    s[r][c] = even + odd;
+                }
         }
         part_sync();                                                       // K(ch) has been read
         if (ch + kSplit < ch1) fetch(sK, Kb, p.ks.t, ch + kSplit, c_hi, true); else fetch_commit();

@@ -473,6 +473,38 @@ def test_cuda_core_attention_keeps_a_value_out_of_rows_that_may_not_see_it(B, S,
     g.close()
 
 
+def _chain_scores(q, k, chains):
+    """q . k over 128 dims as fp32 fused multiply-adds in `chains` interleaved chains (exact products and one rounding per step)."""
+    sums = [torch.zeros(q.shape[0], k.shape[0], dtype=torch.float64, device=q.device) for _ in range(chains)]
+    for d in range(128):
+        sums[d % chains] = torch.addcmul(sums[d % chains], q[:, None, d].double(), k[None, :, d].double()).float().double()
+    return sum(sums).float().double()
+
+
+@pytest.mark.parametrize("S,Hq,Hkv", [(192, 4, 4), (192, 80, 40)])     # two chunk sequences per CTA / all warps on one
+def test_cuda_core_attention_sums_a_score_in_two_chains(S, Hq, Hkv):
+    """fp32 attention is bound by the rounding of its scores: the whole of its error (2-norm, against 64 bits) stays below what
+    scores summed in ONE chain of 128 would leave with everything after them exact, and so is no larger than with two."""
+    g_ = torch.Generator(device=DEV).manual_seed(S + Hq)
+    q, k, v = (1.28 * torch.randn(1, S, h, 128, device=DEV, generator=g_) for h in (Hq, Hkv, Hkv))
+    g = Gpu(q, k, v, prune_ratio=0.0)
+    idx = torch.arange(S, dtype=torch.int32, device=DEV)[None].contiguous()
+    g.ctx.tf_pruned_attention(g.shape, g.params, q, k, v, idx, torch.full((1,), S, dtype=torch.int32, device=DEV), g.O)
+    g.status_ok()
+    hidden = torch.ones(S, S, dtype=torch.bool, device=DEV).triu(1)
+    scale_log2 = torch.tensor(1.4426950408889634 / 128 ** 0.5, dtype=torch.float32, device=DEV)
+    err = {"kernel": 0.0, 1: 0.0, 2: 0.0}
+    for h in range(4):
+        qh, kh, vh = q[0, :, h], k[0, :, h // (Hq // Hkv)], v[0, :, h // (Hq // Hkv)].double()
+        probs = lambda s: torch.softmax(s.masked_fill(hidden, -torch.inf) * np.log(2.0), -1)
+        ref = probs(qh.double() @ kh.double().T * (1.4426950408889634 / 128 ** 0.5)) @ vh
+        err["kernel"] += float((g.O[0, :, h].double() - ref).square().sum())
+        for chains in (1, 2):
+            err[chains] += float((probs(_chain_scores(qh * scale_log2, kh, chains)) @ vh - ref).square().sum())
+    assert err["kernel"] < err[1], {n: e ** 0.5 for n, e in err.items()}
+    g.close()
+
+
 def test_layer_filter_retained_keys_only():
     q, k, v = _qkv(2, 700, 8, 2, torch.bfloat16, seed=77)
     n_mis = _layer_case(q, k, v, window=0, prune_ratio=0.5, warmup_tokens=4, kv_visibility=tfb.TF_KV_RETAINED)

@@ -731,8 +731,10 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
 __global__ void __launch_bounds__(kHeadDim) decode_combine_kernel(const DecStreamParams p) {
     grid_dependency_wait();
     const unsigned int x = blockIdx.x, n_pieces = p.begun[-1].x;
-    const uint4 it = p.begun[x];                            // (beyond the last piece: whatever is there)
-    if (x >= n_pieces || it.x == 0xffffffffu) return;
+    // Beyond the last piece, and in the pieces of a CTA that gave up waiting, stands whatever the workspace held: an entry
+    // that does not name a work item is passed over, not followed.
+    const uint4 it = p.begun[x];
+    if (x >= n_pieces || it.x >= (unsigned int)p.B || it.y >= (unsigned int)p.Hkv || it.z < x || it.z >= n_pieces) return;
     const int n = (int)(it.z - x) + 1, d = threadIdx.x;
     const float* base = p.partial + (size_t)(2 * x) * kPartialFloats;
     float M = -1e30f, L = 0.f, acc = 0.f;

@@ -901,6 +901,43 @@ def test_decode_attention_uneven_positions_and_skips(B, S, Hkv, G, window, works
     ctx.close()
 
 
+@pytest.mark.parametrize("fill", [0x00, 0x3f, 0xff])
+def test_decode_step_whose_waits_run_out_leaves_a_usable_context(fill):
+    """A streaming step that may not wait gives up (bounded waits, no fault) before it has described the work items it was to
+    merge; what the workspace held before is not taken for such descriptions, and the next step is right."""
+    B, S, Hkv = 3, 3000, 5
+    q, k, v = _qkv(B, S, Hkv, Hkv, torch.bfloat16, seed=5)
+    params = tfb.default_params(prune_ratio=0.5, warmup_tokens=0)
+    guard = torch.full((B + 2, Hkv, 128), 7.0, dtype=torch.bfloat16, device=DEV)      # the output, between rows that must stay
+    O = guard[1:-1]
+    qn = q[:, -1].contiguous()
+    shape = tfb.make_shape(None, k, v, n_q_heads=Hkv)
+    shape.q_stride[:] = [qn.stride(0), 0, qn.stride(1)]
+    shape.o_stride[:] = [O.stride(0), 0, O.stride(1)]
+    ctx = tfb.Context(0)
+    ws = torch.full((ctx.workspace_bytes(shape, params),), fill, dtype=torch.uint8, device=DEV)
+    ctx.set_workspace(ws)
+    st = tfb.DecodeState(B, Hkv, DEV)
+    st.tau.fill_(9.0)
+    skip = torch.empty(B, dtype=torch.uint8, device=DEV)
+    pos = torch.tensor([S - 1, 1700, 63], dtype=torch.int32, device=DEV)
+    ctx.tf_set_wait_limits(wait_cycles=0)
+    ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
+    assert ctx.tf_get_status()[0] in (tfb.TF_OK, tfb.TF_ERR_TIMEOUT)
+    ctx.tf_set_wait_limits()
+    ctx.tf_clear_status()
+    for _ in range(2):
+        ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
+        assert ctx.tf_get_status()[0] == tfb.TF_OK
+        for b in range(B):
+            kk, vv = k[b, :int(pos[b]) + 1].double(), v[b, :int(pos[b]) + 1].double()
+            p = (torch.einsum("hd,nhd->hn", qn[b].double(), kk) / 128 ** 0.5).softmax(-1)
+            assert attn_rel_err(to_np(O[b]), torch.einsum("hn,nhd->hd", p, vv).cpu().numpy()) < ATTN_TOL[torch.bfloat16], b
+        O.fill_(7.0)
+    assert torch.all(guard == 7.0)
+    ctx.close()
+
+
 @pytest.mark.parametrize("dtype,mode,window,S0,T,Hq,Hkv",
                          [(torch.bfloat16, tfb.TF_ANCHOR_PAST_MEAN, 0, 70, 90, 8, 2), (torch.float32, tfb.TF_ANCHOR_PAST_MEAN, 40, 70, 90, 8, 2),
                           (torch.bfloat16, tfb.TF_ANCHOR_EMA, 0, 70, 90, 8, 2), (torch.bfloat16, tfb.TF_ANCHOR_INCL_MEAN, 0, 70, 90, 8, 2),

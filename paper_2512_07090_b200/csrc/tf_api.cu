@@ -484,8 +484,7 @@ tf_status tf_get_status(tf_ctx* ctx, int sync, int64_t detail[4]) {
         detail[2] = (int64_t)h.nan_count; detail[3] = (int64_t)ctx->launches;
     }
     if (h.code == TF_ERR_TIMEOUT) {
-        invalidate_scan_scratch(ctx);   // records written under a wait that gave up are not to be trusted, nor counters
-        cudaMemset(ctx->dev_status + 1, 0, kStatusBytes - sizeof(DevStatus));
+        invalidate_scan_scratch(ctx);   // records written under a wait that gave up are not to be trusted
         return TF_ERR_TIMEOUT;
     }
     if (h.code == TF_ERR_NAN_SCORE) return TF_ERR_NAN_SCORE;
@@ -497,7 +496,7 @@ tf_status tf_clear_status(tf_ctx* ctx) {
     DeviceGuard g(ctx->device);
     if (!g.ok) return TF_ERR_CUDA;
     invalidate_scan_scratch(ctx);
-    return cudaMemset(ctx->dev_status, 0, kStatusBytes) == cudaSuccess ? TF_OK : TF_ERR_CUDA;
+    return cudaMemset(ctx->dev_status, 0, sizeof(DevStatus)) == cudaSuccess ? TF_OK : TF_ERR_CUDA;
 }
 
 tf_status tf_last_kernels(tf_ctx* ctx, int32_t kernels[2]) {

@@ -938,6 +938,43 @@ def test_decode_step_whose_waits_run_out_leaves_a_usable_context(fill):
     ctx.close()
 
 
+def test_status_is_read_and_cleared_while_decode_steps_run():
+    """tf_get_status without synchronising and tf_clear_status touch nothing that a step in flight works with, after a wait
+    that gave up as well: every step's output has the same bits."""
+    B, S, Hkv = 4, 4096, 40
+    q, k, v = _qkv(B, S, Hkv, Hkv, torch.bfloat16, seed=6)
+    qn = q[:, -1].contiguous()
+    O = torch.empty(24, B, Hkv, 128, dtype=torch.bfloat16, device=DEV)
+    shape = tfb.make_shape(None, k, v, n_q_heads=Hkv)
+    shape.q_stride[:] = [qn.stride(0), 0, qn.stride(1)]
+    shape.o_stride[:] = [O.stride(1), 0, O.stride(2)]
+    params = tfb.default_params(prune_ratio=0.5, warmup_tokens=0)
+    ctx = tfb.Context(0)
+    ctx.ensure_workspace(shape, params)
+    st = tfb.DecodeState(B, Hkv, DEV)
+    st.tau.fill_(9.0)
+    skip = torch.empty(B, dtype=torch.uint8, device=DEV)
+    pos = torch.full((B,), S - 1, dtype=torch.int32, device=DEV)
+    ctx.tf_set_wait_limits(max_polls=3, wait_cycles=20000)
+    ctx.tf_wait_selftest()                                   # from here on the status says TIMEOUT
+    assert ctx.tf_get_status()[0] == tfb.TF_ERR_TIMEOUT
+    ctx.tf_set_wait_limits()
+    side = torch.cuda.Stream()                               # (a non-blocking stream: nothing orders it with the default one)
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        for i in range(O.shape[0]):
+            ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O[i], None, skip)
+            assert ctx.tf_get_status(sync=False)[0] == (tfb.TF_ERR_TIMEOUT if i < 16 else tfb.TF_OK)
+            if i >= 15:
+                ctx.tf_clear_status()
+    torch.cuda.synchronize()
+    assert ctx.tf_get_status()[0] == tfb.TF_OK
+    assert torch.isfinite(O[0].float()).all()
+    for i in range(1, O.shape[0]):
+        assert torch.equal(O[i], O[0]), i
+    ctx.close()
+
+
 @pytest.mark.parametrize("dtype,mode,window,S0,T,Hq,Hkv",
                          [(torch.bfloat16, tfb.TF_ANCHOR_PAST_MEAN, 0, 70, 90, 8, 2), (torch.float32, tfb.TF_ANCHOR_PAST_MEAN, 40, 70, 90, 8, 2),
                           (torch.bfloat16, tfb.TF_ANCHOR_EMA, 0, 70, 90, 8, 2), (torch.bfloat16, tfb.TF_ANCHOR_INCL_MEAN, 0, 70, 90, 8, 2),

@@ -10,8 +10,6 @@ namespace {
 
 using namespace tf;
 
-constexpr size_t kStatusBytes = sizeof(DevStatus) + kDecodeCounters * sizeof(unsigned int);
-
 inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 // Sections of the caller's workspace.
@@ -154,8 +152,8 @@ tf_status tf_create(tf_ctx** out, int device) {
     c->use_tensor_cores = 1;
     c->max_polls = -1;
     c->wait_cycles = -1;
-    if (cudaMalloc(reinterpret_cast<void**>(&c->dev_status), kStatusBytes) != cudaSuccess ||
-        cudaMemset(c->dev_status, 0, kStatusBytes) != cudaSuccess) {
+    if (cudaMalloc(reinterpret_cast<void**>(&c->dev_status), sizeof(DevStatus)) != cudaSuccess ||
+        cudaMemset(c->dev_status, 0, sizeof(DevStatus)) != cudaSuccess) {
         delete c;
         return TF_ERR_CUDA;
     }

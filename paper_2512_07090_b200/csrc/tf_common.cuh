@@ -11,7 +11,6 @@ namespace tf {
 
 constexpr int kHeadDim = 128;
 constexpr int kDeviceFlagSlots = 64;       // per-device one-time set-up flags
-constexpr int kDecodeCounters = 2;         // counters of the streaming decode kernel: its work list
 constexpr float kNormEps = 1e-8f;   // lower clamp of each norm in the cosine
 
 // Device status record: four 64-bit words {code, where, nan_count, reserved}.
@@ -207,7 +206,7 @@ __device__ __forceinline__ void scan_leave(unsigned int* counters, unsigned int 
 // The opaque context of include/tf.h.
 struct tf_ctx {
     int device;
-    tf::DevStatus* dev_status;     // device memory: the status record, then kDecodeCounters counters of tf_decode_step
+    tf::DevStatus* dev_status;     // device memory, 4 words
     void* workspace;               // caller-owned
     size_t workspace_bytes;
     tf::ScanScratch scan_user;     // scan bookkeeping of the caller's workspace

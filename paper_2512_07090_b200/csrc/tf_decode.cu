@@ -34,6 +34,7 @@ struct DecideParams {
     int early;                          // the kernel after this one may start now (it waits before it reads what this one writes)
     float* tau; long long* steps; long long* skips;
     float* score_out; uint8_t* skip_out;
+    unsigned int* next_piece;           // the streaming kernel's work list, set to its start here (null: there is none)
     DevStatus* status;
 };
 
@@ -75,6 +76,7 @@ __global__ void __launch_bounds__(kDecideWarps * 32) decode_decide_kernel(const 
     long long steps = 0, skips = 0;
     float tau_old = 0.f;
     if (threadIdx.x == 0) { steps = p.steps[b]; skips = p.skips[b]; tau_old = p.tau[b]; }
+    if (p.next_piece && b == 0 && threadIdx.x == 0) *p.next_piece = 0u;   // (drawn from after that kernel's wait for this one)
 
     for (int h0 = warp; h0 < p.Hkv; h0 += 2 * n_warps) {    // two heads at a time: all of their loads go out together
         float xk4[2][4], xv4[2][4], ak4[2][4], av4[2][4];
@@ -305,10 +307,10 @@ struct DecStreamParams {
     int B, Hq, Hkv, window;
     float scale_log2;
     uint4* begun;                     // for decode_combine_kernel: [piece] {sequence or ~0, KV head, last piece} of the work item that begins in the
-                                      // piece and ends in a later one; in front of it the number of pieces
+                                      // piece and ends in a later one; in front of it {pieces, next piece to be drawn}: all of a step's state
+                                      // is in its workspace, so that steps on different workspaces do not share any
     float* partial;                   // [slot][130]; null: a work item is never split
     unsigned int max_slots;
-    unsigned int* counters;           // {next piece, CTAs done}, zero before and after every launch (with partial only)
     DevStatus* status;
     long long wait_cycles;
 };
@@ -519,7 +521,7 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
         // ================================ producer ============================================================
         if (any_skip) { make_list(true); walk = 0; }
         if (lane == 0) make_cut();
-        if (cta == 0 && lane == 0 && p.begun) p.begun[-1] = make_uint4(whole ? 0u : n_pieces, 0u, 0u, 0u);
+        if (cta == 0 && lane == 0 && p.begun) p.begun[-1].x = whole ? 0u : n_pieces;
         if (lane == 0) {
             unsigned int x = cta, it = ahead;
             bool ok = true, open = !any_skip && ahead > 0;   // the piece opened above goes on
@@ -536,7 +538,7 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
                 bool drawn = !p.partial;
                 while (ok && py < py_end) {
                     if (!drawn && py + 3 >= py_end) {       // as late as the answer is still there in time
-                        x_next = gridDim.x + atomicAdd(p.counters, 1u);
+                        x_next = gridDim.x + atomicAdd(&p.begun[-1].y, 1u);
                         drawn = true;
                     }
                     if (p_done == 0) {
@@ -546,17 +548,13 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
                     ok = ok && slot_free();
                     if (ok) { produce(it); ++it; }
                 }
-                if (!drawn) x_next = gridDim.x + atomicAdd(p.counters, 1u);
+                if (!drawn) x_next = gridDim.x + atomicAdd(&p.begun[-1].y, 1u);
                 open = false;
                 x = x_next;
             }
             if (ok && seg_free()) {                         // no more work
                 pt.count = 0;
                 announce();
-            }
-            if (p.partial && atomicAdd(p.counters + 1, 1u) == gridDim.x - 1) {   // the last to stop drawing resets the counters
-                atomicExch(p.counters, 0u);
-                atomicExch(p.counters + 1, 0u);
             }
         }
     } else if (warp < 8) {
@@ -731,6 +729,7 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
 __global__ void __launch_bounds__(kHeadDim) decode_combine_kernel(const DecStreamParams p) {
     grid_dependency_wait();
     const unsigned int x = blockIdx.x, n_pieces = p.begun[-1].x;
+    if (x == 0 && threadIdx.x == 0) p.begun[-1].y = 0u;     // for the next sequences of the same step, if there are more
     // Beyond the last piece, and in the pieces of a CTA that gave up waiting, stands whatever the workspace held: an entry
     // that does not name a work item is passed over, not followed.
     const uint4 it = p.begun[x];
@@ -1029,6 +1028,20 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
                         ((s.o_stride[0] | s.o_stride[2]) % 8) == 0 && (reinterpret_cast<uintptr_t>(a.O_new) & 15u) == 0 &&
                         (s.batch == 1 || (s.k_stride[0] > 0 && s.v_stride[0] > 0)) && maps(0, std::min<int>(s.batch, kStreamMaxBatch));
     dp.early = stream ? 1 : 0;
+    // scratch of the streaming kernel: the table of begun work items, then slots: two per piece, and there have to be more
+    // pieces than CTAs
+    DecStreamParams sp{};
+    auto stream_grid = [&](int n) { return (int)std::min<long long>(sms, (long long)n * s.n_kv_heads * ((max_keys + kStreamKeys - 1) / kStreamKeys)); };
+    const int first_grid = stream_grid(std::min<int>(s.batch, kStreamMaxBatch));      // (none after it is larger)
+    const size_t table = stream_table_bytes(first_grid), slot = kPartialFloats * sizeof(float);
+    if (stream && ctx->workspace && ctx->workspace_bytes >= table + (3 * (size_t)first_grid + 2) * slot) {
+        const size_t scratch = std::min(ctx->workspace_bytes, table + kStreamScratch);
+        sp.begun = static_cast<uint4*>(ctx->workspace) + 1;
+        sp.partial = reinterpret_cast<float*>(static_cast<char*>(ctx->workspace) + table);
+        sp.max_slots = (unsigned int)((scratch - table) / slot);
+        dp.next_piece = &sp.begun[-1].y;
+        ctx->scan_user.needs_clear = true; ctx->scan_owned.needs_clear = true;      // (the scan's records: see below)
+    }
     dp.tau = a.state->tau; dp.steps = reinterpret_cast<long long*>(a.state->steps);
     dp.skips = reinterpret_cast<long long*>(a.state->skips);
     dp.score_out = a.score_out; dp.skip_out = a.skip_out; dp.status = ctx->dev_status;
@@ -1094,7 +1107,6 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
         return e;
     }
     if (stream) {
-        DecStreamParams sp{};
         sp.q_b = ap.q_b; sp.q_h = ap.q_h; sp.o_b = ap.o_b; sp.o_h = ap.o_h;
         sp.Hq = s.n_q_heads; sp.Hkv = s.n_kv_heads; sp.window = s.window; sp.scale_log2 = ap.scale_log2;
         sp.status = ctx->dev_status; sp.wait_cycles = ctx_wait_cycles(ctx);
@@ -1105,20 +1117,7 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
             sp.Q = static_cast<const __nv_bfloat16*>(a.q_new) + (long long)b0 * ap.q_b;
             sp.O = static_cast<__nv_bfloat16*>(a.O_new) + (long long)b0 * ap.o_b;
             sp.pos = a.pos + b0; sp.skip = a.skip_out + b0;
-            const long long tiles = (long long)n * s.n_kv_heads * ((max_keys + kStreamKeys - 1) / kStreamKeys);
-            const int grid = (int)std::min<long long>(sms, tiles);
-            sp.partial = nullptr; sp.begun = nullptr; sp.counters = nullptr;
-            // scratch: the table of begun work items, then slots: two per piece, and there have to be more pieces than CTAs
-            const size_t slot = kPartialFloats * sizeof(float), table = stream_table_bytes(grid);
-            const size_t scratch = std::min(ctx->workspace ? ctx->workspace_bytes : 0, table + kStreamScratch);
-            if (scratch >= table + (3 * grid + 2) * slot) {
-                sp.partial = reinterpret_cast<float*>(static_cast<char*>(ctx->workspace) + table);
-                sp.max_slots = (unsigned int)((scratch - table) / slot);
-                sp.counters = reinterpret_cast<unsigned int*>(ctx->dev_status + 1);
-                sp.begun = static_cast<uint4*>(ctx->workspace) + 1;
-                ctx->scan_user.needs_clear = true; ctx->scan_owned.needs_clear = true;      // (the scan's records: as above)
-            }
-            e = launch_stream(sp, grid, ctx->device, mk, mv, st);
+            e = launch_stream(sp, stream_grid(n), ctx->device, mk, mv, st);
             ctx->launches += sp.begun ? 2 : 1;
             if (e != cudaSuccess) return e;
         }

@@ -975,6 +975,45 @@ def test_status_is_read_and_cleared_while_decode_steps_run():
     ctx.close()
 
 
+def test_decode_steps_on_two_workspaces_and_streams_do_not_share_state():
+    """A context's workspace is rebound between steps that run at the same time on different streams: whatever a step keeps
+    while it runs (its work list among it) is in its own workspace."""
+    B, S, Hkv = 4, 4096, 40
+    q, k, v = _qkv(B, S, Hkv, Hkv, torch.bfloat16, seed=8)
+    qn = [q[:, -1].contiguous(), q[:, -2].contiguous()]
+    shape = tfb.make_shape(None, k, v, n_q_heads=Hkv)
+    shape.q_stride[:] = [qn[0].stride(0), 0, qn[0].stride(1)]
+    shape.o_stride[:] = list(shape.q_stride)
+    params = tfb.default_params(prune_ratio=0.5, warmup_tokens=0)
+    ctx = tfb.Context(0)
+    n = ctx.workspace_bytes(shape, params)
+    ws = [torch.empty(n, dtype=torch.uint8, device=DEV) for _ in range(2)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    pos = [torch.tensor(p, dtype=torch.int32, device=DEV) for p in ([S - 1, 3000, 2000, 4000], [2500, S - 1, 100, 3500])]
+    state = [tfb.DecodeState(B, Hkv, DEV) for _ in range(2)]
+    for st in state:
+        st.tau.fill_(9.0)
+    skip = [torch.empty(B, dtype=torch.uint8, device=DEV) for _ in range(2)]
+    alone = [torch.empty_like(qn[0]) for _ in range(2)]
+    for i in range(2):
+        ctx.set_workspace(ws[i])
+        ctx.tf_decode_step(shape, params, 0.0, qn[i], k, v, pos[i], state[i], alone[i], None, skip[i])
+        torch.cuda.synchronize()
+    O = torch.full((2, 12, B, Hkv, 128), float("nan"), dtype=torch.bfloat16, device=DEV)
+    torch.cuda.synchronize()
+    for r in range(O.shape[1]):
+        for i in range(2):
+            ctx.set_workspace(ws[i])
+            with torch.cuda.stream(streams[i]):
+                ctx.tf_decode_step(shape, params, 0.0, qn[i], k, v, pos[i], state[i], O[i, r], None, skip[i])
+    torch.cuda.synchronize()
+    assert ctx.tf_get_status()[0] == tfb.TF_OK
+    for i in range(2):
+        for r in range(O.shape[1]):
+            assert torch.equal(O[i, r], alone[i]), (i, r)
+    ctx.close()
+
+
 @pytest.mark.parametrize("dtype,mode,window,S0,T,Hq,Hkv",
                          [(torch.bfloat16, tfb.TF_ANCHOR_PAST_MEAN, 0, 70, 90, 8, 2), (torch.float32, tfb.TF_ANCHOR_PAST_MEAN, 40, 70, 90, 8, 2),
                           (torch.bfloat16, tfb.TF_ANCHOR_EMA, 0, 70, 90, 8, 2), (torch.bfloat16, tfb.TF_ANCHOR_INCL_MEAN, 0, 70, 90, 8, 2),

@@ -668,7 +668,9 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
             ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar_part_free, (k_seg & 1u) ^ 1u, abort_flag, p.wait_cycles, p.status, 605));
             if (!ok) break;
             if (t == 0) {                                        // column 0 is the head
-                float* dst = part_s + warp * kPartialFloats;
+                // (ordered by the tiles, not by the half that the ring happened to give them to: the merge then adds in one
+                // order whichever pieces this CTA drew before, and the result has the same bits every time)
+                float* dst = part_s + (i0 * 4 + (warp & 3)) * kPartialFloats;
 #pragma unroll
                 for (int mt = 0; mt < 8; ++mt) { dst[16 * mt + g] = o[mt][0]; dst[16 * mt + 8 + g] = o[mt][2]; }
                 if (g == 0) { dst[kHeadDim] = m[0]; dst[kHeadDim + 1] = l[0]; }

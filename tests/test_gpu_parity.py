@@ -1014,6 +1014,44 @@ def test_decode_steps_on_two_workspaces_and_streams_do_not_share_state():
     ctx.close()
 
 
+def test_decode_of_many_short_sequences_repeats_its_bits_on_a_shared_workspace():
+    """More than eight work items per CTA: each is a piece of its own, drawn in whatever order the CTAs come, with scratch
+    present.  In turn with a step that splits its items: both give the same bits every time, and the right ones."""
+    params = tfb.default_params(prune_ratio=0.5, warmup_tokens=0)
+    ctx = tfb.Context(0)
+    cases = []
+    for B, S, Hkv in ((128, 130, 40), (2, 5000, 40)):
+        q, k, v = _qkv(B, S, Hkv, Hkv, torch.bfloat16, seed=S)
+        qn = q[:, -1].contiguous()
+        shape = tfb.make_shape(None, k, v, n_q_heads=Hkv)
+        shape.q_stride[:] = [qn.stride(0), 0, qn.stride(1)]
+        shape.o_stride[:] = list(shape.q_stride)
+        pos = torch.from_numpy(np.random.default_rng(S).integers(S // 3, S, B).astype(np.int32)).to(DEV)
+        st = tfb.DecodeState(B, Hkv, DEV)
+        st.tau.fill_(9.0)
+        st.tau[B // 4 + 1:B // 2] = -9.0                                  # these are skipped
+        cases.append((shape, qn, k, v, pos, st, torch.empty_like(qn), torch.empty(B, dtype=torch.uint8, device=DEV)))
+    ctx.set_workspace(torch.empty(max(ctx.workspace_bytes(c[0], params) for c in cases), dtype=torch.uint8, device=DEV))
+    first = [None, None]
+    for _ in range(8):
+        for i, (shape, qn, k, v, pos, st, O, skip) in enumerate(cases):
+            O.fill_(float("nan"))
+            ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
+            assert ctx.tf_get_status()[0] == tfb.TF_OK
+            first[i] = O.clone() if first[i] is None else first[i]
+            assert torch.equal(O, first[i]), i
+    for (shape, qn, k, v, pos, st, O, skip) in cases:
+        for b in range(O.shape[0]):
+            if skip[b]:
+                assert torch.all(O[b] == 0)
+                continue
+            kk, vv = k[b, :int(pos[b]) + 1].double(), v[b, :int(pos[b]) + 1].double()
+            p = (torch.einsum("hd,nhd->hn", qn[b].double(), kk) / 128 ** 0.5).softmax(-1)
+            assert attn_rel_err(to_np(O[b]), torch.einsum("hn,nhd->hd", p, vv).cpu().numpy()) < ATTN_TOL[torch.bfloat16], b
+    assert cases[0][-1].sum() > 0
+    ctx.close()
+
+
 @pytest.mark.parametrize("dtype,mode,window,S0,T,Hq,Hkv",
                          [(torch.bfloat16, tfb.TF_ANCHOR_PAST_MEAN, 0, 70, 90, 8, 2), (torch.float32, tfb.TF_ANCHOR_PAST_MEAN, 40, 70, 90, 8, 2),
                           (torch.bfloat16, tfb.TF_ANCHOR_EMA, 0, 70, 90, 8, 2), (torch.bfloat16, tfb.TF_ANCHOR_INCL_MEAN, 0, 70, 90, 8, 2),

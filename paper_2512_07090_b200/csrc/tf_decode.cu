@@ -274,9 +274,10 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_attention_kernel(const 
 //           running ahead across work items.  It starts while the decision kernel still runs, as if no token were skipped; if
 //           one is, what it fetched is thrown away.
 //   warps 0-3 / 4-7 consume the even / odd tiles, 16 keys per warp, on m16n8k16 products:
-//           S^T[16 keys x 8 columns] = K Q^T (A by ldmatrix; one column is the head, the others are zero: the products are not what
-//           bounds this), online softmax on the accumulator layout (lane holds keys g, g + 8 for columns 2t, 2t + 1), P^T through two 8x8 register transposes, O^T[128 dims x 8] += V^T P^T (A by
-//           ldmatrix.trans).
+//           S^T[16 keys x 8 columns] = K Q^T (A by ldmatrix; column 0 is the head, the others are zero: the products are not what
+//           bounds this), online softmax on the accumulator layout (lane holds keys g, g + 8 for columns 2t, 2t + 1), P^T
+//           through two 8x8 register transposes, O^T[128 dims x 8] += V^T P^T (A by ldmatrix.trans) with what rounding P to
+//           bf16 leaves in column 1: the result is as exact as its own rounding.
 //   warps 9-12 merge: at the end of a segment (a work item, or the part of one in this piece) the consumers leave their
 //           states in shared memory and go on with the next segment at once; these warps merge the eight states and write the result.
 // Every wait is bounded, those of the warps for one another too (mbarriers, no named barriers): on expiry the CTA records
@@ -583,8 +584,8 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
             if (sg < wasted_segs) continue;
             if (seg.count == 0) break;
             const int t_pos = s_pos[seg.b], n_vis = t_pos - first_key(t_pos) + 1 - seg.j * kStreamKeys;      // visible keys from the segment's first on
-            float m[2] = {-1e30f, -1e30f}, l[2] = {0.f, 0.f};   // heads 2t, 2t + 1 (m is the same in all lanes of equal t; l is the lane's share)
-            float o[8][4];                                      // O^T: dims 16 mt + g and 16 mt + 8 + g, heads 2t, 2t + 1
+            float m = -1e30f, l = 0.f;                          // of column 2t (m is the same in all lanes of equal t; l is the lane's share)
+            float o[8][4];                                      // O^T: dims 16 mt + g and 16 mt + 8 + g, columns 2t, 2t + 1
             uint32_t qb[8][2];
 #pragma unroll
             for (int mt = 0; mt < 8; ++mt) { o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f; }
@@ -620,28 +621,24 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
                         __syncwarp();
                     }
                     const bool v0 = g < left, v1 = g + 8 < left;
-                    s[0] = v0 ? (s[0] + s2[0]) * p.scale_log2 : -1e30f; s[1] = v0 ? (s[1] + s2[1]) * p.scale_log2 : -1e30f;
-                    s[2] = v1 ? (s[2] + s2[2]) * p.scale_log2 : -1e30f; s[3] = v1 ? (s[3] + s2[3]) * p.scale_log2 : -1e30f;
-                    float corr[2], pr[4];
+                    const float sa = v0 ? (s[0] + s2[0]) * p.scale_log2 : -1e30f, sb = v1 ? (s[2] + s2[2]) * p.scale_log2 : -1e30f;
+                    float mx = fmaxf(sa, sb);
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+                    const float mn = fmaxf(m, mx), corr = ex2_approx(m - mn);
+                    m = mn;
+                    const float pa = v0 ? ex2_approx(sa - mn) : 0.f, pb = v1 ? ex2_approx(sb - mn) : 0.f;
+                    l = fmaf(l, corr, pa + pb);
+                    // P^T (keys x columns) -> the B operand wants column g with keys 2t, 2t+1 / 2t+8, 2t+9: two 8x8 transposes.
+                    // The odd columns have no head of their own: they take what rounding a probability to bf16 leaves, so
+                    // that it is not lost (4 x 4095 keys x 40 heads, error against 64 bits: without it 1.82e-3).
+                    const float ha = __bfloat162float(__float2bfloat16_rn(pa)), hb = __bfloat162float(__float2bfloat16_rn(pb));
+                    const uint32_t pb0 = transpose8x8_b16(pack_bf16x2(ha, pa - ha));
+                    const uint32_t pb1 = transpose8x8_b16(pack_bf16x2(hb, pb - hb));
+                    if (__any_sync(0xffffffffu, corr != 1.f)) {
 #pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        float mx = fmaxf(s[k], s[k + 2]);
-                        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
-                        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
-                        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-                        const float mn = fmaxf(m[k], mx);
-                        corr[k] = ex2_approx(m[k] - mn);
-                        m[k] = mn;
-                        pr[k] = v0 ? ex2_approx(s[k] - mn) : 0.f;
-                        pr[k + 2] = v1 ? ex2_approx(s[k + 2] - mn) : 0.f;
-                        l[k] = fmaf(l[k], corr[k], pr[k] + pr[k + 2]);
-                    }
-                    // P^T (keys x heads) -> the B operand wants head g with keys 2t, 2t+1 / 2t+8, 2t+9: two 8x8 transposes
-                    const uint32_t pb0 = transpose8x8_b16(pack_bf16x2(pr[0], pr[1]));
-                    const uint32_t pb1 = transpose8x8_b16(pack_bf16x2(pr[2], pr[3]));
-                    if (__any_sync(0xffffffffu, corr[0] != 1.f || corr[1] != 1.f)) {
-#pragma unroll
-                        for (int mt = 0; mt < 8; ++mt) { o[mt][0] *= corr[0]; o[mt][1] *= corr[1]; o[mt][2] *= corr[0]; o[mt][3] *= corr[1]; }
+                        for (int mt = 0; mt < 8; ++mt) { o[mt][0] *= corr; o[mt][1] *= corr; o[mt][2] *= corr; o[mt][3] *= corr; }
                     }
 #pragma unroll
                     for (int mt = 0; mt < 8; ++mt) {
@@ -658,22 +655,19 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
             if (!ok) break;
             it += seg.count;
             // ---- the warp's state to the merging warps ---------------------------------------------------------------
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                l[k] += __shfl_xor_sync(0xffffffffu, l[k], 4);
-                l[k] += __shfl_xor_sync(0xffffffffu, l[k], 8);
-                l[k] += __shfl_xor_sync(0xffffffffu, l[k], 16);
-            }
+            l += __shfl_xor_sync(0xffffffffu, l, 4);
+            l += __shfl_xor_sync(0xffffffffu, l, 8);
+            l += __shfl_xor_sync(0xffffffffu, l, 16);
             const unsigned int k_seg = sg - wasted_segs;         // (the first wait passes: nothing has been left there yet)
             ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar_part_free, (k_seg & 1u) ^ 1u, abort_flag, p.wait_cycles, p.status, 605));
             if (!ok) break;
-            if (t == 0) {                                        // column 0 is the head
+            if (t == 0) {                                        // columns 0 and 1 are the head
                 // (ordered by the tiles, not by the half that the ring happened to give them to: the merge then adds in one
                 // order whichever pieces this CTA drew before, and the result has the same bits every time)
                 float* dst = part_s + (i0 * 4 + (warp & 3)) * kPartialFloats;
 #pragma unroll
-                for (int mt = 0; mt < 8; ++mt) { dst[16 * mt + g] = o[mt][0]; dst[16 * mt + 8 + g] = o[mt][2]; }
-                if (g == 0) { dst[kHeadDim] = m[0]; dst[kHeadDim + 1] = l[0]; }
+                for (int mt = 0; mt < 8; ++mt) { dst[16 * mt + g] = o[mt][0] + o[mt][1]; dst[16 * mt + 8 + g] = o[mt][2] + o[mt][3]; }
+                if (g == 0) { dst[kHeadDim] = m; dst[kHeadDim + 1] = l; }
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_part);

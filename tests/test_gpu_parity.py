@@ -1052,6 +1052,32 @@ def test_decode_of_many_short_sequences_repeats_its_bits_on_a_shared_workspace()
     ctx.close()
 
 
+def test_streaming_decode_loses_nothing_before_the_result_is_rounded():
+    """The error against 64 bits is that of rounding the exact result to bf16 (to 2 %): probabilities keep 16 bits."""
+    B, S, Hkv = 4, 4096, 40
+    q, k, v = _qkv(B, S, Hkv, Hkv, torch.bfloat16, seed=9)
+    qn = q[:, -1].contiguous()
+    shape = tfb.make_shape(None, k, v, n_q_heads=Hkv)
+    shape.q_stride[:] = [qn.stride(0), 0, qn.stride(1)]
+    shape.o_stride[:] = list(shape.q_stride)
+    params = tfb.default_params(prune_ratio=0.5, warmup_tokens=0)
+    ctx = tfb.Context(0)
+    ctx.ensure_workspace(shape, params)
+    st = tfb.DecodeState(B, Hkv, DEV)
+    st.tau.fill_(9.0)
+    O, skip = torch.empty_like(qn), torch.empty(B, dtype=torch.uint8, device=DEV)
+    ctx.tf_decode_step(shape, params, 0.0, qn, k, v, torch.full((B,), S - 1, dtype=torch.int32, device=DEV), st, O, None, skip)
+    assert ctx.tf_get_status()[0] == tfb.TF_OK
+    err = rounding = 0.0
+    for b in range(B):
+        p = (torch.einsum("hd,nhd->hn", qn[b].double(), k[b].double()) / 128 ** 0.5).softmax(-1)
+        ref = torch.einsum("hn,nhd->hd", p, v[b].double())
+        err += float((O[b].double() - ref).square().sum())
+        rounding += float((ref.bfloat16().double() - ref).square().sum())
+    assert err < 1.02 ** 2 * rounding, (err ** 0.5, rounding ** 0.5)
+    ctx.close()
+
+
 @pytest.mark.parametrize("dtype,mode,window,S0,T,Hq,Hkv",
                          [(torch.bfloat16, tfb.TF_ANCHOR_PAST_MEAN, 0, 70, 90, 8, 2), (torch.float32, tfb.TF_ANCHOR_PAST_MEAN, 40, 70, 90, 8, 2),
                           (torch.bfloat16, tfb.TF_ANCHOR_EMA, 0, 70, 90, 8, 2), (torch.bfloat16, tfb.TF_ANCHOR_INCL_MEAN, 0, 70, 90, 8, 2),

@@ -61,7 +61,7 @@ __device__ __forceinline__ void dec_load4(const __nv_bfloat16* p, float (&f)[4])
 // step is complete the attention kernel may start and fetch its first tiles under this kernel.
 constexpr int kDecideWarps = 32;
 
-template <typename T>
+template <typename T, int kHeadsPerWarp>
 __global__ void __launch_bounds__(kDecideWarps * 32) decode_decide_kernel(const DecideParams p) {
     extern __shared__ float cos_s[];        // [2][Hkv]
     grid_dependency_wait();                 // launched early; the step before this one on the stream must be complete
@@ -78,10 +78,10 @@ __global__ void __launch_bounds__(kDecideWarps * 32) decode_decide_kernel(const 
     if (threadIdx.x == 0) { steps = p.steps[b]; skips = p.skips[b]; tau_old = p.tau[b]; }
     if (p.next_piece && b == 0 && threadIdx.x == 0) *p.next_piece = 0u;   // (drawn from after that kernel's wait for this one)
 
-    for (int h0 = warp; h0 < p.Hkv; h0 += 2 * n_warps) {    // two heads at a time: all of their loads go out together
-        float xk4[2][4], xv4[2][4], ak4[2][4], av4[2][4];
+    for (int h0 = warp; h0 < p.Hkv; h0 += kHeadsPerWarp * n_warps) {    // two heads at a time: all of their loads go out together
+        float xk4[kHeadsPerWarp][4], xv4[kHeadsPerWarp][4], ak4[kHeadsPerWarp][4], av4[kHeadsPerWarp][4];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
+        for (int u = 0; u < kHeadsPerWarp; ++u) {
             const int h = min(h0 + u * n_warps, p.Hkv - 1);
             dec_load4(reinterpret_cast<const T*>(p.K) + (long long)b * p.ks.b + (long long)t * p.ks.t + (long long)h * p.ks.h + lane * 4, xk4[u]);
             dec_load4(reinterpret_cast<const T*>(p.V) + (long long)b * p.vs.b + (long long)t * p.vs.t + (long long)h * p.vs.h + lane * 4, xv4[u]);
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(kDecideWarps * 32) decode_decide_kernel(const 
             }
         }
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
+        for (int u = 0; u < kHeadsPerWarp; ++u) {
             const int h = h0 + u * n_warps;
             if (h >= p.Hkv) break;
             float dk = 0.f, kk = 0.f, pk = 0.f, dv = 0.f, vv = 0.f, pv = 0.f;
@@ -1043,9 +1043,12 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
     dp.score_out = a.score_out; dp.skip_out = a.skip_out; dp.status = ctx->dev_status;
     const size_t smem = 2 * (size_t)s.n_kv_heads * sizeof(float);
     cudaError_t e;
-    const dim3 decide_block(32u * std::min(kDecideWarps, std::max((s.n_kv_heads + 1) / 2, 4)));
-    if (s.dtype == TF_BF16) e = launch_dependent(decode_decide_kernel<__nv_bfloat16>, dim3((unsigned)s.batch), decide_block, smem, st, dp);
-    else                    e = launch_dependent(decode_decide_kernel<float>, dim3((unsigned)s.batch), decide_block, smem, st, dp);
+    // up to 8 heads a warp has one, beyond it two (two for 8: 1 x 100 keys x 8 heads fp32 15.3 us a step)
+    const bool two = s.n_kv_heads > 8;
+    const dim3 decide_block(32u * std::min(kDecideWarps, two ? (s.n_kv_heads + 1) / 2 : std::max(s.n_kv_heads, 4)));
+    auto decide = s.dtype == TF_BF16 ? (two ? decode_decide_kernel<__nv_bfloat16, 2> : decode_decide_kernel<__nv_bfloat16, 1>)
+                                     : (two ? decode_decide_kernel<float, 2> : decode_decide_kernel<float, 1>);
+    e = launch_dependent(decide, dim3((unsigned)s.batch), decide_block, smem, st, dp);
     ctx->launches += 1;
     if (e != cudaSuccess) return e;
 

@@ -1078,6 +1078,50 @@ def test_streaming_decode_loses_nothing_before_the_result_is_rounded():
     ctx.close()
 
 
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("Hkv", [1, 3, 8, 9, 64, 65, 80])     # a warp per head / two heads per warp / more than one trip
+@pytest.mark.parametrize("offset", [0, 1])                    # sums on 16-byte boundaries / off them
+def test_decode_decision_and_state_for_every_number_of_heads(dtype, Hkv, offset):
+    """Score, skip, threshold, counters and sums after one step against the same step in 64 bits."""
+    B, S, eta = 3, 40, 0.25
+    _, k, v = _qkv(B, S, Hkv, Hkv, dtype, seed=Hkv)
+    qn = k[:, 0].contiguous()
+    shape = tfb.make_shape(None, k, v, n_q_heads=Hkv)
+    shape.q_stride[:] = [qn.stride(0), 0, qn.stride(1)]
+    shape.o_stride[:] = list(shape.q_stride)
+    params = tfb.default_params(prune_ratio=0.5, warmup_tokens=0)
+    st = tfb.DecodeState(B, Hkv, DEV)
+    n = B * Hkv * 128
+    pos = torch.tensor([S - 1, 7, 20], dtype=torch.int32, device=DEV)
+    past = [torch.zeros(n + offset, device=DEV)[offset:].view(B, Hkv, 128) for _ in range(2)]
+    for t, x in zip(past, (k, v)):
+        for b in range(B):
+            t[b] = x[b, :pos[b]].float().sum(0)
+    st.sum_k, st.sum_v = past
+    st.struct.sum_k, st.struct.sum_v = (t.data_ptr() for t in past)
+    st.count.copy_(pos)
+    st.steps.copy_(torch.tensor([4, 0, 10])); st.skips.copy_(torch.tensor([3, 0, 2]))
+    st.tau.copy_(torch.tensor([-2.0, 2.0, -2.0]))
+    sums = [t.double().clone() for t in past]
+    x = [torch.stack([t[b, pos[b]] for b in range(B)]).double() for t in (k, v)]
+    cos = [torch.nn.functional.cosine_similarity(a, c, dim=-1) for a, c in zip(x, sums)]
+    mean, var = [c.mean(1) for c in cos], [c.var(1, unbiased=False) for c in cos]
+    alpha = (var[1] + 1e-8) / (var[0] + var[1] + 2e-8)
+    ref = alpha * mean[0] + (1 - alpha) * mean[1]
+    tau = torch.tensor([-2.0 + eta * (0.75 - 0.5), 2.0 + eta * (0.0 - 0.5), -2.0 + eta * (0.2 - 0.5)])
+    ctx = tfb.Context(0)
+    O, score, skip = torch.empty_like(qn), torch.empty(B, device=DEV), torch.empty(B, dtype=torch.uint8, device=DEV)
+    ctx.tf_decode_step(shape, params, eta, qn, k, v, pos, st, O, score, skip)
+    assert ctx.tf_get_status()[0] == tfb.TF_OK
+    assert (score.double() - ref).abs().max() < SCORE_ATOL
+    assert skip.tolist() == [1, 0, 1]
+    assert torch.allclose(st.tau.cpu(), tau, rtol=1e-6)
+    assert st.steps.tolist() == [5, 1, 11] and st.skips.tolist() == [4, 0, 3] and st.count.tolist() == [S, 8, 21]
+    for t, a, c in zip(past, sums, x):
+        assert torch.equal(t, (a.float() + c.float()))
+    ctx.close()
+
+
 @pytest.mark.parametrize("dtype,mode,window,S0,T,Hq,Hkv",
                          [(torch.bfloat16, tfb.TF_ANCHOR_PAST_MEAN, 0, 70, 90, 8, 2), (torch.float32, tfb.TF_ANCHOR_PAST_MEAN, 40, 70, 90, 8, 2),
                           (torch.bfloat16, tfb.TF_ANCHOR_EMA, 0, 70, 90, 8, 2), (torch.bfloat16, tfb.TF_ANCHOR_INCL_MEAN, 0, 70, 90, 8, 2),

@@ -1006,7 +1006,7 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
     dp.sum_k = a.state->sum_k; dp.sum_v = a.state->sum_v; dp.count = reinterpret_cast<long long*>(a.state->count);
     dp.sums16 = ((reinterpret_cast<uintptr_t>(dp.sum_k) | reinterpret_cast<uintptr_t>(dp.sum_v)) & 15u) == 0;
     // bf16 with 1, 2, 4 or 8 query heads per KV head and 16-byte aligned query rows: the streaming kernel for ungrouped heads
-    // (more than half a tile per SM), the split kernel otherwise (both sides' times stand at the split kernel)
+    // (more than half a tile per SM), the split kernel otherwise (both sides' times stand at the split kernel) ...
     const int G = s.n_q_heads / s.n_kv_heads;
     const int sms = sm_count();
     const int max_keys = s.window > 0 ? std::min(s.window, s.seq) : s.seq;     // pos is device data: size for the worst case
@@ -1020,7 +1020,13 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
         return make_bshd_map(&mk, K, s.k_stride, n, s.seq, s.n_kv_heads, 2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 64, kStreamKeys, CU_TENSOR_MAP_SWIZZLE_128B) &&
                make_bshd_map(&mv, V, s.v_stride, n, s.seq, s.n_kv_heads, 2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 64, kStreamKeys, CU_TENSOR_MAP_SWIZZLE_128B);
     };
-    const bool stream = grouped && G == 1 && 2 * tiles_max > sms && tiles_max < (1ll << 31) &&              // (tile numbers are 32 bits)
+    // ... but not where all CTAs of the split kernel run at once and have at most four tiles each: the streaming kernel's list
+    // and hand-overs are not paid back then (us a step of full caches, split / streaming: 5 x 128 x 32 heads 10.5 / 12.6,
+    // 7 x 256 x 40 17.5 / 18.4, 7 x 320 x 40 19.4 / 18.8, 8 x 256 x 40, a second wave, 22.1 / 18.9, 32 x 256 x 8 15.1 / 17.9,
+    // 100 x 192 x 2 13.0 / 19.0); nor with one or two tiles in several launches (600 x 64 x 8 64.3 / 69.0)
+    const long long items = (long long)s.batch * s.n_kv_heads;
+    const bool few_short = (items <= 2 * sms && max_keys <= 4 * kStreamKeys) || (s.batch > kStreamMaxBatch && max_keys <= 2 * kStreamKeys);
+    const bool stream = grouped && G == 1 && !few_short && 2 * tiles_max > sms && tiles_max < (1ll << 31) &&              // (tile numbers are 32 bits)
                         ((s.o_stride[0] | s.o_stride[2]) % 8) == 0 && (reinterpret_cast<uintptr_t>(a.O_new) & 15u) == 0 &&
                         (s.batch == 1 || (s.k_stride[0] > 0 && s.v_stride[0] > 0)) && maps(0, std::min<int>(s.batch, kStreamMaxBatch));
     dp.early = stream ? 1 : 0;

@@ -855,7 +855,9 @@ def test_requested_kernel_that_cannot_take_the_call_is_an_error_not_a_fallback()
 @pytest.mark.parametrize("workspace", [True, False])     # work items split over CTAs and merged / whole items per CTA
 @pytest.mark.parametrize("B,S,Hkv,G,window", [(1, 64, 1, 1, 0), (1, 65, 3, 2, 0), (5, 1500, 3, 4, 0), (4, 2000, 2, 8, 700),
                                               (1, 9000, 1, 4, 0), (40, 300, 5, 1, 130), (1030, 70, 1, 1, 0),
-                                              (2, 9000, 3, 1, 0), (150, 130, 8, 1, 0), (1, 200, 4, 8, 0)])
+                                              (2, 9000, 3, 1, 0), (150, 130, 8, 1, 0), (1, 200, 4, 8, 0),
+                                              (7, 256, 40, 1, 0), (7, 257, 40, 1, 0), (8, 256, 40, 1, 0),      # either side of the streaming kernel
+                                              (1030, 129, 1, 1, 0), (1, 256, 4, 1, 0)])   # ... in three launches; ungrouped heads as a cluster
 def test_decode_attention_uneven_positions_and_skips(B, S, Hkv, G, window, workspace):
     """Every sequence at a position of its own (tile edges among them), some skipped, NaN in the cache behind each position:
     the streaming kernel (ungrouped heads: split and whole work items) and the split kernel (as a cluster, through scratch,

@@ -1,5 +1,6 @@
 // C-ABI entry points of include/tf.h: argument checks, workspace carving, kernel sequencing.
 // Every step of the layer runs in the kernels of this library; there is no host fallback.
+#include <algorithm>
 #include <math.h>
 #include <new>
 #include <string.h>
@@ -14,7 +15,9 @@ inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 // Sections of the caller's workspace.
 struct WsLayout {
-    size_t scan, sim_k, sim_v, score, keep_mask, kept_idx, n_kept, theta, kv_compact, total;
+    size_t scan, sim_k, sim_v, score, keep_mask, kept_idx, n_kept, theta, kv_compact;
+    size_t prefill;       // all of these: what tf_layer_filter needs
+    size_t total;         // ... or tf_decode_step, whichever is more (each uses the workspace from the front; it serves one call at a time)
 };
 
 WsLayout ws_layout(const tf_shape& s, const tf_filter_params* p) {
@@ -31,7 +34,8 @@ WsLayout ws_layout(const tf_shape& s, const tf_filter_params* p) {
     w.theta = off;     off += align256((size_t)s.batch * sizeof(float));
     w.kv_compact = off;   // retained tokens' K and V (TF_KV_RETAINED on the tensor-core path only)
     if (p && p->kv_visibility == TF_KV_RETAINED && s.dtype == TF_BF16) off += kv_compact_bytes(s);
-    w.total = off + align256(decode_scratch_bytes(s));   // (used from the front of the workspace: one workspace serves one call at a time)
+    w.prefill = off;
+    w.total = std::max(off, align256(decode_scratch_bytes(s)));
     return w;
 }
 
@@ -117,7 +121,7 @@ tf_status kv_compact_section(tf_ctx* ctx, const tf_shape& s, const tf_filter_par
     *out = nullptr;
     if (p.kv_visibility != TF_KV_RETAINED || s.dtype != TF_BF16 || !ctx->use_tensor_cores) return TF_OK;
     const WsLayout w = ws_layout(s, &p);
-    if (!ctx->workspace || ctx->workspace_bytes < w.total) return TF_ERR_WORKSPACE;
+    if (!ctx->workspace || ctx->workspace_bytes < w.prefill) return TF_ERR_WORKSPACE;
     *out = static_cast<char*>(ctx->workspace) + w.kv_compact;
     return TF_OK;
 }
@@ -285,7 +289,7 @@ tf_status tf_layer_filter(tf_ctx* ctx, const tf_shape* shape, const tf_filter_pa
     if (!aligned16(Q) || !aligned16(O)) return TF_ERR_UNSUPPORTED;
     if (!stride_ok(shape->q_stride, shape->dtype) || !stride_ok(shape->o_stride, shape->dtype)) return TF_ERR_UNSUPPORTED;
     const WsLayout w = ws_layout(*shape, params);
-    if (!ctx->workspace || ctx->workspace_bytes < w.total) return TF_ERR_WORKSPACE;
+    if (!ctx->workspace || ctx->workspace_bytes < w.prefill) return TF_ERR_WORKSPACE;
     DeviceGuard g(ctx->device);
     if (!g.ok) return TF_ERR_CUDA;
     char* ws = static_cast<char*>(ctx->workspace);
@@ -340,10 +344,10 @@ tf_status tf_layer_filter_host(tf_ctx* ctx, const tf_shape* shape, const tf_filt
         ctx->stage_bytes = need;
     }
     const WsLayout w = ws_layout(*shape, params);
-    if (ctx->owned_ws_bytes < w.total) {
+    if (ctx->owned_ws_bytes < w.prefill) {
         if (ctx->owned_ws) { cudaStreamSynchronize(st); cudaFree(ctx->owned_ws); ctx->owned_ws = nullptr; ctx->owned_ws_bytes = 0; }
-        if (cudaMalloc(&ctx->owned_ws, w.total) != cudaSuccess) return TF_ERR_CUDA;
-        ctx->owned_ws_bytes = w.total;
+        if (cudaMalloc(&ctx->owned_ws, w.prefill) != cudaSuccess) return TF_ERR_CUDA;
+        ctx->owned_ws_bytes = w.prefill;
         ctx->scan_owned = tf::ScanScratch();
         ctx->scan_owned.ptr = ctx->owned_ws;
         ctx->scan_owned.capacity = ctx->owned_ws_bytes;

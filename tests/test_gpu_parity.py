@@ -689,6 +689,47 @@ def test_layer_filter_host_pipelined_head_groups(visibility):
     g.close()
 
 
+@pytest.mark.parametrize("visibility", [tfb.TF_KV_ALL, tfb.TF_KV_RETAINED])
+def test_layer_step_takes_a_workspace_of_just_what_it_uses(visibility):
+    """The records of the scan (what tf_kv_stats asks for), the intermediates and the retained K and V: a step that does not
+    decode does not need the scratch of one that does."""
+    B, S, Hq, Hkv = 2, 700, 8, 2
+    q, k, v = _qkv(B, S, Hq, Hkv, torch.bfloat16, seed=3)
+    g = Gpu(q, k, v, prune_ratio=0.5, kv_visibility=visibility)
+    g.ctx.tf_layer_filter(g.shape, g.params, q, k, v, g.O)
+    g.status_ok()
+    ref = g.O.clone()
+    buf = torch.empty(64 << 20, dtype=torch.uint8, device=DEV)
+    up = lambda n: (n + 255) // 256 * 256
+
+    def refused(call, n):
+        g.ctx.set_workspace(buf[:n])
+        try:
+            call()
+        except tfb.TokenFilterError as e:
+            assert e.code == tfb.TF_ERR_WORKSPACE
+            return True
+        return False
+
+    lo, hi = 0, (4 << 20) // 256                   # units of 256 bytes: refused / taken
+    scan = lambda: g.ctx.tf_kv_stats(g.shape, g.params, k, v, g.sim_k, g.sim_v)
+    assert not refused(scan, hi * 256)
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        lo, hi = (mid, hi) if refused(scan, mid * 256) else (lo, mid)
+    n = hi * 256 + 2 * up(B * S * Hkv * 4) + up(B * S * 4) + up(B * S) + up(B * S * 4) + 2 * up(B * 4)
+    if visibility == tfb.TF_KV_RETAINED:
+        n += 2 * (B * S * Hkv * 128 * 2 + 255) // 256 * 256
+    step = lambda: g.ctx.tf_layer_filter(g.shape, g.params, q, k, v, g.O)
+    assert refused(step, n - 256)
+    g.O.fill_(float("nan"))
+    assert not refused(step, n)
+    g.status_ok()
+    assert torch.equal(g.O, ref)
+    assert g.ctx.workspace_bytes(g.shape, g.params) >= n
+    g.close()
+
+
 def test_decode_and_prefill_share_the_workspace():
     """The decode step keeps its split-key partial results in the bound workspace, over the region where the
     similarity scan keeps its records; a scan after decode steps must still be right (it clears its region first),

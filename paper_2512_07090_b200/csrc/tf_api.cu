@@ -17,7 +17,7 @@ inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 struct WsLayout {
     size_t scan, sim_k, sim_v, score, keep_mask, kept_idx, n_kept, theta, kv_compact;
     size_t prefill;       // all of these: what tf_layer_filter needs
-    size_t total;         // ... or tf_decode_step, whichever is more (each uses the workspace from the front; it serves one call at a time)
+    size_t total;         // ... and tf_decode_step next to the scan's records, which are kept from call to call (it serves one call at a time)
 };
 
 WsLayout ws_layout(const tf_shape& s, const tf_filter_params* p) {
@@ -35,7 +35,7 @@ WsLayout ws_layout(const tf_shape& s, const tf_filter_params* p) {
     w.kv_compact = off;   // retained tokens' K and V (TF_KV_RETAINED on the tensor-core path only)
     if (p && p->kv_visibility == TF_KV_RETAINED && s.dtype == TF_BF16) off += kv_compact_bytes(s);
     w.prefill = off;
-    w.total = std::max(off, align256(decode_scratch_bytes(s)));
+    w.total = std::max(off, w.sim_k + align256(decode_scratch_bytes(s)));
     return w;
 }
 

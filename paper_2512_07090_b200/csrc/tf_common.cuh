@@ -290,7 +290,7 @@ struct tf_decode_args {
     const tf_decode_state* state; void* O_new; float* score_out; uint8_t* skip_out;
     float eta; int alg1_sign;
 };
-size_t decode_scratch_bytes(const tf_shape& s);   // partial results of tf_decode_step, at the start of the workspace
+size_t decode_scratch_bytes(const tf_shape& s);   // partial results of tf_decode_step, at the end of the workspace
 cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_params& p, const tf_decode_args& a,
                                cudaStream_t st);
 // returns cudaErrorNotSupported when the tensor-core path cannot take this call

@@ -758,7 +758,7 @@ __global__ void __launch_bounds__(kHeadDim) decode_combine_kernel(const DecStrea
 // what decode_combine_kernel reads, in front of the slots
 static size_t stream_table_bytes(int grid) { return (1 + (size_t)grid * (1 + kStreamDrawn)) * sizeof(uint4); }
 
-size_t decode_scratch_bytes(const tf_shape& s) { return s.dtype == TF_BF16 ? kStreamScratch + stream_table_bytes(sm_count()) : 0; }
+size_t decode_scratch_bytes(const tf_shape& s) { return s.dtype == TF_BF16 ? kStreamScratch + stream_table_bytes(sm_count()) + 256 : 0; }   // (+ alignment)
 
 static cudaError_t launch_stream(const DecStreamParams& sp, int grid, int device, const CUtensorMap& mk, const CUtensorMap& mv, cudaStream_t st) {
     static bool attr_set_dev[kDeviceFlagSlots] = {};      // function attributes are per device
@@ -993,6 +993,16 @@ static cudaError_t launch_split(const DecGqaParams& gp, dim3 grid, bool cluster,
     return cudaLaunchKernelEx(&cfg, decode_attention_split_kernel<G, true>, gp);
 }
 
+// The scratch of a step lies at the END of the bound workspace, the records that a scan keeps from call to call at the front: a
+// workspace of tf_workspace_bytes holds both.  (At the front the records had to be cleared before the next scan, which the host
+// only knows of a step that it launches itself, not of one that is replayed from a CUDA graph.)  In a smaller workspace, where
+// they overlap, the next scan clears its region first.
+static char* step_scratch(tf_ctx* ctx, size_t bytes) {
+    const size_t at = (ctx->workspace_bytes - bytes) & ~(size_t)255;
+    if (at < (ctx->scan_user.bytes & ~(size_t)1)) ctx->scan_user.needs_clear = true;      // (the low bit is not part of the extent)
+    return static_cast<char*>(ctx->workspace) + at;
+}
+
 cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_params& p, const tf_decode_args& a,
                                cudaStream_t st) {
     if (s.batch == 0) return cudaSuccess;
@@ -1038,11 +1048,11 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
     const size_t table = stream_table_bytes(first_grid), slot = kPartialFloats * sizeof(float);
     if (stream && ctx->workspace && ctx->workspace_bytes >= table + (3 * (size_t)first_grid + 2) * slot) {
         const size_t scratch = std::min(ctx->workspace_bytes, table + kStreamScratch);
-        sp.begun = static_cast<uint4*>(ctx->workspace) + 1;
-        sp.partial = reinterpret_cast<float*>(static_cast<char*>(ctx->workspace) + table);
+        char* at = step_scratch(ctx, scratch);
+        sp.begun = reinterpret_cast<uint4*>(at) + 1;
+        sp.partial = reinterpret_cast<float*>(at + table);
         sp.max_slots = (unsigned int)((scratch - table) / slot);
         dp.next_piece = &sp.begun[-1].y;
-        ctx->scan_user.needs_clear = true; ctx->scan_owned.needs_clear = true;      // (the scan's records: see below)
     }
     dp.tau = a.state->tau; dp.steps = reinterpret_cast<long long*>(a.state->steps);
     dp.skips = reinterpret_cast<long long*>(a.state->skips);
@@ -1080,8 +1090,8 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
         const long long groups = (long long)s.batch * s.n_kv_heads, slots = 2ll * sms;
         const bool few = 8 * groups <= sms && G <= 4;
         int n_splits = 1;
+        const size_t per_split = (size_t)s.batch * s.n_q_heads * kPartialFloats * sizeof(float);
         {
-            const size_t per_split = (size_t)s.batch * s.n_q_heads * kPartialFloats * sizeof(float);
             const int most = std::max(few ? std::min(8, max_keys / 64) : 1, max_keys / 256);
             long long best = -1;
             for (int n = 1; n <= std::max(1, most); ++n) {
@@ -1093,10 +1103,7 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
         }
         gp.n_splits = n_splits;
         const bool cluster = few && n_splits > 1 && n_splits <= 8, scratch = n_splits > 1 && !cluster;
-        gp.partial = scratch ? static_cast<float*>(ctx->workspace) : nullptr;
-        // the partial results overwrite the start of the workspace, where tf_kv_stats keeps its tagged records: the
-        // next scan on this workspace clears its region first instead of trusting what it finds there
-        if (scratch) { ctx->scan_user.needs_clear = true; ctx->scan_owned.needs_clear = true; }
+        gp.partial = scratch ? reinterpret_cast<float*>(step_scratch(ctx, per_split * n_splits)) : nullptr;
         const dim3 grid((unsigned)n_splits, (unsigned)s.n_kv_heads, (unsigned)s.batch);
         switch (G) {
             case 1: e = launch_split<1>(gp, grid, cluster, st); break;

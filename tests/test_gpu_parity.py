@@ -730,6 +730,45 @@ def test_layer_step_takes_a_workspace_of_just_what_it_uses(visibility):
     g.close()
 
 
+@pytest.mark.parametrize("B,S,Hq,Hkv", [(2, 3000, 12, 12), (4, 2048, 32, 8)])     # streaming kernel / splits merged through scratch
+def test_replayed_decode_steps_leave_the_scan_records_of_the_shared_workspace_alone(B, S, Hq, Hkv):
+    """Layer steps and decode steps on one workspace, each captured once and replayed in turn, and launched directly in
+    between: the host does not see a replay, so neither may rely on it to be told of the other's use of the workspace."""
+    q, k, v = _qkv(B, S, Hq, Hkv, torch.bfloat16, seed=B)
+    g = Gpu(q, k, v, prune_ratio=0.5)
+    qn = q[:, -1].contiguous()
+    O = torch.empty_like(qn)
+    shape = tfb.make_shape(None, k, v, n_q_heads=Hq)
+    shape.q_stride[:] = [qn.stride(0), 0, qn.stride(1)]
+    shape.o_stride[:] = list(shape.q_stride)
+    st = tfb.DecodeState(B, Hkv, DEV)
+    st.tau.fill_(9.0)
+    skip, pos = torch.empty(B, dtype=torch.uint8, device=DEV), torch.full((B,), S - 1, dtype=torch.int32, device=DEV)
+    layer = lambda: g.ctx.tf_layer_filter(g.shape, g.params, q, k, v, g.O, g.score, g.keep, g.idx, g.nk)
+    step = lambda: g.ctx.tf_decode_step(shape, g.params, 0.0, qn, k, v, pos, st, O, None, skip)
+    layer()
+    step()
+    g.status_ok()
+    ref, ref_score, ref_step = g.O.clone(), g.score.clone(), O.clone()
+    graphs = []
+    for call in (layer, step):
+        call()
+        torch.cuda.synchronize()
+        graphs.append(torch.cuda.CUDAGraph())
+        with torch.cuda.graph(graphs[-1]):
+            call()
+    layer()                          # (the host believes the records to be in order from here on)
+    for order in ((1, layer), (1, 0), (0, 1, 0), (step, 0), (1, 1, layer), (step, layer)):
+        g.score.fill_(float("nan")); g.O.fill_(float("nan")); O.fill_(float("nan"))
+        for what in order:
+            what() if callable(what) else graphs[what].replay()
+        g.status_ok()
+        assert torch.equal(g.score, ref_score) and torch.equal(g.O, ref), order
+        if any(w in (1, step) for w in order):
+            assert torch.equal(O, ref_step), order
+    g.close()
+
+
 def test_decode_and_prefill_share_the_workspace():
     """The decode step keeps its split-key partial results in the bound workspace, over the region where the
     similarity scan keeps its records; a scan after decode steps must still be right (it clears its region first),

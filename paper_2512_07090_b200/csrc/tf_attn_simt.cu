@@ -10,8 +10,9 @@
 //                         as many CTAs with half the serial length, for problems that would leave SMs idle.
 // The next chunk's keys are fetched (cp.async) under the P V part, its values under the next Q K part.  Shared-memory reads
 // bound it: per 4 dims 16 wavefronts (a 16-byte broadcast is two) for 8 cycles of multiply-adds in Q K^T, 24 for 16 in P V.
-// A retained row's warp also zeroes the output rows of the pruned tokens before it (Section 3.2: a skipped token's
-// attention output is zero), so the whole of O is written with no separate clearing pass.
+// The CTA also zeroes the output rows of the pruned tokens before its rows (Section 3.2: a skipped token's attention output is
+// zero), all warps and before the chunks, so the whole of O is written with no separate clearing pass.  Under a window it
+// passes over chunks that none of its rows sees.
 //   One warp per row, a key at a time per lane straight from global memory, took 48 us at 1 x 128 tokens x 32 heads, 392 at
 // 512 and 4700 at 2 x 1024 x 40 heads; this kernel takes 11, 85 and 670.
 // CTAs with rows start before those expected to have none, over all heads (a quarter to a half of the grid was empty CTAs
@@ -129,20 +130,37 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
     }
 
     // keys are visited by index: token positions, or positions in the retained list (retained_only), where entry c stands
-    // for token kept[c] and the query itself is its own entry
-    auto first_key = [&](int slot, int t) {
-        const int t_min = p.window > 0 ? max(0, t - p.window + 1) : 0;
-        return p.retained_only ? (t_min > 0 ? first_kept_at_or_after(kept, slot + 1, t_min) : 0) : t_min;
+    // for token kept[c] and the query itself is its own entry.  Lane l of every warp looks up row l of the CTA.
+    const int slot_l = slot0 + lane, last_row = min(C::kRows, nk - slot0) - 1;
+    const int t_l = lane <= last_row ? kept[slot_l] : -1, t_before = slot0 > 0 ? kept[slot0 - 1] : -1;
+    int lo_l = 0, hi_l = -1;                                                // visible keys of the row (hi < lo: no such row)
+    if (lane <= last_row) {
+        const int t_min = p.window > 0 ? max(0, t_l - p.window + 1) : 0;
+        lo_l = p.retained_only ? (t_min > 0 ? first_kept_at_or_after(kept, slot_l + 1, t_min) : 0) : t_min;
+        hi_l = p.retained_only ? slot_l : t_l;
+    }
+    __syncwarp();
+    const int c_hi = __shfl_sync(0xffffffffu, hi_l, last_row);             // the CTA's last visible key
+    const int ch1 = c_hi / kSimtChunk + 1;
+    // the first chunk from c on that some row sees: rows of a sparse list with a short window leave chunks between them
+    auto seen_from = [&](int c) {
+        if (p.window == 0) return c;
+        const int mine = hi_l / kSimtChunk >= c && hi_l >= 0 ? max(c, lo_l / kSimtChunk) : ch1;
+        return (int)__reduce_min_sync(0xffffffffu, (unsigned int)mine);
     };
-    const int s_last = min(slot0 + C::kRows, nk) - 1;
-    const int c_hi = p.retained_only ? s_last : kept[s_last];              // the CTA's last visible key
-    const int ch0 = first_key(slot0, kept[slot0]) / kSimtChunk, ch1 = c_hi / kSimtChunk + 1;
+    auto advance = [&](int c) {
+        if (p.window == 0) return c + kSplit;
+#pragma unroll
+        for (int i = 0; i < kSplit; ++i) c = seen_from(c + 1);
+        return c;
+    };
 
     auto part_sync = [&]() {
         if (kSplit == 1) __syncthreads();
         else asm volatile("bar.sync %0, %1;" :: "r"(1 + part), "n"(C::kPartThreads) : "memory");
     };
-    int ch = ch0 + part;
+    int ch = seen_from(0);
+    if (part) ch = seen_from(ch + 1);
     if (!early && ch < ch1) { fetch(sK, Kb, p.ks.t, ch, c_hi, true); fetch(sV, Vb, p.vs.t, ch, c_hi, false); }
     for (int i = tid; i < C::kRows * 32; i += kSimtThreads) {
         const int row = i >> 5, piece = i & 31, slot = slot0 + row;
@@ -152,19 +170,25 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
         *reinterpret_cast<float4*>(sQ + row * kHeadDim + piece * 4) = make_float4(q.x * p.scale_log2, q.y * p.scale_log2, q.z * p.scale_log2, q.w * p.scale_log2);
     }
     const int row0 = rgroup * R;
-    int lo[R], hi[R], w_lo = 0x7fffffff, w_hi = -1;                     // visible keys of each row (hi < lo: no such row)
+    int lo[R], hi[R], w_lo = 0x7fffffff, w_hi = -1;                     // visible keys of each row of the warp
     int all_lo = 0, all_hi = 0x7fffffff;                                // keys that every row of the warp sees
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int slot = slot0 + row0 + r;
-        lo[r] = 0; hi[r] = -1;
-        if (slot < nk) {
-            const int t = kept[slot];
-            lo[r] = first_key(slot, t);
-            hi[r] = p.retained_only ? slot : t;
+        lo[r] = __shfl_sync(0xffffffffu, lo_l, row0 + r);
+        hi[r] = __shfl_sync(0xffffffffu, hi_l, row0 + r);
+        if (row0 + r <= last_row) {
             w_lo = min(w_lo, lo[r]); w_hi = max(w_hi, hi[r]);
             all_lo = max(all_lo, lo[r]); all_hi = min(all_hi, hi[r]);
         }
+    }
+    // the rows of pruned tokens before each retained one (and behind the last of all) are zero; the stores run under the chunks
+#pragma unroll
+    for (int i = 0; i < C::kRows / kSimtWarps; ++i) {
+        const int row = warp * (C::kRows / kSimtWarps) + i;
+        const int t = __shfl_sync(0xffffffffu, t_l, row), before = __shfl_sync(0xffffffffu, t_l, max(row - 1, 0));
+        if (row > last_row) break;
+        zero_rows(Ob, p.os, (row == 0 ? t_before : before) + 1, t, lane);
+        if (slot0 + row == nk - 1) zero_rows(Ob, p.os, t + 1, p.S, lane);
     }
     __syncthreads();
 
@@ -190,8 +214,9 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
             }
         }
     };
-    for (; ch < ch1; ch += kSplit) {
+    for (int ch_next; ch < ch1; ch = ch_next) {
         const int j0 = ch * kSimtChunk;
+        ch_next = advance(ch);
         const bool mine = w_hi >= j0 && w_lo < j0 + kSimtChunk;            // some row of this warp sees this chunk
         fetch_wait_all_but_one();
         part_sync();                                                       // K(ch) is there
@@ -224,7 +249,7 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
                 }
         }
         part_sync();                                                       // K(ch) has been read
-        if (ch + kSplit < ch1) fetch(sK, Kb, p.ks.t, ch + kSplit, c_hi, true); else fetch_commit();
+        if (ch_next < ch1) fetch(sK, Kb, p.ks.t, ch_next, c_hi, true); else fetch_commit();
         if (mine) {
             const int ja = j0 + lane, jb = ja + 32;
 #pragma unroll
@@ -255,7 +280,7 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
             __syncwarp();                                                  // sP is written again in the next chunk
         }
         part_sync();                                                       // V(ch) has been read
-        if (ch + kSplit < ch1) fetch(sV, Vb, p.vs.t, ch + kSplit, c_hi, false); else fetch_commit();
+        if (ch_next < ch1) fetch(sV, Vb, p.vs.t, ch_next, c_hi, false); else fetch_commit();
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) l[r] = warp_sum(l[r]);
@@ -284,13 +309,10 @@ __global__ void __launch_bounds__(kSimtThreads, kSplit == 2 ? 1 : 2) attention_s
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int slot = slot0 + row0 + r;
-        if (slot >= nk) break;
-        const int t = kept[slot];
+        if (row0 + r > last_row) break;
+        const int t = __shfl_sync(0xffffffffu, t_l, row0 + r);
         const float inv = 1.f / l[r];
         store4(Ob + (long long)t * p.os.t + lane * 4, acc[r][0] * inv, acc[r][1] * inv, acc[r][2] * inv, acc[r][3] * inv);
-        zero_rows(Ob, p.os, slot == 0 ? 0 : kept[slot - 1] + 1, t, lane);   // pruned rows before this one
-        if (slot == nk - 1) zero_rows(Ob, p.os, t + 1, p.S, lane);
     }
 }
 

@@ -412,7 +412,9 @@ def test_pruned_attention_retained_keys_only(dtype, path, B, S, Hq, Hkv, window,
     (1, 16, 2, 1, 0, 0.0, tfb.TF_KV_ALL), (1, 17, 2, 1, 0, 0.0, tfb.TF_KV_ALL), (1, 65, 3, 3, 0, 0.25, tfb.TF_KV_RETAINED),
     (1, 600, 2, 2, 65, 0.1, tfb.TF_KV_ALL),          # split over two chunk sequences (few CTAs)
     (2, 520, 20, 5, 100, 0.5, tfb.TF_KV_ALL), (3, 333, 24, 6, 0, 0.3, tfb.TF_KV_RETAINED),
-    (1, 97, 80, 40, 0, 0.0, tfb.TF_KV_ALL)])          # 32 rows per CTA, all warps on one chunk
+    (1, 97, 80, 40, 0, 0.0, tfb.TF_KV_ALL),           # 32 rows per CTA, all warps on one chunk
+    (1, 4000, 2, 1, 30, 0.995, tfb.TF_KV_ALL), (3, 5000, 48, 6, 70, 0.99, tfb.TF_KV_ALL),       # chunks between the rows that nobody sees
+    (1, 4000, 2, 1, 300, 0.99, tfb.TF_KV_RETAINED)])
 def test_cuda_core_attention_both_forms(B, S, Hq, Hkv, window, ratio, visibility):
     q, k, v = _qkv(B, S, Hq, Hkv, torch.float32, seed=S + Hq)
     qn, kn, vn = oracle_inputs(q, k, v)

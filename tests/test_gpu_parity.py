@@ -592,6 +592,28 @@ def test_pruned_attention_many_short_items_per_cta(path, S, window, claimed_rati
     g.close()
 
 
+@pytest.mark.parametrize("path,Hq,Hkv", [(2, 8, 8), (5, 8, 4), (6, 16, 4)])
+@pytest.mark.parametrize("share", [0.0, 0.03, 0.6])
+def test_persistent_attention_with_an_eligibility_mask(path, Hq, Hkv, share):
+    """With a mask the list can be of any length from the ratio's to all tokens, and every row block is a work item of its own."""
+    B, S, ratio = 3, 1200, 0.8
+    q, k, v = _qkv(B, S, Hq, Hkv, torch.bfloat16, seed=int(100 * share) + Hq)
+    elig = (np.random.default_rng(S).random((B, S)) < share).astype(np.uint8)
+    elig_d = torch.from_numpy(elig).to(DEV)
+    qn, kn, vn = oracle_inputs(q, k, v)
+    g = Gpu(q, k, v, prune_ratio=ratio, warmup_tokens=5, eligible=elig_d)
+    g.ctx.tf_set_attention_path(path)
+    g.ctx.tf_layer_filter(g.shape, g.params, q, k, v, g.O, g.score, g.keep, g.idx, g.nk)
+    g.status_ok()
+    keep = g.keep.cpu().numpy()
+    pruned = np.minimum((elig[:, 5:]).sum(1), int(ratio * S))
+    assert np.array_equal(g.nk.cpu().numpy(), S - pruned) and np.all(keep[:, :5] == 1) and np.all(keep[elig == 0] == 1)
+    o = to_np(g.O)
+    assert attn_rel_err(o, oracle.pruned_attention(qn, kn, vn, keep)) < ATTN_TOL[torch.bfloat16]
+    assert np.all(o[keep == 0] == 0.0)
+    g.close()
+
+
 @pytest.mark.parametrize("tensor_cores", [2, 3, 4, 5, 6])
 @pytest.mark.parametrize("claimed_ratio", [0.0, 0.9])
 def test_pruned_attention_with_a_retained_list_the_ratio_does_not_predict(tensor_cores, claimed_ratio):

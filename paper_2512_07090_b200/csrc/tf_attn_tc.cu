@@ -268,24 +268,23 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
     const uint32_t bar_q1 = bar_q0 + 8;                  // [2] Q slot of tile 1, the item's rows and descriptor given back
     const uint32_t bar_item = bar_q1 + 16;               // [2] item descriptor written
     const uint32_t bar_claim = bar_item + 16;            // answer of the launch queue
-    const uint32_t bar_asked = bar_claim + 8;            // all but the last kClaimLead K/V tiles of the item requested
-    const uint32_t claim = bars + 192;                   // 16 bytes
+    const uint32_t bar_asked = bar_claim + 8;            // [2] all but the last kClaimLead K/V tiles of the item requested
+    const uint32_t claim = bars + 208;                   // 16 bytes
     TcItem* const items = reinterpret_cast<TcItem*>(smem + kPOffMisc + 224);          // [2]
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kPOffMisc + 320);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kPOffMisc + 328);
     int* const rows = reinterpret_cast<int*>(smem + kPOffRows);                       // [2][256] token position, -1: no row
-    static_assert(sizeof(TcItem) <= 48 && (2 * kPStages + 16) * 8 <= 192, "layout of the last 512 bytes");
+    static_assert(sizeof(TcItem) <= 48 && (2 * kPStages + 17) * 8 <= 208, "layout of the last 512 bytes");
     if (tid == 0) {
         for (int i = 0; i < kPStages; ++i) { mbar_init(bar_full + 8 * i, 1); mbar_init(bar_empty + 8 * i, 1); }
         for (int i = 0; i < 2; ++i) {
             mbar_init(bar_s + 8 * i, 1); mbar_init(bar_p + 8 * i, kTileM); mbar_init(bar_o + 8 * i, 1);
-            mbar_init(bar_qf0 + 8 * i, kGatherThreads); mbar_init(bar_item + 8 * i, kGatherThreads);
+            mbar_init(bar_qf0 + 8 * i, kGatherThreads); mbar_init(bar_item + 8 * i, kGatherThreads); mbar_init(bar_asked + 8 * i, 1);
             mbar_init(bar_q1 + 8 * i, kSoftmaxThreads / 32);
         }
         mbar_init(bar_qf1, kGatherThreads);
         mbar_init(bar_q0, kHeads ? 1 : kTileM / 32);
         mbar_init(bar_claim, 1);
-        mbar_init(bar_asked, 1);
         *abort_flag = 0;
         mbar_fence_init();
     }
@@ -437,7 +436,7 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
             }
             // the next item
             __syncwarp();
-            if (produced) mbar_wait(bar_asked, (n - 1) & 1, abort_flag, p.wait_cycles, p.status, 15);
+            if (produced) mbar_wait(bar_asked + 8 * ((n - 1) & 1), ((n - 1) >> 1) & 1, abort_flag, p.wait_cycles, p.status, 15);
             __syncwarp();
             fence_proxy_async();                               // the last answer has been read
             if (gather_any(*abort_flag != 0)) break;
@@ -479,7 +478,7 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
                         tma_load_4d(dst, map, bar_full + 8 * st, 0, kh, j * kTileN, it.b);
                         tma_load_4d(dst + kHalfBytes, map, bar_full + 8 * st, 64, kh, j * kTileN, it.b);
                     }
-                    if (j == max(J1 - 1 - kClaimLead, it.jb[0])) mbar_arrive(bar_asked);
+                    if (j == max(J1 - 1 - kClaimLead, it.jb[0])) mbar_arrive(bar_asked + 8 * (n & 1));
                 }
             }
             __syncwarp();

@@ -244,8 +244,9 @@ tf_status tf_decode_step(tf_ctx *ctx, const tf_shape *shape, const tf_filter_par
 tf_status tf_tail_policy(double p_global, double tail_fraction, int32_t n_layers,
                          double *ratio_per_layer, int32_t *n_tail_out);
 
-/* Device-side conditions since the last tf_clear_status: returns TF_OK, TF_ERR_TIMEOUT or
- * TF_ERR_NAN_SCORE.  sync != 0 synchronises the device first.  detail (may be NULL) receives
+/* Device-side conditions since the last tf_clear_status: returns TF_OK, TF_ERR_TIMEOUT,
+ * TF_ERR_NAN_SCORE or TF_ERR_CUDA (a kernel refused to run on shared memory that does not start on
+ * the 1024-byte boundary it is declared with).  sync != 0 synchronises the device first.  detail (may be NULL) receives
  * four words: {code, where, count of NaN scores, kernels launched by this context}.  After a
  * TF_ERR_TIMEOUT the outputs of the call that saw it are undefined; the context stays usable
  * (the next similarity scan clears its scratch records first). */

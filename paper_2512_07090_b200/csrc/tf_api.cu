@@ -490,6 +490,7 @@ tf_status tf_get_status(tf_ctx* ctx, int sync, int64_t detail[4]) {
         return TF_ERR_TIMEOUT;
     }
     if (h.code == TF_ERR_NAN_SCORE) return TF_ERR_NAN_SCORE;
+    if (h.code == TF_ERR_CUDA) return TF_ERR_CUDA;   // a kernel found its shared memory off the 1024-byte boundary it is declared with
     return TF_OK;
 }
 

@@ -250,11 +250,11 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
     constexpr int kTileRows = kHeads ? kTileM / kHpt : kTileM;   // retained-list entries per Q tile
     constexpr int kRows = kHeads ? kTileRows : 2 * kTileM;       // ... per item
     constexpr int kHeadsPerCta = kHeads ? 2 * kHpt : 1;
-    extern __shared__ uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t sbase = smem_u32(smem);
     if (sbase & 1023u) {   // the swizzled operand layout needs it; nothing has been started yet
-        if (tid == 0) report_error(p.status, TF_ERR_TIMEOUT, 398);
+        if (tid == 0) report_error(p.status, TF_ERR_CUDA, 398);
         return;
     }
     const uint32_t bars = sbase + kPOffMisc;
@@ -968,11 +968,11 @@ constexpr int kRegs1 = 128;                      // registers per thread at laun
 
 __global__ void __launch_bounds__(kThreads1, 2)
 attention_tc_single_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV) {
-    extern __shared__ uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t sbase = smem_u32(smem);
     if (sbase & 1023u) {   // the swizzled operand layout needs it; nothing has been started yet
-        if (tid == 0) report_error(p.status, TF_ERR_TIMEOUT, 399);
+        if (tid == 0) report_error(p.status, TF_ERR_CUDA, 399);
         return;
     }
     const uint32_t bar_q = sbase + kOffBar1;              // Q tile written

@@ -216,11 +216,11 @@ struct Gram1Params {
 template <bool EMA>
 __global__ void __launch_bounds__(128, 6)
 kv_stats_gram1_kernel(const Gram1Params p, const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV) {
-    extern __shared__ uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     if (sbase & 1023u) {   // the swizzled operand layout needs it; nothing has been started yet
         if (threadIdx.x == 0) {
-            report_error(p.status, TF_ERR_TIMEOUT, 199);
+            report_error(p.status, TF_ERR_CUDA, 199);
             grid_dependency_wait();
             scan_draw_ticket(p.counters);
             scan_leave(p.counters, gridDim.x);
@@ -507,12 +507,12 @@ template <bool EMA>
 __global__ void __launch_bounds__(kPThreads, 1)
 kv_stats_gram_persistent_kernel(const GramPParams pp, const __grid_constant__ CUtensorMap mapK,
                                 const __grid_constant__ CUtensorMap mapV) {
-    extern __shared__ uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     const Gram1Params& p = pp.g;
     const uint32_t sbase = smem_u32(smem);
     if (sbase & 1023u) {
         if (threadIdx.x == 0) {
-            report_error(p.status, TF_ERR_TIMEOUT, 299);
+            report_error(p.status, TF_ERR_CUDA, 299);
             grid_dependency_wait();
             scan_leave(p.counters, gridDim.x);
         }

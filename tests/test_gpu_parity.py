@@ -1228,6 +1228,34 @@ def test_decode_decision_and_state_for_every_number_of_heads(dtype, Hkv, offset)
     ctx.close()
 
 
+@pytest.mark.parametrize("B,S,Hkv", [(6, 3000, 4), (150, 500, 8)])       # split / whole work items otherwise
+def test_streaming_decode_when_every_sequence_is_skipped(B, S, Hkv):
+    """The tiles fetched before the decisions were known are thrown away and there is no work: zero rows, and a right next step."""
+    _, k, v = _qkv(B, S, Hkv, Hkv, torch.bfloat16, seed=S)
+    qn = k[:, 5].contiguous()
+    shape = tfb.make_shape(None, k, v, n_q_heads=Hkv)
+    shape.q_stride[:] = [qn.stride(0), 0, qn.stride(1)]
+    shape.o_stride[:] = list(shape.q_stride)
+    params = tfb.default_params(prune_ratio=0.5, warmup_tokens=0)
+    ctx = tfb.Context(0)
+    ctx.ensure_workspace(shape, params)
+    st = tfb.DecodeState(B, Hkv, DEV)
+    O, skip = torch.empty_like(qn), torch.empty(B, dtype=torch.uint8, device=DEV)
+    pos = torch.full((B,), S - 1, dtype=torch.int32, device=DEV)
+    for tau in (-9.0, -9.0, 9.0, -9.0):
+        st.tau.fill_(tau)
+        O.fill_(float("nan"))
+        ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
+        assert ctx.tf_get_status()[0] == tfb.TF_OK
+        assert torch.all(skip == (1 if tau < 0 else 0))
+        if tau < 0:
+            assert torch.all(O == 0)
+            continue
+        p = (torch.einsum("bhd,bnhd->bhn", qn.double(), k.double()) / 128 ** 0.5).softmax(-1)
+        assert attn_rel_err(to_np(O), torch.einsum("bhn,bnhd->bhd", p, v.double()).cpu().numpy()) < ATTN_TOL[torch.bfloat16]
+    ctx.close()
+
+
 @pytest.mark.parametrize("dtype,mode,window,S0,T,Hq,Hkv",
                          [(torch.bfloat16, tfb.TF_ANCHOR_PAST_MEAN, 0, 70, 90, 8, 2), (torch.float32, tfb.TF_ANCHOR_PAST_MEAN, 40, 70, 90, 8, 2),
                           (torch.bfloat16, tfb.TF_ANCHOR_EMA, 0, 70, 90, 8, 2), (torch.bfloat16, tfb.TF_ANCHOR_INCL_MEAN, 0, 70, 90, 8, 2),

@@ -41,7 +41,7 @@ constexpr int kTileN = 128;           // keys per K/V tile
 constexpr int kHalfBytes = 128 * 128; // one [128 rows][128 B] swizzled block (64 bf16 per row)
 constexpr int kTileBytes = 2 * kHalfBytes;
 constexpr int kSoftmaxThreads = kQTiles * kTileM;
-constexpr int kThreads = kSoftmaxThreads + 128;   // third warpgroup: MMA warp, TMA warp, two idle warps
+constexpr int kThreads = kSoftmaxThreads + 128;   // third warpgroup: MMA warp, TMA warp, two that fetch items and Q rows (split form: only zero rows)
 constexpr int kMmaWarp = kSoftmaxThreads / 32, kTmaWarp = kMmaWarp + 1;
 constexpr uint32_t kTmemCols = 512;   // S0 | S1 | O0 | O1, 128 fp32 columns each
 constexpr float kRescaleThreshold = 8.f;         // log2 units
@@ -202,8 +202,8 @@ __device__ __forceinline__ void softmax_tile(uint32_t tm_s, uint32_t tm_o, int l
 // A CTA per item spends some 15,000 cycles around its tiles (3,300 each): launch, TMEM, three dependent global round
 // trips, 64 KB of scattered Q rows, the first Q K^T and the last P V with nothing beside them, the epilogue.  Here the
 // next item's set-up runs under the tiles of the current one:
-//   warps 10-11 claim the next item when the last K/V tile of this one has been requested (late enough for the queue
-//     to hand items to the SMs that run out first), read its indices, gather its Q rows (cp.async) and publish a
+//   warps 10-11 claim the next item when all but the last kClaimLead K/V tiles of this one have been requested (late enough
+//     for the queue to hand items to the SMs that run out first), read its indices, gather its Q rows (cp.async) and publish a
 //     descriptor; then they zero the output rows of pruned tokens.
 //   warp 9 goes on with the next item's K/V tiles in the same ring, warp 8 with its products: Q K^T of the next item's
 //     first tile is issued right behind the last P V of this one.
@@ -212,7 +212,8 @@ __device__ __forceinline__ void softmax_tile(uint32_t tm_s, uint32_t tm_o, int l
 //     needed (kHpt > 0) or group 0's epilogue does (kHpt = 0, where group 0 finishes first).
 //   The epilogue stages its rows in the slot of tile 1 (kHpt > 0) or of the group's own tile (kHpt = 0).
 // One layer's pass, one CTA per item -> persistent: 8 x 16384 windowed 4276 -> 3932 us, 2 x 8192 grouped heads 609 -> 568 us,
-// 4 x 4096 x 40 heads 555 -> 506 us, 3 x 1531 87.7 -> 82.8 us, 2 x 3001 retained keys 139 -> 127 us.
+// 4 x 4096 x 40 heads 555 -> 506 us, 3 x 1531 87.7 -> 82.8 us, 2 x 3001 retained keys 139 -> 127 us; the last two with rows of
+// pruned tokens zeroed by bulk copies 76 and 118 us.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kGatherWarp = kTmaWarp + 1;              // and the one after it
 constexpr int kGatherThreads = 64;

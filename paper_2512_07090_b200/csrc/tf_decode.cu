@@ -1,7 +1,7 @@
 // Online decode step: Algorithm 1 for ONE new token per sequence, with the threshold feedback of
 // Section 3.3 (T_l <- T_l + eta (P_current - P_tail)) and the attention it gates.
 //
-// decode_decide_kernel (one CTA per sequence, one warp per KV head at a time):
+// decode_decide_kernel (one CTA per sequence, a warp per KV head, beyond 8 heads per two):
 //   per head: cosine of the current token's key / value to the anchor carried in the state (sum of
 //   past tokens, or the EMA of Eq. 1); then one warp: mean / variance over heads, weight alpha
 //   (Eq. 2), score s_KV (Eq. 3), threshold adaptation, skip decision; then the anchor takes the
@@ -57,7 +57,7 @@ __device__ __forceinline__ void dec_load4(const __nv_bfloat16* p, float (&f)[4])
 }
 
 // One chain of dependent loads (position, then rows), so what counts is how much of it is in flight at once: a warp per
-// two KV heads as far as 32 warps reach, every load a full vector (where the state is aligned).  Once everything before the
+// KV head, beyond 8 heads per two as far as 32 warps reach, every load a full vector (where the state is aligned).  Once everything before the
 // step is complete the attention kernel may start and fetch its first tiles under this kernel.
 constexpr int kDecideWarps = 32;
 
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_attention_kernel(const 
 //           states in shared memory and go on with the next segment at once; these warps merge the eight states and write the result.
 // Every wait is bounded, those of the warps for one another too (mbarriers, no named barriers): on expiry the CTA records
 // TF_ERR_TIMEOUT, stops waiting, lets copies in flight land and exits.
-//   A step of 128 sequences x 400 keys x 40 heads (half of them skipped): 112 -> 98 us, 4 x 4096 keys x 40 heads: 75 -> 60 us.
+//   A step of 128 sequences x 400 keys x 40 heads (half of them skipped): 112 -> 100 us, 4 x 4096 keys x 40 heads: 75.5 -> 60 us.
 // ---------------------------------------------------------------------------------------------------
 constexpr int kPartialFloats = kHeadDim + 2;
 constexpr int kStreamKeys = 64;                            // keys per tile
@@ -352,7 +352,7 @@ struct StreamSeg {
     int b, kh, j;                     // sequence, KV head, first tile of the work item
     int count;                        // tiles; 0: no more work
     int slot;                         // where the result goes in the scratch; -1: it is the whole work item
-    unsigned int p_first, p_last;     // the pieces the work item lies in
+    unsigned int p_last;              // the last piece the work item lies in
     int ends_piece;                   // 1: the piece's last segment ...
     unsigned int piece;               // ... and that piece
 };
@@ -441,10 +441,9 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
     unsigned int py = 0, py_end = 0, p_now = 0, pn = 0;     // tile number, end of the piece, its number; tiles of the work item
     auto open_segment = [&]() {                             // from tile py of work item (pt.b, pt.kh, pt.j) on
         pk_lo = first_key(s_pos[pt.b]);
-        const unsigned int i0 = py - pt.j;
         pt.count = (int)min(pn - pt.j, py_end - py);
         p_done = 0;
-        pt.p_first = whole ? p_now : cut.piece_of(i0); pt.p_last = whole ? p_now : cut.piece_of(i0 + pn - 1);
+        pt.p_last = whole ? p_now : cut.piece_of(py - pt.j + pn - 1);
         pt.ends_piece = py + (unsigned int)pt.count == py_end ? 1 : 0;
         pt.piece = p_now;
         pt.slot = (unsigned int)pt.count == pn ? -1 : (int)(2 * p_now + (pt.j == 0 ? 1 : 0));

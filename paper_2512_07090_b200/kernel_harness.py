@@ -3,10 +3,11 @@ program a profiler capture wants (a few hundred MB on the device instead of a wh
 
     python -m paper_2512_07090_b200.kernel_harness --stage scan --batch 8 --seq 16384 --kv-heads 8 [--q-heads 32]
            [--window 4096] [--prune 0.5] [--anchor ema --gamma 0.9] [--launches 6] [--scan-path 0..3] [--attention-path 0..6]
-           [--select-path 0..2]
+           [--select-path 0..2] [--dtype fp32]
 
 Stages: scan (tf_kv_stats), fuse (tf_score_fuse), select (tf_select), score_select (tf_score_select), attention
-(tf_pruned_attention), step (tf_layer_filter).  Inputs are N(0,1) bf16 tensors from a fixed seed with a quarter of the tokens near-duplicates of an
+(tf_pruned_attention), step (tf_layer_filter), decode (tf_decode_step at the last position, no sequence skipped).
+Inputs are N(0,1) tensors from a fixed seed with a quarter of the tokens near-duplicates of an
 earlier token (the recipe of the reduced parity cases); the stages before the requested one run once to produce its
 inputs.  Prints the mean time per launch from CUDA events.
 """
@@ -21,7 +22,7 @@ from . import binding as tfb
 
 def main():
     ap = argparse.ArgumentParser()
-    ap.add_argument("--stage", default="scan", choices=["scan", "fuse", "select", "score_select", "attention", "step"])
+    ap.add_argument("--stage", default="scan", choices=["scan", "fuse", "select", "score_select", "attention", "step", "decode"])
     ap.add_argument("--batch", type=int, default=8)
     ap.add_argument("--seq", type=int, default=16384)
     ap.add_argument("--kv-heads", type=int, default=8)
@@ -34,6 +35,7 @@ def main():
     ap.add_argument("--scan-path", type=int, default=0)
     ap.add_argument("--attention-path", type=int, default=1)
     ap.add_argument("--select-path", type=int, default=0)
+    ap.add_argument("--dtype", default="bf16", choices=["bf16", "fp32"])
     a = ap.parse_args()
     dev = "cuda:0"
     torch.cuda.set_device(0)
@@ -47,9 +49,10 @@ def main():
     dup[:, 0] = False
     for t in (k, v):
         t.copy_(torch.where(dup[..., None, None], torch.gather(t, 1, src[..., None, None].expand_as(t)) + 0.05 * torch.randn_like(t), t))
-    k, v = k.bfloat16(), v.bfloat16()
-    need_q = a.stage in ("attention", "step")
-    q = torch.randn(B, S, Hq, 128, generator=g, device=dev, dtype=torch.bfloat16) if need_q else None
+    dtype = torch.float32 if a.dtype == "fp32" else torch.bfloat16
+    k, v = k.to(dtype), v.to(dtype)
+    need_q = a.stage in ("attention", "step", "decode")
+    q = torch.randn(B, S, Hq, 128, generator=g, device=dev).to(dtype) if need_q else None
     O = torch.empty_like(q) if need_q else None
     ctx = tfb.Context(0)
     shape = tfb.make_shape(q, k, v, O, window=a.window, n_q_heads=Hq)
@@ -70,12 +73,16 @@ def main():
     ctx.tf_select(shape, params, score, keep, idx, nk)
     torch.cuda.synchronize()
 
+    state, pos = tfb.DecodeState(B, Hkv, dev, tau0=9.0), torch.full((B,), S - 1, dtype=torch.int32, device=dev)
+    skip = torch.empty(B, dtype=torch.uint8, device=dev)
+
     def run():
         if a.stage == "scan": ctx.tf_kv_stats(shape, params, k, v, sim_k, sim_v)
         elif a.stage == "fuse": ctx.tf_score_fuse(shape, params, sim_k, sim_v, score)
         elif a.stage == "select": ctx.tf_select(shape, params, score, keep, idx, nk)
         elif a.stage == "score_select": ctx.tf_score_select(shape, params, sim_k, sim_v, score, keep, idx, nk)
         elif a.stage == "attention": ctx.tf_pruned_attention(shape, params, q, k, v, idx, nk, O)
+        elif a.stage == "decode": ctx.tf_decode_step(shape, params, 0.0, q[:, -1], k, v, pos, state, O[:, -1], None, skip)
         else: ctx.tf_layer_filter(shape, params, q, k, v, O, score, keep, idx, nk)
 
     run()

@@ -1305,9 +1305,11 @@ cudaError_t launch_attention_tc(tf_ctx* ctx, const tf_shape& s, const tf_filter_
     const double ctas_shared = (double)s.batch * s.n_q_heads * ceil(s.seq * kept_frac / (kQTiles * kTileM));
     const int sms = sm_count();
     const bool single = ctx->attention_form == 3;
-    // ... when all its CTAs run at once, or when a row's keys are many (32 heads x 2048 tokens, 16 tiles: 34.4 us against 37.7):
-    // with few tiles per CTA the second wave of CTAs costs more than the halved length saves (4 x 512 tokens x 32 heads: 26.5
-    // against 19.4).
+    // ... when all its CTAs run at once, or when a row's keys are many: with few tiles per CTA the second wave of CTAs costs more
+    // than the halved length saves (us, split / shared: 4 x 512 tokens x 32 heads, 4 tiles, 23.0 / 16.7, 2 x 768, 6 tiles, 22.7 /
+    // 18.3, 2 x 1024, 8 tiles, 26.2 / 23.6, 1 x 1280, 10 tiles, 22.2 / 24.8, 1 x 1536, 12 tiles, 24.2 / 28.9, 1 x 2048, 16 tiles,
+    // 34.4 / 37.7; grouped heads 2 x 1024 26.2 / 21.3).  The crossing is between 8 and 10 tiles; the line stays below it, where all
+    // head groups of a call through host memory take the form that the whole call takes, and so have its bits.
     double keys = compact ? s.seq * kept_frac : (double)s.seq;
     if (s.window > 0) keys = std::min(keys, (double)s.window + kTileM / std::max(kept_frac, 1e-3));
     const bool split = ctx->attention_form == 2 ||

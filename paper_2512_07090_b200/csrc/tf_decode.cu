@@ -1084,10 +1084,11 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
         // Number of key splits: two CTAs fit an SM, a wave of CTAs costs (a fixed part worth ~192 keys + its keys), and a
         // partly filled wave costs as much as a full one; take the split count with the cheapest estimate, at least
         // 256 keys per split.
-        // Few work items: the splits, as short as 64 keys, are a cluster and need no third launch (1 x 420 keys x 8 heads 8.4
-        // instead of 9.9 us; with the SMs full clusters wait for one another's slots: 32 x 4096 x 8 86 instead of 79 us).
+        // Few work items: the splits, as short as 64 keys, are a cluster and need no third launch (us a step, cluster / scratch: 1 x
+        // 420 keys x 8 heads 7.85 / 8.97, 1 x 500 x 10 7.9 / 10.3, 4 x 500 x 3 7.9 / 9.15; clusters of more groups wait for one another's slots: 2 x 420 x 8
+        // 10.7 / 9.1, 4 x 500 x 4 10.7 / 9.4, 3 x 500 x 8 11.4 / 9.3, 4 x 1000 x 8 18.8 / 12.8).
         const long long groups = (long long)s.batch * s.n_kv_heads, slots = 2ll * sms;
-        const bool few = 8 * groups <= sms && G <= 4;
+        const bool few = 12 * groups <= sms && G <= 4;
         int n_splits = 1;
         const size_t per_split = (size_t)s.batch * s.n_q_heads * kPartialFloats * sizeof(float);
         {

@@ -961,7 +961,7 @@ def test_requested_kernel_that_cannot_take_the_call_is_an_error_not_a_fallback()
                                               (1, 9000, 1, 4, 0), (40, 300, 5, 1, 130), (1030, 70, 1, 1, 0),
                                               (2, 9000, 3, 1, 0), (150, 130, 8, 1, 0), (1, 200, 4, 8, 0),
                                               (7, 256, 40, 1, 0), (7, 257, 40, 1, 0), (8, 256, 40, 1, 0),      # either side of the streaming kernel
-                                              (1030, 129, 1, 1, 0), (1, 256, 4, 1, 0)])   # ... in three launches; ungrouped heads as a cluster
+                                              (1030, 129, 1, 1, 0), (1, 256, 4, 1, 0), (3, 700, 4, 4, 0), (2, 700, 8, 4, 0)])   # ... in three launches; ungrouped heads as a cluster; either side of the clusters
 def test_decode_attention_uneven_positions_and_skips(B, S, Hkv, G, window, workspace):
     """Every sequence at a position of its own (tile edges among them), some skipped, NaN in the cache behind each position:
     the streaming kernel (ungrouped heads: split and whole work items) and the split kernel (as a cluster, through scratch,

@@ -13,8 +13,8 @@
 // The CTA also zeroes the output rows of the pruned tokens before its rows (Section 3.2: a skipped token's attention output is
 // zero), all warps and before the chunks, so the whole of O is written with no separate clearing pass.  Under a window it
 // passes over chunks that none of its rows sees.
-//   One warp per row, a key at a time per lane straight from global memory, took 48 us at 1 x 128 tokens x 32 heads, 392 at
-// 512 and 4700 at 2 x 1024 x 40 heads; this kernel takes 11, 85 and 670.
+//   One warp per row, a key at a time per lane straight from global memory, took 48 us at 1 x 128 tokens x 32 heads (half of them
+// retained); this kernel takes 11.8, 32 at 300 tokens and 405 at 2 x 1024 x 40 heads (71 % of the shared-memory wavefronts).
 // CTAs with rows start before those expected to have none, over all heads (a quarter to a half of the grid was empty CTAs
 // between the others), and inside a layer step the first chunk is fetched while the selection runs: per pass 1 x 300 x 32
 // heads 63.5 -> 52.4 us, 1 x 700 143 -> 119, 2 x 1000 571 -> 506.

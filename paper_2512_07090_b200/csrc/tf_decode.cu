@@ -13,6 +13,7 @@
 //   is zero (Section 3.2).  The 8 warps take interleaved blocks of 32 keys, each with its own online softmax; the
 //   partial results are merged through shared memory.
 #include <algorithm>
+#include <atomic>
 #include <cooperative_groups.h>
 
 #include "tf_ptx.cuh"
@@ -72,10 +73,10 @@ __global__ void __launch_bounds__(kDecideWarps * 32) decode_decide_kernel(const 
     const bool ema = p.anchor_mode == TF_ANCHOR_EMA, incl = p.anchor_mode == TF_ANCHOR_INCL_MEAN;
     const float a = ema ? p.gamma : 1.f, w = ema ? 1.f - p.gamma : 1.f;
     const long long n_cmp = n0 + (incl ? 1 : 0);            // tokens the anchor covers when it is compared
-    // the controller's state is read now, under the row loads below, not after the block barrier
+    // the controller's state is read, and the threshold adapted, under the row loads below, not after the block barrier
     long long steps = 0, skips = 0;
-    float tau_old = 0.f;
-    if (threadIdx.x == 0) { steps = p.steps[b]; skips = p.skips[b]; tau_old = p.tau[b]; }
+    float tau = 0.f;
+    if (threadIdx.x == 0) { steps = p.steps[b]; skips = p.skips[b]; tau = p.tau[b]; }
     if (p.next_piece && b == 0 && threadIdx.x == 0) *p.next_piece = 0u;   // (drawn from after that kernel's wait for this one)
 
     for (int h0 = warp; h0 < p.Hkv; h0 += kHeadsPerWarp * n_warps) {    // two heads at a time: all of their loads go out together
@@ -94,6 +95,12 @@ __global__ void __launch_bounds__(kDecideWarps * 32) decode_decide_kernel(const 
 #pragma unroll
                 for (int i = 0; i < 4; ++i) { ak4[u][i] = p.sum_k[off + i]; av4[u][i] = p.sum_v[off + i]; }
             }
+        }
+        if (threadIdx.x == 0 && h0 == 0) {
+            // ratio and step in double, the threshold itself is an fp32 state word
+            const double rho = steps > 0 ? (double)skips / (double)steps : 0.0;
+            const double delta = (double)p.eta * (p.alg1_sign ? (p.target - rho) : (rho - p.target));
+            tau += (float)delta;
         }
 #pragma unroll
         for (int u = 0; u < kHeadsPerWarp; ++u) {
@@ -157,10 +164,6 @@ __global__ void __launch_bounds__(kDecideWarps * 32) decode_decide_kernel(const 
             }
             float s = alpha * mk + (1.f - alpha) * mv;
             s += 0.f;
-            // ratio and step in double, the threshold itself is an fp32 state word
-            const double rho = steps > 0 ? (double)skips / (double)steps : 0.0;
-            const double delta = (double)p.eta * (p.alg1_sign ? (p.target - rho) : (rho - p.target));
-            const float tau = tau_old + (float)delta;
             const bool decide = s > tau;              // false for NaN
             const bool skip = decide && t >= p.warmup;
             p.tau[b] = tau;
@@ -782,16 +785,20 @@ static cudaError_t launch_stream(const DecStreamParams& sp, int grid, int device
 }
 
 // ---------------------------------------------------------------------------------------------------
-// Grouped heads, and ungrouped ones in a very short step: one CTA per (split of the visible keys, KV head, sequence), two CTAs
-// per SM.  No list of work to make: a grouped cache is a G-th of the bytes, and the head start of this form outweighs the equal
-// shares of the streaming kernel (us a step, this / streaming: 1 x 8192 16 / 24, 8 x 4096 keys of 16384 31 / 32, 128 x 1024 68 / 80;
-// ungrouped 40 heads: 1 x 8192 44 / 36, 4 x 4096 75 / 60, 128 x 512 112 / 98).  Operands come straight from global memory, no shared
-// memory: a dot product does not care in which order the dims are visited, so lane (g, t) loads 16-byte pieces t, t+4, t+8,
-// t+12 of its two key rows (g, g+8) and of query head g; of its four value rows (2t, 2t+1, 2t+8, 2t+9) it loads dims 16g ..
-// 16g+15, and the pairs "same dim, two consecutive keys" the A operand wants are byte permutes.  The 8 warps take key blocks 8 apart
-// and are merged through shared memory.  The splits of a short step are a thread-block cluster (kCluster): they are merged through
-// distributed shared memory, without scratch and without a third launch; otherwise the CTA leaves (max, sum, unnormalised
-// output) per head in scratch and decode_merge_splits_kernel merges the splits.
+// Grouped heads, and ungrouped ones in a short step: one CTA per (split of the visible keys, KV head, sequence), two CTAs per SM.
+// No list of work to make, and the head start of this form outweighs the equal shares of the streaming kernel: always for grouped
+// heads (whose cache is a G-th of the bytes; us a step, this / streaming with four heads a tile: 1 x 8192 14.6 / 23.3, 8 x 4096
+// 28.6 / 30.3, 64 x 1000 48.6 / 52.7, 128 x 4000 327 / 323), for ungrouped ones as far as launch_decode_step says.  Operands come
+// straight from global memory, no shared memory: a dot product does not care in which order the dims are visited, so lane (g, t)
+// loads 16-byte pieces t, t+4, t+8, t+12 of its two key rows (g, g+8) and of the query head of column g; of its four value rows (2t,
+// 2t+1, 2t+8, 2t+9) it loads dims 16g .. 16g+15, and the pairs "same dim, two consecutive keys" the A operand wants are byte permutes.
+// The 8 warps take key blocks 8 apart and are merged through shared memory.  The splits of a short step are a thread-block cluster
+// (kAsCluster): they are merged through distributed shared memory, without scratch and without a third launch; otherwise the CTA
+// leaves (max, sum, unnormalised output) per head in scratch and decode_merge_splits_kernel merges the splits.
+//   The kernel starts while the decision is made: keys, values, queries and positions are not written by the decision kernel, which
+// lets this one start once all work before it is complete.  A CTA waits for the decision with its first keys in flight (kEarly), a
+// short one of a cluster only when its products are done: one stream of 420 keys 7.9 -> 6.5 us, of 2000 9.6 -> 6.7, 8 x 4096 keys
+// 30.1 -> 28.7.  Letting the kernel after this one start as early made every step slower (1 x 8192 14.7 -> 16.5).
 // ---------------------------------------------------------------------------------------------------
 struct DecGqaParams {
     const __nv_bfloat16* Q; const __nv_bfloat16* K; const __nv_bfloat16* V; __nv_bfloat16* O;
@@ -799,62 +806,84 @@ struct DecGqaParams {
     Strides3 ks, vs;
     const int32_t* pos; const uint8_t* skip;
     int Hq, Hkv, window, n_splits;
+    int n_early;                      // the CTAs that start while the decision kernel runs
     float scale_log2;
     float* partial;                   // [B][Hq][n_splits][130] when n_splits > 1
 };
 
+// loads ahead of the wait go past L1, which may hold what a row held before the kernels that are complete by now
+template <bool kPastL1> __device__ __forceinline__ uint4 load16(const void* p) {
+    return kPastL1 ? __ldcg(reinterpret_cast<const uint4*>(p)) : ldg16(p);
+}
 __device__ __forceinline__ uint32_t word_of(const uint4& r, int w) { return w == 0 ? r.x : w == 1 ? r.y : w == 2 ? r.z : r.w; }
 
-template <int G, bool kCluster>
-__global__ void __launch_bounds__(256, kCluster ? 1 : 2) decode_attention_split_kernel(const DecGqaParams p) {
+// When a CTA waits for the decision: before its first loads, with its first keys' loads in flight, or when its products are done
+enum SplitForm { kAfterDecision, kEarly, kAsCluster };
+
+template <int G, int kForm>
+__global__ void __launch_bounds__(256, kForm == kAsCluster ? 1 : 2) decode_attention_split_kernel(const DecGqaParams p) {
+    constexpr bool kCluster = kForm == kAsCluster;
+    // column 2h of the products is head h, column 2h + 1 what rounding its probabilities to bf16 leaves (as in the streaming kernel); or
+    // column h is head h: eight heads fill them, and with two CTAs per SM grouped heads have no registers left for the remainder (G = 4:
+    // 20 bytes spilled, 32 x 5000 keys x 8 heads 110.8 instead of 103.4 us)
+    constexpr bool kRest = G == 1 || (G <= 4 && kCluster);
+    constexpr int kCols = kRest ? 1 : 2;             // heads of a lane: t, or 2t and 2t + 1
     __shared__ float part_s[8][G][kPartialFloats];
     __shared__ float merge_s[kCluster ? 8 : 1][kCluster ? G : 1][kPartialFloats];   // the splits' results, in the first CTA of a cluster
-    grid_dependency_wait();
     const int split = blockIdx.x, kh = blockIdx.y, b = blockIdx.z;
-    if (p.skip[b]) {
-        if (split == 0 && (kCluster || p.n_splits == 1))
-            for (int i = threadIdx.x; i < G * kHeadDim; i += 256)
-                p.O[(long long)b * p.o_b + (long long)(kh * G + i / kHeadDim) * p.o_h + (i % kHeadDim)] = __float2bfloat16_rn(0.f);
-        return;
-    }
     if constexpr (kCluster) cooperative_groups::this_cluster().barrier_arrive();   // this CTA's shared memory may be written from now on
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int t_pos = p.pos[b];
+    const int t_pos = __ldcg(p.pos + b);
     const int j_lo = (p.window > 0) ? max(0, t_pos - p.window + 1) : 0;
     const int n_vis = t_pos - j_lo + 1;
     const int per = ((n_vis + p.n_splits - 1) / p.n_splits + 15) / 16 * 16;     // keys per split, a multiple of 16
     const int k_lo = j_lo + split * per, k_hi = min(t_pos + 1, k_lo + per);       // [k_lo, k_hi)
     const uint4 zero4 = make_uint4(0, 0, 0, 0);
 
-    // Q^T as the B operand of the 8 score products: head g, pieces t + 4i; product 2i + u takes words 2u, 2u + 1
+    // Q^T as the B operand of the 8 score products: column g, pieces t + 4i; product 2i + u takes words 2u, 2u + 1
     uint32_t qb[8][2];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const uint4 r = (g < G) ? ldg16(p.Q + (long long)b * p.q_b + (long long)(kh * G + g) * p.q_h + 8 * (t + 4 * i)) : zero4;
+        const bool head = kRest ? (g & 1) == 0 && g < 2 * G : g < G;
+        const uint4 r = head ? load16<kForm != kAfterDecision>(p.Q + (long long)b * p.q_b + (long long)(kh * G + (kRest ? g >> 1 : g)) * p.q_h + 8 * (t + 4 * i)) : zero4;
         qb[2 * i][0] = r.x; qb[2 * i][1] = r.y; qb[2 * i + 1][0] = r.z; qb[2 * i + 1][1] = r.w;
     }
     const __nv_bfloat16* Kb = p.K + (long long)b * p.ks.b + (long long)kh * p.ks.h;
     const __nv_bfloat16* Vb = p.V + (long long)b * p.vs.b + (long long)kh * p.vs.h + 16 * g;
 
-    // this lane's part of the state: heads 2t and 2t + 1 (m is the same in all lanes of equal t; l is the lane's share)
-    float m[2] = {-1e30f, -1e30f}, l[2] = {0.f, 0.f};
-    float o[8][4];                                   // O^T: product mt, rows (dims) 16g + mt and 16g + 8 + mt, columns (heads) 2t, 2t + 1
+    // this lane's part of the state (m is the same in all lanes of equal t; l is the lane's share)
+    float m[kCols], l[kCols];
+#pragma unroll
+    for (int c = 0; c < kCols; ++c) { m[c] = -1e30f; l[c] = 0.f; }
+    float o[8][4];                                   // O^T: product mt, rows (dims) 16g + mt and 16g + 8 + mt, columns 2t, 2t + 1
 #pragma unroll
     for (int mt = 0; mt < 8; ++mt) { o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f; }
 
-    for (int kb = k_lo + 16 * warp; kb < k_hi; kb += 16 * 8) {       // warp-uniform bounds: the shuffles below name all lanes
+    bool decided = false, skipped = false;
+    auto decision = [&]() {
+        grid_dependency_wait();
+        decided = true;
+        skipped = __ldcg(p.skip + b) != 0;
+    };
+    // (the CTAs of a later wave start after the decision: theirs costs nothing to know, and may save them their loads)
+    if (kForm == kAfterDecision || (kForm == kEarly && split + p.n_splits * (kh + p.Hkv * b) >= p.n_early)) decision();
+    for (int kb = k_lo + 16 * warp; kb < k_hi && !skipped; kb += 16 * 8) {       // warp-uniform bounds: the shuffles below name all lanes
         uint4 kr[2][4], vr[4][2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int j = kb + g + 8 * h;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) kr[h][i] = (j < k_hi) ? ldg16(Kb + (long long)j * p.ks.t + 8 * (t + 4 * i)) : zero4;
+            for (int i = 0; i < 4; ++i) kr[h][i] = (j < k_hi) ? load16<kForm != kAfterDecision>(Kb + (long long)j * p.ks.t + 8 * (t + 4 * i)) : zero4;
         }
 #pragma unroll
         for (int q4 = 0; q4 < 4; ++q4) {
             const int j = kb + 2 * t + (q4 & 1) + 8 * (q4 >> 1);
 #pragma unroll
-            for (int i = 0; i < 2; ++i) vr[q4][i] = (j < k_hi) ? ldg16(Vb + (long long)j * p.vs.t + 8 * i) : zero4;
+            for (int i = 0; i < 2; ++i) vr[q4][i] = (j < k_hi) ? load16<kForm != kAfterDecision>(Vb + (long long)j * p.vs.t + 8 * i) : zero4;
+        }
+        if (kForm == kEarly && !decided) {
+            decision();
+            if (skipped) break;
         }
         // ---- scores: rows = keys g, g + 8; columns = heads 2t, 2t + 1 -----------------------------------------
         float s[4] = {0.f, 0.f, 0.f, 0.f};
@@ -864,28 +893,34 @@ __global__ void __launch_bounds__(256, kCluster ? 1 : 2) decode_attention_split_
             mma_bf16_16816(s, kr[0][i].z, kr[1][i].z, kr[0][i].w, kr[1][i].w, qb[2 * i + 1][0], qb[2 * i + 1][1]);
         }
         const bool v0 = kb + g < k_hi, v1 = kb + g + 8 < k_hi;
-        s[0] = v0 ? s[0] * p.scale_log2 : -1e30f; s[1] = v0 ? s[1] * p.scale_log2 : -1e30f;
-        s[2] = v1 ? s[2] * p.scale_log2 : -1e30f; s[3] = v1 ? s[3] * p.scale_log2 : -1e30f;
-        float corr[2], pr[4];
+        float corr[kCols], pr[2 * kCols];
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            float mx = fmaxf(s[c], s[c + 2]);
+        for (int c = 0; c < kCols; ++c) {
+            const float sa = v0 ? s[c] * p.scale_log2 : -1e30f, sb = v1 ? s[c + 2] * p.scale_log2 : -1e30f;
+            float mx = fmaxf(sa, sb);
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
             const float mn = fmaxf(m[c], mx);
             corr[c] = ex2_approx(m[c] - mn);
             m[c] = mn;
-            pr[c] = v0 ? ex2_approx(s[c] - mn) : 0.f;
-            pr[c + 2] = v1 ? ex2_approx(s[c + 2] - mn) : 0.f;
-            l[c] = fmaf(l[c], corr[c], pr[c] + pr[c + 2]);
+            pr[c] = v0 ? ex2_approx(sa - mn) : 0.f;
+            pr[c + kCols] = v1 ? ex2_approx(sb - mn) : 0.f;
+            l[c] = fmaf(l[c], corr[c], pr[c] + pr[c + kCols]);
         }
-        // P^T (keys x heads) -> the B operand wants head g with keys 2t, 2t+1 / 2t+8, 2t+9: two 8x8 transposes
-        const uint32_t pb0 = transpose8x8_b16(pack_bf16x2(pr[0], pr[1]));
-        const uint32_t pb1 = transpose8x8_b16(pack_bf16x2(pr[2], pr[3]));
+        // P^T (keys x columns) -> the B operand wants column g with keys 2t, 2t+1 / 2t+8, 2t+9: two 8x8 transposes
+        uint32_t pb0, pb1;
+        if constexpr (kRest) {
+            const float ha = __bfloat162float(__float2bfloat16_rn(pr[0])), hb = __bfloat162float(__float2bfloat16_rn(pr[1]));
+            pb0 = transpose8x8_b16(pack_bf16x2(ha, pr[0] - ha));
+            pb1 = transpose8x8_b16(pack_bf16x2(hb, pr[1] - hb));
+        } else {
+            pb0 = transpose8x8_b16(pack_bf16x2(pr[0], pr[1]));
+            pb1 = transpose8x8_b16(pack_bf16x2(pr[2], pr[3]));
+        }
 #pragma unroll
         for (int mt = 0; mt < 8; ++mt) {
-            o[mt][0] *= corr[0]; o[mt][1] *= corr[1]; o[mt][2] *= corr[0]; o[mt][3] *= corr[1];
+            o[mt][0] *= corr[0]; o[mt][1] *= corr[kCols - 1]; o[mt][2] *= corr[0]; o[mt][3] *= corr[kCols - 1];
             const int w = mt >> 1;
             const uint32_t sel = (mt & 1) ? 0x7632u : 0x5410u;     // the high / low halves of two rows' words
             const uint32_t a0 = __byte_perm(word_of(vr[0][0], w), word_of(vr[1][0], w), sel);   // dim 16g + mt,     keys 2t, 2t+1
@@ -895,21 +930,29 @@ __global__ void __launch_bounds__(256, kCluster ? 1 : 2) decode_attention_split_
             mma_bf16_16816(o[mt], a0, a1, a2, a3, pb0, pb1);
         }
     }
+    if (!decided) decision();
+    if (skipped) {                                   // the whole cluster (it has one sequence)
+        if (split == 0 && (kCluster || p.n_splits == 1))
+            for (int i = threadIdx.x; i < G * kHeadDim; i += 256)
+                p.O[(long long)b * p.o_b + (long long)(kh * G + i / kHeadDim) * p.o_h + (i % kHeadDim)] = __float2bfloat16_rn(0.f);
+        if constexpr (kCluster) cooperative_groups::this_cluster().barrier_wait();
+        return;
+    }
     // ---- the lane's share of l -> the sum over the 8 lanes of equal t; then everything into shared memory ---------
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
+    for (int c = 0; c < kCols; ++c) {
         l[c] += __shfl_xor_sync(0xffffffffu, l[c], 4);
         l[c] += __shfl_xor_sync(0xffffffffu, l[c], 8);
         l[c] += __shfl_xor_sync(0xffffffffu, l[c], 16);
     }
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        const int h = 2 * t + c;
+    for (int c = 0; c < kCols; ++c) {
+        const int h = kCols * t + c;
         if (h < G) {
 #pragma unroll
             for (int mt = 0; mt < 8; ++mt) {
-                part_s[warp][h][16 * g + mt] = o[mt][c];
-                part_s[warp][h][16 * g + 8 + mt] = o[mt][c + 2];
+                part_s[warp][h][16 * g + mt] = kRest ? o[mt][0] + o[mt][1] : o[mt][c];
+                part_s[warp][h][16 * g + 8 + mt] = kRest ? o[mt][2] + o[mt][3] : o[mt][c + 2];
             }
             if (g == 0) { part_s[warp][h][kHeadDim] = m[c]; part_s[warp][h][kHeadDim + 1] = l[c]; }
         }
@@ -987,18 +1030,42 @@ __global__ void __launch_bounds__(kHeadDim) decode_merge_splits_kernel(const Dec
     *out = skip ? __float2bfloat16_rn(0.f) : __float2bfloat16_rn(acc / L);
 }
 
-template <int G>
-static cudaError_t launch_split(const DecGqaParams& gp, dim3 grid, bool cluster, cudaStream_t st) {
-    if (!cluster) return launch_dependent(decode_attention_split_kernel<G, false>, grid, dim3(256), 0, st, gp);
+// the launch of a grid of clusters of grid.x CTAs (attr: two entries that outlive the call)
+static cudaLaunchConfig_t cluster_config(dim3 grid, cudaStream_t st, cudaLaunchAttribute* attr) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = 0; cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = grid.x; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = grid.x; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, decode_attention_split_kernel<G, true>, gp);
+    return cfg;
+}
+template <int G>
+static cudaError_t launch_split(const DecGqaParams& gp, dim3 grid, bool cluster, bool early, cudaStream_t st) {
+    if (G > 4 || !cluster) return launch_dependent(early ? decode_attention_split_kernel<G, kEarly> : decode_attention_split_kernel<G, kAfterDecision>, grid, dim3(256), 0, st, gp);
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = cluster_config(grid, st, attr);
+    return cudaLaunchKernelEx(&cfg, decode_attention_split_kernel<(G > 4 ? 4 : G), kAsCluster>, gp);
+}
+// how many clusters of n CTAs (2 .. 8) the device runs at once: a property of the device and the kernel, asked for once
+static int max_clusters(int device, int G, int n) {
+    static std::atomic<int> known[kDeviceFlagSlots][3][9] = {};      // + 1; 0: not asked yet
+    std::atomic<int>& k = known[device >= 0 && device < kDeviceFlagSlots ? device : 0][G >> 1][n];
+    int v = k.load(std::memory_order_relaxed);
+    if (v == 0) {
+        cudaLaunchAttribute attr[2];
+        cudaLaunchConfig_t cfg = cluster_config(dim3((unsigned)n), nullptr, attr);
+        cfg.numAttrs = 1;
+        int most = 0;
+        const cudaError_t e = G == 1 ? cudaOccupancyMaxActiveClusters(&most, decode_attention_split_kernel<1, kAsCluster>, &cfg)
+                            : G == 2 ? cudaOccupancyMaxActiveClusters(&most, decode_attention_split_kernel<2, kAsCluster>, &cfg)
+                                     : cudaOccupancyMaxActiveClusters(&most, decode_attention_split_kernel<4, kAsCluster>, &cfg);
+        if (e != cudaSuccess) { (void)cudaGetLastError(); most = 0; }
+        v = most + 1;
+        k.store(v, std::memory_order_relaxed);
+    }
+    return v - 1;
 }
 
 // The scratch of a step lies at the END of the bound workspace, the records that a scan keeps from call to call at the front: a
@@ -1009,6 +1076,30 @@ static char* step_scratch(tf_ctx* ctx, size_t bytes) {
     const size_t at = (ctx->workspace_bytes - bytes) & ~(size_t)255;
     if (at < (ctx->scan_user.bytes & ~(size_t)1)) ctx->scan_user.needs_clear = true;      // (the low bit is not part of the extent)
     return static_cast<char*>(ctx->workspace) + at;
+}
+
+// How the split kernel divides the visible keys of a (sequence, KV head), at least 256 keys each.  Through scratch: two CTAs fit an
+// SM, a wave of CTAs costs (a fixed part worth ~192 keys + its keys), and a partly filled wave costs as much as a full one; the
+// cheapest estimate.  As a cluster, of as many splits (8 at most, as short as 64 keys) as let the clusters of all groups run at
+// once: no third launch, which is worth ~400 keys of a CTA (us a step, cluster / scratch, 8 KV heads: 1 x 420 keys 6.5 / 7.5, 4 x 500
+// 6.6 / 7.7, 8 x 420 7.3 / 8.9, 4 x 1500 8.8 / 10.5, 1 x 4096 9.2 / 10.3; 8 x 2000 19.6 / 18.6, 4 x 4096 19.7 / 18.7, 1 x 8192
+// 16.9 / 14.5), up to 2048 keys: the check that a step through scratch leaves the scan's records alone makes one of 2304.  Clusters
+// that wait for one another's SMs lose: 2 x 420 keys in 6 splits 6.9, in 7 9.9.
+struct SplitPlan { int n; bool cluster; };
+static size_t split_bytes(const tf_shape& s) { return (size_t)s.batch * s.n_q_heads * kPartialFloats * sizeof(float); }     // of one split
+static SplitPlan split_plan(const tf_ctx* ctx, const tf_shape& s, int G, int max_keys, int sms) {
+    const long long groups = (long long)s.batch * s.n_kv_heads, slots = 2ll * sms;
+    SplitPlan plan{1, false};
+    long long best = -1, keys_at_once = 0;                  // (of a CTA of every wave)
+    for (int n = 1; n <= std::max(1, max_keys / 256); ++n) {
+        if (n > 1 && (!ctx->workspace || ctx->workspace_bytes < split_bytes(s) * n)) break;
+        const long long waves = (groups * n + slots - 1) / slots, keys = (max_keys + n - 1) / n, cost = waves * (192 + keys);
+        if (best < 0 || cost < best) { best = cost; plan.n = n; keys_at_once = waves * keys; }
+    }
+    int n = G <= 4 && max_keys <= 2048 ? (int)std::min<long long>(std::min(8, max_keys / 64), sms / groups) : 1;
+    while (n > 1 && groups > max_clusters(ctx->device, G, n)) --n;
+    if (n > 1 && (max_keys + n - 1) / n <= keys_at_once + (plan.n > 1 ? 400 : 0)) plan = {n, true};
+    return plan;
 }
 
 cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_params& p, const tf_decode_args& a,
@@ -1041,16 +1132,20 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
                     && make_bshd_map(&maps.v[x], V, s.v_stride, n, s.seq, s.n_kv_heads, 2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 64, 16 * (x + 1), CU_TENSOR_MAP_SWIZZLE_128B);
         return ok;
     };
-    // ... but not where all CTAs of the split kernel run at once and have at most four tiles each: the streaming kernel's list
-    // and hand-overs are not paid back then (us a step of full caches, split / streaming: 5 x 128 x 32 heads 10.5 / 12.6,
-    // 7 x 256 x 40 17.5 / 18.4, 7 x 320 x 40 19.4 / 18.8, 8 x 256 x 40, a second wave, 22.1 / 18.9, 32 x 256 x 8 15.1 / 17.9,
-    // 100 x 192 x 2 13.0 / 19.0); nor with one or two tiles in several launches (600 x 64 x 8 64.3 / 69.0)
+    // ... but not for short steps, where the streaming kernel's list and hand-overs are not paid back: up to 18 tiles of 64 keys
+    // per SM, 34 where the split kernel's CTAs fill one or two waves well; nor with one or two tiles in several launches (us a step of
+    // full caches, streaming / split: 1 x 1000 x 40 heads 14.4 / 8.0, 16 x 128 x 32 17.5 / 12.8, 40 x 128 x 32 (17 tiles) 27.5 / 27.6,
+    // 24 x 250 x 32 (21, three waves) 27.5 / 27.8, 12 x 600 x 32 (26, one and a third) 29.6 / 33.2, 16 x 400 x 32 (24) 28.0 / 25.9,
+    // 16 x 600 x 32 (35) 35.1 / 32.4, 1 x 8000 x 40 (34) 35.4 / 33.8, 2 x 4000 x 40 (34) 34.0 / 34.6, 24 x 400 x 32 (36) 35.7 / 37.6; 600 x 64 x 8
+    // 69.0 / 64.3)
     const long long items = (long long)s.batch * s.n_kv_heads;
-    const bool few_short = (items <= 2 * sms && max_keys <= 4 * kStreamKeys) || (s.batch > kStreamMaxBatch && max_keys <= 2 * kStreamKeys);
-    const bool stream = grouped && G == 1 && !few_short && 2 * tiles_max > sms && tiles_max < (1ll << 31) &&              // (tile numbers are 32 bits)
+    const SplitPlan plan = grouped ? split_plan(ctx, s, G, max_keys, sms) : SplitPlan{1, false};
+    const long long split_ctas = items * plan.n, waves = (split_ctas + 2 * sms - 1) / (2 * sms);
+    const bool filled = waves <= 2 && 5 * split_ctas >= 4 * waves * 2 * sms;
+    const bool few_short = tiles_max <= (filled ? 34ll : 18ll) * sms || (s.batch > kStreamMaxBatch && max_keys <= 2 * kStreamKeys);
+    const bool stream = grouped && G == 1 && !few_short && tiles_max < (1ll << 31) &&              // (tile numbers are 32 bits)
                         ((s.o_stride[0] | s.o_stride[2]) % 8) == 0 && (reinterpret_cast<uintptr_t>(a.O_new) & 15u) == 0 &&
                         (s.batch == 1 || (s.k_stride[0] > 0 && s.v_stride[0] > 0)) && make_maps(0, std::min<int>(s.batch, kStreamMaxBatch));
-    dp.early = stream ? 1 : 0;
     // scratch of the streaming kernel: the table of begun work items, then slots: two per piece, and there have to be more
     // pieces than CTAs
     DecStreamParams sp{};
@@ -1068,6 +1163,9 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
     dp.tau = a.state->tau; dp.steps = reinterpret_cast<long long*>(a.state->steps);
     dp.skips = reinterpret_cast<long long*>(a.state->skips);
     dp.score_out = a.score_out; dp.skip_out = a.skip_out; dp.status = ctx->dev_status;
+    // The attention starts while the decisions are made where that is worth it: what it loads for skipped tokens is lost, and with
+    // many waves little is gained (128 x 1024 keys x 8 heads, half of them skipped, 54.8 instead of 51.1 us)
+    dp.early = stream || (grouped && waves <= 2) ? 1 : 0;
     const size_t smem = 2 * (size_t)s.n_kv_heads * sizeof(float);
     cudaError_t e;
     // up to 8 heads a warp has one, beyond it two (two for 8: 1 x 100 keys x 8 heads fp32 15.3 us a step)
@@ -1093,35 +1191,16 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
         gp.q_b = ap.q_b; gp.q_h = ap.q_h; gp.o_b = ap.o_b; gp.o_h = ap.o_h;
         gp.ks = ap.ks; gp.vs = ap.vs; gp.pos = a.pos; gp.skip = a.skip_out;
         gp.Hq = s.n_q_heads; gp.Hkv = s.n_kv_heads; gp.window = s.window; gp.scale_log2 = ap.scale_log2;
-        // Number of key splits: two CTAs fit an SM, a wave of CTAs costs (a fixed part worth ~192 keys + its keys), and a
-        // partly filled wave costs as much as a full one; take the split count with the cheapest estimate, at least
-        // 256 keys per split.
-        // Few work items: the splits, as short as 64 keys, are a cluster and need no third launch (us a step, cluster / scratch: 1 x
-        // 420 keys x 8 heads 7.85 / 8.97, 1 x 500 x 10 7.9 / 10.3, 4 x 500 x 3 7.9 / 9.15; clusters of more groups wait for one another's slots: 2 x 420 x 8
-        // 10.7 / 9.1, 4 x 500 x 4 10.7 / 9.4, 3 x 500 x 8 11.4 / 9.3, 4 x 1000 x 8 18.8 / 12.8).
-        const long long groups = (long long)s.batch * s.n_kv_heads, slots = 2ll * sms;
-        const bool few = 12 * groups <= sms && G <= 4;
-        int n_splits = 1;
-        const size_t per_split = (size_t)s.batch * s.n_q_heads * kPartialFloats * sizeof(float);
-        {
-            const int most = std::max(few ? std::min(8, max_keys / 64) : 1, max_keys / 256);
-            long long best = -1;
-            for (int n = 1; n <= std::max(1, most); ++n) {
-                if ((n > 8 || (n > 1 && !few)) && (!ctx->workspace || ctx->workspace_bytes < per_split * n)) break;
-                const long long waves = (groups * n + slots - 1) / slots;
-                const long long cost = waves * (192 + (max_keys + n - 1) / n);
-                if (best < 0 || cost < best) { best = cost; n_splits = n; }
-            }
-        }
-        gp.n_splits = n_splits;
-        const bool cluster = few && n_splits > 1 && n_splits <= 8, scratch = n_splits > 1 && !cluster;
-        gp.partial = scratch ? reinterpret_cast<float*>(step_scratch(ctx, per_split * n_splits)) : nullptr;
-        const dim3 grid((unsigned)n_splits, (unsigned)s.n_kv_heads, (unsigned)s.batch);
+        gp.n_splits = plan.n;
+        gp.n_early = 2 * sms;
+        const bool scratch = plan.n > 1 && !plan.cluster;
+        gp.partial = scratch ? reinterpret_cast<float*>(step_scratch(ctx, split_bytes(s) * plan.n)) : nullptr;
+        const dim3 grid((unsigned)plan.n, (unsigned)s.n_kv_heads, (unsigned)s.batch);
         switch (G) {
-            case 1: e = launch_split<1>(gp, grid, cluster, st); break;
-            case 2: e = launch_split<2>(gp, grid, cluster, st); break;
-            case 4: e = launch_split<4>(gp, grid, cluster, st); break;
-            default: e = launch_dependent(decode_attention_split_kernel<8, false>, grid, dim3(256), 0, st, gp); break;
+            case 1: e = launch_split<1>(gp, grid, plan.cluster, dp.early != 0, st); break;
+            case 2: e = launch_split<2>(gp, grid, plan.cluster, dp.early != 0, st); break;
+            case 4: e = launch_split<4>(gp, grid, plan.cluster, dp.early != 0, st); break;
+            default: e = launch_split<8>(gp, grid, false, dp.early != 0, st); break;
         }
         ctx->launches += 1;
         if (e == cudaSuccess && scratch) {

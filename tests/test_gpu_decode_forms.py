@@ -1,6 +1,10 @@
 """Decode steps at the sizes where one form of the attention gives way to another, against fp64 softmax attention."""
+import numpy as np
 import pytest
+import torch
 
+from paper_2512_07090_b200 import binding as tfb
+from test_gpu_parity import ATTN_TOL, DEV, _qkv, attn_rel_err, to_np
 from test_gpu_parity import test_decode_attention_uneven_positions_and_skips as _uneven_positions_and_skips
 
 pytestmark = pytest.mark.gpu
@@ -8,6 +12,86 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("workspace", [True, False])
 @pytest.mark.parametrize("B,S,Hkv,G,window", [
+    (8, 420, 8, 4, 0), (4, 777, 8, 4, 0), (1, 300, 40, 1, 0), (2, 512, 8, 4, 100), (3, 129, 10, 2, 0),   # clusters of 2 to 8 splits
+    (1, 2048, 4, 2, 0), (1, 2049, 4, 2, 0),                       # the longest as a cluster, the shortest through scratch
+    (18, 600, 8, 4, 0), (70, 300, 8, 4, 0), (80, 300, 8, 4, 0),   # one wave, two (the attention starts early), three (it does not)
+    (20, 300, 8, 8, 0),                                           # eight heads a group
     (6, 30000, 4, 1, 0), (300, 200, 8, 1, 0)])                    # streaming: pieces of work items, whole ones; last tiles of 1 to 64 keys
 def test_decode_attention_forms(B, S, Hkv, G, window, workspace):
     _uneven_positions_and_skips(B, S, Hkv, G, window, workspace)
+
+
+def _step(B, S, Hkv, G, seed):
+    q, k, v = _qkv(B, S, Hkv * G, Hkv, torch.bfloat16, seed=seed)
+    qn = q[:, -1].contiguous()
+    shape = tfb.make_shape(None, k, v, n_q_heads=Hkv * G)
+    shape.q_stride[:] = [qn.stride(0), 0, qn.stride(1)]
+    shape.o_stride[:] = list(shape.q_stride)
+    params = tfb.default_params(prune_ratio=0.5, warmup_tokens=0)
+    ctx = tfb.Context(0)
+    st = tfb.DecodeState(B, Hkv, DEV)
+    st.tau.fill_(9.0)
+    return ctx, shape, params, qn, k, v, st, torch.empty_like(qn), torch.empty(B, dtype=torch.uint8, device=DEV)
+
+
+def _exact(qn, k, v, b, n):
+    Hkv = k.shape[2]
+    s = torch.einsum("hgd,nhd->hgn", qn[b].double().view(Hkv, -1, 128), k[b, :n].double()) / 128 ** 0.5
+    return torch.einsum("hgn,nhd->hgd", s.softmax(-1), v[b, :n].double()).reshape(-1, 128)
+
+
+@pytest.mark.parametrize("B,S,Hkv,G,launches", [(1, 1000, 8, 4, 2), (1, 600, 40, 1, 2), (3, 500, 6, 2, 2), (1, 4000, 40, 1, 3), (16, 500, 32, 1, 2)])
+def test_split_decode_loses_nothing_before_the_result_is_rounded(B, S, Hkv, G, launches):
+    """The error against 64 bits is that of rounding the exact result to bf16 (to 2 %): clusters of every group size, ungrouped
+    heads through scratch and unsplit."""
+    ctx, shape, params, qn, k, v, st, O, skip = _step(B, S, Hkv, G, seed=S)
+    ctx.ensure_workspace(shape, params)
+    n0 = ctx.launches
+    ctx.tf_decode_step(shape, params, 0.0, qn, k, v, torch.full((B,), S - 1, dtype=torch.int32, device=DEV), st, O, None, skip)
+    assert ctx.launches - n0 == launches
+    assert ctx.tf_get_status()[0] == tfb.TF_OK
+    err = rounding = 0.0
+    for b in range(B):
+        ref = _exact(qn, k, v, b, S)
+        err += float((O[b].double() - ref).square().sum())
+        rounding += float((ref.bfloat16().double() - ref).square().sum())
+    assert err < 1.02 ** 2 * rounding, (err ** 0.5, rounding ** 0.5)
+    ctx.close()
+
+
+@pytest.mark.parametrize("fill", [0x00, 0xff])
+def test_long_streaming_step_whose_waits_run_out_leaves_a_usable_context(fill):
+    """As for a shorter one in test_gpu_parity.py, at a size that the streaming kernel takes."""
+    B, S, Hkv = 3, 30000, 8
+    ctx, shape, params, qn, k, v, st, O, skip = _step(B, S, Hkv, 1, seed=5)
+    ctx.set_workspace(torch.full((ctx.workspace_bytes(shape, params),), fill, dtype=torch.uint8, device=DEV))
+    pos = torch.tensor([S - 1, 1700, 63], dtype=torch.int32, device=DEV)
+    ctx.tf_set_wait_limits(wait_cycles=0)
+    ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
+    assert ctx.tf_get_status()[0] in (tfb.TF_OK, tfb.TF_ERR_TIMEOUT)
+    ctx.tf_set_wait_limits()
+    ctx.tf_clear_status()
+    for _ in range(2):
+        O.fill_(float("nan"))
+        ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
+        assert ctx.tf_get_status()[0] == tfb.TF_OK
+        for b in range(B):
+            assert attn_rel_err(to_np(O[b]), _exact(qn, k, v, b, int(pos[b]) + 1).cpu().numpy()) < ATTN_TOL[torch.bfloat16], b
+    ctx.close()
+
+
+def test_long_streaming_steps_in_which_every_sequence_is_skipped():
+    """As for a shorter one in test_gpu_parity.py: tiles fetched in vain, then a right step."""
+    B, S, Hkv = 6, 30000, 4
+    ctx, shape, params, qn, k, v, st, O, skip = _step(B, S, Hkv, 1, seed=7)
+    ctx.ensure_workspace(shape, params)
+    pos = torch.full((B,), S - 1, dtype=torch.int32, device=DEV)
+    for tau in (-9.0, 9.0, -9.0):
+        st.tau.fill_(tau)
+        O.fill_(float("nan"))
+        ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
+        assert ctx.tf_get_status()[0] == tfb.TF_OK
+        for b in range(B):
+            ref = np.zeros((Hkv, 128)) if tau < 0 else _exact(qn, k, v, b, S).cpu().numpy()
+            assert np.all(to_np(O[b]) == 0) if tau < 0 else attn_rel_err(to_np(O[b]), ref) < ATTN_TOL[torch.bfloat16], b
+    ctx.close()

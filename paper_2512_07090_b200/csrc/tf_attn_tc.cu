@@ -131,16 +131,16 @@ __device__ __forceinline__ void softmax_tile(uint32_t tm_s, uint32_t tm_o, int l
     tmem_wait_ld();
     const bool full = (j0 >= lo) && (j0 + kTileN - 1 <= hi);
     if (!full) {   // columns below c_lo or above c_hi are invisible to this row: -inf
+        // One bit per column, both bounds at once: a select on a bit of a word is one instruction beside the moves of bits to
+        // predicates, and rows cut at either end take the same path (three variants with two compares a column before: 2048 tokens
+        // 61.2 -> 60.1 us per pass, 4 x 4096 x 40 heads 521 -> 513, 2 x 8192 grouped 578 -> 573, 8 x 16384 windowed 3939 -> 3917)
         const int c_lo = lo - j0, c_hi = hi - j0;
-        if (c_lo <= 0) {
 #pragma unroll
-            for (int c = 0; c < 128; ++c) if (c > c_hi) sreg[c] = 0xff800000u;
-        } else if (c_hi >= kTileN - 1) {
+        for (int w = 0; w < 4; ++w) {
+            const int up = min(max(c_hi - 32 * w + 1, 0), 32), dn = min(max(c_lo - 32 * w, 0), 32);
+            const uint32_t vis = (uint32_t)((1ull << up) - 1ull) & ~(uint32_t)((1ull << dn) - 1ull);
 #pragma unroll
-            for (int c = 0; c < 128; ++c) if (c < c_lo) sreg[c] = 0xff800000u;
-        } else {
-#pragma unroll
-            for (int c = 0; c < 128; ++c) if (c < c_lo || c > c_hi) sreg[c] = 0xff800000u;
+            for (int e = 0; e < 32; ++e) sreg[32 * w + e] = (vis & (1u << e)) ? sreg[32 * w + e] : 0xff800000u;
         }
     }
     float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};   // four chains, not one of 128

@@ -87,6 +87,14 @@ __device__ __forceinline__ void work_item(const TcParams& p, unsigned int item, 
     bh = g * p.bh_group + within % g_size;
 }
 
+// The key that the first K/V tile of an item starts at, k_first being the first that any of its rows sees.  Under a window tiles
+// start there, not at a multiple of their length: a window of 4096 and rows that span 127 positions then take 33 or 34 tiles instead of
+// always 34, one of them cut by the window's start instead of two (per pass: 8 x 16384 grouped 3917 -> 3862 us, 1 x 20000 x 32 heads 3 %
+// with the masks).  Compacted keys are only defined up to a multiple of the tile.
+__device__ __forceinline__ int first_tile_key(const TcParams& p, int k_first) {
+    return p.window <= 0 ? 0 : p.compact ? k_first / kTileN * kTileN : k_first;
+}
+
 // bounded wait; after the first expiry in this CTA nobody waits any more
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long budget_cycles,
                                           DevStatus* status, unsigned long long where) {
@@ -232,6 +240,7 @@ constexpr int kClaimLead = 2;
 struct TcItem {
     int valid;            // 0: there is no further item
     int b, qh, slot0, nk;
+    int k0;               // K/V tile j holds keys k0 + 128 j ..
     int jb[2], je[2];     // K/V tiles jb .. je - 1 of each Q tile
 };
 
@@ -352,7 +361,7 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
                     k1[1] = e0 + kTileM + 32 + lane < nk ? kept[e0 + kTileM + 32 + lane] : -1;
                 }
                 TcItem d;
-                d.valid = 1; d.b = b; d.qh = qh; d.slot0 = slot0; d.nk = nk;
+                d.valid = 1; d.b = b; d.qh = qh; d.slot0 = slot0; d.nk = nk; d.k0 = 0;
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {     // which K/V tiles each Q tile needs
                     const int s_lo = slot0 + (kHeads ? 0 : i * kTileM);
@@ -366,8 +375,9 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
                             k_first = p.window > 0 ? first_kept_at_or_after(kept, s_lo + 1, k_first) : 0;
                             k_last = s_last;
                         }
-                        d.jb[i] = k_first / kTileN;
-                        d.je[i] = k_last / kTileN + 1;
+                        if (i == 0) d.k0 = first_tile_key(p, k_first);
+                        d.jb[i] = (k_first - d.k0) / kTileN;
+                        d.je[i] = (k_last - d.k0) / kTileN + 1;
                     }
                 }
                 // the slot of tile 0, the descriptor and the row positions are those of item n - 2
@@ -476,8 +486,8 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
                         const uint32_t dst = sbase + kPOffRing + st * kTileBytes;
                         const CUtensorMap* map = kv ? &mapV : &mapK;
                         mbar_expect_tx(bar_full + 8 * st, kTileBytes);
-                        tma_load_4d(dst, map, bar_full + 8 * st, 0, kh, j * kTileN, it.b);
-                        tma_load_4d(dst + kHalfBytes, map, bar_full + 8 * st, 64, kh, j * kTileN, it.b);
+                        tma_load_4d(dst, map, bar_full + 8 * st, 0, kh, it.k0 + j * kTileN, it.b);
+                        tma_load_4d(dst + kHalfBytes, map, bar_full + 8 * st, 64, kh, it.k0 + j * kTileN, it.b);
                     }
                     if (j == max(J1 - 1 - kClaimLead, it.jb[0])) mbar_arrive(bar_asked + 8 * (n & 1));
                 }
@@ -596,7 +606,7 @@ attention_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap mapK, 
                 mbar_wait(bar_s + 8 * i, tiles & 1, abort_flag, p.wait_cycles, p.status, 30 + i);
                 __syncwarp();
                 tc_fence_after();
-                softmax_tile(tm_s, tm_o, lo, hi, j * kTileN, p.scale_log2, j > jb, m_ref, l_run);
+                softmax_tile(tm_s, tm_o, lo, hi, it.k0 + j * kTileN, p.scale_log2, j > jb, m_ref, l_run);
                 tmem_wait_st();
                 tc_fence_before();
                 mbar_arrive(bar_p + 8 * i);
@@ -742,7 +752,8 @@ attention_tc_split_kernel(const TcParams p, const __grid_constant__ CUtensorMap 
         k_first = p.window > 0 ? first_kept_at_or_after(kept, slot0 + 1, k_first) : 0;
         k_last = s_last;
     }
-    const int J0 = k_first / kTileN, J1 = k_last / kTileN + 1;
+    const int k0 = first_tile_key(p, k_first);
+    const int J0 = (k_first - k0) / kTileN, J1 = (k_last - k0) / kTileN + 1;
     const int jb[2] = {J0, J0 + 1};
     const int kh = qh / (p.Hq / p.Hkv);
 
@@ -782,8 +793,8 @@ attention_tc_split_kernel(const TcParams p, const __grid_constant__ CUtensorMap 
                     const uint32_t dst = sbase + kOffRing + st * kTileBytes;
                     const CUtensorMap* map = kv ? &mapV : &mapK;
                     mbar_expect_tx(bar_full + 8 * st, kTileBytes);
-                    tma_load_4d(dst, map, bar_full + 8 * st, 0, kh, j * kTileN, b);
-                    tma_load_4d(dst + kHalfBytes, map, bar_full + 8 * st, 64, kh, j * kTileN, b);
+                    tma_load_4d(dst, map, bar_full + 8 * st, 0, kh, k0 + j * kTileN, b);
+                    tma_load_4d(dst + kHalfBytes, map, bar_full + 8 * st, 64, kh, k0 + j * kTileN, b);
                 }
             }
         }
@@ -870,7 +881,7 @@ attention_tc_split_kernel(const TcParams p, const __grid_constant__ CUtensorMap 
         float m_ref = -INFINITY, l_run = 0.f;
         for (int j = jb[i]; j < J1; j += kStep) {
             const int c_it = (j - jb[i]) / kStep;
-            const int j0 = j * kTileN;
+            const int j0 = k0 + j * kTileN;
             mbar_wait(bar_s + 8 * i, c_it & 1, abort_flag, p.wait_cycles, p.status, 30 + i);
             __syncwarp();
             tc_fence_after();

@@ -791,7 +791,7 @@ static cudaError_t launch_stream(const DecStreamParams& sp, int grid, int device
 // 28.6 / 30.3, 64 x 1000 48.6 / 52.7, 128 x 4000 327 / 323), for ungrouped ones as far as launch_decode_step says.  Operands come
 // straight from global memory, no shared memory: a dot product does not care in which order the dims are visited, so lane (g, t)
 // loads 16-byte pieces t, t+4, t+8, t+12 of its two key rows (g, g+8) and of the query head of column g; of its four value rows (2t,
-// 2t+1, 2t+8, 2t+9) it loads dims 16g .. 16g+15, and the pairs "same dim, two consecutive keys" the A operand wants are byte permutes.
+// 2t+1, 2t+8, 2t+9) it loads 16 dims, and the pairs "same dim, two consecutive keys" the A operand wants are byte permutes.
 // The 8 warps take key blocks 8 apart and are merged through shared memory.  The splits of a short step are a thread-block cluster
 // (kAsCluster): they are merged through distributed shared memory, without scratch and without a third launch; otherwise the CTA
 // leaves (max, sum, unnormalised output) per head in scratch and decode_merge_splits_kernel merges the splits.
@@ -828,6 +828,11 @@ __global__ void __launch_bounds__(256, kForm == kAsCluster ? 1 : 2) decode_atten
     // 20 bytes spilled, 32 x 5000 keys x 8 heads 110.8 instead of 103.4 us)
     constexpr bool kRest = G == 1 || (G <= 4 && kCluster);
     constexpr int kCols = kRest ? 1 : 2;             // heads of a lane: t, or 2t and 2t + 1
+    // dims of a lane's value rows: 16g .. 16g + 15, or 8g .. and 64 + 8g .., where a load instruction takes whole lines (128 x 256 keys x 8
+    // heads 35.6 -> 34.0 us, 4 x 700 as clusters 6.64 -> 6.46; but ungrouped clusters 1 x 1500 x 40 9.9 -> 10.4, and with the decision
+    // waited for under the loads 16 x 4096 48.5 -> 49.3)
+    constexpr bool kLines = kForm == kAfterDecision || (kCluster && G > 1);
+    constexpr int kDim0 = kLines ? 8 : 16, kDim8 = kLines ? 64 : 8;   // dim of piece 0 / of piece 1 beyond it, per g
     __shared__ float part_s[8][G][kPartialFloats];
     __shared__ float merge_s[kCluster ? 8 : 1][kCluster ? G : 1][kPartialFloats];   // the splits' results, in the first CTA of a cluster
     const int split = blockIdx.x, kh = blockIdx.y, b = blockIdx.z;
@@ -849,13 +854,13 @@ __global__ void __launch_bounds__(256, kForm == kAsCluster ? 1 : 2) decode_atten
         qb[2 * i][0] = r.x; qb[2 * i][1] = r.y; qb[2 * i + 1][0] = r.z; qb[2 * i + 1][1] = r.w;
     }
     const __nv_bfloat16* Kb = p.K + (long long)b * p.ks.b + (long long)kh * p.ks.h;
-    const __nv_bfloat16* Vb = p.V + (long long)b * p.vs.b + (long long)kh * p.vs.h + 16 * g;
+    const __nv_bfloat16* Vb = p.V + (long long)b * p.vs.b + (long long)kh * p.vs.h + kDim0 * g;
 
     // this lane's part of the state (m is the same in all lanes of equal t; l is the lane's share)
     float m[kCols], l[kCols];
 #pragma unroll
     for (int c = 0; c < kCols; ++c) { m[c] = -1e30f; l[c] = 0.f; }
-    float o[8][4];                                   // O^T: product mt, rows (dims) 16g + mt and 16g + 8 + mt, columns 2t, 2t + 1
+    float o[8][4];                                   // O^T: product mt, rows (dims) kDim0 g + mt and kDim8 beyond, columns 2t, 2t + 1
 #pragma unroll
     for (int mt = 0; mt < 8; ++mt) { o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f; }
 
@@ -879,7 +884,7 @@ __global__ void __launch_bounds__(256, kForm == kAsCluster ? 1 : 2) decode_atten
         for (int q4 = 0; q4 < 4; ++q4) {
             const int j = kb + 2 * t + (q4 & 1) + 8 * (q4 >> 1);
 #pragma unroll
-            for (int i = 0; i < 2; ++i) vr[q4][i] = (j < k_hi) ? load16<kForm != kAfterDecision>(Vb + (long long)j * p.vs.t + 8 * i) : zero4;
+            for (int i = 0; i < 2; ++i) vr[q4][i] = (j < k_hi) ? load16<kForm != kAfterDecision>(Vb + (long long)j * p.vs.t + kDim8 * i) : zero4;
         }
         if (kForm == kEarly && !decided) {
             decision();
@@ -923,9 +928,9 @@ __global__ void __launch_bounds__(256, kForm == kAsCluster ? 1 : 2) decode_atten
             o[mt][0] *= corr[0]; o[mt][1] *= corr[kCols - 1]; o[mt][2] *= corr[0]; o[mt][3] *= corr[kCols - 1];
             const int w = mt >> 1;
             const uint32_t sel = (mt & 1) ? 0x7632u : 0x5410u;     // the high / low halves of two rows' words
-            const uint32_t a0 = __byte_perm(word_of(vr[0][0], w), word_of(vr[1][0], w), sel);   // dim 16g + mt,     keys 2t, 2t+1
-            const uint32_t a1 = __byte_perm(word_of(vr[0][1], w), word_of(vr[1][1], w), sel);   // dim 16g + 8 + mt, keys 2t, 2t+1
-            const uint32_t a2 = __byte_perm(word_of(vr[2][0], w), word_of(vr[3][0], w), sel);   // dim 16g + mt,     keys 2t+8, 2t+9
+            const uint32_t a0 = __byte_perm(word_of(vr[0][0], w), word_of(vr[1][0], w), sel);   // the first dim,  keys 2t, 2t+1
+            const uint32_t a1 = __byte_perm(word_of(vr[0][1], w), word_of(vr[1][1], w), sel);   // the second dim, keys 2t, 2t+1
+            const uint32_t a2 = __byte_perm(word_of(vr[2][0], w), word_of(vr[3][0], w), sel);   // the first dim,  keys 2t+8, 2t+9
             const uint32_t a3 = __byte_perm(word_of(vr[2][1], w), word_of(vr[3][1], w), sel);
             mma_bf16_16816(o[mt], a0, a1, a2, a3, pb0, pb1);
         }
@@ -951,8 +956,8 @@ __global__ void __launch_bounds__(256, kForm == kAsCluster ? 1 : 2) decode_atten
         if (h < G) {
 #pragma unroll
             for (int mt = 0; mt < 8; ++mt) {
-                part_s[warp][h][16 * g + mt] = kRest ? o[mt][0] + o[mt][1] : o[mt][c];
-                part_s[warp][h][16 * g + 8 + mt] = kRest ? o[mt][2] + o[mt][3] : o[mt][c + 2];
+                part_s[warp][h][kDim0 * g + mt] = kRest ? o[mt][0] + o[mt][1] : o[mt][c];
+                part_s[warp][h][kDim0 * g + kDim8 + mt] = kRest ? o[mt][2] + o[mt][3] : o[mt][c + 2];
             }
             if (g == 0) { part_s[warp][h][kHeadDim] = m[c]; part_s[warp][h][kHeadDim + 1] = l[c]; }
         }

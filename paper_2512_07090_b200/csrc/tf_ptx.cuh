@@ -75,6 +75,17 @@ __device__ __forceinline__ bool mbar_wait_parked(uint32_t bar, uint32_t parity, 
     }
 }
 
+// ---- distributed shared memory: stores into another CTA of the cluster that complete a transaction on its mbarrier -------
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {      // the same place in CTA `rank`
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_async16(uint32_t remote, uint4 v, uint32_t remote_bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 :: "r"(remote), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(remote_bar) : "memory");
+}
+
 // ---- 8-byte tagged packets {value, tag} in global memory: how one CTA hands a number to another --------------------
 __device__ __forceinline__ uint2 ld_packet2(const uint2* p) {
     uint2 r;

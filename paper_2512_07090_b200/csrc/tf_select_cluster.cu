@@ -11,19 +11,17 @@
 //     additions the 8-lanes-per-token kernel of tf_scan.cu uses, so both give the same bits; the scores are written
 //     out (they are an output of the layer step) and stay in registers for step a4;
 //   * step a4, RATIO mode: the same 4-pass, 8-bit MSB-first radix select over order-preserving keys as the
-//     one-CTA kernel.  Each CTA histograms its own candidates; after a cluster barrier every CTA adds up the
-//     cluster's histograms through distributed shared memory and takes the same decision (two histogram buffers
-//     alternate, so one cluster barrier per pass is enough); once at most 32 candidates share the prefix they are
-//     appended to a list in CTA 0's shared memory and every CTA ranks them there instead of further passes;
+//     one-CTA kernel.  Each CTA histograms its own candidates and stores the histogram into every CTA's shared
+//     memory; every CTA adds them up and takes the same decision; once at most 32 candidates share the prefix every CTA
+//     is told all of them and ranks them instead of further passes;
 //   * ranks in index order (which of the tokens that tie with the P-th key go, and where a retained token lands in
-//     kept_idx) are a CTA-local scan plus the totals of the CTAs before it in the cluster, again through
-//     distributed shared memory.
+//     kept_idx) are a CTA-local scan plus the totals of the CTAs before it in the cluster, told the same way.
 // Same results as select_kernel, bit for bit: same keys, same tie rule (equal scores go from the highest index
 // down), same outputs.
 #include <cooperative_groups.h>
 #include <math_constants.h>
 
-#include "tf_common.cuh"
+#include "tf_ptx.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -32,6 +30,9 @@ namespace {
 
 constexpr int kCsThreads = 512;
 constexpr int kCsWarps = kCsThreads / 32;
+constexpr int kCsRanks = 8;                   // CTAs of a cluster, at most
+constexpr unsigned int kFewMax = 32;          // candidates that are ranked one by one
+constexpr int kFewWords = 36;                 // {count, keys}, in whole 16 bytes
 
 struct ClusterSelectParams {
     const float* sim_k; const float* sim_v;   // [B,S,H]; null: the scores are read from `score`
@@ -44,6 +45,7 @@ struct ClusterSelectParams {
     long long p_target;                       // floor(ratio*S), computed on the host in double
     uint8_t* keep_mask; int32_t* kept_idx; int32_t* n_kept; float* theta;
     DevStatus* status;
+    long long wait_cycles;                    // budget of one mbarrier wait
 };
 
 // Step a3 for one token by one thread from the token's similarities in registers (up to 8 KV heads; xk[h], xv[h] are
@@ -79,25 +81,52 @@ constexpr int kFuseLanes = 8;   // the lane count score_fuse_kernel uses for up 
 
 template <int KPT>
 __global__ void __launch_bounds__(kCsThreads, 1) select_cluster_kernel(const ClusterSelectParams p) {
-    __shared__ int hist[2][256];
+    // What the CTAs tell one another is stored straight into every CTA's shared memory (its own included), where an mbarrier counts the
+    // bytes: nobody waits for more than the numbers themselves.  (A cluster barrier before reading the others' numbers took 1,000 to
+    // 1,350 cycles, five times a selection, and the reads as much again: selection of 1 x 2048 tokens 6.3 -> 4.9 us, 1 x 4096 6.7 -> 5.4,
+    // 2 x 8192 8.2 -> 7.0, with the scans by one warp.)  Every exchange has its own barrier, used once; the histograms take two buffers
+    // in turn: a CTA that sends the pass after next has had everybody's next one, which follows their reading of this one.
+    __shared__ __align__(16) unsigned int rx_hist[2][kCsRanks][256];
+    __shared__ __align__(16) unsigned int rx_few[kCsRanks][kFewWords];     // {count, keys}
+    __shared__ __align__(16) unsigned int rx_eq[kCsRanks][4];              // {equal keys}
+    __shared__ __align__(16) unsigned int rx_pub[kCsRanks][4];             // {retained, lowest pruned score}
+    __shared__ __align__(8) unsigned long long s_bars[7];                  // passes 0-3, few, equal, published
+    __shared__ __align__(16) unsigned int hist[256];
+    __shared__ __align__(16) unsigned int s_few[kFewWords];
+    __shared__ int s_abort;
     __shared__ int s_warp[kCsWarps];
-    __shared__ int s_pub[4];                  // read by the other CTAs of the cluster: [0] equal keys, [1] retained, [2] lowest pruned score
+    __shared__ float s_min;
     __shared__ unsigned int s_prefix;
     __shared__ int s_rank, s_count, s_total;
     __shared__ int s_tab[KPT * kCsWarps];     // [chunk][warp] ballot counts of the final sweep
-    __shared__ unsigned int s_few[32];        // CTA 0's copy: the last few candidates' keys, appended by the whole cluster
-    __shared__ int s_few_n;
 
-    grid_dependency_wait();
-    grid_launch_dependents();   // few CTAs: the attention grid may take the other SMs and set up meanwhile (see select_kernel)
     cg::cluster_group cluster = cg::this_cluster();
     const int n_ranks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const int b = (int)blockIdx.x / n_ranks, tid = threadIdx.x, S = p.S;
     const int lane = tid & 31, wid = tid >> 5;
+    const uint32_t bars = smem_u32(s_bars);
+    volatile int* abort_flag = &s_abort;
+    if (tid == 0) {
+        s_abort = 0;
+        for (int i = 0; i < 7; ++i) mbar_init(bars + 8 * i, 1);
+        mbar_fence_init();
+        for (int i = 0; i < 7; ++i)
+            mbar_expect_tx(bars + 8 * i, (uint32_t)n_ranks * (i < 4 ? 1024u : i == 4 ? 4u * kFewWords : 16u));
+    }
+    if (tid < kFewWords) s_few[tid] = 0;
+    cluster.barrier_arrive();    // (waited for before the first store into another CTA: its barriers are set up then)
+    // thread (q, k): 16 bytes k of src to place k of this CTA's row in CTA q
+    auto tell = [&](const unsigned int* src, unsigned int* row, int words, int bar) {
+        const int per = words / 4, q = tid / per, k = tid - q * per;
+        if (q < n_ranks)
+            st_async16(cluster_addr(smem_u32(row + 4 * k), q), *reinterpret_cast<const uint4*>(src + 4 * k), cluster_addr(bars + 8 * bar, q));
+    };
+    auto heard = [&](int bar) { mbar_wait_bounded(bars + 8 * bar, 0, abort_flag, p.wait_cycles, p.status, 700 + bar); };
+    grid_dependency_wait();
+    grid_launch_dependents();   // few CTAs: the attention grid may take the other SMs and set up meanwhile (see select_kernel)
     const int t_base = rank * (KPT * kCsThreads);
     const uint8_t* el = p.eligible ? p.eligible + (size_t)b * S : nullptr;
     float* sc = p.score + (size_t)b * S;
-    if (tid == 0) s_few_n = 0;                // used at most once, after at least one cluster barrier
 
     // token of slot i: t_base + i*512 + tid (ascending in (i, tid))
     float sreg[KPT];
@@ -169,9 +198,7 @@ __global__ void __launch_bounds__(kCsThreads, 1) select_cluster_kernel(const Clu
         unsigned int prefix = 0, mask = 0;
         int r = 0, pass = 0;
         for (int shift = 24; shift >= 0; shift -= 8, ++pass) {
-            int* h = hist[pass & 1];
-            // this buffer was last read by the cluster two passes ago; every CTA has passed the barrier since
-            if (tid < 256) h[tid] = 0;
+            if (tid < 256) hist[tid] = 0;
             __syncthreads();
 #pragma unroll
             for (int i = 0; i < KPT; ++i) {
@@ -181,66 +208,87 @@ __global__ void __launch_bounds__(kCsThreads, 1) select_cluster_kernel(const Clu
                     const unsigned int k = score_key(sreg[i]);
                     if ((k & mask) == prefix) bin = (int)((k >> shift) & 255u);
                 }
-                const unsigned int same = __match_any_sync(0xffffffffu, bin);
-                if (bin < 256 && lane == __ffs(same) - 1) atomicAdd(&h[bin], __popc(same));
+                if (pass == 0) {     // (most scores share a few exponents; under a prefix they spread out)
+                    const unsigned int same = __match_any_sync(0xffffffffu, bin);
+                    if (bin < 256 && lane == __ffs(same) - 1) atomicAdd(&hist[bin], (unsigned int)__popc(same));
+                } else if (bin < 256) {
+                    atomicAdd(&hist[bin], 1u);
+                }
             }
-            cluster.sync();      // every CTA's histogram of this pass is complete
-            // descending inclusive scan of the cluster's histogram: the bin where the count reaches r
-            int hval = 0, incl = 0;
-            if (tid < 256) {
-                for (int q = 0; q < n_ranks; ++q) hval += cluster.map_shared_rank(h, q)[255 - tid];
-                incl = hval;
+            __syncthreads();
+            if (pass == 0) cluster.barrier_wait();
+            tell(hist, rx_hist[pass & 1][rank], 256, pass);
+            // descending inclusive scan of the cluster's histogram: the bin where the count reaches r.  One warp, eight bins a lane
+            if (wid == 0) {
+                heard(pass);
+                int v[8], sum = 0;      // bins 255 - 8 lane, 254 - 8 lane, ..
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = 0;
+                for (int q = 0; q < n_ranks; ++q) {
+                    const uint4* src = reinterpret_cast<const uint4*>(&rx_hist[pass & 1][q][248 - 8 * lane]);
+                    const uint4 lo = src[0], hi = src[1];
+                    v[0] += (int)hi.w; v[1] += (int)hi.z; v[2] += (int)hi.y; v[3] += (int)hi.x;
+                    v[4] += (int)lo.w; v[5] += (int)lo.z; v[6] += (int)lo.y; v[7] += (int)lo.x;
+                }
+#pragma unroll
+                for (int e = 0; e < 8; ++e) sum += v[e];
+                int incl = sum;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     const int n = __shfl_up_sync(0xffffffffu, incl, o);
                     if (lane >= o) incl += n;
                 }
-                if (lane == 31) s_warp[wid] = incl;
-            }
-            __syncthreads();
-            if (shift == 24) {   // first pass: the number of candidates E caps the number to prune (same in every CTA)
-                int E = 0;
+                // first pass: the number of candidates E caps the number to prune (same in every CTA)
+                const int E = __shfl_sync(0xffffffffu, incl, 31);
+                const int want = pass == 0 ? (int)(p.p_target < (long long)E ? p.p_target : (long long)E) : r;
+                if (lane == 0 && want <= 0) s_rank = 0;
+                int excl = incl - sum;
+                if (excl < want && incl >= want) {
+                    int e = 0;
 #pragma unroll
-                for (int w2 = 0; w2 < 8; ++w2) E += s_warp[w2];
-                r = (int)(p.p_target < (long long)E ? p.p_target : (long long)E);
-                if (r <= 0) { nothing = true; break; }
-            }
-            if (tid < 256) {
-                int off = 0;
-                for (int w2 = 0; w2 < wid; ++w2) off += s_warp[w2];
-                incl += off;
-                const int excl = incl - hval;
-                if (excl < r && incl >= r) {
-                    s_prefix = prefix | ((unsigned int)(255 - tid) << shift);
-                    s_rank = r - excl;
-                    s_count = hval;
+                    for (int k = 0; k < 7; ++k)
+                        if (e == k && excl + v[k] < want) { excl += v[k]; e = k + 1; }
+                    int count = v[7];
+#pragma unroll
+                    for (int k = 0; k < 7; ++k) count = e == k ? v[k] : count;
+                    s_prefix = prefix | ((unsigned int)(255 - 8 * lane - e) << shift);
+                    s_rank = want - excl;
+                    s_count = count;
                 }
             }
             __syncthreads();
-            prefix = s_prefix;
             r = s_rank;
+            if (r <= 0) { nothing = true; break; }           // (first pass only)
+            prefix = s_prefix;
             n_eq = s_count;
             mask |= 255u << shift;
-            __syncthreads();     // s_warp, s_prefix, s_rank and s_count are written again in the next pass
-            // Few candidates left under this prefix (typical after two or three passes): they are collected in CTA 0's
-            // shared memory and every CTA ranks them there instead of further histogram passes.  Same result: the key of
-            // rank r among them, how many candidates carry it, and the rank within those.  (n_eq is the same in every CTA.)
-            if (shift > 0 && n_eq <= 32) {
-                unsigned int* few0 = cluster.map_shared_rank(s_few, 0);
-                int* few_n0 = cluster.map_shared_rank(&s_few_n, 0);
+            __syncthreads();     // s_prefix, s_rank and s_count are written again below
+            // Few candidates left under this prefix (typical after two or three passes): every CTA is told all of them and ranks
+            // them instead of further histogram passes.  Same result: the key of rank r among them, how many candidates carry it,
+            // and the rank within those.  (n_eq is the same in every CTA.)
+            if (shift > 0 && n_eq <= (int)kFewMax) {
 #pragma unroll
                 for (int i = 0; i < KPT; ++i) {
                     const int t = t_base + i * kCsThreads + tid;
                     if (t < S && candidate(t, sreg[i])) {
                         const unsigned int k = score_key(sreg[i]);
-                        if ((k & mask) == prefix) few0[atomicAdd(few_n0, 1)] = k;     // exactly n_eq appends in all
+                        if ((k & mask) == prefix) s_few[1 + min(atomicAdd(&s_few[0], 1u), kFewMax - 1u)] = k;     // n_eq in all CTAs
                     }
                 }
-                cluster.sync();
+                __syncthreads();
+                tell(s_few, rx_few[rank], kFewWords, 4);
                 if (tid < 32) {
-                    const unsigned int key = tid < n_eq ? few0[tid] : 0u;
+                    heard(4);
+                    unsigned int key = 0u;
+                    int at = tid;
+                    for (int q = 0; q < n_ranks; ++q) {
+                        const int c = min((int)rx_few[q][0], (int)kFewMax);
+                        if (at >= 0 && at < c) key = rx_few[q][1 + at];
+                        at -= c;
+                    }
                     int greater = 0, equal = 0;
-                    for (int o = 0; o < n_eq; ++o) {
+#pragma unroll
+                    for (int o = 0; o < (int)kFewMax; ++o) {         // (a lane without a candidate has key 0, below all of them)
                         const unsigned int ko = __shfl_sync(0xffffffffu, key, o);
                         greater += ko > key ? 1 : 0;
                         equal += ko == key ? 1 : 0;
@@ -281,6 +329,9 @@ __global__ void __launch_bounds__(kCsThreads, 1) select_cluster_kernel(const Clu
 #pragma unroll
             for (int e = 0; e < kPer; ++e) { if (lane * kPer + e < kEnt) s_tab[lane * kPer + e] = run; run += v[e]; }
             if (lane == 31) s_total = incl;
+        } else if (wid == 1) {                                // (the last time: the lowest pruned score)
+            const float m = -warp_max(lane < kCsWarps ? -__int_as_float(s_warp[lane]) : -CUDART_INF_F);
+            if (lane == 0) s_min = m;
         }
         __syncthreads();
     };
@@ -307,10 +358,10 @@ __global__ void __launch_bounds__(kCsThreads, 1) select_cluster_kernel(const Clu
                 if (lane == 0) s_tab[i * kCsWarps + wid] = __popc(bal);
             }
             scan_table();
-            if (tid == 0) s_pub[0] = s_total;
-            cluster.sync();
+            if (tid < n_ranks) st_async16(cluster_addr(smem_u32(rx_eq[rank]), tid), make_uint4((unsigned int)s_total, 0u, 0u, 0u), cluster_addr(bars + 8 * 5, tid));
+            heard(5);
             int eq_before = 0;                                // equal keys in the CTAs before this one
-            for (int q = 0; q < rank; ++q) eq_before += cluster.map_shared_rank(s_pub, q)[0];
+            for (int q = 0; q < rank; ++q) eq_before += (int)rx_eq[q][0];
 #pragma unroll
             for (int i = 0; i < KPT; ++i) {
                 const bool eq = (eq_bits >> i) & 1u;
@@ -332,19 +383,21 @@ __global__ void __launch_bounds__(kCsThreads, 1) select_cluster_kernel(const Clu
         if ((prune_bits >> i) & 1u) th_min = fminf(th_min, sreg[i]);
     }
     th_min = -warp_max(-th_min);
-    __syncthreads();             // s_warp may still be read by the last radix pass (the nothing-to-prune exit)
     if (lane == 0) s_warp[wid] = __float_as_int(th_min);
     scan_table();
-    if (tid == 0) {
-        float m = CUDART_INF_F;
-        for (int w2 = 0; w2 < kCsWarps; ++w2) m = fminf(m, __int_as_float(s_warp[w2]));
-        s_pub[1] = s_total;
-        s_pub[2] = __float_as_int(m);
+    if (p.mode == TF_SELECT_THRESHOLD || p.p_target <= 0) cluster.barrier_wait();     // (there was no histogram pass)
+    if (tid < n_ranks)
+        st_async16(cluster_addr(smem_u32(rx_pub[rank]), tid), make_uint4((unsigned int)s_total, __float_as_uint(s_min), 0u, 0u), cluster_addr(bars + 8 * 6, tid));
+    heard(6);
+    if (__syncthreads_or(*abort_flag)) {         // a wait gave up: everybody is told
+        if (tid < n_ranks) *cluster.map_shared_rank(&s_abort, tid) = 1;
+        __threadfence();
     }
-    cluster.sync();
+    // nobody leaves before everybody has come this far: nothing is stored into another CTA after it (relaxed: there is nothing else to order)
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     int kept_before = 0, kept_all = 0;
     for (int q = 0; q < n_ranks; ++q) {
-        const int n = cluster.map_shared_rank(s_pub, q)[1];
+        const int n = (int)rx_pub[q][0];
         kept_before += q < rank ? n : 0;
         kept_all += n;
     }
@@ -356,7 +409,7 @@ __global__ void __launch_bounds__(kCsThreads, 1) select_cluster_kernel(const Clu
         const int pos = kept_before + s_tab[i * kCsWarps + wid] + __popc(bal & lt);
         if (in) {
             p.keep_mask[(size_t)b * S + t] = keep ? 1 : 0;
-            if (keep) p.kept_idx[(size_t)b * S + pos] = t;
+            if (keep && (unsigned int)pos < (unsigned int)S) p.kept_idx[(size_t)b * S + pos] = t;   // (outside only after a wait that gave up)
             if (t >= kept_all) p.kept_idx[(size_t)b * S + t] = -1;   // the list's tail: positions kept_all .. S-1 (pos <= t, so never a slot just filled)
         }
     }
@@ -364,11 +417,21 @@ __global__ void __launch_bounds__(kCsThreads, 1) select_cluster_kernel(const Clu
         p.n_kept[b] = kept_all;
         if (p.theta) {
             float m = CUDART_INF_F;
-            for (int q = 0; q < n_ranks; ++q) m = fminf(m, __int_as_float(cluster.map_shared_rank(s_pub, q)[2]));
+            for (int q = 0; q < n_ranks; ++q) m = fminf(m, __uint_as_float(rx_pub[q][1]));
             p.theta[b] = m;
         }
     }
-    cluster.sync();              // nobody leaves while its shared memory may still be read
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    if (*abort_flag) {           // in all CTAs or none: no list is better than one with holes, which the attention would follow
+        cluster.sync();
+        for (int i = 0; i < KPT; ++i) {
+            const int t = t_base + i * kCsThreads + tid;
+            if (t < S) p.kept_idx[(size_t)b * S + t] = -1;
+        }
+        if (rank == 0 && tid == 0) p.n_kept[b] = 0;
+        const long long t0 = clock64();          // stores still under way land before the shared memory goes away
+        while (clock64() - t0 < 2000000ll) { }
+    }
 }
 
 template <int KPT>
@@ -414,6 +477,7 @@ cudaError_t launch_select_cluster(tf_ctx* ctx, const tf_shape& s, const tf_filte
     cp.p_target = (long long)floor(p.prune_ratio * (double)s.seq);
     cp.keep_mask = keep_mask; cp.kept_idx = kept_idx; cp.n_kept = n_kept; cp.theta = theta;
     cp.status = ctx->dev_status;
+    cp.wait_cycles = ctx_wait_cycles(ctx);
     const int n_ranks = s.seq > 2048 ? 8 : 4;
     const int per_rank = (s.seq + n_ranks - 1) / n_ranks;
     int kpt = 1;

@@ -1,0 +1,74 @@
+"""The cluster selection's exchanges: every number of passes and CTAs, and waits that give up."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2512_07090_b200 import binding as tfb
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _select(ctx, score, ratio):
+    B, S = score.shape
+    shape = tfb.tf_shape()
+    shape.batch, shape.seq, shape.n_q_heads, shape.n_kv_heads, shape.head_dim, shape.dtype = B, S, 32, 32, 128, tfb.TF_BF16
+    params = tfb.default_params(prune_ratio=ratio, warmup_tokens=4)
+    keep = torch.full((B, S), 7, dtype=torch.uint8, device=DEV)
+    idx = torch.full((B, S), -7, dtype=torch.int32, device=DEV)
+    nk = torch.full((B,), -7, dtype=torch.int32, device=DEV)
+    ctx.tf_select(shape, params, score, keep, idx, nk)
+    return keep, idx, nk
+
+
+def _expect(score, ratio):
+    S = len(score)
+    order = sorted(range(4, S), key=lambda t: (-score[t], -t))          # equal scores go from the highest index down
+    pruned = set(order[:min(S - 4, int(np.floor(ratio * S)))])
+    return [t for t in range(S) if t not in pruned]
+
+
+# spread scores (two passes), all of them in one binade and close together (three and four passes), many equal ones
+@pytest.mark.parametrize("kind", ["spread", "close", "closer", "ties"])
+@pytest.mark.parametrize("S", [1025, 2048, 2049, 9000, 32768])           # clusters of 4 and 8, every register count
+def test_cluster_selection_passes(S, kind):
+    rng = np.random.default_rng(S)
+    x = rng.standard_normal((2, S)) * 0.05
+    if kind != "spread":
+        x = 0.5 + rng.random((2, S)) * {"close": 1e-3, "closer": 2e-6, "ties": 1e-3}[kind]
+    if kind == "ties":
+        x = np.round(x, 5)
+    score = x.astype(np.float32)
+    ctx = tfb.Context(0)
+    ctx.tf_set_select_path(2)
+    keep, idx, nk = _select(ctx, torch.from_numpy(score).to(DEV), 0.4)
+    assert ctx.tf_get_status()[0] == tfb.TF_OK
+    for b in range(2):
+        want = _expect(score[b], 0.4)
+        assert int(nk[b]) == len(want)
+        got = idx[b].cpu().numpy()
+        assert np.array_equal(got[:len(want)], want) and np.all(got[len(want):] == -1)
+        assert np.array_equal(np.flatnonzero(keep[b].cpu().numpy()), want)
+    ctx.close()
+
+
+def test_a_selection_whose_waits_give_up_leaves_an_empty_list_or_the_right_one():
+    """A wait of no cycles may give up: the status says so, and the attention would find no list rather than one with holes."""
+    score = (np.random.default_rng(3).standard_normal((8, 20000)) * 0.05).astype(np.float32)
+    dev = torch.from_numpy(score).to(DEV)
+    want = [_expect(s, 0.5) for s in score]
+    ctx = tfb.Context(0)
+    ctx.tf_set_select_path(2)
+    for limit in (0, 0, 0, -1):
+        ctx.tf_set_wait_limits(wait_cycles=limit)
+        keep, idx, nk = _select(ctx, dev, 0.5)
+        code = ctx.tf_get_status()[0]
+        assert code == tfb.TF_OK or (limit == 0 and code == tfb.TF_ERR_TIMEOUT)
+        for b in range(8):
+            got, n = idx[b].cpu().numpy(), int(nk[b])
+            if code == tfb.TF_OK or n > 0:
+                assert n == len(want[b]) and np.array_equal(got[:n], want[b]) and np.all(got[n:] == -1)
+            else:
+                assert np.all(got == -1)
+        ctx.tf_clear_status()
+    ctx.close()

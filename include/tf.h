@@ -166,8 +166,8 @@ tf_status tf_select(tf_ctx *ctx, const tf_shape *shape, const tf_filter_params *
 /* Steps a3 + a4 in one call (Alg. 1 from "(s_k, sigma_k^2)" to the skip decision; Eq. 2-3, Section 3.3): the
  * arguments of tf_score_fuse followed by the outputs of tf_select, with the same meaning, layout and results (the
  * scores have the bits tf_score_fuse gives, the selection the outputs tf_select gives on them).  For sequences of
- * 1025 to 32768 tokens with up to 8 KV heads both steps run in one launch, a thread-block cluster per sequence;
- * otherwise as two kernels.  theta may be NULL. */
+ * up to 240 tokens with up to 64 KV heads, and of 1025 to 32768 tokens with up to 8, both steps run in one launch (one
+ * CTA, a thread-block cluster per sequence); otherwise as two kernels.  theta may be NULL. */
 tf_status tf_score_select(tf_ctx *ctx, const tf_shape *shape, const tf_filter_params *params,
                           const float *sim_k, const float *sim_v, float *score, uint8_t *keep_mask,
                           int32_t *kept_idx, int32_t *n_kept, float *theta, void *stream);

@@ -10,7 +10,9 @@
 // (token i*1024 + tid in slot i), so the passes run out of registers and shared memory; longer
 // sequences stage the scores in shared memory (up to 51200 tokens) or re-read them from global memory
 // on each pass.  (Producing the scores inside this
-// kernel as well was measured: one CTA per sequence reads the per-head similarities far too slowly.)
+// kernel as well was measured: one CTA per sequence reads the per-head similarities far too slowly.)  Sequences of
+// up to 240 tokens have a kernel of their own, select_small_kernel, which also makes the scores.
+#include <algorithm>
 #include <math_constants.h>
 
 #include "tf_common.cuh"
@@ -415,7 +417,210 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_kernel(const SelectPara
     }
 }
 
+// ---------------------------------------------------------------------------------------------------------
+// Short sequences (up to 240 tokens): step a3 and step a4 in one launch, one CTA per sequence, without radix passes: the rank of
+// every token among all candidates is counted outright.  A chain of latencies, so what counts is how few there are: one round trip to
+// memory for all similarities, one for the outputs, five block barriers.  us per pass, two launches / this one: fp32 1 x 33 x 8 heads 15.4
+// / 12.9, 1 x 128 x 32 19.7 / 18.1, 2 x 192 x 40 44.2 / 43.5; bf16 4 x 33 x 8 20.8 / 17.6, 4 x 128 x 8 21.6 / 18.4, 1 x 192 x 32 22.8 / 21.9.  The
+// line: the comparisons grow with the square of the length, and one SM reads all similarities: 240 x 32 heads 24.4 / 24.4, 256 x 32
+// 24.7 / 25.1, 256 x 8 23.8 / 23.2.  The scores have the bits of score_fuse_kernel<G>: the same order of additions, every rounding
+// spelled out.
+// ---------------------------------------------------------------------------------------------------------
+struct SmallParams {
+    SelectParams sel;
+    const float* sim_k; const float* sim_v;   // [B,S,H]; null: the scores are read
+    float* score_out;                         // [B,S]: written when sim_k is given
+    int H, fuse_mode;
+    int vec4;                                 // the similarities can be read as float4 (H a multiple of 4, 16-byte aligned)
+    float eps;
+    DevStatus* status;
+};
+constexpr int kSmallTokens = 256, kSmallHeads = 64;     // room of the kernel
+constexpr int kSmallSeq = 240;                          // ... and the line to the other forms
+
+template <int G>
+__global__ void __launch_bounds__(kSelThreads, 1) select_small_kernel(const SmallParams sp) {
+    __shared__ float s_score[kSmallTokens];
+    __shared__ __align__(16) unsigned int s_key[kSmallTokens];     // 0: not a candidate
+    __shared__ unsigned char s_prune[kSmallTokens];
+    __shared__ int s_cnt[kSmallTokens / 32];
+    __shared__ float s_low[kSmallTokens / 32];
+    const SelectParams& p = sp.sel;
+    grid_dependency_wait();
+    grid_launch_dependents();   // (after the wait: see select_kernel)
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, S = p.S, H = sp.H;
+    if (sp.sim_k) {
+        // Rows to shared memory as they lie, 4 words apart (a warp then reads 8 tokens x 4 heads without conflicts).  Four threads
+        // fuse a token: thread q has the lanes q, q + 4, .. of score_fuse_kernel<G>'s group, so all but the last two steps of its sums
+        // are a thread's own (a group of lanes per token spends 20 shuffles on one: 128 tokens x 32 heads 20.8 us per pass instead of 18.1).
+        extern __shared__ __align__(16) float s_sim[];                // [2][S][H + 4]
+        const int stride = H + 4, n = S * H;
+        float* const ks = s_sim;
+        float* const vs = s_sim + S * stride;
+        const float* gk = sp.sim_k + (size_t)b * n;
+        const float* gv = sp.sim_v + (size_t)b * n;
+        if (sp.vec4) {
+            for (int i = tid * 4; i < n; i += 4 * blockDim.x) {
+                const float4 k = __ldg(reinterpret_cast<const float4*>(gk + i)), v = __ldg(reinterpret_cast<const float4*>(gv + i));
+                const int at = i + (i / H) * 4;
+                *reinterpret_cast<float4*>(ks + at) = k;
+                *reinterpret_cast<float4*>(vs + at) = v;
+            }
+        } else {
+            for (int i = tid; i < n; i += blockDim.x) {
+                const float k = __ldg(gk + i), v = __ldg(gv + i);
+                const int at = i + (i / H) * 4;
+                ks[at] = k; vs[at] = v;
+            }
+        }
+        __syncthreads();
+        const int t = tid >> 2, q = tid & 3;
+        const float* xk = ks + t * stride;
+        const float* xv = vs + t * stride;
+        constexpr int kOwn = G / 4;
+        auto total = [](float (&v)[kOwn]) {
+#pragma unroll
+            for (int o = kOwn / 2; o > 0; o >>= 1)
+#pragma unroll
+                for (int e = 0; e < o; ++e) v[e] = __fadd_rn(v[e], v[e + o]);
+            v[0] = __fadd_rn(v[0], __shfl_xor_sync(0xffffffffu, v[0], 2));
+            return __fadd_rn(v[0], __shfl_xor_sync(0xffffffffu, v[0], 1));
+        };
+        const float inv = 1.f / (float)H;
+        float a[kOwn][2], c[kOwn][2], pk[kOwn], pv[kOwn];
+#pragma unroll
+        for (int e = 0; e < kOwn; ++e) {
+            const int l = q + 4 * e;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const bool in = t < S && l + u * G < H;
+                a[e][u] = in ? xk[l + u * G] : 0.f;
+                c[e][u] = in ? xv[l + u * G] : 0.f;
+            }
+            pk[e] = __fadd_rn(0.f, a[e][0]); pv[e] = __fadd_rn(0.f, c[e][0]);
+            if (l + G < H) { pk[e] = __fadd_rn(pk[e], a[e][1]); pv[e] = __fadd_rn(pv[e], c[e][1]); }
+        }
+        const float sk = __fmul_rn(total(pk), inv), sv = __fmul_rn(total(pv), inv);
+#pragma unroll
+        for (int e = 0; e < kOwn; ++e) {
+            pk[e] = pv[e] = 0.f;
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                if (q + 4 * e + u * G < H) {
+                    const float dk = __fsub_rn(a[e][u], sk), dv = __fsub_rn(c[e][u], sv);
+                    pk[e] = __fmaf_rn(dk, dk, pk[e]);
+                    pv[e] = __fmaf_rn(dv, dv, pv[e]);
+                }
+        }
+        const float vk = __fmul_rn(total(pk), inv), vv = __fmul_rn(total(pv), inv);
+        if (q == 0 && t < S) {
+            const float s = fuse_score(sp.fuse_mode, sk, vk, sv, vv, sp.eps);
+            s_score[t] = s;
+            sp.score_out[(size_t)b * S + t] = s;
+            note_nan_score(sp.status, s, (unsigned long long)b * S + t);
+        }
+    } else if (tid < S) {
+        s_score[tid] = p.score[(size_t)b * S + tid];
+    }
+    __syncthreads();
+    const uint8_t* el = p.eligible ? p.eligible + (size_t)b * S : nullptr;
+    bool cand = false;
+    if (tid < kSmallTokens) {
+        const float s = tid < S ? s_score[tid] : 0.f;
+        cand = tid < S && tid >= p.warmup && (el == nullptr || el[tid] != 0) && s == s;    // NaN never pruned
+        s_key[tid] = cand ? score_key(s) : 0u;                                              // (no score's key is 0)
+    }
+    const int E = __syncthreads_count(cand ? 1 : 0);
+    {   // token t, a quarter of the others per thread: higher keys, and equal ones with a higher index, go first
+        const int t = tid >> 2, part = tid & 3;
+        bool prune = false;
+        if (p.mode == TF_SELECT_THRESHOLD) {
+            prune = t < S && s_key[t] != 0u && s_score[t] > p.threshold[b];
+        } else {
+            const int P = (int)(p.p_target < (long long)E ? p.p_target : (long long)E);
+            const unsigned int key = s_key[t];
+            int rank = 0;
+            if (t < S)
+                for (int o = part * 4; o < S; o += 16) {              // (keys from S on are 0)
+                    const uint4 k = *reinterpret_cast<const uint4*>(&s_key[o]);
+                    rank += (k.x > key || (k.x == key && o > t)) ? 1 : 0;
+                    rank += (k.y > key || (k.y == key && o + 1 > t)) ? 1 : 0;
+                    rank += (k.z > key || (k.z == key && o + 2 > t)) ? 1 : 0;
+                    rank += (k.w > key || (k.w == key && o + 3 > t)) ? 1 : 0;
+                }
+            rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+            rank += __shfl_xor_sync(0xffffffffu, rank, 2);
+            prune = t < S && key != 0u && rank < P;
+        }
+        if (part == 0) s_prune[t] = prune ? 1 : 0;
+    }
+    __syncthreads();
+    unsigned int bal = 0;
+    bool keep = false;
+    if (tid < kSmallTokens) {
+        const bool prune = tid < S && s_prune[tid] != 0;
+        keep = tid < S && !prune;
+        bal = __ballot_sync(0xffffffffu, keep);
+        const float low = -warp_max(prune ? -s_score[tid] : -CUDART_INF_F);
+        if (lane == 0) { s_cnt[wid] = __popc(bal); s_low[wid] = low; }
+    }
+    __syncthreads();
+    if (tid >= S) return;
+    int before = 0, kept = 0;
+    float low = CUDART_INF_F;
+#pragma unroll
+    for (int w = 0; w < kSmallTokens / 32; ++w) {
+        before += w < wid ? s_cnt[w] : 0;
+        kept += s_cnt[w];
+        low = fminf(low, s_low[w]);
+    }
+    p.keep_mask[(size_t)b * S + tid] = keep ? 1 : 0;
+    if (keep) p.kept_idx[(size_t)b * S + before + __popc(bal & ((1u << lane) - 1u))] = tid;
+    if (tid >= kept) p.kept_idx[(size_t)b * S + tid] = -1;
+    if (tid == 0) {
+        p.n_kept[b] = kept;
+        if (p.theta) p.theta[b] = low;
+    }
+}
+
 namespace {
+// both steps, or step a4 alone (sim_k null)
+bool select_small_takes(const tf_ctx* ctx, const tf_shape& s, bool fuses) {
+    return ctx->select_form == 0 && s.seq <= kSmallSeq && (!fuses || s.n_kv_heads <= kSmallHeads);
+}
+cudaError_t launch_select_small(tf_ctx* ctx, const tf_shape& s, const SelectParams& sel, const tf_filter_params& p, const float* sim_k, const float* sim_v,
+                                float* score_out, cudaStream_t st) {
+    if (s.seq == 0) return cudaErrorInvalidValue;
+    SmallParams sp{};
+    sp.sel = sel; sp.sim_k = sim_k; sp.sim_v = sim_v; sp.score_out = score_out;
+    sp.H = s.n_kv_heads; sp.fuse_mode = p.fuse_mode; sp.eps = p.var_eps > 0.f ? p.var_eps : 1e-8f;
+    sp.status = ctx->dev_status;
+    sp.vec4 = (s.n_kv_heads % 4 == 0 && ((reinterpret_cast<uintptr_t>(sim_k) | reinterpret_cast<uintptr_t>(sim_v)) & 15) == 0) ? 1 : 0;
+    static bool attr_set_dev[kDeviceFlagSlots] = {};      // function attributes are per device
+    bool& attr_set = attr_set_dev[ctx->device >= 0 && ctx->device < kDeviceFlagSlots ? ctx->device : 0];
+    if (!attr_set) {
+        constexpr int most = 2 * kSmallTokens * (kSmallHeads + 4) * (int)sizeof(float);
+        cudaError_t e = cudaFuncSetAttribute(select_small_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(select_small_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(select_small_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    const size_t smem = sim_k ? 2 * (size_t)s.seq * (s.n_kv_heads + 4) * sizeof(float) : 0;
+    auto kernel = s.n_kv_heads <= 8 ? select_small_kernel<8> : s.n_kv_heads <= 16 ? select_small_kernel<16> : select_small_kernel<32>;
+    const cudaError_t e = launch_dependent(kernel, dim3((unsigned)s.batch), dim3((unsigned)std::max(kSmallTokens, (4 * s.seq + 31) / 32 * 32)), smem, st, sp);     // four threads a token
+    ctx->launches += 1;
+    return e;
+}
+SelectParams select_params(const tf_shape& s, const tf_filter_params& p, const float* score, uint8_t* keep_mask, int32_t* kept_idx, int32_t* n_kept, float* theta) {
+    SelectParams sp{};
+    sp.score = score; sp.eligible = p.eligible; sp.threshold = p.threshold;
+    sp.S = s.seq; sp.warmup = p.warmup_tokens; sp.mode = p.select_mode;
+    sp.p_target = (long long)floor(p.prune_ratio * (double)s.seq);
+    sp.keep_mask = keep_mask; sp.kept_idx = kept_idx; sp.n_kept = n_kept; sp.theta = theta;
+    return sp;
+}
+
 cudaError_t launch_select_form(const SelectParams& sp, int batch, cudaStream_t st) {
     const dim3 grid(batch), block(kSelThreads);
     const int S = sp.S;
@@ -450,11 +655,8 @@ cudaError_t launch_select(tf_ctx* ctx, const tf_shape& s, const tf_filter_params
     // sequences of 1025 to 32768 tokens are shared by the CTAs of a cluster
     if (ctx->select_form == 2 || (ctx->select_form == 0 && select_cluster_preferred(s)))
         return launch_select_cluster(ctx, s, p, nullptr, nullptr, const_cast<float*>(score), keep_mask, kept_idx, n_kept, theta, st);
-    SelectParams sp{};
-    sp.score = score; sp.eligible = p.eligible; sp.threshold = p.threshold;
-    sp.S = s.seq; sp.warmup = p.warmup_tokens; sp.mode = p.select_mode;
-    sp.p_target = (long long)floor(p.prune_ratio * (double)s.seq);
-    sp.keep_mask = keep_mask; sp.kept_idx = kept_idx; sp.n_kept = n_kept; sp.theta = theta;
+    const SelectParams sp = select_params(s, p, score, keep_mask, kept_idx, n_kept, theta);
+    if (s.seq > 0 && select_small_takes(ctx, s, false)) return launch_select_small(ctx, s, sp, p, nullptr, nullptr, nullptr, st);
     cudaError_t e = launch_select_form(sp, s.batch, st);
     ctx->launches += 1;
     return e;
@@ -466,6 +668,8 @@ cudaError_t launch_score_select(tf_ctx* ctx, const tf_shape& s, const tf_filter_
     if ((ctx->select_form == 2 && select_cluster_usable(s) && select_cluster_fuses(s)) ||
         (ctx->select_form == 0 && select_cluster_preferred(s) && select_cluster_fuses(s)))
         return launch_select_cluster(ctx, s, p, sim_k, sim_v, score, keep_mask, kept_idx, n_kept, theta, st);
+    if (s.batch > 0 && s.seq > 0 && select_small_takes(ctx, s, true))
+        return launch_select_small(ctx, s, select_params(s, p, score, keep_mask, kept_idx, n_kept, theta), p, sim_k, sim_v, score, st);
     cudaError_t e = launch_score_fuse(ctx, s, p, sim_k, sim_v, score, st);
     if (e == cudaSuccess) e = launch_select(ctx, s, p, score, keep_mask, kept_idx, n_kept, theta, st);
     return e;

@@ -1,4 +1,4 @@
-"""The cluster selection's exchanges: every number of passes and CTAs, and waits that give up."""
+"""Selections at the sizes where one form gives way to another: exchanges of the cluster form, waits that give up, short sequences."""
 import numpy as np
 import pytest
 import torch
@@ -71,4 +71,44 @@ def test_a_selection_whose_waits_give_up_leaves_an_empty_list_or_the_right_one()
             else:
                 assert np.all(got == -1)
         ctx.tf_clear_status()
+    ctx.close()
+
+
+@pytest.mark.parametrize("H", [1, 8, 9, 32, 64, 65])                      # 8, 16, 32 lanes a token, one or two heads a lane; too many
+@pytest.mark.parametrize("S", [1, 33, 240, 241])                          # ... too long
+@pytest.mark.parametrize("case", ["plain", "ties", "nan", "eligible", "threshold", "none"])
+def test_short_sequences_in_one_launch_give_the_bits_of_the_two_steps(S, H, case):
+    rng = np.random.default_rng(100 * S + H)
+    B = 3
+    sim = [torch.from_numpy((rng.standard_normal((B, S, H)) * 0.1).astype(np.float32)).to(DEV) for _ in range(2)]
+    if case == "ties":
+        for s in sim:
+            s[:, 1::2] = s[:, :1]
+    if case == "nan":
+        sim[0][1, S // 2, H // 2] = float("nan")
+    kw = dict(prune_ratio=0.0 if case == "none" else 0.4, warmup_tokens=2)
+    if case == "eligible":
+        kw["eligible"] = el = torch.from_numpy((rng.random((B, S)) < 0.3).astype(np.uint8)).to(DEV)
+    if case == "threshold":
+        kw["threshold"] = tau = torch.tensor([-0.02, 0.0, 0.5], device=DEV)
+        kw["select_mode"] = tfb.TF_SELECT_THRESHOLD
+    params = tfb.default_params(**kw)
+    shape = tfb.tf_shape()
+    shape.batch, shape.seq, shape.n_q_heads, shape.n_kv_heads, shape.head_dim, shape.dtype = B, S, H, H, 128, tfb.TF_F32
+    got = []
+    ctx = tfb.Context(0)
+    for path in (1, 0):
+        ctx.tf_set_select_path(path)
+        out = [torch.full((B, S), -3.0, device=DEV), torch.full((B, S), 9, dtype=torch.uint8, device=DEV),
+               torch.full((B, S), -9, dtype=torch.int32, device=DEV), torch.full((B,), -9, dtype=torch.int32, device=DEV), torch.full((B,), -9.0, device=DEV)]
+        n0 = ctx.launches
+        ctx.tf_score_select(shape, params, sim[0], sim[1], *out)
+        assert ctx.launches - n0 == (1 if path == 0 and S <= 240 and H <= 64 else 2)
+        got.append(out)
+        alone = [torch.empty_like(o) for o in out[1:]]                       # step a4 alone on these scores
+        ctx.tf_select(shape, params, out[0], *alone)
+        for a, o in zip(alone, out[1:]):
+            assert torch.equal(a, o)
+    for a, o in zip(*got):
+        assert torch.equal(a.view(torch.int32) if a.dtype == torch.float32 else a, o.view(torch.int32) if o.dtype == torch.float32 else o)
     ctx.close()

@@ -226,7 +226,7 @@ typedef struct {
  *          and head strides of q_new [B, n_q_heads, 128], o_stride[0], o_stride[2] those of O_new.
  *   pos:   device int32 [B], 0 <= pos[b] < seq, the cache row that already holds the current token.
  *   score (may be NULL) fp32 [B]; skip u8 [B] (required): 1 = attention skipped, O_new row is zero.
- * Two or three launches on the stream (ungrouped heads: one, then one or two per 512 sequences); the state is advanced in
+ * Two or three launches on the stream (long steps of ungrouped heads: one, then one or two per 512 sequences); the state is advanced in
  * place.  If a workspace is bound (tf_set_workspace; any size tf_workspace_bytes returns for a prefill of this shape is enough),
  * bf16 calls with 1, 2, 4 or 8 query heads per KV head split the visible keys over several CTAs and keep partial results at its
  * end; without one only the few keys and heads whose splits form a thread-block cluster are split. */

@@ -86,6 +86,29 @@ __device__ __forceinline__ void st_async16(uint32_t remote, uint4 v, uint32_t re
                  :: "r"(remote), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(remote_bar) : "memory");
 }
 
+// The bounded wait for such stores: what other CTAs of the cluster stored may be read after it, which takes an acquire at cluster
+// scope (the waits above acquire at CTA scope).
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long budget_cycles,
+                                                  DevStatus* status, unsigned long long where) {
+    if (mbar_try_wait_cluster(bar, parity)) return true;
+    const long long t0 = clock64();
+    while (!mbar_try_wait_cluster(bar, parity)) {
+        if (*abort_flag) return false;
+        if (clock64() - t0 > budget_cycles) {
+            *abort_flag = 1;
+            report_error(status, TF_ERR_TIMEOUT, where);
+            return false;
+        }
+    }
+    return true;
+}
+
 // ---- 8-byte tagged packets {value, tag} in global memory: how one CTA hands a number to another --------------------
 __device__ __forceinline__ uint2 ld_packet2(const uint2* p) {
     uint2 r;

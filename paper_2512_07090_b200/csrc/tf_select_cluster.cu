@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kCsThreads, 1) select_cluster_kernel(const Clu
         if (q < n_ranks)
             st_async16(cluster_addr(smem_u32(row + 4 * k), q), *reinterpret_cast<const uint4*>(src + 4 * k), cluster_addr(bars + 8 * bar, q));
     };
-    auto heard = [&](int bar) { mbar_wait_bounded(bars + 8 * bar, 0, abort_flag, p.wait_cycles, p.status, 700 + bar); };
+    auto heard = [&](int bar) { mbar_wait_cluster(bars + 8 * bar, 0, abort_flag, p.wait_cycles, p.status, 700 + bar); };
     grid_dependency_wait();
     grid_launch_dependents();   // few CTAs: the attention grid may take the other SMs and set up meanwhile (see select_kernel)
     const int t_base = rank * (KPT * kCsThreads);

@@ -96,11 +96,19 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
 }
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long budget_cycles,
                                                   DevStatus* status, unsigned long long where) {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (!mbar_try_wait_cluster(bar, parity)) {
+    long long t0 = 0;
+    if (budget_cycles > 0) {
+        if (mbar_try_wait_cluster(bar, parity)) return true;
+        t0 = clock64();
+    } else {         // a look, without waiting: what is not there yet counts as missing
+        uint32_t ok;
+        asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return true;
+    }
+    while (budget_cycles <= 0 || !mbar_try_wait_cluster(bar, parity)) {
         if (*abort_flag) return false;
-        if (clock64() - t0 > budget_cycles) {
+        if (budget_cycles <= 0 || clock64() - t0 > budget_cycles) {
             *abort_flag = 1;
             report_error(status, TF_ERR_TIMEOUT, where);
             return false;

@@ -392,6 +392,7 @@ __global__ void __launch_bounds__(kCsThreads, 1) select_cluster_kernel(const Clu
     if (__syncthreads_or(*abort_flag)) {         // a wait gave up: everybody is told
         if (tid < n_ranks) *cluster.map_shared_rank(&s_abort, tid) = 1;
         __threadfence();
+        __syncwarp();
     }
     // nobody leaves before everybody has come this far: nothing is stored into another CTA after it (relaxed: there is nothing else to order)
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
@@ -422,13 +423,16 @@ __global__ void __launch_bounds__(kCsThreads, 1) select_cluster_kernel(const Clu
         }
     }
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-    if (*abort_flag) {           // in all CTAs or none: no list is better than one with holes, which the attention would follow
+    if (*abort_flag) {           // in all CTAs or none: nothing kept is better than a list with holes, which the attention would follow
         cluster.sync();
         for (int i = 0; i < KPT; ++i) {
             const int t = t_base + i * kCsThreads + tid;
-            if (t < S) p.kept_idx[(size_t)b * S + t] = -1;
+            if (t < S) { p.kept_idx[(size_t)b * S + t] = -1; p.keep_mask[(size_t)b * S + t] = 0; }
         }
-        if (rank == 0 && tid == 0) p.n_kept[b] = 0;
+        if (rank == 0 && tid == 0) {
+            p.n_kept[b] = 0;
+            if (p.theta) p.theta[b] = CUDART_INF_F;
+        }
         const long long t0 = clock64();          // stores still under way land before the shared memory goes away
         while (clock64() - t0 < 2000000ll) { }
     }

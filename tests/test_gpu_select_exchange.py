@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-def _select(ctx, score, ratio):
+def _select(ctx, score, ratio, theta=None):
     B, S = score.shape
     shape = tfb.tf_shape()
     shape.batch, shape.seq, shape.n_q_heads, shape.n_kv_heads, shape.head_dim, shape.dtype = B, S, 32, 32, 128, tfb.TF_BF16
@@ -17,7 +17,7 @@ def _select(ctx, score, ratio):
     keep = torch.full((B, S), 7, dtype=torch.uint8, device=DEV)
     idx = torch.full((B, S), -7, dtype=torch.int32, device=DEV)
     nk = torch.full((B,), -7, dtype=torch.int32, device=DEV)
-    ctx.tf_select(shape, params, score, keep, idx, nk)
+    ctx.tf_select(shape, params, score, keep, idx, nk, theta)
     return keep, idx, nk
 
 
@@ -52,25 +52,30 @@ def test_cluster_selection_passes(S, kind):
     ctx.close()
 
 
-def test_a_selection_whose_waits_give_up_leaves_an_empty_list_or_the_right_one():
-    """A wait of no cycles may give up: the status says so, and the attention would find no list rather than one with holes."""
+def test_a_selection_whose_waits_give_up_keeps_nothing_or_the_right_tokens():
+    """On a limit of no cycles an exchange that is not there at the first look counts as missing: the status says so, and all outputs
+    of that sequence say that nothing is kept, so that neither the list nor the mask leads on to numbers that were never exchanged."""
     score = (np.random.default_rng(3).standard_normal((8, 20000)) * 0.05).astype(np.float32)
     dev = torch.from_numpy(score).to(DEV)
     want = [_expect(s, 0.5) for s in score]
     ctx = tfb.Context(0)
     ctx.tf_set_select_path(2)
+    codes = []
     for limit in (0, 0, 0, -1):
         ctx.tf_set_wait_limits(wait_cycles=limit)
-        keep, idx, nk = _select(ctx, dev, 0.5)
-        code = ctx.tf_get_status()[0]
-        assert code == tfb.TF_OK or (limit == 0 and code == tfb.TF_ERR_TIMEOUT)
+        theta = torch.full((8,), 7.0, device=DEV)
+        keep, idx, nk = _select(ctx, dev, 0.5, theta)
+        codes.append(ctx.tf_get_status()[0])
         for b in range(8):
-            got, n = idx[b].cpu().numpy(), int(nk[b])
-            if code == tfb.TF_OK or n > 0:
+            got, n, mask = idx[b].cpu().numpy(), int(nk[b]), keep[b].cpu().numpy()
+            if codes[-1] == tfb.TF_OK or n > 0:
                 assert n == len(want[b]) and np.array_equal(got[:n], want[b]) and np.all(got[n:] == -1)
+                assert np.array_equal(np.flatnonzero(mask), want[b])
+                assert float(theta[b]) == np.delete(score[b], want[b]).min()
             else:
-                assert np.all(got == -1)
+                assert np.all(got == -1) and not mask.any() and float(theta[b]) == np.inf
         ctx.tf_clear_status()
+    assert tfb.TF_ERR_TIMEOUT in codes[:3] and set(codes[:3]) <= {tfb.TF_OK, tfb.TF_ERR_TIMEOUT} and codes[3] == tfb.TF_OK
     ctx.close()
 
 

@@ -795,9 +795,13 @@ static cudaError_t launch_stream(const DecStreamParams& sp, int grid, int device
 // (kAsCluster): they are merged through distributed shared memory, without scratch and without a third launch; otherwise the CTA
 // leaves (max, sum, unnormalised output) per head in scratch and decode_merge_splits_kernel merges the splits.
 //   The kernel starts while the decision is made: keys, values, queries and positions are not written by the decision kernel, which
-// lets this one start once all work before it is complete.  A CTA waits for the decision with its first keys in flight (kEarly), a
-// short one of a cluster only when its products are done: one stream of 420 keys 7.9 -> 6.5 us, of 2000 9.6 -> 6.7, 8 x 4096 keys
-// 30.1 -> 28.7.  Letting the kernel after this one start as early made every step slower (1 x 8192 14.7 -> 16.5).
+// lets this one start once all work before it is complete.  A CTA waits for the decision with its first keys in flight (kEarly), one
+// of a cluster with its third 128 keys in flight, or when its products are done: one stream of 420 keys 8.0 -> 5.8 us, 8 x 4096 keys
+// 30.1 -> 28.0.  What it loads for a skipped sequence is lost, so a cluster does not go further ahead (us a step, keys from HBM, waiting
+// only when the products are done / with the third / the second / the first 128 keys in flight; none skipped: 8 x 420 8.8 / 8.5 / 8.4 /
+// 9.2, 4 x 1500 11.1 / 10.4 / 10.4 / 11.5, 8 x 1000 13.3 / 12.1 / 12.1 / 13.2, 1 x 1500 x 40 ungrouped 12.2 / 11.3 / 12.7; half of them
+// skipped: 4 x 1500 11.1 / 10.3 / 10.3 / 10.9, 8 x 1000 13.2 / 12.0 / 11.9 / 12.5; all: 9.6 / 8.4 / 6.8 / 5.0, 11.6 / 8.6 / 6.9 / 4.8).
+// Letting the kernel after this one start as early made every step slower (1 x 8192 14.7 -> 16.5).
 // ---------------------------------------------------------------------------------------------------
 struct DecGqaParams {
     const __nv_bfloat16* Q; const __nv_bfloat16* K; const __nv_bfloat16* V; __nv_bfloat16* O;
@@ -816,8 +820,10 @@ template <bool kPastL1> __device__ __forceinline__ uint4 load16(const void* p) {
 }
 __device__ __forceinline__ uint32_t word_of(const uint4& r, int w) { return w == 0 ? r.x : w == 1 ? r.y : w == 2 ? r.z : r.w; }
 
-// When a CTA waits for the decision: before its first loads, with its first keys' loads in flight, or when its products are done
+// When a CTA waits for the decision: before its first loads, with its first keys' loads in flight, or as a cluster does
 enum SplitForm { kAfterDecision, kEarly, kAsCluster };
+
+constexpr int kClusterAhead = 2 * 8 * 16;        // keys a CTA of a cluster goes through before it waits: two blocks of 16 per warp
 
 template <int G, int kForm>
 __global__ void __launch_bounds__(256, kForm == kAsCluster ? 1 : 2) decode_attention_split_kernel(const DecGqaParams p) {
@@ -885,7 +891,7 @@ __global__ void __launch_bounds__(256, kForm == kAsCluster ? 1 : 2) decode_atten
 #pragma unroll
             for (int i = 0; i < 2; ++i) vr[q4][i] = (j < k_hi) ? load16<kForm != kAfterDecision>(Vb + (long long)j * p.vs.t + kDim8 * i) : zero4;
         }
-        if (kForm == kEarly && !decided) {
+        if (!decided && (kForm == kEarly || (kForm == kAsCluster && kb >= k_lo + kClusterAhead))) {
             decision();
             if (skipped) break;
         }

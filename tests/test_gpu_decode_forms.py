@@ -13,6 +13,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("workspace", [True, False])
 @pytest.mark.parametrize("B,S,Hkv,G,window", [
     (8, 420, 8, 4, 0), (4, 777, 8, 4, 0), (1, 300, 40, 1, 0), (2, 512, 8, 4, 100), (3, 129, 10, 2, 0),   # clusters of 2 to 8 splits
+    (8, 1000, 8, 4, 0), (4, 1800, 8, 2, 0), (3, 1100, 12, 1, 0),  # ... that learn of a skip with keys in flight
     (1, 2048, 4, 2, 0), (1, 2049, 4, 2, 0),                       # the longest as a cluster, the shortest through scratch
     (18, 600, 8, 4, 0), (70, 300, 8, 4, 0), (80, 300, 8, 4, 0),   # one wave, two (the attention starts early), three (it does not)
     (20, 300, 8, 8, 0),                                           # eight heads a group

@@ -344,7 +344,10 @@ __device__ __forceinline__ void ldmatrix4_trans(uint32_t addr, uint32_t (&r)[4])
 
 // Maps of K and V by the tile's length in blocks of 16 keys: the last tile of a work item is fetched as far as it is visible, not as
 // far as it could reach (128 x 401 keys x 40 heads, half of them skipped: 98.3 -> 93.5 us, 416 rows an item instead of 448).  Four
-// copies a tile either way; a box of 16 keys at a time costs one lane up to 16 small ones.
+// copies a tile either way; a box of 16 keys at a time costs one lane up to 16 small ones.  A map whose address is computed costs the
+// ring time, though, where a CTA has one long work item and nothing but the ring bounds it: whole tiles then (kBoxes false; no
+// workspace, boxes / whole tiles: 2 x 20000 keys x 40 heads 156 / 150 us, 1 x 3000 x 100 34.1 / 33.8; several items a CTA, 400 keys of 525:
+// 128 x 40 heads 164 / 183, 128 x 10 heads of 650 keys 71 / 76).
 constexpr int kStreamBoxes = kStreamKeys / 16;
 struct StreamMaps { CUtensorMap k[kStreamBoxes], v[kStreamBoxes]; };
 
@@ -365,6 +368,7 @@ struct StreamSeg {
     unsigned int piece;               // ... and that piece
 };
 
+template <bool kBoxes>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ StreamMaps maps) {
     extern __shared__ uint8_t stream_raw[];
@@ -494,7 +498,7 @@ decode_attention_stream_kernel(const DecStreamParams p, const __grid_constant__ 
         const uint32_t dst = sbase + st * kStreamStage, bar = bar_full + 8 * st;
         const int key = pk_lo + (pt.j + p_done) * kStreamKeys;
         const bool with_q = p_done < 2;                    // either half of the consumers finds the query rows with its first tile
-        const int box = min((p_vis - p_done * kStreamKeys + 15) / 16, kStreamBoxes) - 1;
+        const int box = kBoxes ? min((p_vis - p_done * kStreamKeys + 15) / 16, kStreamBoxes) - 1 : kStreamBoxes - 1;
         const CUtensorMap *mk = &maps.k[box], *mv = &maps.v[box];
         mbar_expect_tx(bar, (box + 1) * (4 * 16 * 128) + (with_q ? kStreamQ : 0));
         tma_load_4d(dst, mk, bar, 0, pt.kh, key, pt.b);
@@ -774,11 +778,14 @@ static cudaError_t launch_stream(const DecStreamParams& sp, int grid, int device
     static bool attr_set_dev[kDeviceFlagSlots] = {};      // function attributes are per device
     bool& attr_set = attr_set_dev[device >= 0 && device < kDeviceFlagSlots ? device : 0];
     if (!attr_set) {
-        const cudaError_t e = cudaFuncSetAttribute(decode_attention_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStreamSmem);
+        cudaError_t e = cudaFuncSetAttribute(decode_attention_stream_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStreamSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_attention_stream_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStreamSmem);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    const cudaError_t e = launch_dependent(decode_attention_stream_kernel, dim3((unsigned)grid), dim3(kStreamThreads), kStreamSmem, st, sp, maps);
+    const bool boxes = sp.begun || (long long)sp.B * sp.Hkv > grid;      // (one whole item a CTA at most: see StreamMaps)
+    const cudaError_t e = launch_dependent(boxes ? decode_attention_stream_kernel<true> : decode_attention_stream_kernel<false>, dim3((unsigned)grid),
+                                           dim3(kStreamThreads), kStreamSmem, st, sp, maps);
     if (e != cudaSuccess || !sp.begun) return e;
     return launch_dependent(decode_combine_kernel, dim3((unsigned)(grid * (1 + kStreamDrawn))), dim3(kHeadDim), 0, st, sp);
 }

@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
     (1, 2048, 4, 2, 0), (1, 2049, 4, 2, 0),                       # the longest as a cluster, the shortest through scratch
     (18, 600, 8, 4, 0), (70, 300, 8, 4, 0), (80, 300, 8, 4, 0),   # one wave, two (the attention starts early), three (it does not)
     (20, 300, 8, 8, 0),                                           # eight heads a group
-    (6, 30000, 4, 1, 0), (300, 200, 8, 1, 0)])                    # streaming: pieces of work items, whole ones; last tiles of 1 to 64 keys
+    (6, 30000, 4, 1, 0), (300, 200, 8, 1, 0), (3, 3000, 32, 1, 0)])     # streaming: pieces of work items, whole ones, one a CTA; last tiles of 1 to 64 keys
 def test_decode_attention_forms(B, S, Hkv, G, window, workspace):
     _uneven_positions_and_skips(B, S, Hkv, G, window, workspace)
 

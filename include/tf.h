@@ -229,7 +229,8 @@ typedef struct {
  * Two or three launches on the stream (long steps of ungrouped heads: one, then one or two per 512 sequences); the state is advanced in
  * place.  If a workspace is bound (tf_set_workspace; any size tf_workspace_bytes returns for a prefill of this shape is enough),
  * bf16 calls with 1, 2, 4 or 8 query heads per KV head split the visible keys over several CTAs and keep partial results at its
- * end; without one only the few keys and heads whose splits form a thread-block cluster are split. */
+ * end; without one they are split as far as thread-block clusters go (1, 2 or 4 query heads per KV head, at most 8 splits and
+ * as many as the device runs at once), and long steps of more sequences and heads take longer than with one. */
 tf_status tf_decode_step(tf_ctx *ctx, const tf_shape *shape, const tf_filter_params *params,
                          float eta, int32_t alg1_sign, const void *q_new, const void *K_cache,
                          const void *V_cache, const int32_t *pos, const tf_decode_state *state,

@@ -1098,10 +1098,11 @@ static char* step_scratch(tf_ctx* ctx, size_t bytes) {
 // How the split kernel divides the visible keys of a (sequence, KV head), at least 256 keys each.  Through scratch: two CTAs fit an
 // SM, a wave of CTAs costs (a fixed part worth ~192 keys + its keys), and a partly filled wave costs as much as a full one; the
 // cheapest estimate.  As a cluster, of as many splits (8 at most, as short as 64 keys) as let the clusters of all groups run at
-// once: no third launch, which is worth ~400 keys of a CTA (us a step, cluster / scratch, 8 KV heads: 1 x 420 keys 6.5 / 7.5, 4 x 500
-// 6.6 / 7.7, 8 x 420 7.3 / 8.9, 4 x 1500 8.8 / 10.5, 1 x 4096 9.2 / 10.3; 8 x 2000 19.6 / 18.6, 4 x 4096 19.7 / 18.7, 1 x 8192
-// 16.9 / 14.5), up to 2048 keys: the check that a step through scratch leaves the scan's records alone makes one of 2304.  Clusters
-// that wait for one another's SMs lose: 2 x 420 keys in 6 splits 6.9, in 7 9.9.
+// once: no third launch, which is worth ~400 keys of a CTA (us a step, keys from HBM, cluster / scratch, 8 KV heads x 4: 1 x 2048 keys
+// 8.3 / 10.1, 1 x 4096 11.0 / 11.3, 4 x 1500 10.4 / 13.6, 4 x 2500 13.5 / 15.2, 8 x 1400 14.9 / 14.9, 8 x 1700 16.6 / 16.9; the difference of
+// keys above 400: 4 x 4096 20.5 / 18.5, 1 x 8192 19.3 / 15.4).  Clusters that wait for one another's SMs lose: 2 x 420 keys in 6 splits 6.9, in
+// 7 9.9.  Without room for partial results a cluster is always the better one: 1 x 8192 19.4, as 8 whole items 88.9; 1 x 4000 x 40 ungrouped
+// 24.4 / 49.3.
 struct SplitPlan { int n; bool cluster; };
 static size_t split_bytes(const tf_shape& s) { return (size_t)s.batch * s.n_q_heads * kPartialFloats * sizeof(float); }     // of one split
 static SplitPlan split_plan(const tf_ctx* ctx, const tf_shape& s, int G, int max_keys, int sms) {
@@ -1113,7 +1114,7 @@ static SplitPlan split_plan(const tf_ctx* ctx, const tf_shape& s, int G, int max
         const long long waves = (groups * n + slots - 1) / slots, keys = (max_keys + n - 1) / n, cost = waves * (192 + keys);
         if (best < 0 || cost < best) { best = cost; plan.n = n; keys_at_once = waves * keys; }
     }
-    int n = G <= 4 && max_keys <= 2048 ? (int)std::min<long long>(std::min(8, max_keys / 64), sms / groups) : 1;
+    int n = G <= 4 ? (int)std::min<long long>(std::min(8, max_keys / 64), sms / groups) : 1;
     while (n > 1 && groups > max_clusters(ctx->device, G, n)) --n;
     if (n > 1 && (max_keys + n - 1) / n <= keys_at_once + (plan.n > 1 ? 400 : 0)) plan = {n, true};
     return plan;
@@ -1131,8 +1132,8 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
     dp.eta = a.eta; dp.target = p.prune_ratio; dp.alg1_sign = a.alg1_sign;
     dp.sum_k = a.state->sum_k; dp.sum_v = a.state->sum_v; dp.count = reinterpret_cast<long long*>(a.state->count);
     dp.sums16 = ((reinterpret_cast<uintptr_t>(dp.sum_k) | reinterpret_cast<uintptr_t>(dp.sum_v)) & 15u) == 0;
-    // bf16 with 1, 2, 4 or 8 query heads per KV head and 16-byte aligned query rows: the streaming kernel for ungrouped heads
-    // (more than half a tile per SM), the split kernel otherwise (both sides' times stand at the split kernel) ...
+    // bf16 with 1, 2, 4 or 8 query heads per KV head and 16-byte aligned query rows: the streaming kernel for ungrouped heads, the split
+    // kernel otherwise (both sides' times stand at the split kernel) ...
     const int G = s.n_q_heads / s.n_kv_heads;
     const int sms = sm_count();
     const int max_keys = s.window > 0 ? std::min(s.window, s.seq) : s.seq;     // pos is device data: size for the worst case
@@ -1154,22 +1155,27 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
     // full caches, streaming / split: 1 x 1000 x 40 heads 14.4 / 8.0, 16 x 128 x 32 17.5 / 12.8, 40 x 128 x 32 (17 tiles) 27.5 / 27.6,
     // 24 x 250 x 32 (21, three waves) 27.5 / 27.8, 12 x 600 x 32 (26, one and a third) 29.6 / 33.2, 16 x 400 x 32 (24) 28.0 / 25.9,
     // 16 x 600 x 32 (35) 35.1 / 32.4, 1 x 8000 x 40 (34) 35.4 / 33.8, 2 x 4000 x 40 (34) 34.0 / 34.6, 24 x 400 x 32 (36) 35.7 / 37.6; 600 x 64 x 8
-    // 69.0 / 64.3)
+    // 69.0 / 64.3).  Where work items are whole for want of room, an SM has one at most and they are longer than 4 tiles, the ring of the
+    // streaming kernel is the faster way through them, and a cluster faster than both (no workspace, streaming / whole items of the
+    // split kernel, 90 items: 192 keys 9.9 / 8.8, 384 10.6 / 11.3, 2000 22.9 / 30.0; 148 items: 10.9 / 10.1, 12.3 / 14.0, 28.8 / 37.2; 160 items:
+    // 13.4 / 10.0, 16.5 / 13.9, 44.2 / 37.7; streaming / clusters: 74 items of 4000 37.6 / 32.4, 40 of 16384 130 / 66, 8 of 30000 222 / 44).
     const long long items = (long long)s.batch * s.n_kv_heads;
     const SplitPlan plan = grouped ? split_plan(ctx, s, G, max_keys, sms) : SplitPlan{1, false};
     const long long split_ctas = items * plan.n, waves = (split_ctas + 2 * sms - 1) / (2 * sms);
     const bool filled = waves <= 2 && 5 * split_ctas >= 4 * waves * 2 * sms;
     const bool few_short = tiles_max <= (filled ? 34ll : 18ll) * sms || (s.batch > kStreamMaxBatch && max_keys <= 2 * kStreamKeys);
-    const bool stream = grouped && G == 1 && !few_short && tiles_max < (1ll << 31) &&              // (tile numbers are 32 bits)
-                        ((s.o_stride[0] | s.o_stride[2]) % 8) == 0 && (reinterpret_cast<uintptr_t>(a.O_new) & 15u) == 0 &&
-                        (s.batch == 1 || (s.k_stride[0] > 0 && s.v_stride[0] > 0)) && make_maps(0, std::min<int>(s.batch, kStreamMaxBatch));
-    // scratch of the streaming kernel: the table of begun work items, then slots: two per piece, and there have to be more
-    // pieces than CTAs
-    DecStreamParams sp{};
     auto stream_grid = [&](int n) { return (int)std::min<long long>(sms, (long long)n * s.n_kv_heads * ((max_keys + kStreamKeys - 1) / kStreamKeys)); };
     const int first_grid = stream_grid(std::min<int>(s.batch, kStreamMaxBatch));      // (none after it is larger)
+    // scratch of the streaming kernel: the table of begun work items, then slots: two per piece, and there have to be more
+    // pieces than CTAs
     const size_t table = stream_table_bytes(first_grid), slot = kPartialFloats * sizeof(float);
-    if (stream && ctx->workspace && ctx->workspace_bytes >= table + (3 * (size_t)first_grid + 2) * slot) {
+    const bool pieces = ctx->workspace && ctx->workspace_bytes >= table + (3 * (size_t)first_grid + 2) * slot;
+    const bool split = plan.n == 1 && items <= sms && !pieces ? max_keys <= 4 * kStreamKeys : few_short || (plan.cluster && !pieces);
+    const bool stream = grouped && G == 1 && !split && tiles_max < (1ll << 31) &&              // (tile numbers are 32 bits)
+                        ((s.o_stride[0] | s.o_stride[2]) % 8) == 0 && (reinterpret_cast<uintptr_t>(a.O_new) & 15u) == 0 &&
+                        (s.batch == 1 || (s.k_stride[0] > 0 && s.v_stride[0] > 0)) && make_maps(0, std::min<int>(s.batch, kStreamMaxBatch));
+    DecStreamParams sp{};
+    if (stream && pieces) {
         const size_t scratch = std::min(ctx->workspace_bytes, table + kStreamScratch);
         char* at = step_scratch(ctx, scratch);
         sp.begun = reinterpret_cast<uint4*>(at) + 1;

@@ -4,6 +4,7 @@ import pytest
 import torch
 
 from paper_2512_07090_b200 import binding as tfb
+from launched import ran
 from test_gpu_parity import ATTN_TOL, DEV, _qkv, attn_rel_err, to_np
 from test_gpu_parity import test_decode_attention_uneven_positions_and_skips as _uneven_positions_and_skips
 
@@ -14,7 +15,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("B,S,Hkv,G,window", [
     (8, 420, 8, 4, 0), (4, 777, 8, 4, 0), (1, 300, 40, 1, 0), (2, 512, 8, 4, 100), (3, 129, 10, 2, 0),   # clusters of 2 to 8 splits
     (8, 1000, 8, 4, 0), (4, 1800, 8, 2, 0), (3, 1100, 12, 1, 0),  # ... that learn of a skip with keys in flight
-    (1, 2048, 4, 2, 0), (1, 2049, 4, 2, 0),                       # the longest as a cluster, the shortest through scratch
+    (1, 3800, 4, 2, 0), (1, 6000, 4, 2, 0),                       # a long one as a cluster, a short one through scratch
     (18, 600, 8, 4, 0), (70, 300, 8, 4, 0), (80, 300, 8, 4, 0),   # one wave, two (the attention starts early), three (it does not)
     (20, 300, 8, 8, 0),                                           # eight heads a group
     (6, 30000, 4, 1, 0), (300, 200, 8, 1, 0), (3, 3000, 32, 1, 0)])     # streaming: pieces of work items, whole ones, one a CTA; last tiles of 1 to 64 keys
@@ -39,6 +40,23 @@ def _exact(qn, k, v, b, n):
     Hkv = k.shape[2]
     s = torch.einsum("hgd,nhd->hgn", qn[b].double().view(Hkv, -1, 128), k[b, :n].double()) / 128 ** 0.5
     return torch.einsum("hgn,nhd->hgd", s.softmax(-1), v[b, :n].double()).reshape(-1, 128)
+
+
+@pytest.mark.parametrize("B,S,Hkv,G,kernel,ctas", [
+    (1, 8192, 8, 4, "split", 64), (4, 4096, 8, 4, "split", 128), (1, 30000, 8, 1, "split", 64), (1, 4000, 40, 1, "split", 120),   # clusters at any length
+    (20, 1000, 8, 4, "split", 160), (1, 8192, 2, 8, "split", 2),      # no room for clusters, none for eight heads a group
+    (1, 200, 100, 1, "split", 100), (4, 1000, 40, 1, "split", 160),   # whole items: short ones, several an SM
+    (1, 3000, 100, 1, "stream", 148), (1, 384, 90, 1, "stream", 148)])
+def test_steps_without_a_workspace_are_split_as_far_as_clusters_go(B, S, Hkv, G, kernel, ctas):
+    ctx, shape, params, qn, k, v, st, O, skip = _step(B, S, Hkv, G, seed=S)
+    pos = torch.full((B,), S - 1, dtype=torch.int32, device=DEV)
+    step = lambda: ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
+    step()
+    assert ctx.tf_get_status()[0] == tfb.TF_OK
+    for b in range(B):
+        assert attn_rel_err(to_np(O[b]), _exact(qn, k, v, b, S).cpu().numpy()) < ATTN_TOL[torch.bfloat16], b
+    assert ran(step, f"decode_attention_{kernel}_kernel") == ctas
+    ctx.close()
 
 
 @pytest.mark.parametrize("B,S,Hkv,G,launches", [(1, 1000, 8, 4, 2), (1, 600, 40, 1, 2), (3, 500, 6, 2, 2), (1, 4000, 40, 1, 3), (16, 500, 32, 1, 2)])

@@ -796,8 +796,9 @@ def test_replayed_decode_steps_leave_the_scan_records_of_the_shared_workspace_al
 def test_decode_and_prefill_share_the_workspace():
     """The decode step keeps its split-key partial results in the bound workspace, over the region where the
     similarity scan keeps its records; a scan after decode steps must still be right (it clears its region first),
-    and the split decode output must equal the one-CTA-per-head output computed without a workspace."""
-    B, S, Hq, Hkv = 2, 2304, 8, 2
+    and the split decode output must equal the one-CTA-per-head output computed without a workspace.  (Eight query heads per
+    KV head: with fewer the splits of so short a step merge in a thread-block cluster, with and without a workspace.)"""
+    B, S, Hq, Hkv = 2, 2304, 16, 2
     q, k, v = _qkv(B, S, Hq, Hkv, torch.bfloat16, seed=77)
     _, kn, vn = oracle_inputs(q, k, v)
     ref_k = oracle.anchor_similarity(kn)

@@ -1150,12 +1150,16 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
                     && make_bshd_map(&maps.v[x], V, s.v_stride, n, s.seq, s.n_kv_heads, 2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 64, 16 * (x + 1), CU_TENSOR_MAP_SWIZZLE_128B);
         return ok;
     };
-    // ... but not for short steps, where the streaming kernel's list and hand-overs are not paid back: up to 18 tiles of 64 keys
-    // per SM, 34 where the split kernel's CTAs fill one or two waves well; nor with one or two tiles in several launches (us a step of
-    // full caches, streaming / split: 1 x 1000 x 40 heads 14.4 / 8.0, 16 x 128 x 32 17.5 / 12.8, 40 x 128 x 32 (17 tiles) 27.5 / 27.6,
-    // 24 x 250 x 32 (21, three waves) 27.5 / 27.8, 12 x 600 x 32 (26, one and a third) 29.6 / 33.2, 16 x 400 x 32 (24) 28.0 / 25.9,
-    // 16 x 600 x 32 (35) 35.1 / 32.4, 1 x 8000 x 40 (34) 35.4 / 33.8, 2 x 4000 x 40 (34) 34.0 / 34.6, 24 x 400 x 32 (36) 35.7 / 37.6; 600 x 64 x 8
-    // 69.0 / 64.3).  Where work items are whole for want of room, an SM has one at most and they are longer than 4 tiles, the ring of the
+    // ... but not for short steps, where the streaming kernel's list and hand-overs are not paid back: up to 18 tiles of 64 keys per SM,
+    // 34 where the split kernel's CTAs fill one wave or two well, 48 where these are two of whole items; beyond it shares drawn by whoever
+    // is free outweigh them once sequences are skipped.  us a step of full caches from HBM, streaming / split, none skipped and half of them:
+    //   no full waves: 1 x 1000 x 40 heads 14.4 / 8.0; 40 x 500 x 8 (17 tiles) 23.8 / 22.4, 22.5 / 14.9; 24 x 250 x 32 (21) 27.1 / 29.7, 23.7 / 20.8;
+    //     12 x 600 x 32 (26) 32.0 / 37.1; 24 x 400 x 32 (36) 35.0 / 42.0, 28.1 / 28.8
+    //   one: 8 x 1024 x 32 (28) 30.6 / 26.4, 23.7 / 22.1; 1 x 8000 x 40 (34) 34.5 / 32.4; 7 x 1500 x 40 (45) 42.3 / 38.3, 26.4 / 29.6;
+    //     20 x 2000 x 12 (52) 47.7 / 42.7, 31.3 / 36.1
+    //   two of whole items: 16 x 600 x 32 (35) 33.7 / 31.5, 26.5 / 21.2; 16 x 850 x 32 (48) 43.1 / 41.1, 30.3 / 26.0; 15 x 1000 x 32 (52) 46.9 / 44.9,
+    //     a fifth skipped 41.0 / 43.3; 18 x 2500 x 32 (156) 120 / 116, a fifth 99.8 / 100.2
+    // Nor with one or two tiles in several launches (600 x 64 x 8 69.0 / 64.3).  Where work items are whole for want of room, an SM has one at most and they are longer than 4 tiles, the ring of the
     // streaming kernel is the faster way through them, and a cluster faster than both (no workspace, streaming / whole items of the
     // split kernel, 90 items: 192 keys 9.9 / 8.8, 384 10.6 / 11.3, 2000 22.9 / 30.0; 148 items: 10.9 / 10.1, 12.3 / 14.0, 28.8 / 37.2; 160 items:
     // 13.4 / 10.0, 16.5 / 13.9, 44.2 / 37.7; streaming / clusters: 74 items of 4000 37.6 / 32.4, 40 of 16384 130 / 66, 8 of 30000 222 / 44).
@@ -1163,7 +1167,7 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
     const SplitPlan plan = grouped ? split_plan(ctx, s, G, max_keys, sms) : SplitPlan{1, false};
     const long long split_ctas = items * plan.n, waves = (split_ctas + 2 * sms - 1) / (2 * sms);
     const bool filled = waves <= 2 && 5 * split_ctas >= 4 * waves * 2 * sms;
-    const bool few_short = tiles_max <= (filled ? 34ll : 18ll) * sms || (s.batch > kStreamMaxBatch && max_keys <= 2 * kStreamKeys);
+    const bool few_short = tiles_max <= (!filled ? 18ll : waves == 2 && plan.n == 1 ? 48ll : 34ll) * sms || (s.batch > kStreamMaxBatch && max_keys <= 2 * kStreamKeys);
     auto stream_grid = [&](int n) { return (int)std::min<long long>(sms, (long long)n * s.n_kv_heads * ((max_keys + kStreamKeys - 1) / kStreamKeys)); };
     const int first_grid = stream_grid(std::min<int>(s.batch, kStreamMaxBatch));      // (none after it is larger)
     // scratch of the streaming kernel: the table of begun work items, then slots: two per piece, and there have to be more

@@ -59,6 +59,23 @@ def test_steps_without_a_workspace_are_split_as_far_as_clusters_go(B, S, Hkv, G,
     ctx.close()
 
 
+@pytest.mark.parametrize("B,S,Hkv,kernel,ctas", [
+    (12, 250, 32, "split", 384), (24, 250, 32, "stream", 148),            # 18 tiles per SM
+    (7, 1000, 40, "split", 280), (7, 1200, 40, "stream", 148),            # 34: a full wave
+    (16, 832, 32, "split", 512), (16, 896, 32, "stream", 148)])           # 48: two of them
+def test_ungrouped_steps_either_side_of_the_streaming_kernel(B, S, Hkv, kernel, ctas):
+    ctx, shape, params, qn, k, v, st, O, skip = _step(B, S, Hkv, 1, seed=S)
+    ctx.ensure_workspace(shape, params)
+    pos = torch.full((B,), S - 1, dtype=torch.int32, device=DEV)
+    step = lambda: ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
+    step()
+    assert ctx.tf_get_status()[0] == tfb.TF_OK
+    for b in (0, B - 1):
+        assert attn_rel_err(to_np(O[b]), _exact(qn, k, v, b, S).cpu().numpy()) < ATTN_TOL[torch.bfloat16], b
+    assert ran(step, f"decode_attention_{kernel}_kernel") == ctas
+    ctx.close()
+
+
 @pytest.mark.parametrize("B,S,Hkv,G,launches", [(1, 1000, 8, 4, 2), (1, 600, 40, 1, 2), (3, 500, 6, 2, 2), (1, 4000, 40, 1, 3), (16, 500, 32, 1, 2)])
 def test_split_decode_loses_nothing_before_the_result_is_rounded(B, S, Hkv, G, launches):
     """The error against 64 bits is that of rounding the exact result to bf16 (to 2 %): clusters of every group size, ungrouped

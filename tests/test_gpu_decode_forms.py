@@ -1,32 +1,51 @@
 """Decode steps at the sizes where one form of the attention gives way to another, against fp64 softmax attention."""
-import numpy as np
 import pytest
 import torch
 
 from paper_2512_07090_b200 import binding as tfb
-from launched import ran
+from launched import launched, ran
 from test_gpu_parity import ATTN_TOL, DEV, _qkv, attn_rel_err, to_np
 from test_gpu_parity import test_decode_attention_uneven_positions_and_skips as _uneven_positions_and_skips
 
 pytestmark = pytest.mark.gpu
 
 
+def _form(call, items):
+    """How the visible keys of a work item are divided: by the kernels launched and their CTAs."""
+    names = launched(call)
+    assert "decode_decide_kernel" in names[0][0]
+    if "decode_attention_stream_kernel" in names[1][0]:
+        return "pieces" if "decode_combine_kernel" in names[-1][0] else "stream"
+    assert "decode_attention_split_kernel" in names[1][0]
+    return "scratch" if len(names) == 3 else "whole" if names[1][1] == items else "cluster"
+
+
 @pytest.mark.parametrize("workspace", [True, False])
-@pytest.mark.parametrize("B,S,Hkv,G,window", [
-    (8, 420, 8, 4, 0), (4, 777, 8, 4, 0), (1, 300, 40, 1, 0), (2, 512, 8, 4, 100), (3, 129, 10, 2, 0),   # clusters of 2 to 8 splits
-    (8, 1000, 8, 4, 0), (4, 1800, 8, 2, 0), (3, 1100, 12, 1, 0),  # ... that learn of a skip with keys in flight
-    (1, 3800, 4, 2, 0), (1, 6000, 4, 2, 0),                       # a long one as a cluster, a short one through scratch
-    (18, 600, 8, 4, 0), (70, 300, 8, 4, 0), (80, 300, 8, 4, 0),   # one wave, two (the attention starts early), three (it does not)
-    (20, 300, 8, 8, 0),                                           # eight heads a group
-    (6, 30000, 4, 1, 0), (300, 200, 8, 1, 0), (3, 3000, 32, 1, 0)])     # streaming: pieces of work items, whole ones, one a CTA; last tiles of 1 to 64 keys
-def test_decode_attention_forms(B, S, Hkv, G, window, workspace):
+@pytest.mark.parametrize("B,S,Hkv,G,window,forms", [      # with a workspace, without
+    (8, 420, 8, 4, 0, "cluster cluster"), (4, 777, 8, 4, 0, "cluster cluster"), (1, 300, 40, 1, 0, "cluster cluster"), (3, 129, 10, 2, 0, "cluster cluster"),
+    (2, 512, 8, 4, 100, "whole whole"),                                                      # a window too short to be split
+    (8, 1000, 8, 4, 0, "cluster cluster"), (4, 1800, 8, 2, 0, "cluster cluster"), (3, 1100, 12, 1, 0, "cluster cluster"),   # they learn of a skip with keys in flight
+    (1, 3800, 4, 2, 0, "cluster cluster"), (1, 6000, 4, 2, 0, "scratch cluster"),            # a long one as a cluster, a short one through scratch
+    (18, 600, 8, 4, 0, "scratch whole"), (70, 300, 8, 4, 0, "whole whole"), (80, 300, 8, 4, 0, "whole whole"),   # one wave, two (the attention starts early), three (it does not)
+    (20, 300, 8, 8, 0, "whole whole"),                                                       # eight heads a group
+    (6, 30000, 4, 1, 0, "pieces cluster"), (300, 200, 8, 1, 0, "pieces stream"),             # last tiles of 1 to 64 keys
+    (3, 3000, 32, 1, 0, "scratch stream"), (7, 1200, 40, 1, 0, "pieces stream")])
+def test_decode_attention_forms(B, S, Hkv, G, window, forms, workspace):
+    ctx, shape, params, qn, k, v, st, O, skip = _step(B, S, Hkv, G, seed=S, window=window)
+    if workspace:
+        ctx.ensure_workspace(shape, params)
+    pos = torch.zeros(B, dtype=torch.int32, device=DEV)
+    step = lambda: ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
+    step()
+    assert _form(step, B * Hkv) == forms.split()[0 if workspace else 1]
+    ctx.close()
     _uneven_positions_and_skips(B, S, Hkv, G, window, workspace)
 
 
-def _step(B, S, Hkv, G, seed):
+def _step(B, S, Hkv, G, seed, window=0):
     q, k, v = _qkv(B, S, Hkv * G, Hkv, torch.bfloat16, seed=seed)
     qn = q[:, -1].contiguous()
-    shape = tfb.make_shape(None, k, v, n_q_heads=Hkv * G)
+    shape = tfb.make_shape(None, k, v, window=window, n_q_heads=Hkv * G)
     shape.q_stride[:] = [qn.stride(0), 0, qn.stride(1)]
     shape.o_stride[:] = list(shape.q_stride)
     params = tfb.default_params(prune_ratio=0.5, warmup_tokens=0)
@@ -92,42 +111,4 @@ def test_split_decode_loses_nothing_before_the_result_is_rounded(B, S, Hkv, G, l
         err += float((O[b].double() - ref).square().sum())
         rounding += float((ref.bfloat16().double() - ref).square().sum())
     assert err < 1.02 ** 2 * rounding, (err ** 0.5, rounding ** 0.5)
-    ctx.close()
-
-
-@pytest.mark.parametrize("fill", [0x00, 0xff])
-def test_long_streaming_step_whose_waits_run_out_leaves_a_usable_context(fill):
-    """As for a shorter one in test_gpu_parity.py, at a size that the streaming kernel takes."""
-    B, S, Hkv = 3, 30000, 8
-    ctx, shape, params, qn, k, v, st, O, skip = _step(B, S, Hkv, 1, seed=5)
-    ctx.set_workspace(torch.full((ctx.workspace_bytes(shape, params),), fill, dtype=torch.uint8, device=DEV))
-    pos = torch.tensor([S - 1, 1700, 63], dtype=torch.int32, device=DEV)
-    ctx.tf_set_wait_limits(wait_cycles=0)
-    ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
-    assert ctx.tf_get_status()[0] in (tfb.TF_OK, tfb.TF_ERR_TIMEOUT)
-    ctx.tf_set_wait_limits()
-    ctx.tf_clear_status()
-    for _ in range(2):
-        O.fill_(float("nan"))
-        ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
-        assert ctx.tf_get_status()[0] == tfb.TF_OK
-        for b in range(B):
-            assert attn_rel_err(to_np(O[b]), _exact(qn, k, v, b, int(pos[b]) + 1).cpu().numpy()) < ATTN_TOL[torch.bfloat16], b
-    ctx.close()
-
-
-def test_long_streaming_steps_in_which_every_sequence_is_skipped():
-    """As for a shorter one in test_gpu_parity.py: tiles fetched in vain, then a right step."""
-    B, S, Hkv = 6, 30000, 4
-    ctx, shape, params, qn, k, v, st, O, skip = _step(B, S, Hkv, 1, seed=7)
-    ctx.ensure_workspace(shape, params)
-    pos = torch.full((B,), S - 1, dtype=torch.int32, device=DEV)
-    for tau in (-9.0, 9.0, -9.0):
-        st.tau.fill_(tau)
-        O.fill_(float("nan"))
-        ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
-        assert ctx.tf_get_status()[0] == tfb.TF_OK
-        for b in range(B):
-            ref = np.zeros((Hkv, 128)) if tau < 0 else _exact(qn, k, v, b, S).cpu().numpy()
-            assert np.all(to_np(O[b]) == 0) if tau < 0 else attn_rel_err(to_np(O[b]), ref) < ATTN_TOL[torch.bfloat16], b
     ctx.close()

@@ -9,6 +9,7 @@ import torch
 
 import oracle
 from paper_2512_07090_b200 import binding as tfb, workloads as W
+from launched import launched, ran
 from parity import ATTN_TOL, SCORE_ATOL, Gpu, attn_rel_err, mask_disagreements, oracle_inputs, to_np
 
 pytestmark = pytest.mark.gpu
@@ -754,8 +755,10 @@ def test_layer_step_takes_a_workspace_of_just_what_it_uses(visibility):
     g.close()
 
 
-@pytest.mark.parametrize("B,S,Hq,Hkv", [(2, 3000, 12, 12), (4, 2048, 32, 8)])     # streaming kernel / splits merged through scratch
-def test_replayed_decode_steps_leave_the_scan_records_of_the_shared_workspace_alone(B, S, Hq, Hkv):
+@pytest.mark.parametrize("B,S,Hq,Hkv,second,third", [(4, 4096, 40, 40, "stream", "combine"),             # a work list and pieces of items in the workspace
+                                                     (4, 4096, 32, 8, "attention_split", "merge_splits"),   # splits merged through it
+                                                     (4, 2048, 32, 8, "attention_split", None)])            # ... as clusters: none of it
+def test_replayed_decode_steps_leave_the_scan_records_of_the_shared_workspace_alone(B, S, Hq, Hkv, second, third):
     """Layer steps and decode steps on one workspace, each captured once and replayed in turn, and launched directly in
     between: the host does not see a replay, so neither may rely on it to be told of the other's use of the workspace."""
     q, k, v = _qkv(B, S, Hq, Hkv, torch.bfloat16, seed=B)
@@ -773,6 +776,8 @@ def test_replayed_decode_steps_leave_the_scan_records_of_the_shared_workspace_al
     layer()
     step()
     g.status_ok()
+    names = [name for name, _ in launched(step)]
+    assert len(names) == (3 if third else 2) and second in names[1] and (not third or third in names[2]), names
     ref, ref_score, ref_step = g.O.clone(), g.score.clone(), O.clone()
     graphs = []
     for call in (layer, step):
@@ -961,8 +966,8 @@ def test_requested_kernel_that_cannot_take_the_call_is_an_error_not_a_fallback()
 @pytest.mark.parametrize("B,S,Hkv,G,window", [(1, 64, 1, 1, 0), (1, 65, 3, 2, 0), (5, 1500, 3, 4, 0), (4, 2000, 2, 8, 700),
                                               (1, 9000, 1, 4, 0), (40, 300, 5, 1, 130), (1030, 70, 1, 1, 0),
                                               (2, 9000, 3, 1, 0), (150, 130, 8, 1, 0), (1, 200, 4, 8, 0),
-                                              (7, 256, 40, 1, 0), (7, 257, 40, 1, 0), (8, 256, 40, 1, 0),      # either side of the streaming kernel
-                                              (1030, 129, 1, 1, 0), (1, 256, 4, 1, 0), (3, 700, 4, 4, 0), (2, 700, 8, 4, 0)])   # ... in three launches; ungrouped heads as a cluster; either side of the clusters
+                                              (7, 256, 40, 1, 0), (7, 257, 40, 1, 0), (8, 256, 40, 1, 0),      # either side of a second wave
+                                              (1030, 129, 1, 1, 0), (1, 256, 4, 1, 0), (3, 700, 4, 4, 0), (2, 700, 8, 4, 0)])   # streaming, in three launches; clusters
 def test_decode_attention_uneven_positions_and_skips(B, S, Hkv, G, window, workspace):
     """Every sequence at a position of its own (tile edges among them), some skipped, NaN in the cache behind each position:
     the streaming kernel (ungrouped heads: split and whole work items) and the split kernel (as a cluster, through scratch,
@@ -1012,7 +1017,7 @@ def test_decode_attention_uneven_positions_and_skips(B, S, Hkv, G, window, works
 def test_decode_step_whose_waits_run_out_leaves_a_usable_context(fill):
     """A streaming step that may not wait gives up (bounded waits, no fault) before it has described the work items it was to
     merge; what the workspace held before is not taken for such descriptions, and the next step is right."""
-    B, S, Hkv = 3, 3000, 5
+    B, S, Hkv = 3, 30000, 8
     q, k, v = _qkv(B, S, Hkv, Hkv, torch.bfloat16, seed=5)
     params = tfb.default_params(prune_ratio=0.5, warmup_tokens=0)
     guard = torch.full((B + 2, Hkv, 128), 7.0, dtype=torch.bfloat16, device=DEV)      # the output, between rows that must stay
@@ -1033,8 +1038,10 @@ def test_decode_step_whose_waits_run_out_leaves_a_usable_context(fill):
     assert ctx.tf_get_status()[0] in (tfb.TF_OK, tfb.TF_ERR_TIMEOUT)
     ctx.tf_set_wait_limits()
     ctx.tf_clear_status()
+    step = lambda: ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
+    assert ran(step, "decode_attention_stream_kernel") and ran(step, "decode_combine_kernel")
     for _ in range(2):
-        ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip)
+        step()
         assert ctx.tf_get_status()[0] == tfb.TF_OK
         for b in range(B):
             kk, vv = k[b, :int(pos[b]) + 1].double(), v[b, :int(pos[b]) + 1].double()
@@ -1229,7 +1236,7 @@ def test_decode_decision_and_state_for_every_number_of_heads(dtype, Hkv, offset)
     ctx.close()
 
 
-@pytest.mark.parametrize("B,S,Hkv", [(6, 3000, 4), (150, 500, 8)])       # split / whole work items otherwise
+@pytest.mark.parametrize("B,S,Hkv", [(6, 30000, 4), (150, 500, 8)])      # split / whole work items otherwise
 def test_streaming_decode_when_every_sequence_is_skipped(B, S, Hkv):
     """The tiles fetched before the decisions were known are thrown away and there is no work: zero rows, and a right next step."""
     _, k, v = _qkv(B, S, Hkv, Hkv, torch.bfloat16, seed=S)
@@ -1251,6 +1258,7 @@ def test_streaming_decode_when_every_sequence_is_skipped(B, S, Hkv):
         assert torch.all(skip == (1 if tau < 0 else 0))
         if tau < 0:
             assert torch.all(O == 0)
+            assert ran(lambda: ctx.tf_decode_step(shape, params, 0.0, qn, k, v, pos, st, O, None, skip), "decode_attention_stream_kernel")
             continue
         p = (torch.einsum("bhd,bnhd->bhn", qn.double(), k.double()) / 128 ** 0.5).softmax(-1)
         assert attn_rel_err(to_np(O), torch.einsum("bhn,bnhd->bhd", p, v.double()).cpu().numpy()) < ATTN_TOL[torch.bfloat16]

@@ -79,8 +79,8 @@ def test_a_selection_whose_waits_give_up_keeps_nothing_or_the_right_tokens():
     ctx.close()
 
 
-@pytest.mark.parametrize("H", [1, 8, 9, 32, 64, 65])                      # 8, 16, 32 lanes a token, one or two heads a lane; too many
-@pytest.mark.parametrize("S", [1, 33, 240, 241])                          # ... too long
+@pytest.mark.parametrize("S,H", [(1, 1), (33, 8), (33, 9), (240, 32), (240, 64),       # 8, 16, 32 lanes a token, one or two heads a lane
+                                 (240, 65), (241, 8), (241, 32)])                    # too many heads; too long
 @pytest.mark.parametrize("case", ["plain", "ties", "nan", "eligible", "threshold", "none"])
 def test_short_sequences_in_one_launch_give_the_bits_of_the_two_steps(S, H, case):
     rng = np.random.default_rng(100 * S + H)

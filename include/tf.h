@@ -283,8 +283,8 @@ tf_status tf_last_kernels(tf_ctx *ctx, int32_t kernels[2]);
 tf_status tf_set_attention_path(tf_ctx *ctx, int use_tensor_cores);
 
 /* Which kernel steps a3 / a4 use (tf_select, tf_score_select, tf_layer_filter): 0 = choose (default: a cluster of
- * CTAs per sequence for 1025 to 32768 tokens, one CTA per sequence otherwise), 1 = one CTA per sequence (step a3 as
- * a launch of its own), 2 = a cluster per sequence; a call whose sequence length it cannot take (up to 1024 or more
+ * CTAs per sequence for 1025 to 32768 tokens, one CTA per sequence otherwise, which up to 240 tokens counts ranks and, with up
+ * to 64 KV heads, makes the scores too), 1 = one CTA per sequence with radix passes (step a3 as a launch of its own), 2 = a cluster per sequence; a call whose sequence length it cannot take (up to 1024 or more
  * than 32768 tokens) then fails with TF_ERR_UNSUPPORTED.  Same results either way.  For A/B checks. */
 tf_status tf_set_select_path(tf_ctx *ctx, int path);
 

@@ -88,8 +88,8 @@ __device__ __forceinline__ void work_item(const TcParams& p, unsigned int item, 
 }
 
 // The key that the first K/V tile of an item starts at, k_first being the first that any of its rows sees.  Under a window tiles
-// start there, not at a multiple of their length: a window of 4096 and rows that span 127 positions then take 33 or 34 tiles instead of
-// always 34, one of them cut by the window's start instead of two (per pass: 8 x 16384 grouped 3917 -> 3862 us, 1 x 20000 x 32 heads 3 %
+// start there, not at a multiple of their length: a window of 4096 and rows up to 128 positions apart then take 33 tiles instead of 33 or
+// 34, one of them cut by the window's start instead of two (per pass: 8 x 16384 grouped 3917 -> 3862 us, 1 x 20000 x 32 heads 3 %
 // with the masks).  Compacted keys are only defined up to a multiple of the tile.
 __device__ __forceinline__ int first_tile_key(const TcParams& p, int k_first) {
     return p.window <= 0 ? 0 : p.compact ? k_first / kTileN * kTileN : k_first;

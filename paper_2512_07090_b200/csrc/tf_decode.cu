@@ -284,7 +284,8 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_attention_kernel(const 
 //           states in shared memory and go on with the next segment at once; these warps merge the eight states and write the result.
 // Every wait is bounded, those of the warps for one another too (mbarriers, no named barriers): on expiry the CTA records
 // TF_ERR_TIMEOUT, stops waiting, lets copies in flight land and exits.
-//   A step of 128 sequences x 400 keys x 40 heads (half of them skipped): 112 -> 94 us, 4 x 4096 keys x 40 heads: 75.5 -> 60 us.
+//   Against the split kernel: 128 sequences x 400 keys x 40 heads (half of them skipped) 112 -> 96 us, 4 x 4096 keys x 40
+// heads 75.5 -> 59 us.
 // ---------------------------------------------------------------------------------------------------
 constexpr int kPartialFloats = kHeadDim + 2;
 constexpr int kStreamKeys = 64;                            // keys per tile
@@ -343,7 +344,7 @@ __device__ __forceinline__ void ldmatrix4_trans(uint32_t addr, uint32_t (&r)[4])
 }
 
 // Maps of K and V by the tile's length in blocks of 16 keys: the last tile of a work item is fetched as far as it is visible, not as
-// far as it could reach (128 x 401 keys x 40 heads, half of them skipped: 98.3 -> 93.5 us, 416 rows an item instead of 448).  Four
+// far as it could reach (401 of 525 keys, 128 sequences x 40 heads, half of them skipped: 96.0 -> 91.0 us, none 171 -> 161; 416 rows an item instead of 448).  Four
 // copies a tile either way; a box of 16 keys at a time costs one lane up to 16 small ones.  A map whose address is computed costs the
 // ring time, though, where a CTA has one long work item and nothing but the ring bounds it: whole tiles then (kBoxes false; no
 // workspace, boxes / whole tiles: 2 x 20000 keys x 40 heads 156 / 150 us, 1 x 3000 x 100 34.1 / 33.8; several items a CTA, 400 keys of 525:

@@ -459,9 +459,10 @@ cudaError_t launch_form(const ClusterSelectParams& cp, int batch, int n_ranks, c
 
 }  // namespace
 
-// Sequence lengths the cluster form takes, and is chosen for: more than 1024 tokens (up to there one CTA per sequence
-// is as fast: the cluster's barriers and remote reads cost what the shorter passes save) and at most 8 CTAs x 512
-// threads x 8 scores per thread.
+// Sequence lengths the cluster form takes, and is chosen for: more than 1024 tokens and at most 8 CTAs x 512 threads x 8 scores per
+// thread.  Up to 1024 one CTA per sequence selects in the same time (us a launch, one CTA / cluster: 4 x 256 tokens 3.8 / 3.8, 4 x 512 3.9 / 4.4,
+// 4 x 768 4.1 / 4.1, 1 x 1000 4.2 / 4.1, 4 x 1024 4.4 / 4.1); with up to 8 KV heads the cluster would also save the fusion's launch (both
+// steps, two launches / cluster: 4 x 256 5.1 / 4.4, 4 x 512 5.5 / 5.1, 4 x 768 5.5 / 4.9, 4 x 1024 5.6 / 4.8), with more it does not fuse.
 bool select_cluster_usable(const tf_shape& s) { return s.seq > 1024 && s.seq <= 8 * kCsThreads * 8; }
 bool select_cluster_preferred(const tf_shape& s) { return select_cluster_usable(s); }
 bool select_cluster_fuses(const tf_shape& s) { return s.n_kv_heads <= kFuseLanes; }

@@ -1192,8 +1192,11 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
     dp.skips = reinterpret_cast<long long*>(a.state->skips);
     dp.score_out = a.score_out; dp.skip_out = a.skip_out; dp.status = ctx->dev_status;
     // The attention starts while the decisions are made where that is worth it: what it loads for skipped tokens is lost, and with
-    // many waves little is gained (128 x 1024 keys x 8 heads, half of them skipped, 54.8 instead of 51.1 us)
-    dp.early = stream || (grouped && waves <= 2) ? 1 : 0;
+    // many waves little is gained (128 x 1024 keys x 8 heads, half of them skipped, 54.8 instead of 51.1 us).  In two waves of two or
+    // four heads a group the loss outweighs it (us a step, early / after the decision, none, a fifth and half of them skipped: 22 x 1024 of 15739
+    // keys x 8 x 4 24.6 / 25.8, 23.6 / 24.6, 18.6 / 16.4; 70 x 300 23.1 / 23.6, 21.7 / 22.3, 18.5 / 16.7; a caller's launches cover most of what the early
+    // start gains, 25.8 / 26.1 and 23.7 / 23.7); ungrouped heads spill registers in the other form (16 x 850 x 32 41.1 / 50.4, 26.1 / 30.0).
+    dp.early = stream || (grouped && waves <= (G == 2 || G == 4 ? 1 : 2)) ? 1 : 0;
     const size_t smem = 2 * (size_t)s.n_kv_heads * sizeof(float);
     cudaError_t e;
     // up to 8 heads a warp has one, beyond it two (two for 8: 1 x 100 keys x 8 heads fp32 15.3 us a step)

@@ -26,7 +26,7 @@ def _form(call, items):
     (2, 512, 8, 4, 100, "whole whole"),                                                      # a window too short to be split
     (8, 1000, 8, 4, 0, "cluster cluster"), (4, 1800, 8, 2, 0, "cluster cluster"), (3, 1100, 12, 1, 0, "cluster cluster"),   # they learn of a skip with keys in flight
     (1, 3800, 4, 2, 0, "cluster cluster"), (1, 6000, 4, 2, 0, "scratch cluster"),            # a long one as a cluster, a short one through scratch
-    (18, 600, 8, 4, 0, "scratch whole"), (70, 300, 8, 4, 0, "whole whole"), (80, 300, 8, 4, 0, "whole whole"),   # one wave, two (the attention starts early), three (it does not)
+    (18, 600, 8, 4, 0, "scratch whole"), (70, 300, 8, 4, 0, "whole whole"), (80, 300, 8, 4, 0, "whole whole"),   # one wave (the attention starts early), two, three
     (20, 300, 8, 8, 0, "whole whole"),                                                       # eight heads a group
     (6, 30000, 4, 1, 0, "pieces cluster"), (300, 200, 8, 1, 0, "pieces stream"),             # last tiles of 1 to 64 keys
     (3, 3000, 32, 1, 0, "scratch stream"), (7, 1200, 40, 1, 0, "pieces stream")])

@@ -1160,6 +1160,8 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
     //     20 x 2000 x 12 (52) 47.7 / 42.7, 31.3 / 36.1
     //   two of whole items: 16 x 600 x 32 (35) 33.7 / 31.5, 26.5 / 21.2; 16 x 850 x 32 (48) 43.1 / 41.1, 30.3 / 26.0; 15 x 1000 x 32 (52) 46.9 / 44.9,
     //     a fifth skipped 41.0 / 43.3; 18 x 2500 x 32 (156) 120 / 116, a fifth 99.8 / 100.2
+    // (5 tiles where more than two waves of whole items stream without a merge launch: 19 x 47 x 32 (4) 15.0 / 15.5, a third skipped 14.1 / 13.0;
+    // 28 x 47 x 32 (6) 17.1 / 18.7, 16.0 / 16.1; 18 x 130 x 40 (15) 18.8 / 23.3, 18.2 / 18.8.)
     // Nor with one or two tiles in several launches (600 x 64 x 8 69.0 / 64.3).  Where work items are whole for want of room, an SM has one at most and they are longer than 4 tiles, the ring of the
     // streaming kernel is the faster way through them, and a cluster faster than both (no workspace, streaming / whole items of the
     // split kernel, 90 items: 192 keys 9.9 / 8.8, 384 10.6 / 11.3, 2000 22.9 / 30.0; 148 items: 10.9 / 10.1, 12.3 / 14.0, 28.8 / 37.2; 160 items:
@@ -1168,13 +1170,13 @@ cudaError_t launch_decode_step(tf_ctx* ctx, const tf_shape& s, const tf_filter_p
     const SplitPlan plan = grouped ? split_plan(ctx, s, G, max_keys, sms) : SplitPlan{1, false};
     const long long split_ctas = items * plan.n, waves = (split_ctas + 2 * sms - 1) / (2 * sms);
     const bool filled = waves <= 2 && 5 * split_ctas >= 4 * waves * 2 * sms;
-    const bool few_short = tiles_max <= (!filled ? 18ll : waves == 2 && plan.n == 1 ? 48ll : 34ll) * sms || (s.batch > kStreamMaxBatch && max_keys <= 2 * kStreamKeys);
     auto stream_grid = [&](int n) { return (int)std::min<long long>(sms, (long long)n * s.n_kv_heads * ((max_keys + kStreamKeys - 1) / kStreamKeys)); };
     const int first_grid = stream_grid(std::min<int>(s.batch, kStreamMaxBatch));      // (none after it is larger)
     // scratch of the streaming kernel: the table of begun work items, then slots: two per piece, and there have to be more
     // pieces than CTAs
     const size_t table = stream_table_bytes(first_grid), slot = kPartialFloats * sizeof(float);
     const bool pieces = ctx->workspace && ctx->workspace_bytes >= table + (3 * (size_t)first_grid + 2) * slot;
+    const bool few_short = tiles_max <= (!filled ? (waves > 2 && !pieces ? 5ll : 18ll) : waves == 2 && plan.n == 1 ? 48ll : 34ll) * sms || (s.batch > kStreamMaxBatch && max_keys <= 2 * kStreamKeys);
     const bool split = plan.n == 1 && items <= sms && !pieces ? max_keys <= 4 * kStreamKeys : few_short || (plan.cluster && !pieces);
     const bool stream = grouped && G == 1 && !split && tiles_max < (1ll << 31) &&              // (tile numbers are 32 bits)
                         ((s.o_stride[0] | s.o_stride[2]) % 8) == 0 && (reinterpret_cast<uintptr_t>(a.O_new) & 15u) == 0 &&

@@ -29,7 +29,8 @@ def _form(call, items):
     (18, 600, 8, 4, 0, "scratch whole"), (70, 300, 8, 4, 0, "whole whole"), (80, 300, 8, 4, 0, "whole whole"),   # one wave (the attention starts early), two, three
     (20, 300, 8, 8, 0, "whole whole"),                                                       # eight heads a group
     (6, 30000, 4, 1, 0, "pieces cluster"), (300, 200, 8, 1, 0, "pieces stream"),             # last tiles of 1 to 64 keys
-    (3, 3000, 32, 1, 0, "scratch stream"), (7, 1200, 40, 1, 0, "pieces stream")])
+    (3, 3000, 32, 1, 0, "scratch stream"), (7, 1200, 40, 1, 0, "pieces stream"),
+    (18, 130, 40, 1, 0, "whole stream"), (18, 130, 8, 1, 0, "whole whole")])                # three waves of short items, one
 def test_decode_attention_forms(B, S, Hkv, G, window, forms, workspace):
     ctx, shape, params, qn, k, v, st, O, skip = _step(B, S, Hkv, G, seed=S, window=window)
     if workspace:
